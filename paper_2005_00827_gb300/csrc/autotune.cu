@@ -60,15 +60,15 @@ extern "C" qpfrg_status qpfrg_autotune(qpfrg_t c, double lambda, qpfrg_tuning *o
     c->prof = false;    // tuning launches are not part of any profile
     EventPair ev;
     qpfrg_status st = QPFRG_OK;
-    const long N = c->pb.N, NN = N * N, n3 = NN * N;
+    const long N = c->pb.N, NN = N * N;
     const bool mixed = c->opt.precision != QPFRG_FP64;
     const void *Vin = c->d_V;
     double best_b = 0.0, best_s = 0.0, best_c = 0.0;
     do {
         if (mixed) {
-            if ((st = launch_convert_f32(c, c->d_V, c->d_Vf, n3)) != QPFRG_OK) break;
             Vin = c->d_Vf;
         }
+        if ((st = launch_stage_prep(c, c->d_V, c->d_Z, state_form(c).mode == 2 ? 1 : 0)) != QPFRG_OK) break;
         // loop kernels: transfers per CTA and per warp pass (4 only in FP32)
         {
             const int cand[] = {8, 16, 32, 64, 128, 256};
@@ -81,7 +81,7 @@ extern "C" qpfrg_status qpfrg_autotune(qpfrg_t c, double lambda, qpfrg_tuning *o
                     c->tune.bubble_transfers = hw;
                     const double ms = time_launch(
                         c, ev,
-                        [&] { return launch_bubbles(c, lambda, c->d_Z, c->c4v_state, nullptr, c->c4v_state); }, st);
+                        [&] { return launch_bubbles(c, lambda, c->d_Z, c->c4v_state, nullptr, state_form(c)); }, st);
                     if (ms < 0.0) break;
                     if (ms < best) {
                         best = ms;
@@ -94,7 +94,7 @@ extern "C" qpfrg_status qpfrg_autotune(qpfrg_t c, double lambda, qpfrg_tuning *o
             c->tune.bubble_transfers = pick_h;
             best_b = best;
             // leave the loop-kernel rows of the fastest shape for the contraction below
-            if ((st = launch_bubbles(c, lambda, c->d_Z, c->c4v_state, nullptr, c->c4v_state)) != QPFRG_OK) break;
+            if ((st = launch_bubbles(c, lambda, c->d_Z, c->c4v_state, nullptr, state_form(c))) != QPFRG_OK) break;
         }
         // tensor-core contraction: split-K per channel (0 = the wave-filling heuristic)
         if (c->opt.precision == QPFRG_MIXED_TC) {

@@ -45,13 +45,17 @@ struct BubbleArgs {
     int qchunk;
     // C4v-reduced launch (symmetry.cu; tasks == nullptr: every row evaluated):
     // CTA task (family, patch, first representative, count); per
-    // representative its transfer and its image rows (Q', a' | g << 16); img
-    // == nullptr with tasks: the contraction's representative rows, each
-    // written once to row kq of the compact table
+    // representative its transfer and its image rows (Q', a' | g << 16)
     const int4 *tasks;
     const int *repQ;
     const int *nimg;
     const int2 *img;
+    int ntask;
+    // representative rows of the row orbits (the form sym selects): their tasks and transfers
+    const int4 *rtasks;
+    const int *rrep;
+    int n_rtask;
+    SymMode sym;
     // batched flows: a device flag read by every CTA; 0 = nothing to do
     const int *active;
     // tensor-core path: the table in tiles (tc_table_index; tRT = 0: row-major)
@@ -311,7 +315,8 @@ __device__ __forceinline__ void table_row(const BubbleArgs<R> &A, const R *row, 
 // its image rows.  A warp carries H transfers at once (H = 2 or 4): one
 // shared-memory read of a point serves all of them.
 template <typename R, bool PP, bool TFLOW, bool TP0, int H, bool FULL>
-__device__ __forceinline__ void bubble_body(const BubbleArgs<R> &A, unsigned char *smem_raw, int a, int q0, int q1)
+__device__ __forceinline__ void bubble_body(const BubbleArgs<R> &A, unsigned char *smem_raw, int a, int q0, int q1,
+                                            const int *repQ, const int2 *img)
 {
     const int N = A.pb.N, P = A.pb.P, M = A.pb.M;
     const long NN = (long)N * N;
@@ -380,7 +385,7 @@ __device__ __forceinline__ void bubble_body(const BubbleArgs<R> &A, unsigned cha
 #pragma unroll
         for (int h = 0; h < H; ++h) {
             const int kq = h < nq ? Q0 + h * nwarp : Q0;
-            const int Q = A.repQ ? A.repQ[kq] : kq;
+            const int Q = repQ ? repQ[kq] : kq;
             cQx[h] = Qt.cx[Q];
             sQx[h] = Qt.sx[Q];
             cQy[h] = Qt.cy[Q];
@@ -520,11 +525,11 @@ __device__ __forceinline__ void bubble_body(const BubbleArgs<R> &A, unsigned cha
             // the row's image rows: (Q', a', g) of the representative, or the
             // row itself (unreduced launch: row Q; representative rows of the
             // contraction's row orbits: row kq of the compact table)
-            const int nimg = A.img ? A.nimg[kq] : 1;
+            const int nimg = img ? A.nimg[kq] : 1;
             for (int im = 0; im < nimg; ++im) {
                 int Qi = kq, ai = a, g = 0;
-                if (A.img) {
-                    const int2 e = A.img[8 * (long)kq + im];
+                if (img) {
+                    const int2 e = img[8 * (long)kq + im];
                     Qi = e.x;
                     ai = e.y & 0xffff;
                     g = e.y >> 16;
@@ -545,32 +550,44 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (H == 2 ? 3 : 2) : 1) bu
     if (A.active && *A.active == 0) return;      // uniform over the grid
     const bool tflow = A.pb.regulator == QPFRG_REG_TEMPERATURE;
     int fam, a, q0, q1;
-    if (A.tasks) {
-        const int4 t = A.tasks[blockIdx.x];
+    // the grid covers every form the launch may take; a CTA past its form's
+    // tasks returns (uniform over the CTA)
+    const int *repQ = nullptr;
+    const int2 *img = nullptr;
+    const bool compact = sym_compact(A.sym);
+    if (compact || A.tasks) {
+        if ((int)blockIdx.x >= (compact ? A.n_rtask : A.ntask)) return;
+        const int4 t = (compact ? A.rtasks : A.tasks)[blockIdx.x];
         fam = t.x;
         a = t.y;
         q0 = t.z;
         q1 = t.z + t.w;
+        repQ = compact ? A.rrep : A.repQ;
+        img = compact ? nullptr : A.img;
     } else {
-        const long NN = (long)A.pb.N * A.pb.N;
-        fam = blockIdx.z;
-        a = blockIdx.x;
-        q0 = blockIdx.y * A.qchunk;
+        const int N = A.pb.N;
+        const long NN = (long)N * N;
+        const int nch = (int)((NN + A.qchunk - 1) / A.qchunk);
+        const int id = blockIdx.x / N, ch = id % nch;
+        a = blockIdx.x - id * N;
+        fam = id / nch;
+        if (fam > 1) return;
+        q0 = ch * A.qchunk;
         q1 = (int)min((long)q0 + A.qchunk, NN);
     }
     if (fam == 0) {
-        if (tflow) bubble_body<R, true, true, TP0, H, FULL>(A, smem_raw, a, q0, q1);
-        else bubble_body<R, true, false, TP0, H, FULL>(A, smem_raw, a, q0, q1);
+        if (tflow) bubble_body<R, true, true, TP0, H, FULL>(A, smem_raw, a, q0, q1, repQ, img);
+        else bubble_body<R, true, false, TP0, H, FULL>(A, smem_raw, a, q0, q1, repQ, img);
     } else {
-        if (tflow) bubble_body<R, false, true, TP0, H, FULL>(A, smem_raw, a, q0, q1);
-        else bubble_body<R, false, false, TP0, H, FULL>(A, smem_raw, a, q0, q1);
+        if (tflow) bubble_body<R, false, true, TP0, H, FULL>(A, smem_raw, a, q0, q1, repQ, img);
+        else bubble_body<R, false, false, TP0, H, FULL>(A, smem_raw, a, q0, q1, repQ, img);
     }
 }
 
 template <typename R>
 static qpfrg_status launch_r(qpfrg_ctx *c, double lambda, const double *d_Z, const double *d_K, bool z_symmetric,
                              const FineTable<R> &fine, const TransferTable<R> &qpp, const TransferTable<R> &qph,
-                             R thr, bool compact = false)
+                             R thr, const SymMode &sym)
 {
     const Problem &pb = c->pb;
     BubbleArgs<R> A{};
@@ -609,21 +626,28 @@ static qpfrg_status launch_r(qpfrg_ctx *c, double lambda, const double *d_Z, con
     // C4v-reduced launch: one row per orbit (the Z-free loop kernels of
     // quasi-particle lines depend on Z, which must then be symmetric)
     const bool red = c->loop_red && (pb.propagator == QPFRG_PROP_PAPER || z_symmetric);
-    int ntask = 0;
-    if (compact) {
+    A.sym = sym;
+    long ctas = 0;
+    if (sym.mode != 0) {
         // representative rows of the contraction's row orbits, all patches a
-        A.qchunk = std::max(8, A.qchunk);
-        qpfrg_status st = row_tasks(c, A.qchunk, &ntask);
+        qpfrg_status st = row_tasks(c, std::max(8, A.qchunk), &A.n_rtask);
         if (st != QPFRG_OK) return st;
-        A.tasks = c->d_rtask;
-        A.repQ = c->d_rrep;
-    } else if (red) {
-        qpfrg_status st = loop_tasks(c, A.qchunk, &ntask);
-        if (st != QPFRG_OK) return st;
-        A.tasks = c->d_ltask;
-        A.repQ = c->d_lrepQ;
-        A.nimg = c->d_lnimg;
-        A.img = c->d_limg;
+        A.rtasks = c->d_rtask;
+        A.rrep = c->d_rrep;
+        ctas = A.n_rtask;
+    }
+    if (sym.mode != 1) {
+        long n = 2L * pb.N * qchunks;
+        if (red) {
+            qpfrg_status st = loop_tasks(c, A.qchunk, &A.ntask);
+            if (st != QPFRG_OK) return st;
+            A.tasks = c->d_ltask;
+            A.repQ = c->d_lrepQ;
+            A.nimg = c->d_lnimg;
+            A.img = c->d_limg;
+            n = A.ntask;
+        }
+        ctas = std::max(ctas, n);
     }
     // transfers per warp pass: 4 only in FP32 (the packed pairs of the
     // temperature flow), 2 otherwise or when tuned so
@@ -645,9 +669,8 @@ static qpfrg_status launch_r(qpfrg_ctx *c, double lambda, const double *d_Z, con
         if (H == 4) kern = pb.tp == 0.0 ? bubble_kernel<R, true, 4, false> : bubble_kernel<R, false, 4, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(c, e, "bubble smem attribute");
-    const dim3 grid = (compact || red) ? dim3(ntask) : dim3(pb.N, qchunks, 2);
     prof_begin(c);
-    kern<<<grid, nthr, smem, c->stream>>>(A);
+    kern<<<(unsigned)ctas, nthr, smem, c->stream>>>(A);
     prof_end(c, K_BUBBLE);
     e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "bubble_kernel");
@@ -663,20 +686,17 @@ constexpr double kThrF64 = 1e-5;
 constexpr float kThrF32 = 6e-3f;
 
 qpfrg_status launch_bubbles(qpfrg_ctx *c, double lambda, const double *d_Z, bool z_symmetric, const double *d_K,
-                            bool state_symmetric)
+                            const SymMode &sym)
 {
-    c->rows_compact = false;
+    c->rhs_sym = sym;
+    c->rows_compact = sym.mode == 1;
     if (c->opt.precision == QPFRG_FP64)
-        return launch_r<double>(c, lambda, d_Z, d_K, z_symmetric, c->f64, c->qpp64, c->qph64, kThrF64);
+        return launch_r<double>(c, lambda, d_Z, d_K, z_symmetric, c->f64, c->qpp64, c->qph64, kThrF64, sym);
     if (c->opt.precision == QPFRG_MIXED_TC) {
         qpfrg_status s = launch_tc_prep(c);       // B operands and V^T of this stage
         if (s != QPFRG_OK) return s;
     }
-    const bool compact = c->rows_ok && state_symmetric && c->opt.precision == QPFRG_MIXED_TC;
-    const qpfrg_status s =
-        launch_r<float>(c, lambda, d_Z, d_K, z_symmetric, c->f32, c->qpp32, c->qph32, kThrF32, compact);
-    c->rows_compact = compact && s == QPFRG_OK;
-    return s;
+    return launch_r<float>(c, lambda, d_Z, d_K, z_symmetric, c->f32, c->qpp32, c->qph32, kThrF32, sym);
 }
 
 // The loop kernel alone into an explicit buffer (batched flows): the table
@@ -687,8 +707,9 @@ qpfrg_status launch_loop_rows(qpfrg_ctx *c, double lambda, float *rows, const in
 {
     c->loop_out = rows;
     c->loop_active = active;
-    const qpfrg_status s =
-        launch_r<float>(c, lambda, c->d_ones, nullptr, true, c->f32, c->qpp32, c->qph32, kThrF32, compact && c->rows_ok);
+    SymMode sym;
+    sym.mode = compact && c->rows_ok ? 1 : 0;
+    const qpfrg_status s = launch_r<float>(c, lambda, c->d_ones, nullptr, true, c->f32, c->qpp32, c->qph32, kThrF32, sym);
     c->loop_out = nullptr;
     c->loop_active = nullptr;
     return s;

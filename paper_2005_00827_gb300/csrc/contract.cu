@@ -7,169 +7,225 @@
 //   cr (Q = k3-k2 = (l,j)):  dV[i,j,l] -= sum_k B_ph[l,j][k] V[b,j,l] * V[i,a,b]
 //   d  (Q = k1-k3 = (i,l)):  dV[i,j,l] += sum_k B_ph[i,l][k] {(2V[i,a,l] - V[a,i,l]) V[b,j,a]
 //                                                          - V[i,a,l] V[j,b,a]}
-// Each channel is a GEMM with N^2 rows r, K = N^2 (2N^2 for d) and N
-// columns n, whose A operand is a row of a bubble table times a vertex
-// factor (formed while staging into shared memory) and whose B operand is a
-// permuted view of V:
-//   pp: r = (i,j), n = l;  cr: r = (j,l), n = i;  d: r = (i,l), n = j.
-// Output: out[index(r,n)] += scale * sign * sum.
+// Each channel is a GEMM with the table's rows Q as rows, K = N^2 and N
+// columns n (n = l, i, j), whose A operand is a table row times a vertex factor
+// (formed while staging into shared memory) and whose B operand is a permuted
+// view of V; d is two such GEMMs of the same size.  FP64 and FP32 (SIMT):
+//   stage_prep_kernel   the permuted views P[k][n] of cr, d1, d2, the FP32 copy
+//                       and the C4v test of the inputs, one launch
+//   contract_kernel     the four GEMMs, one launch, into partial rows
+//   reduce_kernel       sums the partial rows
+//   expand_kernel       sums the channels into out
+// A C4v-symmetric (V, Z) tables and contracts one row per orbit of transfer
+// pairs (row orbits, symmetry.cu); the expansion permutes the columns.  Which
+// form a right-hand side takes may be decided on the device (SymMode), so that
+// the call stays asynchronous.
 #include <algorithm>
 
 #include "qpfrg_internal.h"
 
 namespace qpfrg {
 
-constexpr int BM = 64, BN = 32, BK = 16, TM = 4, TN = 2;
+constexpr int CBK = 16;      // reduction columns b per staged block
 
-template <typename R, typename VR, int CH>
-struct ChannelOps {
-    const R *B;      // bubble table family (pp or ph), [Q][a][b]
-    const VR *V;     // vertex (FP64 or FP32)
-    int N;
-    long NN;
-
-    // A operand: row r, reduction index k (k >= NN: second product of d)
-    __device__ __forceinline__ R a_elem(int r, long k) const
-    {
-        if (CH == 0) {                         // pp: r = i*N + j
-            const int a = (int)(k / N);
-            return B[(long)r * NN + k] * (R)V[(long)r * N + a];
-        } else if (CH == 1) {                  // cr: r = j*N + l, table row Q = (l, j)
-            const int j = r / N, l = r % N;
-            const int a = (int)(k / N), b = (int)(k % N);
-            (void)a;
-            return B[((long)l * N + j) * NN + k] * (R)V[((long)b * N + j) * N + l];
-        } else {                               // d: r = i*N + l
-            const int i = r / N, l = r % N;
-            const bool second = k >= NN;
-            const long kk = second ? k - NN : k;
-            const int a = (int)(kk / N);
-            const R bt = B[(long)r * NN + kk];
-            const R v_ial = (R)V[((long)i * N + a) * N + l];
-            if (!second) return bt * (R(2) * v_ial - (R)V[((long)a * N + i) * N + l]);
-            return -bt * v_ial;
-        }
-    }
-    // B operand: reduction index k, column n
-    __device__ __forceinline__ R b_elem(long k, int n) const
-    {
-        if (CH == 0) return (R)V[k * N + n];                  // V[a,b,l]
-        if (CH == 1) return (R)V[(long)n * NN + k];           // V[i,a,b]
-        const bool second = k >= NN;
-        const long kk = second ? k - NN : k;
-        const int a = (int)(kk / N), b = (int)(kk % N);
-        if (!second) return (R)V[((long)b * N + n) * N + a];  // V[b,j,a]
-        return (R)V[((long)n * N + b) * N + a];               // V[j,b,a]
-    }
-    __device__ __forceinline__ long out_index(int r, int n) const
-    {
-        if (CH == 0) return (long)r * N + n;                  // (i,j,l) = (r, n)
-        if (CH == 1) return (long)n * NN + r;                 // i = n, (j,l) = r
-        const int i = r / N, l = r % N;
-        return ((long)i * N + n) * N + l;                     // j = n
-    }
+// Rows of the table and split of the reduction over a, per form of the RHS.
+struct ContractShape {
+    int rows, mtiles, splits, a_per;
 };
 
-template <typename R, typename VR, int CH>
-__global__ void __launch_bounds__(256) contract_kernel(ChannelOps<R, VR, CH> ops, double *out,
-                                                       double scale, double sign)
-{
-    const int N = ops.N;
-    const long NN = ops.NN;
-    const long K = CH == 2 ? 2 * NN : NN;
-    const int r0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int tid = threadIdx.x;
-    const int tr = tid / (BN / TN), tn = tid % (BN / TN);   // 16 x 16 thread grid
+template <typename R>
+struct ContractArgs {
+    const R *B;                  // bubble tables [f][row][a][b], family stride N^4
+    const R *V;                  // stage vertex
+    const R *P;                  // permuted views [cr, d1, d2][a][b][n]
+    const int *rep;              // compact form: transfer pair of a row
+    double *part;                // [split][job][row][n]
+    int N, ntiles, njobs;
+    int jobs[4];                 // 0 pp, 1 cr, 2 d first product, 3 d second product
+    ContractShape sh[2];         // every row, representative rows
+    SymMode sym;
+};
 
-    __shared__ R As[BK][BM + 1];
-    __shared__ R Bs[BK][BN + 1];
-    R acc[TM][TN];
+// One CTA: rows m0 .. m0 + 16 TM - 1, columns n0 .. n0 + 16 NB - 1, one job and
+// one range of a; 256 threads as 16 x 16, TM rows x NB columns each.
+//
+// What bounds it: GB300 issues 2 FP64 FMAs per clock and SM (64 clocks per warp
+// instruction and scheduler), so in FP64 the staging, its index arithmetic and
+// the two shared reads per FMA hide behind the FMA pipe, and what counts is the
+// number of rows contracted and an even share of the SMs (the split over a).  In FP32
+// 12 FMAs per 5 shared reads keep the FMA pipe ahead of shared memory.  The
+// next block's table values and factors are loaded while the present one is
+// multiplied.  The crossed channel's factor depends on b, not on a: its blocks
+// run with b outside and a inside, so the gathered factor is read once per b.
+// np48, 16 x 16 points, symmetric vertex: FP64 6232 -> 350 us, FP32 1487 -> 28 us
+// (every row, one launch per channel -> representative rows, one launch).
+template <typename R, int TM, int NB>
+__global__ void __launch_bounds__(256) contract_kernel(const ContractArgs<R> A)
+{
+    constexpr int BM = 16 * TM, BN = 16 * NB;
+    const bool compact = sym_compact(A.sym);
+    const ContractShape sh = A.sh[compact ? 1 : 0];
+    int id = blockIdx.x;
+    const int mt = id % sh.mtiles;
+    id /= sh.mtiles;
+    const int nt = id % A.ntiles;
+    id /= A.ntiles;
+    const int ji = id % A.njobs, sp = id / A.njobs;
+    if (sp >= sh.splits) return;            // CTAs of the other form's grid
+    const int job = A.jobs[ji];
+    const int N = A.N, m0 = mt * BM, n0 = nt * BN;
+    const long NN = (long)N * N;
+    const int a0 = sp * sh.a_per, a1 = min(N, a0 + sh.a_per);
+    const int tid = threadIdx.x, tr = tid >> 4, tn = tid & 15;
+
+    __shared__ R As[2][CBK][BM + 4];
+    __shared__ R Bs[2][CBK][BN];
+
+    // staged A elements of this thread: rows (tid / 16) + 16 e, column tid % 16
+    const int kk = tid & 15;
+    const R *Brow[TM];
+    const R *frow[TM], *grow[TM];           // factor of (row, x): frow[x fstride] (and grow for d1)
+    bool rok[TM];
+    // pp: V[i,j,a]; cr: V[b,j,l]; d1: 2V[i,a,l] - V[a,i,l]; d2: -V[i,a,l]
+    const long fstride = job == 0 ? 1 : (job == 1 ? NN : N);
+#pragma unroll
+    for (int e = 0; e < TM; ++e) {
+        const int m = m0 + (tid >> 4) + 16 * e;
+        rok[e] = m < sh.rows;
+        const int mm = rok[e] ? m : 0;
+        const int Q = compact ? A.rep[mm] : mm;
+        const int q1 = Q / N, q2 = Q - q1 * N;
+        Brow[e] = A.B + (job == 0 ? 0 : NN * NN) + (long)mm * NN;
+        frow[e] = A.V + (job == 0 ? (long)Q * N : (job == 1 ? (long)q2 * N + q1 : (long)q1 * NN + q2));
+        grow[e] = A.V + (long)q1 * N + q2;   // + a N^2
+    }
+    const R *Pj = job == 0 ? A.V : A.P + (job - 1) * NN * N;
+
+    R acc[TM][NB];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = R(0);
+        for (int j = 0; j < NB; ++j) acc[i][j] = R(0);
 
-    for (long k0 = 0; k0 < K; k0 += BK) {
-        // stage A: BM x BK, 4 elements per thread
+    R an[TM], fn[TM], bn[NB];
+    auto load = [&](int a, int b0, bool newfac) {
+        const int b = b0 + kk;
+        const bool bok = b < N;
 #pragma unroll
-        for (int e = 0; e < (BM * BK) / 256; ++e) {
-            const int idx = tid + e * 256;
-            const int rr = idx / BK, kk = idx % BK;
-            const int r = r0 + rr;
-            const long k = k0 + kk;
-            As[kk][rr] = (r < NN && k < K) ? ops.a_elem(r, k) : R(0);
+        for (int e = 0; e < TM; ++e) {
+            an[e] = (rok[e] && bok) ? Brow[e][(long)a * N + b] : R(0);
+            if (newfac) {
+                const int x = job == 1 ? (bok ? b : 0) : a;
+                R f = frow[e][x * fstride];
+                if (job == 2) f = R(2) * f - grow[e][(long)a * NN];
+                else if (job == 3) f = -f;
+                fn[e] = f;
+            }
         }
-        // stage B: BK x BN, 2 elements per thread
 #pragma unroll
-        for (int e = 0; e < (BK * BN) / 256; ++e) {
-            const int idx = tid + e * 256;
-            const int kk = idx / BN, nn = idx % BN;
-            const int n = n0 + nn;
-            const long k = k0 + kk;
-            Bs[kk][nn] = (n < N && k < K) ? ops.b_elem(k, n) : R(0);
+        for (int e = 0; e < NB; ++e) {
+            const int idx = tid + 256 * e, kb = idx / BN, n = n0 + idx % BN;
+            bn[e] = (b0 + kb < N && n < N) ? Pj[((long)a * N + b0 + kb) * N + n] : R(0);
         }
-        __syncthreads();
+    };
+    const int nbc = (N + CBK - 1) / CBK, na = a1 - a0;
+    const int total = na * nbc;
+    int a = a0, b0 = 0;
+    if (total > 0) load(a, b0, true);
+    for (int t = 0; t < total; ++t) {
+        const int s = t & 1;
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            R av[TM], bv[TN];
+        for (int e = 0; e < TM; ++e) As[s][kk][(tid >> 4) + 16 * e] = an[e] * fn[e];
 #pragma unroll
-            for (int i = 0; i < TM; ++i) av[i] = As[kk][tr * TM + i];
+        for (int e = 0; e < NB; ++e) {
+            const int idx = tid + 256 * e;
+            Bs[s][idx / BN][idx % BN] = bn[e];
+        }
+        __syncthreads();     // also: every warp is past the block of two trips ago
+        bool nf;
+        if (job == 1) {      // b outside, a inside
+            nf = ++a == a1;
+            if (nf) {
+                a = a0;
+                b0 += CBK;
+            }
+        } else {
+            b0 += CBK;
+            nf = b0 >= N;
+            if (nf) {
+                b0 = 0;
+                ++a;
+            }
+        }
+        if (t + 1 < total) load(a, b0, nf);
 #pragma unroll
-            for (int j = 0; j < TN; ++j) bv[j] = Bs[kk][tn * TN + j];
+        for (int k = 0; k < CBK; ++k) {
+            R av[TM], bv[NB];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) av[i] = As[s][k][tr * TM + i];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) bv[j] = Bs[s][k][tn + 16 * j];
 #pragma unroll
             for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] += av[i] * bv[j];
+                for (int j = 0; j < NB; ++j) acc[i][j] += av[i] * bv[j];
         }
-        __syncthreads();
     }
-    const double s = scale * sign;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
-        const int r = r0 + tr * TM + i;
-        if (r >= NN) continue;
+        const int m = m0 + tr * TM + i;
+        if (m >= sh.rows) continue;
+        double *dst = A.part + (((long)sp * A.njobs + ji) * sh.rows + m) * N;
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int n = n0 + tn * TN + j;
-            if (n >= N) continue;
-            const long o = ops.out_index(r, n);
-            out[o] += s * (double)acc[i][j];
+        for (int j = 0; j < NB; ++j) {
+            const int n = n0 + tn + 16 * j;
+            if (n < N) dst[n] = (double)acc[i][j];
         }
     }
 }
 
-template <typename R, typename VR, int CH>
-static qpfrg_status launch_channel(qpfrg_ctx *c, const R *B, const VR *V, double scale, double sign,
-                                   double *out, int kid)
-{
-    ChannelOps<R, VR, CH> ops;
-    ops.B = B;
-    ops.V = V;
-    ops.N = c->pb.N;
-    ops.NN = (long)c->pb.N * c->pb.N;
-    dim3 grid(div_up(ops.NN, BM), div_up(c->pb.N, BN));
-    prof_begin(c);
-    contract_kernel<R, VR, CH><<<grid, 256, 0, c->stream>>>(ops, out, scale, sign);
-    prof_end(c, kid);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "contract_kernel");
-}
+// Channel rows outc[0 pp, 1 cr, 2 d][row][n] = the signed sums of the partial
+// rows over splits (and both products of d), in split order, so that the result
+// does not depend on the launch; then out[k1,k2,k3] = scale * (pp + cr + d): pp
+// row (k1,k2) column k3, cr row (k3,k2) column k1, d row (k1,k3) column k2.
+// Compact form: row Q = g rep at column n is the representative's at g^-1 n.
+// Two launches: an expansion that summed the splits itself read each partial
+// row once per image (np48 symmetric: 34 us against 4 + 4).
+struct ExpandArgs {
+    const double *part;
+    double *outc;
+    const int *rowmap;
+    double *out;
+    double scale;
+    int N, ns, njobs;
+    int first[3], count[3];          // jobs of a channel
+    int rows[2], splits[2];
+    SymMode sym;
+};
 
-template <typename R, typename VR>
-static qpfrg_status launch_all(qpfrg_ctx *c, const VR *V, double scale, double *out)
+__global__ void __launch_bounds__(128) reduce_kernel(const ExpandArgs A)
 {
-    const R *B = reinterpret_cast<const R *>(c->d_B);
-    const long table = (long)c->pb.N * c->pb.N * c->pb.N * c->pb.N;
-    const R *Bpp = B, *Bph = B + table;
-    const unsigned ch = c->pb.channels;
-    qpfrg_status s = QPFRG_OK;
-    if ((ch & QPFRG_CH_PP) && (s = launch_channel<R, VR, 0>(c, Bpp, V, scale, -1.0, out, K_CONTRACT_PP)))
-        return s;
-    if ((ch & QPFRG_CH_CR) && (s = launch_channel<R, VR, 1>(c, Bph, V, scale, -1.0, out, K_CONTRACT_CR)))
-        return s;
-    if ((ch & QPFRG_CH_D) && (s = launch_channel<R, VR, 2>(c, Bph, V, scale, 1.0, out, K_CONTRACT_D)))
-        return s;
-    return QPFRG_OK;
+    const int c = sym_compact(A.sym) ? 1 : 0, ch = blockIdx.y, nj = A.count[ch], ns = A.splits[c];
+    if (nj == 0) return;
+    const long stride = (long)A.rows[c] * A.N, per = stride * A.njobs;
+    const double *src = A.part + A.first[ch] * stride;
+    for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < stride; o += (long)gridDim.x * blockDim.x) {
+        double v = 0.0;
+        // 16 loads in flight (one after the other they cost 18 us at 32 partial rows)
+        for (int j = 0; j < nj; ++j)
+            for (int k0 = 0; k0 < ns; k0 += 16) {
+                double t[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) t[u] = k0 + u < ns ? __ldg(src + (k0 + u) * per + j * stride + o) : 0.0;
+                // as a tree: an FP64 add waits long for its operands
+#pragma unroll
+                for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+                    for (int u = 0; u < w; ++u) t[u] += t[u + w];
+                v += t[0];
+            }
+        A.outc[ch * stride + o] = ch < 2 ? -v : v;
+    }
 }
 
 // C4v element g on patch j (wedge part, ns shells per wedge, Na wedges)
@@ -180,6 +236,259 @@ __device__ __forceinline__ int c4v_patch(int g, int j, int ns, int Na)
     int r = (g & 4) ? off - w : w + off;      // in (-Na, 2 Na)
     r = r >= Na ? r - Na : (r < 0 ? r + Na : r);
     return r * ns + sh;
+}
+
+// Block (k2, k1).
+__global__ void expand_kernel(const ExpandArgs A)
+{
+    const bool c = sym_compact(A.sym);
+    const int N = A.N, Na = N / A.ns, k1 = blockIdx.y, k2 = blockIdx.x;
+    const long stride = (long)A.rows[c ? 1 : 0] * N;
+    double *row = A.out + ((long)k1 * N + k2) * N;
+    for (int k3 = threadIdx.x; k3 < N; k3 += blockDim.x) {
+        double v = 0.0;
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+            if (A.count[ch] == 0) continue;
+            const int Q = ch == 0 ? k1 * N + k2 : (ch == 1 ? k3 * N + k2 : k1 * N + k3);
+            const int n = ch == 0 ? k3 : (ch == 1 ? k1 : k2);
+            long o = (long)Q * N + n;
+            if (c) {
+                const int e = __ldg(A.rowmap + Q);
+                o = (long)(e & 0xffffff) * N + c4v_patch(c4v_inverse(e >> 24), n, A.ns, Na);
+            }
+            v += __ldg(A.outc + ch * stride + o);
+        }
+        row[k3] = A.scale * v;
+    }
+}
+
+// ---- stage operands ---------------------------------------------------------
+// Job blockIdx.y (all when 0 < gridDim.y; a missing output skips its job): 0
+// the C4v test of (V, Z) and the FP32 copy of V; 1, 2, 3 the permuted views
+// V[n,a,b], V[b,n,a], V[n,b,a] as [a][b][n].  One warp per row of N values.
+//
+// The C4v test reduces max|V| and the largest deviation under the two
+// generators (rotation by 90 degrees, reflection); any image differs by at most
+// three generator steps, so a deviation below a third of the tolerance
+// guarantees every image.  A non-finite value counts as asymmetric: an infinite
+// deviation against the maximum of the finite values.
+template <typename IN, typename R>
+__global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ V, const double *__restrict__ Z, int nz, int N,
+                                                         int ns, unsigned long long *sym, float *__restrict__ Vf,
+                                                         R *__restrict__ P)
+{
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int w0 = blockIdx.x * nw + (threadIdx.x >> 5), ws = gridDim.x * nw;
+    const int NN = N * N, job = blockIdx.y;
+    if (job > 0) {
+        if (!P) return;
+        R *dst = P + (long)(job - 1) * NN * N;
+        for (int r = w0; r < NN; r += ws) {
+            const int a = r / N, b = r - a * N;
+            for (int n = lane; n < N; n += 32) {
+                const long o = job == 1 ? (long)n * NN + r : (job == 2 ? ((long)b * N + n) * N + a : ((long)n * N + b) * N + a);
+                dst[(long)r * N + n] = (R)V[o];
+            }
+        }
+        return;
+    }
+    if (!sym && !Vf) return;
+    __shared__ short ir[256], is[256];       // images under the generators
+    for (int x = threadIdx.x; sym && x < N; x += blockDim.x) {
+        ir[x] = (short)c4v_apply(1, x, N, ns);
+        is[x] = (short)c4v_apply(4, x, N, ns);
+    }
+    __syncthreads();
+    double m = 0.0, d = 0.0;
+    const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    for (int r = w0; r < NN; r += ws) {
+        const int i = r / N, j = r - i * N;
+        const IN *row = V + (long)r * N;
+        const IN *rr = nullptr, *rs = nullptr;
+        if (sym) {
+            rr = V + ((long)ir[i] * N + ir[j]) * N;
+            rs = V + ((long)is[i] * N + is[j]) * N;
+        }
+        for (int l = lane; l < N; l += 32) {
+            const double v = (double)row[l];
+            if (Vf) Vf[(long)r * N + l] = (float)v;
+            if (!sym) continue;
+            const double e = fmax(fabs((double)rr[ir[l]] - v), fabs((double)rs[is[l]] - v));
+            d = isfinite(v) ? fmax(d, e) : inf;
+            if (isfinite(v)) m = fmax(m, fabs(v));
+        }
+    }
+    if (!sym) return;
+    auto reduce = [&](double x, unsigned long long *slot) {
+        for (int off = 16; off > 0; off >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, off));
+        // non-negative values order like their bits
+        if (lane == 0 && x > 0.0) atomicMax(slot, (unsigned long long)__double_as_longlong(x));
+    };
+    reduce(m, sym);
+    reduce(d, sym + 1);
+    if (w0 == 0) {
+        double mz = 0.0, dz = 0.0;
+        for (int y = lane; y < nz * N; y += 32) {
+            const int x = y % N;
+            const double *Zy = Z + (y - x);
+            const double z = Zy[x];
+            const double e = fmax(fabs(Zy[ir[x]] - z), fabs(Zy[is[x]] - z));
+            dz = isfinite(z) ? fmax(dz, e) : inf;
+            if (isfinite(z)) mz = fmax(mz, fabs(z));
+        }
+        reduce(mz, sym + 2);
+        reduce(dz, sym + 3);
+    }
+}
+
+// The C4v test of V and of nz arrays of N weights Z into c->d_sym (read by
+// sym_compact; nz = 0: no test), the FP32 copy
+// when Vf is given and, outside the tensor-core precision, the permuted views.
+static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const double *d_Z, int nz, float *Vf)
+{
+    const bool test = nz > 0;
+    const int N = c->pb.N, ns = c->pb.n_shell;
+    cudaError_t e;
+    if (test && (e = cudaMemsetAsync(c->d_sym, 0, 4 * sizeof(unsigned long long), c->stream)) != cudaSuccess)
+        return cuda_fail(c, e, "memset symmetry test");
+    unsigned long long *sym = test ? c->d_sym : nullptr;
+    const bool views = c->opt.precision != QPFRG_MIXED_TC;
+    const dim3 grid(std::max(1, std::min(div_up((long)N * N, 8), 304)), views ? 4 : 1);
+    prof_begin(c);
+    if (c->opt.precision == QPFRG_FP64)
+        stage_prep_kernel<double, double><<<grid, 256, 0, c->stream>>>((const double *)V, d_Z, nz, N, ns, sym, nullptr,
+                                                                       (double *)c->d_views);
+    else if (v64)
+        stage_prep_kernel<double, float><<<grid, 256, 0, c->stream>>>((const double *)V, d_Z, nz, N, ns, sym, Vf,
+                                                                      views ? (float *)c->d_views : nullptr);
+    else
+        stage_prep_kernel<float, float><<<grid, 256, 0, c->stream>>>((const float *)V, d_Z, nz, N, ns, sym, nullptr,
+                                                                     (float *)c->d_views);
+    prof_end(c, K_CONVERT);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "stage_prep_kernel");
+}
+
+// Operands of one right-hand side of the given FP64 vertex (qpfrg_rhs, the
+// first stage of a step): C4v test of V and nz weight arrays (nz = 0: none),
+// FP32 copy in the mixed precisions, permuted views of the SIMT contraction.
+qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz)
+{
+    return launch_prep(c, d_V, true, d_Z, nz, c->opt.precision == QPFRG_FP64 ? nullptr : c->d_Vf);
+}
+
+// The same of a later stage's vertex (FP64, or FP32 in mixed precision).
+qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z, int nz)
+{
+    if (c->opt.precision == QPFRG_MIXED_TC) return QPFRG_OK;
+    return launch_prep(c, d_Vin, c->opt.precision == QPFRG_FP64, d_Z, nz, nullptr);
+}
+
+// Columns per thread: the count (1..3) whose 16-wide tiles pad N least.
+static int contract_nb(int N)
+{
+    int best = 3;
+    for (int nb = 3; nb >= 1; --nb)
+        if (div_up(N, 16 * nb) * nb < div_up(N, 16 * best) * best) best = nb;
+    return best;
+}
+
+// Shape of the contraction of `rows` rows: two CTAs per SM where the reduction
+// can be split that far (every split costs partial rows to write and sum).
+static ContractShape contract_shape(const qpfrg_ctx *c, int rows)
+{
+    const int N = c->pb.N, tm = c->opt.precision == QPFRG_FP64 ? 2 : 4;
+    ContractShape s;
+    s.rows = rows;
+    s.mtiles = div_up(rows, 16 * tm);
+    const long per = 4L * s.mtiles * div_up(N, 16 * contract_nb(N));
+    int sp = (int)std::min<long>(N, std::max<long>(1, (2 * 152 + per - 1) / per));
+    s.a_per = div_up(N, sp);
+    s.splits = div_up(N, s.a_per);
+    return s;
+}
+
+// Partial rows and permuted views of the SIMT contraction, sized for both forms.
+qpfrg_status contract_alloc(qpfrg_ctx *c)
+{
+    const long N = c->pb.N, n3 = N * N * N;
+    const ContractShape all = contract_shape(c, (int)(N * N));
+    long n = (long)all.splits * all.rows;
+    if (c->rows_ok) {
+        const ContractShape rep = contract_shape(c, c->n_rrep);
+        n = std::max(n, (long)rep.splits * rep.rows);
+    }
+    const size_t rsz = c->opt.precision == QPFRG_FP64 ? sizeof(double) : sizeof(float);
+    cudaError_t e = cudaMalloc((void **)&c->d_partial, (size_t)n * 4 * N * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_outc, 3 * n3 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_views, 3 * n3 * rsz);
+    if (e == cudaSuccess) return QPFRG_OK;
+    cudaGetLastError();
+    return cuda_fail(c, e, "cudaMalloc(contraction work space)");
+}
+
+template <typename R>
+static qpfrg_status launch_simt(qpfrg_ctx *c, const R *V, double scale, double *out)
+{
+    const int N = c->pb.N;
+    ContractArgs<R> A{};
+    A.B = reinterpret_cast<const R *>(c->d_B);
+    A.V = V;
+    A.P = reinterpret_cast<const R *>(c->d_views);
+    A.rep = c->d_rrep;
+    A.part = c->d_partial;
+    A.N = N;
+    const int nb = contract_nb(N);
+    A.ntiles = div_up(N, 16 * nb);
+    const unsigned ch = c->pb.channels;
+    if (ch & QPFRG_CH_PP) A.jobs[A.njobs++] = 0;
+    if (ch & QPFRG_CH_CR) A.jobs[A.njobs++] = 1;
+    if (ch & QPFRG_CH_D) {
+        A.jobs[A.njobs++] = 2;
+        A.jobs[A.njobs++] = 3;
+    }
+    A.sh[0] = contract_shape(c, N * N);
+    A.sh[1] = c->rows_ok ? contract_shape(c, c->n_rrep) : A.sh[0];
+    A.sym = c->rhs_sym;
+    const int m = c->rhs_sym.mode;
+    const long g0 = (long)A.sh[0].mtiles * A.sh[0].splits, g1 = (long)A.sh[1].mtiles * A.sh[1].splits;
+    const long ctas = (m == 0 ? g0 : (m == 1 ? g1 : std::max(g0, g1))) * A.ntiles * A.njobs;
+    constexpr int TM = sizeof(R) == 8 ? 2 : 4;
+    if (ctas > 0) {
+        prof_begin(c);
+        if (nb == 1) contract_kernel<R, TM, 1><<<(unsigned)ctas, 256, 0, c->stream>>>(A);
+        else if (nb == 2) contract_kernel<R, TM, 2><<<(unsigned)ctas, 256, 0, c->stream>>>(A);
+        else contract_kernel<R, TM, 3><<<(unsigned)ctas, 256, 0, c->stream>>>(A);
+        prof_end(c, K_CONTRACT_PP);   // one launch for every channel
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(c, e, "contract_kernel");
+    }
+    ExpandArgs E{};
+    E.part = c->d_partial;
+    E.outc = c->d_outc;
+    E.rowmap = c->d_rowmap;
+    E.out = out;
+    E.scale = scale;
+    E.N = N;
+    E.ns = c->pb.n_shell;
+    E.njobs = A.njobs;
+    for (int k = 0; k < A.njobs; ++k) {
+        const int q = std::min(A.jobs[k], 2);
+        if (E.count[q]++ == 0) E.first[q] = k;
+    }
+    for (int k = 0; k < 2; ++k) {
+        E.rows[k] = A.sh[k].rows;
+        E.splits[k] = A.sh[k].splits;
+    }
+    E.sym = c->rhs_sym;
+    const long rows = m == 1 ? E.rows[1] : E.rows[0];
+    prof_begin(c);
+    reduce_kernel<<<dim3((unsigned)std::min(div_up(rows * N, 128), 1216), 3), 128, 0, c->stream>>>(E);
+    expand_kernel<<<dim3(N, N), std::min(256, (N + 31) / 32 * 32), 0, c->stream>>>(E);
+    prof_end(c, K_ROWS_EXPAND);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "expand_kernel");
 }
 
 // Expansion of the representative rows (row orbits, symmetry.cu): with a
@@ -245,9 +554,11 @@ qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, 
         qpfrg_status s = QPFRG_OK;
         // representative rows only (row orbits): into the compact rows, then expanded
         double *dst[3] = {d_out, d_out, d_out};
+        cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)c->pb.N * c->pb.N * c->pb.N * sizeof(double), c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "memset right-hand side");
         if (c->rows_compact) {
             const long per = (long)c->n_rrep * c->pb.N;
-            cudaError_t e = cudaMemsetAsync(c->d_outc, 0, 3 * per * sizeof(double), c->stream);
+            e = cudaMemsetAsync(c->d_outc, 0, 3 * per * sizeof(double), c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "memset representative rows");
             for (int k = 0; k < 3; ++k) dst[k] = c->d_outc + k * per;
         }
@@ -260,14 +571,14 @@ qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, 
             rows_expand_kernel<<<dim3(N, N), thr, 0, c->stream>>>(c->d_outc, c->d_rowmap, c->n_rrep, N,
                                                                   c->pb.n_shell, ch, d_out);
             prof_end(c, K_ROWS_EXPAND);
-            cudaError_t e = cudaGetLastError();
+            e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(c, e, "rows_expand_kernel");
         }
         return QPFRG_OK;
     }
     if (c->opt.precision == QPFRG_FP64)
-        return launch_all<double, double>(c, reinterpret_cast<const double *>(d_Vin), scale, d_out);
-    return launch_all<float, float>(c, reinterpret_cast<const float *>(d_Vin), scale, d_out);
+        return launch_simt<double>(c, reinterpret_cast<const double *>(d_Vin), scale, d_out);
+    return launch_simt<float>(c, reinterpret_cast<const float *>(d_Vin), scale, d_out);
 }
 
 }  // namespace qpfrg

@@ -142,24 +142,25 @@ static qpfrg_status zka(qpfrg_ctx *c, const double *y, double g)
 qpfrg_status gflow_enqueue_stages(qpfrg_ctx *c, double x, double h)
 {
     const int N = c->pb.N, nom = c->opt.n_omega;
-    const long n3 = (long)N * N * N, L = gflow_small_len(c), ng = (long)N * nom;
+    const long L = gflow_small_len(c), ng = (long)N * nom;
     const bool mixed = c->opt.precision != QPFRG_FP64;
     const double T = c->pb.T_fixed;
     const double cst[4] = {0.0, 0.5, 0.5, 1.0};
     const double *Zs = c->d_gzka, *Ks = Zs + N, *Ab = Ks + 2 * N;
     qpfrg_status s;
     cudaError_t e;
-    if (mixed && (s = launch_convert_f32(c, c->d_V, c->d_Vf, n3)) != QPFRG_OK) return s;
     const double *Vst = c->d_V;                  // FP64 vertex of the stage (two-loop term)
     const void *Vin = mixed ? (const void *)c->d_Vf : (const void *)c->d_V;
     const double *yst = c->d_gy;
     for (int st = 0; st < 4; ++st) {
         const double gs = x + cst[st] * h;
         if ((s = zka(c, yst, gs)) != QPFRG_OK) return s;
+        // operands of the stage, with the symmetry test of V and of (Z, K)
+        const int nz = state_form(c).mode == 2 ? 2 : 0;
+        if ((s = st == 0 ? launch_stage_prep(c, c->d_V, Zs, nz) : launch_stage_views(c, Vin, Zs, nz)) != QPFRG_OK)
+            return s;
         // vertex: loop kernels with Z and K on the lines, contraction
-        if ((s = launch_bubbles(c, gs, Zs, true, c->opt.katanin ? Ks : nullptr, c->c4v_state)) != QPFRG_OK) return s;
-        if ((e = cudaMemsetAsync(c->d_k, 0, n3 * sizeof(double), c->stream)) != cudaSuccess)
-            return cuda_fail(c, e, "memset k");
+        if ((s = launch_bubbles(c, gs, Zs, true, c->opt.katanin ? Ks : nullptr, state_form(c))) != QPFRG_OK) return s;
         if ((s = launch_contractions(c, Vin, 1.0, c->d_k)) != QPFRG_OK) return s;
         // two-loop term: chord slopes at xi_j +- 2T, and the frequency grid
         if ((s = launch_sigma_lines(c, T, Vst, Zs, c->opt.katanin ? Ks : c->d_ones)) != QPFRG_OK) return s;

@@ -7,12 +7,6 @@
 
 namespace qpfrg {
 
-__global__ void convert_f32_kernel(const double *__restrict__ in, float *__restrict__ out, long n)
-{
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        out[i] = (float)in[i];
-}
-
 // stage 1: acc = k;    Vs = V + h/2 k
 // stage 2: acc += 2k;  Vs = V + h/2 k
 // stage 3: acc += 2k;  Vs = V + h k
@@ -102,15 +96,6 @@ static int grid_for(long n)
     long b = (n + 255) / 256;
     if (b > 152L * 16) b = 152L * 16;
     return (int)(b < 1 ? 1 : b);
-}
-
-qpfrg_status launch_convert_f32(qpfrg_ctx *c, const double *d_in, float *d_out, long n)
-{
-    prof_begin(c);
-    convert_f32_kernel<<<grid_for(n), 256, 0, c->stream>>>(d_in, d_out, n);
-    prof_end(c, K_CONVERT);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "convert_f32_kernel");
 }
 
 qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_V, const double *d_k,

@@ -97,6 +97,14 @@ qpfrg_status dev_alloc(qpfrg_ctx *c, T **p, size_t count, const char *what)
     return QPFRG_OK;
 }
 
+// the C4v test read back into h_red[5..8]: deviations within tol of the maxima
+bool c4v_within(const qpfrg_ctx *c, double tol)
+{
+    double r[4];
+    std::memcpy(r, &c->h_red[5], sizeof(r));
+    return r[1] <= tol / 3.0 * r[0] && r[3] <= tol / 3.0 * r[2];
+}
+
 long n3_of(const qpfrg_ctx *c) { return (long)c->pb.N * c->pb.N * c->pb.N; }
 
 }  // namespace
@@ -185,7 +193,7 @@ void qpfrg_destroy(qpfrg_t c)
                         c->tc.Bpp[0], c->tc.Bpp[1], c->tc.Bcr[0], c->tc.Bcr[1], c->tc.Bd[0], c->tc.Bd[1],
                         c->tc.VT, c->d_tc_err, c->d_xij, c->d_bnd, c->d_qxl, c->d_qyl, c->d_kp, c->d_kcs, c->d_xij_f,
                         c->d_ptab, c->d_jgrid, c->d_repgrid, c->d_lrepQ, c->d_lnimg, c->d_limg, c->d_ltask,
-                        c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc};
+                        c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     }
@@ -366,9 +374,11 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
         (s = dev_alloc(c, &c->d_k, n3, "k")) || (s = dev_alloc(c, &c->d_acc, n3, "acc")) ||
         (s = dev_alloc(c, &c->d_Vf, n3, "V fp32")) || (s = dev_alloc(c, &c->d_Z, N, "Z")) ||
         (s = dev_alloc(c, &c->d_Zwork, N, "Z work")) || (s = dev_alloc(c, &c->d_ones, N, "ones")) ||
-        (s = dev_alloc(c, &c->d_sig, 2 * N, "sigma chord")) || (s = dev_alloc(c, &c->d_red, 5, "reduction")))
+        (s = dev_alloc(c, &c->d_sig, 2 * N, "sigma chord")) || (s = dev_alloc(c, &c->d_red, 5, "reduction")) ||
+        (s = dev_alloc(c, &c->d_sym, 4, "symmetry test")))
         return fail(s);
-    e = cudaMallocHost((void **)&c->h_red, 5 * sizeof(unsigned long long));
+    if (!tcmode && (s = contract_alloc(c)) != QPFRG_OK) return fail(s);
+    e = cudaMallocHost((void **)&c->h_red, 9 * sizeof(unsigned long long));
     if (e != cudaSuccess) return fail(cuda_fail(c, e, "cudaMallocHost"));
     if (c->opt.sigma_ode && (s = gflow_alloc(c)) != QPFRG_OK) return fail(s);
 
@@ -417,7 +427,7 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
     if (e != cudaSuccess) return fail(cuda_fail(c, e, "init Z"));
     c->lambda = lambda0;
     c->lambda_end = c->opt.lambda_end;
-    c->c4v_state = pb.mode == QPFRG_GRID_WEDGE || pb.mode == QPFRG_GRID_SHELL;
+    c->c4v_state = c->rows_state = pb.mode == QPFRG_GRID_WEDGE || pb.mode == QPFRG_GRID_SHELL;
     c->steps = 0;
     c->status = QPFRG_FLOW_RUNNING;
     c->max_abs_v = std::fabs(U);
@@ -435,27 +445,27 @@ qpfrg_status qpfrg_rhs(qpfrg_t c, double lambda, const double *d_V, const double
     const bool tflow = c->pb.regulator == QPFRG_REG_TEMPERATURE;
     if (!std::isfinite(lambda) || (tflow && !(lambda > 0.0)))
         return set_err(c, QPFRG_ERR_INVALID, "lambda must be finite (and T > 0)");
-    const long n3 = n3_of(c);
-    const void *Vin = d_V;
+    const void *Vin = c->opt.precision == QPFRG_FP64 ? (const void *)d_V : (const void *)c->d_Vf;
+    const double *Z = d_Z ? d_Z : c->d_ones;
     qpfrg_status s;
-    if (c->opt.precision != QPFRG_FP64) {
-        if ((s = launch_convert_f32(c, d_V, c->d_Vf, n3)) != QPFRG_OK) return s;
-        Vin = c->d_Vf;
-    }
-    // row orbits of the tensor-core contraction need a C4v-symmetric V and Z:
-    // tested on the device (relative 1e-12 of max|V|, max|Z|) and read back
-    bool sym = false;
+    // row orbits need a C4v-symmetric V and Z: tested on the device, where the
+    // FP64 and FP32 contractions also take the decision; the tensor-core
+    // contraction's is read back
+    if ((s = launch_stage_prep(c, d_V, Z, c->rows_ok ? 1 : 0)) != QPFRG_OK) return s;
+    SymMode sym;
     if (c->rows_ok) {
-        if ((s = launch_state_check(c, d_V, d_Z ? d_Z : c->d_ones, true, 1e-12)) != QPFRG_OK) return s;
-        cudaError_t e = cudaMemcpyAsync(&c->h_red[4], &c->d_red[4], sizeof(unsigned long long),
-                                        cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "C4v test of the RHS input");
-        sym = c->h_red[4] == 0;
+        sym.mode = 2;
+        sym.red = c->d_sym;
+        sym.tol = rows_tol(c) / 3.0;
+        if (c->opt.precision == QPFRG_MIXED_TC) {
+            cudaError_t e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 4 * sizeof(unsigned long long),
+                                            cudaMemcpyDeviceToHost, c->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+            if (e != cudaSuccess) return cuda_fail(c, e, "C4v test of the RHS input");
+            sym.mode = c4v_within(c, rows_tol(c)) ? 1 : 0;
+        }
     }
-    if ((s = launch_bubbles(c, lambda, d_Z ? d_Z : c->d_ones, d_Z == nullptr, nullptr, sym)) != QPFRG_OK) return s;
-    cudaError_t e = cudaMemsetAsync(d_dV, 0, n3 * sizeof(double), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "memset dV");
+    if ((s = launch_bubbles(c, lambda, Z, d_Z == nullptr, nullptr, sym)) != QPFRG_OK) return s;
     return launch_contractions(c, Vin, 1.0, d_dV);
 }
 
@@ -531,25 +541,21 @@ static qpfrg_status enqueue_step(qpfrg_ctx *c)
         if (e != cudaSuccess) return cuda_fail(c, e, "copy Z");
     }
 
-    const void *Vin = c->d_V;
-    if (mixed) {
-        if ((s = launch_convert_f32(c, c->d_V, c->d_Vf, n3)) != QPFRG_OK) return s;
-        Vin = c->d_Vf;
-    }
+    const void *Vin = mixed ? (const void *)c->d_Vf : (const void *)c->d_V;
+    if ((s = launch_stage_prep(c, c->d_V, c->d_Z, state_form(c).mode == 2 ? 1 : 0)) != QPFRG_OK) return s;
     const double cst[4] = {0.0, 0.5, 0.5, 1.0};
     for (int st = 0; st < 4; ++st) {
         const double xs = x + cst[st] * h;
         const double lam = tflow ? std::exp(xs) : xs;
         const double scale = tflow ? lam : 1.0;   // dV/d ln T = T dV/dT
-        if ((s = launch_bubbles(c, lam, c->d_Z, c->c4v_state, nullptr, c->c4v_state)) != QPFRG_OK) return s;
-        if ((e = cudaMemsetAsync(c->d_k, 0, n3 * sizeof(double), c->stream)) != cudaSuccess)
-            return cuda_fail(c, e, "memset k");
+        if ((s = launch_bubbles(c, lam, c->d_Z, c->c4v_state, nullptr, state_form(c))) != QPFRG_OK) return s;
         if ((s = launch_contractions(c, Vin, scale, c->d_k)) != QPFRG_OK) return s;
         if (st < 3) {
             s = launch_rk_stage(c, st + 1, h, c->d_V, c->d_k, c->d_acc, mixed ? nullptr : c->d_Vs,
                                 mixed ? c->d_Vf : nullptr);
             if (s != QPFRG_OK) return s;
             Vin = mixed ? (const void *)c->d_Vf : (const void *)c->d_Vs;
+            if ((s = launch_stage_views(c, Vin)) != QPFRG_OK) return s;
         } else if ((s = launch_rk_final(c, h, c->d_V, c->d_acc, c->d_k)) != QPFRG_OK) {
             return s;
         }
@@ -596,6 +602,21 @@ static qpfrg_status finish_step(qpfrg_ctx *c)
     }
     if ((tflow && x_new - x_end <= 1e-12) || (!tflow && x_end - x_new <= 1e-12)) c->status = QPFRG_FLOW_REACHED_END;
     return QPFRG_OK;
+}
+
+// Whether the chord slopes s1, s2 (2N values of a state image, host) keep the
+// point group: every image within tol of the largest magnitude.
+static bool slopes_symmetric(const qpfrg_ctx *c, const double *s, double tol)
+{
+    const int N = c->pb.N;
+    for (int part = 0; part < 2; ++part, s += N) {
+        double m = 0.0;
+        for (int j = 0; j < N; ++j) m = std::fmax(m, std::fabs(s[j]));
+        for (int j = 0; j < N; ++j)
+            for (int g = 1; g < 8; ++g)
+                if (!(std::fabs(s[c4v_apply(g, j, N, c->pb.n_shell)] - s[j]) <= tol * m)) return false;
+    }
+    return true;
 }
 
 static qpfrg_status do_step(qpfrg_ctx *c)
@@ -662,7 +683,7 @@ static qpfrg_status make_child(qpfrg_ctx *parent, double U, double lambda0, doub
     if (!c) return QPFRG_ERR_OOM;
     c->shares_geometry = true;
     c->rtab_tried = true;   // a child reads the parent's table (if built) and never builds its own
-    c->rows_ok = c->rows_compact = false;   // batched flows contract every row
+    c->rows_compact = false;
     c->profiler = new (std::nothrow) Profiler();
     c->prof = false;
     for (auto &sl : c->slots) sl = ProfileSlot();
@@ -681,7 +702,7 @@ static qpfrg_status make_child(qpfrg_ctx *parent, double U, double lambda0, doub
         qpfrg_destroy(c);
         return s;
     }
-    if (cudaMallocHost((void **)&c->h_red, 5 * sizeof(unsigned long long)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&c->h_red, 9 * sizeof(unsigned long long)) != cudaSuccess) {
         qpfrg_destroy(c);
         return QPFRG_ERR_OOM;
     }
@@ -704,7 +725,7 @@ static qpfrg_status make_child(qpfrg_ctx *parent, double U, double lambda0, doub
     c->max_abs_v = std::fabs(U);
     c->lambda_c = 0.0;
     c->pending = false;
-    c->c4v_state = c->pb.mode == QPFRG_GRID_WEDGE || c->pb.mode == QPFRG_GRID_SHELL;
+    c->c4v_state = c->rows_state = c->pb.mode == QPFRG_GRID_WEDGE || c->pb.mode == QPFRG_GRID_SHELL;
     *out = c;
     return QPFRG_OK;
 }
@@ -871,7 +892,11 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
         e = cudaMemcpyAsync(c->d_acc, Z, c->pb.N * sizeof(double), cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "set_state upload");
     qpfrg_status st = launch_state_check(c, c->d_k, c->d_acc, wedge, tol);
+    if (st == QPFRG_OK && c->rows_ok) st = launch_stage_prep(c, c->d_k, c->d_acc, 1);
     if (st != QPFRG_OK) return st;
+    if (c->rows_ok && (e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 4 * sizeof(unsigned long long),
+                                           cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
+        return cuda_fail(c, e, "set_state check");
     if ((e = cudaMemcpyAsync(c->h_red, c->d_red, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                              c->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
@@ -889,6 +914,13 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
                              c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state (self-energy ODE)");
     c->c4v_state = wedge && c->h_red[4] == 0;
+    // The row orbits: every precision's contraction stays within its own
+    // rounding of the unreduced one (the tensor-core flow keeps the tolerance
+    // of the state's symmetry).  The slopes of the self-energy ODE set Z, K and
+    // A, so they have to be symmetric as well.
+    const double rtol = c->opt.precision == QPFRG_FP64 ? rows_tol(c) : (c->opt.precision == QPFRG_MIXED ? 3e-7 : tol);
+    c->rows_state = c->rows_ok && c->c4v_state && (c->opt.precision == QPFRG_MIXED_TC || c4v_within(c, rtol));
+    if (c->d_gy && c->rows_state) c->rows_state = slopes_symmetric(c, Z + c->pb.N, rtol);
     c->status = hd.status;
     c->steps = (int)hd.steps;
     c->lambda = hd.lambda;

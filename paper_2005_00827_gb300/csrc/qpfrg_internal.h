@@ -76,6 +76,26 @@ enum KernelId {
     K_COUNT
 };
 
+// Form of a right-hand side: 0 every row, 1 representative rows of the C4v row
+// orbits, 2 decided on the device by the C4v test of its inputs (red =
+// [max|V|, deviation, max|Z|, deviation] as FP64 bits, tol the tolerance of one
+// generator relative to the maxima: a third of that of any image, which is at
+// most three generator steps away; divided on the host, since an FP64 division
+// at the head of every kernel costs microseconds).
+struct SymMode {
+    int mode = 0;
+    const unsigned long long *red = nullptr;
+    double tol = 0.0;
+};
+
+__device__ __forceinline__ bool sym_compact(const SymMode &s)
+{
+    if (s.mode != 2) return s.mode == 1;
+    const double m = __longlong_as_double((long long)s.red[0]), d = __longlong_as_double((long long)s.red[1]);
+    const double mz = __longlong_as_double((long long)s.red[2]), dz = __longlong_as_double((long long)s.red[3]);
+    return d <= s.tol * m && dz <= s.tol * mz;
+}
+
 // Launch shapes chosen by qpfrg_autotune (0 = built-in heuristic).
 struct Tuning {
     int bubble_qchunk = 0;      // transfers per loop-kernel CTA
@@ -261,13 +281,18 @@ struct qpfrg_ctx {
     long long loop_evals_red = 0;   // loop-kernel evaluations of one reduced RHS
     long loop_mismatch_rows = 0;    // rows evaluated by themselves (covariance broken)
 
-    // C4v row orbits of the tensor-core contraction (symmetry.cu): with a
+    // C4v row orbits of the contraction (symmetry.cu): with a
     // C4v-symmetric state (V, Z) every channel's output row Q = (x, y) at
     // column n equals its representative's row at column g^-1 n, Q = g rep, so
     // only representative rows are tabled and contracted and the result is
     // expanded (contract.cu).  Built when every loop-kernel row is covariant.
     bool rows_ok = false;
     bool rows_compact = false;   // the table of the current RHS holds representative rows only
+    bool rows_state = false;     // the flow state is symmetric enough for the row orbits
+    qpfrg::SymMode rhs_sym;      // form of the current RHS
+    unsigned long long *d_sym = nullptr;   // C4v test of a right-hand side's inputs (SymMode::red)
+    double *d_partial = nullptr; // partial rows of the SIMT contraction [split][job][row][n]
+    void *d_views = nullptr;     // permuted views of the stage vertex [cr, d1, d2][a][b][n] (FP64 or FP32)
     int n_rrep = 0;
     int *d_rrep = nullptr;       // Q of each representative row
     int *d_rowmap = nullptr;     // per Q: representative index | g << 24, Q = g rep
@@ -341,11 +366,30 @@ qpfrg_status upload_geometry(qpfrg_ctx *c);
 // z_symmetric: Z is C4v symmetric (needed by the reduced launch with
 // quasi-particle lines, whose loop kernels depend on Z).
 // d_K: Katanin factors of the interaction flow's S line (nullptr = 1).
-// state_symmetric: V and Z are C4v symmetric, so that (tensor-core precision,
-// row orbits built) only representative rows are tabled; sets c->rows_compact
-// for the contraction of the same RHS.
+// sym: the form of the RHS (every row, or the representative rows of the row
+// orbits), kept in c->rhs_sym for the contraction of the same RHS.
 qpfrg_status launch_bubbles(qpfrg_ctx *c, double lambda, const double *d_Z, bool z_symmetric,
-                            const double *d_K = nullptr, bool state_symmetric = false);
+                            const double *d_K, const SymMode &sym);
+// tolerance of the C4v test that admits the row orbits, relative to the
+// maxima: a few roundings of the precision that computes the right-hand side
+// (an input asymmetry enters its result at first order)
+inline double rows_tol(const qpfrg_ctx *c) { return c->opt.precision == QPFRG_FP64 ? 1e-14 : 1e-12; }
+// the form of a right-hand side of the flow state.  Where the weights come from
+// self-energies that evaluate every patch, the zone-edge patches differ by what
+// the wedge decision of momenta on |k| = pi does (1e-7 .. 1e-5): the stage's test
+// decides on the device, in FP32 within the rounding of its right-hand side.
+inline SymMode state_form(const qpfrg_ctx *c)
+{
+    SymMode s;
+    if (!c->rows_ok || !c->rows_state) return s;
+    s.mode = 1;
+    const bool fp64 = c->opt.precision == QPFRG_FP64;
+    if (c->opt.precision == QPFRG_MIXED_TC || !(c->opt.sigma_ode || (fp64 && c->opt.z_feedback))) return s;
+    s.mode = 2;
+    s.red = c->d_sym;
+    s.tol = (fp64 ? rows_tol(c) : 1e-6) / 3.0;
+    return s;
+}
 
 qpfrg_status launch_loop_rows(qpfrg_ctx *c, double lambda, float *rows, const int *active, bool compact = false);
 
@@ -354,8 +398,12 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c);
 qpfrg_status loop_tasks(qpfrg_ctx *c, int qchunk, int *ntask);
 qpfrg_status row_tasks(qpfrg_ctx *c, int qchunk, int *ntask);
 
-// contract.cu: d_out (N^3 FP64) += scale * contraction of the bubble tables.
-// V input is FP64 (precision FP64) or FP32 (MIXED).
+// contract.cu: d_out (N^3 FP64) = scale * contraction of the bubble tables.
+// V input is FP64 (precision FP64) or FP32 (MIXED); its permuted views are
+// those of the last launch_stage_prep / launch_stage_views.
+qpfrg_status contract_alloc(qpfrg_ctx *c);
+qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz);
+qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z = nullptr, int nz = 0);
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out);
 
 // sigma.cu
@@ -422,7 +470,6 @@ qpfrg_status tc_make_maps(qpfrg_ctx *c);   // TMA maps of the tensor-core operan
 qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, int kid);
 
 // ode.cu
-qpfrg_status launch_convert_f32(qpfrg_ctx *c, const double *d_in, float *d_out, long n);
 qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_V,
                              const double *d_k, double *d_acc, double *d_Vs, float *d_Vf);
 qpfrg_status launch_state_check(qpfrg_ctx *c, const double *d_V, const double *d_Z, bool c4v_test, double tol);

@@ -18,7 +18,7 @@
 //
 // When every row is covariant and V and Z are C4v symmetric, each channel's
 // output is invariant as well, dV_ch(g k1, g k2, g k3) = dV_ch(k1, k2, k3), so
-// the tensor-core contraction needs one output row per orbit of transfer pairs
+// the contraction needs one output row per orbit of transfer pairs
 // Q only (build_row_orbits: representatives, and per pair Q its
 // representative and the g with Q = g rep); contract.cu expands the rows.
 #include <algorithm>
@@ -63,7 +63,7 @@ __global__ void check_covariance_kernel(const uint8_t *__restrict__ part, const 
     }
 }
 
-// Row orbits of the tensor-core contraction: the representative of the
+// Row orbits of the contraction: the representative of the
 // transfer pair Q = (x, y) is its image g Q = (g x, g y) with the smallest
 // index; rowmap[Q] = (representative index | g << 24) with Q = g rep.  Only
 // built when every loop-kernel row passed the covariance check, so that the
@@ -98,7 +98,8 @@ static qpfrg_status build_row_orbits(qpfrg_ctx *c)
     if ((e = cudaMalloc((void **)&c->d_rrep, nr * sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_rowmap, NN * sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_rtask, (2L * N * ((nr + 7) / 8) + 8) * sizeof(int4))) != cudaSuccess ||
-        (e = cudaMalloc((void **)&c->d_outc, 3L * nr * N * sizeof(double))) != cudaSuccess)
+        (c->opt.precision == QPFRG_MIXED_TC &&
+         (e = cudaMalloc((void **)&c->d_outc, 3L * nr * N * sizeof(double))) != cudaSuccess))
         return cuda_fail(c, e, "cudaMalloc(row orbits)");
     e = cudaMemcpy(c->d_rrep, reps.data(), nr * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_rowmap, rowmap.data(), NN * sizeof(int), cudaMemcpyHostToDevice);
@@ -237,7 +238,7 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
     c->loop_evals_red = evals;
     c->loop_mismatch_rows = mism;
     c->loop_red = true;
-    if (mism == 0 && c->opt.precision == QPFRG_MIXED_TC && c->opt.no_loop_symmetry == 0)
+    if (mism == 0 && c->opt.no_loop_symmetry == 0)
         return build_row_orbits(c);
     return QPFRG_OK;
 }
@@ -314,6 +315,14 @@ extern "C" qpfrg_status qpfrg_rhs_work(qpfrg_t c, long long *loop_evals, long lo
 {
     if (!c) return QPFRG_ERR_INVALID;
     const long long full = 2LL * c->pb.N * c->pb.N * c->pb.M;
+    if (c->rhs_sym.mode == 2) {     // the form was decided on the device: read the test
+        double r[4];
+        cudaError_t e = cudaMemcpyAsync(r, c->d_sym, sizeof(r), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return qpfrg::cuda_fail(c, e, "qpfrg_rhs_work");
+        const double tol = c->rhs_sym.tol;
+        c->rows_compact = r[1] <= tol * r[0] && r[3] <= tol * r[2];
+    }
     if (loop_evals) *loop_evals = c->rows_compact ? c->loop_evals_rows : (c->loop_red ? c->loop_evals_red : full);
     if (loop_evals_full) *loop_evals_full = full;
     if (rows_unreduced) *rows_unreduced = c->loop_red ? c->loop_mismatch_rows : 0;
