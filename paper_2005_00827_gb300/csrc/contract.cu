@@ -271,8 +271,8 @@ __global__ void expand_kernel(const ExpandArgs A)
 // The C4v test reduces max|V| and the largest deviation under the two
 // generators (rotation by 90 degrees, reflection); any image differs by at most
 // three generator steps, so a deviation below a third of the tolerance
-// guarantees every image.  A non-finite value counts as asymmetric: an infinite
-// deviation against the maximum of the finite values.
+// guarantees every image.  A non-finite value sets sym[4] and counts as asymmetric:
+// an infinite deviation against the maximum of the finite values.
 template <typename IN, typename R>
 __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ V, const double *__restrict__ Z, int nz, int N,
                                                          int ns, unsigned long long *sym, float *__restrict__ Vf,
@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
     }
     __syncthreads();
     double m = 0.0, d = 0.0;
+    bool fin = true;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
     for (int r = w0; r < NN; r += ws) {
         const int i = r / N, j = r - i * N;
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
             const double e = fmax(fabs((double)rr[ir[l]] - v), fabs((double)rs[is[l]] - v));
             d = isfinite(v) ? fmax(d, e) : inf;
             if (isfinite(v)) m = fmax(m, fabs(v));
+            else fin = false;
         }
     }
     if (!sym) return;
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
     };
     reduce(m, sym);
     reduce(d, sym + 1);
+    if (!fin) atomicOr(&sym[4], 1ull);
     if (w0 == 0) {
         double mz = 0.0, dz = 0.0;
         for (int y = lane; y < nz * N; y += 32) {
@@ -336,29 +339,31 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
             const double e = fmax(fabs(Zy[ir[x]] - z), fabs(Zy[is[x]] - z));
             dz = isfinite(z) ? fmax(dz, e) : inf;
             if (isfinite(z)) mz = fmax(mz, fabs(z));
+            else fin = false;
         }
         reduce(mz, sym + 2);
         reduce(dz, sym + 3);
+        if (!fin) atomicOr(&sym[4], 1ull);
     }
 }
 
 // The C4v test of V and of nz arrays of N weights Z into c->d_sym (read by
 // sym_compact; nz = 0: no test), the FP32 copy
 // when Vf is given and, outside the tensor-core precision, the permuted views.
-static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const double *d_Z, int nz, float *Vf)
+static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const double *d_Z, int nz, float *Vf, bool operands)
 {
     const bool test = nz > 0;
     const int N = c->pb.N, ns = c->pb.n_shell;
     cudaError_t e;
-    if (test && (e = cudaMemsetAsync(c->d_sym, 0, 4 * sizeof(unsigned long long), c->stream)) != cudaSuccess)
+    if (test && (e = cudaMemsetAsync(c->d_sym, 0, 5 * sizeof(unsigned long long), c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "memset symmetry test");
     unsigned long long *sym = test ? c->d_sym : nullptr;
-    const bool views = c->opt.precision != QPFRG_MIXED_TC;
+    const bool views = operands && c->opt.precision != QPFRG_MIXED_TC;
     const dim3 grid(std::max(1, std::min(div_up((long)N * N, 8), 304)), views ? 4 : 1);
     prof_begin(c);
-    if (c->opt.precision == QPFRG_FP64)
+    if (c->opt.precision == QPFRG_FP64 || !operands)
         stage_prep_kernel<double, double><<<grid, 256, 0, c->stream>>>((const double *)V, d_Z, nz, N, ns, sym, nullptr,
-                                                                       (double *)c->d_views);
+                                                                       views ? (double *)c->d_views : nullptr);
     else if (v64)
         stage_prep_kernel<double, float><<<grid, 256, 0, c->stream>>>((const double *)V, d_Z, nz, N, ns, sym, Vf,
                                                                       views ? (float *)c->d_views : nullptr);
@@ -375,14 +380,19 @@ static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const dou
 // FP32 copy in the mixed precisions, permuted views of the SIMT contraction.
 qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz)
 {
-    return launch_prep(c, d_V, true, d_Z, nz, c->opt.precision == QPFRG_FP64 ? nullptr : c->d_Vf);
+    return launch_prep(c, d_V, true, d_Z, nz, c->opt.precision == QPFRG_FP64 ? nullptr : c->d_Vf, true);
 }
 
 // The same of a later stage's vertex (FP64, or FP32 in mixed precision).
 qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z, int nz)
 {
     if (c->opt.precision == QPFRG_MIXED_TC) return QPFRG_OK;
-    return launch_prep(c, d_Vin, c->opt.precision == QPFRG_FP64, d_Z, nz, nullptr);
+    return launch_prep(c, d_Vin, c->opt.precision == QPFRG_FP64, d_Z, nz, nullptr, true);
+}
+
+qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz)
+{
+    return launch_prep(c, d_V, true, d_Z, nz, nullptr, false);
 }
 
 // Columns per thread: the count (1..3) whose 16-wide tiles pad N least.

@@ -349,6 +349,13 @@ static qpfrg_status alloc_transfer(qpfrg_ctx *c, TransferTable<R> &t, const std:
 qpfrg_status upload_geometry(qpfrg_ctx *c)
 {
     const int N = c->pb.N;
+    c->fx_min = 1e300;
+    c->fx_max = -1e300;
+    for (int p = 0; p < c->pb.M; ++p) {
+        const double x = host_xi(c->pb, c->fk[2 * p], c->fk[2 * p + 1]);
+        c->fx_min = std::fmin(c->fx_min, x);
+        c->fx_max = std::fmax(c->fx_max, x);
+    }
     const size_t NN = (size_t)N * N;
     std::vector<double> Qpp(2 * NN), Qph(2 * NN);
     for (int x = 0; x < N; ++x)
@@ -398,12 +405,17 @@ qpfrg_status upload_geometry(qpfrg_ctx *c)
             (e = cudaMalloc((void **)&c->d_qxl, M * sizeof(float))) != cudaSuccess ||
             (e = cudaMalloc((void **)&c->d_qyl, M * sizeof(float))) != cudaSuccess ||
             (e = cudaMalloc((void **)&c->d_kp, (size_t)N * M * sizeof(float4))) != cudaSuccess ||
+            (e = cudaMalloc((void **)&c->d_kfx, (size_t)N * M * sizeof(int2))) != cudaSuccess ||
+            (e = cudaMalloc((void **)&c->d_pfx, M * sizeof(int2))) != cudaSuccess ||
             (e = cudaMalloc((void **)&c->d_kcs, N * sizeof(float4))) != cudaSuccess)
             return cuda_fail(c, e, "cudaMalloc(xi_j, rays, residuals, k+p)");
         cudaMemcpy(c->d_xij, xij.data(), N * sizeof(double), cudaMemcpyHostToDevice);
         cudaMemcpy(c->d_bnd, bnd.data(), N * sizeof(float4), cudaMemcpyHostToDevice);
         cudaMemcpy(c->d_qxl, xl.data(), M * sizeof(float), cudaMemcpyHostToDevice);
         cudaMemcpy(c->d_qyl, yl.data(), M * sizeof(float), cudaMemcpyHostToDevice);
+        std::vector<int2> pfx(M);
+        for (size_t p = 0; p < M; ++p) pfx[p] = make_int2(angle_fx(c->fk[2 * p]), angle_fx(c->fk[2 * p + 1]));
+        cudaMemcpy(c->d_pfx, pfx.data(), M * sizeof(int2), cudaMemcpyHostToDevice);
         if (c->pb.mode == QPFRG_GRID_WEDGE && N <= 254) {
             std::vector<uint8_t> tab = build_proj_table(N);
             const size_t bytes = (tab.size() + 15) / 16 * 16;
@@ -427,29 +439,22 @@ qpfrg_status upload_geometry(qpfrg_ctx *c)
     dim3 grid((unsigned)NN, pblocks < 1 ? 1 : (pblocks > 65535 ? 65535 : pblocks), 2);
     if (c->d_ptab) {
         // wedge mode: fixed-point decisions, FP64 only in the guard bands
-        const size_t M = c->pb.M;
-        std::vector<int2> qfx(2 * NN), pfx(M);
+        std::vector<int2> qfx(2 * NN);
         for (size_t q = 0; q < NN; ++q) {
             qfx[q] = make_int2(angle_fx(Qpp[2 * q]), angle_fx(Qpp[2 * q + 1]));
             qfx[NN + q] = make_int2(angle_fx(Qph[2 * q]), angle_fx(Qph[2 * q + 1]));
         }
-        for (size_t p = 0; p < M; ++p) pfx[p] = make_int2(angle_fx(c->fk[2 * p]), angle_fx(c->fk[2 * p + 1]));
-        int2 *d_qfx = nullptr, *d_pfx = nullptr;
-        if ((e = cudaMalloc((void **)&d_qfx, 2 * NN * sizeof(int2))) != cudaSuccess ||
-            (e = cudaMalloc((void **)&d_pfx, M * sizeof(int2))) != cudaSuccess) {
-            cudaFree(d_qfx);
+        int2 *d_qfx = nullptr;
+        if ((e = cudaMalloc((void **)&d_qfx, 2 * NN * sizeof(int2))) != cudaSuccess)
             return cuda_fail(c, e, "cudaMalloc(fixed-point momenta)");
-        }
         cudaMemcpy(d_qfx, qfx.data(), 2 * NN * sizeof(int2), cudaMemcpyHostToDevice);
-        cudaMemcpy(d_pfx, pfx.data(), M * sizeof(int2), cudaMemcpyHostToDevice);
         prof_begin(c);
-        partner_map_fx_kernel<<<grid, 256, 0, c->stream>>>(d_qfx, c->d_Qpp, c->d_Qph, d_pfx, c->f64.kx, c->f64.ky,
+        partner_map_fx_kernel<<<grid, 256, 0, c->stream>>>(d_qfx, c->d_Qpp, c->d_Qph, c->d_pfx, c->f64.kx, c->f64.ky,
                                                            c->d_ptab, c->d_bnd, c->d_part, c->pb);
         prof_end(c, K_PARTNER_MAP);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);   // before the momenta are released
         cudaFree(d_qfx);
-        cudaFree(d_pfx);
         if (e != cudaSuccess) return cuda_fail(c, e, "partner_map_fx_kernel");
         return QPFRG_OK;
     }

@@ -155,15 +155,18 @@ qpfrg_status gflow_enqueue_stages(qpfrg_ctx *c, double x, double h)
     for (int st = 0; st < 4; ++st) {
         const double gs = x + cst[st] * h;
         if ((s = zka(c, yst, gs)) != QPFRG_OK) return s;
-        // operands of the stage, with the symmetry test of V and of (Z, K)
-        const int nz = state_form(c).mode == 2 ? 2 : 0;
-        if ((s = st == 0 ? launch_stage_prep(c, c->d_V, Zs, nz) : launch_stage_views(c, Vin, Zs, nz)) != QPFRG_OK)
-            return s;
+        // operands of the stage, with the symmetry test of V and of (Z, K) that
+        // the right-hand side and the self-energy decide by
+        const int nz = c->pb.mode == QPFRG_GRID_LATTICE ? 0 : 2;
+        if (st == 0) s = launch_stage_prep(c, c->d_V, Zs, nz);
+        else if (c->opt.precision == QPFRG_MIXED_TC && nz) s = launch_sym_test(c, Vst, Zs, nz);
+        else s = launch_stage_views(c, Vin, Zs, nz);
+        if (s != QPFRG_OK) return s;
         // vertex: loop kernels with Z and K on the lines, contraction
         if ((s = launch_bubbles(c, gs, Zs, true, c->opt.katanin ? Ks : nullptr, state_form(c))) != QPFRG_OK) return s;
         if ((s = launch_contractions(c, Vin, 1.0, c->d_k)) != QPFRG_OK) return s;
         // two-loop term: chord slopes at xi_j +- 2T, and the frequency grid
-        if ((s = launch_sigma_lines(c, T, Vst, Zs, c->opt.katanin ? Ks : c->d_ones)) != QPFRG_OK) return s;
+        if ((s = launch_sigma_lines(c, T, Vst, Zs, c->opt.katanin ? Ks : c->d_ones, c->d_sig + N)) != QPFRG_OK) return s;
         const double *t2re = nullptr, *t2im = nullptr;
         if (nom > 0) {
             if ((s = launch_sigma_grid(c, T, Vst, Zs, c->d_gt2, c->d_gt2 + ng, c->opt.katanin ? Ks : c->d_ones)) !=
@@ -173,7 +176,7 @@ qpfrg_status gflow_enqueue_stages(qpfrg_ctx *c, double x, double h)
             t2im = c->d_gt2 + ng;
         }
         gflow_deriv_kernel<<<(int)std::min<long>((L + 255) / 256, 1216), 256, 0, c->stream>>>(
-            yst, c->d_sig, t2re, t2im, Ab, gs, N, nom, c->d_gk);
+            yst, c->d_sig + N, t2re, t2im, Ab, gs, N, nom, c->d_gk);
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "gflow_deriv_kernel");
         // RK stages of both parts
         const int blocks = (int)std::min<long>((L + 255) / 256, 1216);

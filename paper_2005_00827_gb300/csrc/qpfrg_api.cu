@@ -193,7 +193,7 @@ void qpfrg_destroy(qpfrg_t c)
                         c->tc.Bpp[0], c->tc.Bpp[1], c->tc.Bcr[0], c->tc.Bcr[1], c->tc.Bd[0], c->tc.Bd[1],
                         c->tc.VT, c->d_tc_err, c->d_xij, c->d_bnd, c->d_qxl, c->d_qyl, c->d_kp, c->d_kcs, c->d_xij_f,
                         c->d_ptab, c->d_jgrid, c->d_repgrid, c->d_lrepQ, c->d_lnimg, c->d_limg, c->d_ltask,
-                        c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views};
+                        c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views, c->d_kfx, c->d_pfx, c->d_events};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     }
@@ -374,11 +374,11 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
         (s = dev_alloc(c, &c->d_k, n3, "k")) || (s = dev_alloc(c, &c->d_acc, n3, "acc")) ||
         (s = dev_alloc(c, &c->d_Vf, n3, "V fp32")) || (s = dev_alloc(c, &c->d_Z, N, "Z")) ||
         (s = dev_alloc(c, &c->d_Zwork, N, "Z work")) || (s = dev_alloc(c, &c->d_ones, N, "ones")) ||
-        (s = dev_alloc(c, &c->d_sig, 2 * N, "sigma chord")) || (s = dev_alloc(c, &c->d_red, 5, "reduction")) ||
-        (s = dev_alloc(c, &c->d_sym, 4, "symmetry test")))
+        (s = dev_alloc(c, &c->d_sig, 4 * N + 1, "sigma chord")) || (s = dev_alloc(c, &c->d_red, 5, "reduction")) ||
+        (s = dev_alloc(c, &c->d_sym, 5, "symmetry test")))
         return fail(s);
     if (!tcmode && (s = contract_alloc(c)) != QPFRG_OK) return fail(s);
-    e = cudaMallocHost((void **)&c->h_red, 9 * sizeof(unsigned long long));
+    e = cudaMallocHost((void **)&c->h_red, 10 * sizeof(unsigned long long));
     if (e != cudaSuccess) return fail(cuda_fail(c, e, "cudaMallocHost"));
     if (c->opt.sigma_ode && (s = gflow_alloc(c)) != QPFRG_OK) return fail(s);
 
@@ -400,6 +400,11 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
             return fail(s);
         cudaMemcpy(c->d_jirr, jirr.data(), jirr.size() * sizeof(int), cudaMemcpyHostToDevice);
         cudaMemcpy(c->d_rep, rep.data(), N * sizeof(int), cudaMemcpyHostToDevice);
+        if (c->d_ptab) {
+            // boundary pairs of the reduced self-energies: eight per loop point and target
+            c->max_events = (unsigned)std::min<long>(1L << 21, 8L * pb.M * c->n_irr);
+            if ((s = dev_alloc(c, &c->d_events, c->max_events, "boundary pairs")) != QPFRG_OK) return fail(s);
+        }
         if (pb.mode == QPFRG_GRID_WEDGE) {
             // frequency grid of the wedge kernels: zone-edge patches j = m N/4
             // get slots of their own
@@ -702,7 +707,7 @@ static qpfrg_status make_child(qpfrg_ctx *parent, double U, double lambda0, doub
         qpfrg_destroy(c);
         return s;
     }
-    if (cudaMallocHost((void **)&c->h_red, 9 * sizeof(unsigned long long)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&c->h_red, 10 * sizeof(unsigned long long)) != cudaSuccess) {
         qpfrg_destroy(c);
         return QPFRG_ERR_OOM;
     }
@@ -891,19 +896,15 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->d_acc, Z, c->pb.N * sizeof(double), cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "set_state upload");
-    qpfrg_status st = launch_state_check(c, c->d_k, c->d_acc, wedge, tol);
-    if (st == QPFRG_OK && c->rows_ok) st = launch_stage_prep(c, c->d_k, c->d_acc, 1);
+    qpfrg_status st = launch_sym_test(c, c->d_k, c->d_acc, 1);
     if (st != QPFRG_OK) return st;
-    if (c->rows_ok && (e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 4 * sizeof(unsigned long long),
-                                           cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
-        return cuda_fail(c, e, "set_state check");
-    if ((e = cudaMemcpyAsync(c->h_red, c->d_red, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+    if ((e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                              c->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state check");
-    if (c->h_red[1] || c->h_red[3]) return set_err(c, QPFRG_ERR_NONFINITE, "state image holds NaN or Inf");
+    if (c->h_red[9]) return set_err(c, QPFRG_ERR_NONFINITE, "state image holds NaN or Inf");
     double m = 0.0;
-    std::memcpy(&m, &c->h_red[0], sizeof(double));
+    std::memcpy(&m, &c->h_red[5], sizeof(double));
     if ((e = cudaMemcpyAsync(c->d_V, c->d_k, n3_of(c) * sizeof(double), cudaMemcpyDeviceToDevice, c->stream)) !=
             cudaSuccess ||
         (e = cudaMemcpyAsync(c->d_Z, c->d_acc, c->pb.N * sizeof(double), cudaMemcpyDeviceToDevice, c->stream)) !=
@@ -913,7 +914,7 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
         (e = cudaMemcpyAsync(c->d_gy, Z + c->pb.N, gflow_small_len(c) * sizeof(double), cudaMemcpyHostToDevice,
                              c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state (self-energy ODE)");
-    c->c4v_state = wedge && c->h_red[4] == 0;
+    c->c4v_state = wedge && c4v_within(c, tol);
     // The row orbits: every precision's contraction stays within its own
     // rounding of the unreduced one (the tensor-core flow keeps the tolerance
     // of the state's symmetry).  The slopes of the self-energy ODE set Z, K and

@@ -247,6 +247,7 @@ struct qpfrg_ctx {
     std::vector<double> fk;      // M x 2
     std::vector<double> fw;      // M
     double fw_max = 0.0;         // max of fw
+    double fx_min = 0.0, fx_max = 0.0;   // range of the dispersion over the fine points
     std::vector<int> fpatch;     // M
 
     // device geometry
@@ -259,8 +260,10 @@ struct qpfrg_ctx {
     float *d_xij_f = nullptr;    // N: xi(k_F(j)) in FP32
     float4 *d_bnd = nullptr;     // N: (cos hi, cos lo, sin hi, sin lo) of the ray between wedges j-1 and j
     float *d_qxl = nullptr, *d_qyl = nullptr;   // M: FP32 residuals kx - (float)kx, ky - (float)ky
-    float4 *d_kp = nullptr;      // [target][p]: k_j + p as FP32 hi/lo pairs (self-energy scratch)
-    float4 *d_kcs = nullptr;     // [target]: cos/sin of k_j (self-energy scratch)
+    float4 *d_kp = nullptr;      // [patch j][p]: k_j + p as FP32 hi/lo pairs (self-energy scratch)
+    int2 *d_kfx = nullptr;       // the same in fixed point
+    int2 *d_pfx = nullptr;       // M: fine points in fixed point (angle_fx)
+    float4 *d_kcs = nullptr;     // [patch j]: cos/sin of k_j (self-energy scratch)
     uint8_t *d_rtab = nullptr;   // patch of r per (irreducible target, p, q) of the flow's Z (sigma.cu)
     bool rtab_tried = false;     // built, or found not to fit, once per context
     uint8_t *d_ptab = nullptr;   // W rows x kProjStride bytes: cell table of the FP32 wedge projection (wedge mode, N <= 254)
@@ -320,7 +323,9 @@ struct qpfrg_ctx {
     // Z, K, A (N each) and Abar; the binned two-loop term on the grid
     double *d_gy = nullptr, *d_gys = nullptr, *d_gk = nullptr, *d_gacc = nullptr;
     double *d_gzka = nullptr, *d_gt2 = nullptr;
-    double *d_sig = nullptr;     // N x 2 Re Sigma at xi_j +- 2T
+    double *d_sig = nullptr;     // chord slopes per target slot, per patch, corrections, slopes of every patch (N each), count of d_events
+    int4 *d_events = nullptr;    // pairs on a boundary between patches (sigma.cu)
+    unsigned max_events = 0;
     int *d_jirr = nullptr;       // C4v-irreducible patches 0..N/8 (wedge mode)
     int *d_rep = nullptr;        // slot of each patch's representative in d_jirr
     int n_irr = 0;
@@ -402,18 +407,21 @@ qpfrg_status row_tasks(qpfrg_ctx *c, int qchunk, int *ntask);
 // V input is FP64 (precision FP64) or FP32 (MIXED); its permuted views are
 // those of the last launch_stage_prep / launch_stage_views.
 qpfrg_status contract_alloc(qpfrg_ctx *c);
+// the C4v test of V (FP64) and nz weight arrays alone, into c->d_sym
+qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz);
 qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz);
 qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z = nullptr, int nz = 0);
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out);
 
 // sigma.cu
 qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z,
-                            double *d_Zout, bool use_symmetry);
+                            double *d_Zout, bool state_symmetric);
 // d_K: the interaction flow's line weights with these Katanin factors (the
 // generic kernel); nullptr: the temperature flow's Z_a Z_b Z_c
 qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z,
                                double *d_re, double *d_im, const double *d_K = nullptr);
-qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K);
+qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                                double *d_slopes);
 
 // gflow.cu: interaction flow with the self-energy ODE
 long gflow_small_len(const qpfrg_ctx *c);
@@ -472,7 +480,6 @@ qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, in
 // ode.cu
 qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_V,
                              const double *d_k, double *d_acc, double *d_Vs, float *d_Vf);
-qpfrg_status launch_state_check(qpfrg_ctx *c, const double *d_V, const double *d_Z, bool c4v_test, double tol);
 qpfrg_status launch_rk_final(qpfrg_ctx *c, double h, double *d_V, const double *d_acc,
                              const double *d_k);
 qpfrg_status launch_check_finite(qpfrg_ctx *c, const double *d_x, long n);

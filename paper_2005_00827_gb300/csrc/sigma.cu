@@ -130,13 +130,32 @@ __device__ __forceinline__ float cross_ff(float4 b, float xh, float xl, float yh
     return s + t;
 }
 
+// Wedge of a folded momentum (float-float) from ray tests: the estimated wedge jc
+// and its neighbours.  bnd[m] = (cos hi, cos lo, sin hi, sin lo) of the ray
+// between wedges m-1 and m, at angle (m - 1/2) 2 pi / N.  margin: |r| times the
+// distance to the nearer of the wedge's rays.
+__device__ __forceinline__ int rays_ff(float xh, float xl, float yh, float yl, int jc, int N, const float4 *bnd,
+                                       float &margin)
+{
+    int j = jc;
+    for (int it = 0; it < 3; ++it) {
+        const int jj = j < 0 ? j + N : (j >= N ? j - N : j);
+        const int jn = jj + 1 == N ? 0 : jj + 1;
+        const float lo = cross_ff(bnd[jj], xh, xl, yh, yl), hi = cross_ff(bnd[jn], xh, xl, yh, yl);
+        const bool ccw_lo = lo >= 0.f;   // on or after the lower ray
+        const bool cw_hi = hi < 0.f;     // before the upper ray
+        margin = fminf(fabsf(lo), fabsf(hi));
+        if (ccw_lo && cw_hi) return jj;
+        j = ccw_lo ? jj + 1 : jj - 1;
+    }
+    return j < 0 ? j + N : (j >= N ? j - N : j);
+}
+
 // Guarded cases away from the zone edge: r = (k+p) - q in float-float, folded
-// (|r| < 3 pi; the fold decision is safe away from the zone edge), then the
-// point is tested against the boundary rays of the estimated wedge and its
-// neighbours.  bnd[m] = (cos hi, cos lo, sin hi, sin lo) of the ray between
-// wedges m-1 and m, at angle (m - 1/2) 2 pi / N.
+// (|r| < 3 pi; the fold decision is safe away from the zone edge), then the ray
+// tests.
 __device__ __forceinline__ int project_ff(float kph, float kpl, float kqh, float kql, float qxh, float qxl,
-                                          float qyh, float qyl, int jc, int N, const float4 *bnd)
+                                          float qyh, float qyl, int jc, int N, const float4 *bnd, float &margin)
 {
     const float C1 = 6.28318548f, C2 = -1.7484555e-7f;   // 2 pi = C1 + C2 (float-float)
     float xh, xl, yh, yl, e;
@@ -150,23 +169,16 @@ __device__ __forceinline__ int project_ff(float kph, float kpl, float kqh, float
     xl = xl + e - kx_ * C2;
     two_sum(yh, -ky_ * C1, yh, e);
     yl = yl + e - ky_ * C2;
-    int j = jc;
-    for (int it = 0; it < 3; ++it) {
-        const int jj = j < 0 ? j + N : (j >= N ? j - N : j);
-        const int jn = jj + 1 == N ? 0 : jj + 1;
-        const bool ccw_lo = cross_ff(bnd[jj], xh, xl, yh, yl) >= 0.f;   // on or after the lower ray
-        const bool cw_hi = cross_ff(bnd[jn], xh, xl, yh, yl) < 0.f;     // before the upper ray
-        if (ccw_lo && cw_hi) return jj;
-        j = ccw_lo ? jj + 1 : jj - 1;
-    }
-    return j < 0 ? j + N : (j >= N ? j - N : j);
+    return rays_ff(xh, xl, yh, yl, jc, N, bnd, margin);
 }
 
-// Per target and loop point, once per self-energy call: k_j + p as FP32
-// hi/lo pairs (from the FP64 sum, the same sum as the FP64 path) and, per
-// target, cos/sin of k_j's components.
+// Per target j and loop point, once per self-energy call: k_j + p as FP32
+// hi/lo pairs (from the FP64 sum, the same sum as the FP64 path) and in fixed
+// point, and, per target, cos/sin of k_j's components.  The pair kernels convert
+// nothing in FP64 (a conversion per record and loop point in every CTA took a
+// tenth of the chord kernel at 256 points per patch, 40 % at 64).
 __global__ void kp_table_kernel(const double *kf, const int *jlist, int nj, const double *kx64, const double *ky64,
-                                int M, float4 *kp, float4 *kcs)
+                                int M, float4 *kp, int2 *kfx, float4 *kcs)
 {
     const long total = (long)nj * M;
     for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
@@ -174,12 +186,14 @@ __global__ void kp_table_kernel(const double *kf, const int *jlist, int nj, cons
         const int j = jlist ? jlist[ji] : ji;
         const double x = kf[2 * j] + kx64[p], y = kf[2 * j + 1] + ky64[p];
         const float xh = (float)x, yh = (float)y;
-        kp[idx] = make_float4(xh, (float)(x - xh), yh, (float)(y - yh));
+        const float xl = (float)(x - xh), yl = (float)(y - yh);
+        kp[(long)j * M + p] = make_float4(xh, xl, yh, yl);
+        if (kfx) kfx[(long)j * M + p] = make_int2(angle_fx((double)xh + (double)xl), angle_fx((double)yh + (double)yl));
         if (p == 0) {
             double sx, cx, sy, cy;
             sincos(kf[2 * j], &sx, &cx);
             sincos(kf[2 * j + 1], &sy, &cy);
-            kcs[ji] = make_float4((float)cx, (float)sx, (float)cy, (float)sy);
+            kcs[j] = make_float4((float)cx, (float)sx, (float)cy, (float)sy);
         }
     }
 }
@@ -202,8 +216,8 @@ struct SigmaArgs {
     const double *kx64, *ky64;  // FP64 fine momenta (guarded FP32 projection)
     const double *xij;          // xi(k_F(j)), FP64
     const float4 *bnd;          // boundary rays of the wedges, float-float (FP32 projection fallback)
-    const float4 *kp;           // [target][p]: k_j + p as (x hi, x lo, y hi, y lo)
-    const float4 *kcs;          // [target]: cos, sin of k_j's components
+    const float4 *kp;           // [patch j][p]: k_j + p as (x hi, x lo, y hi, y lo)
+    const float4 *kcs;          // [patch j]: cos, sin of k_j's components
     const float *qxl, *qyl;     // FP32 residuals of the fine momenta
     // scalars of the inner loop in R (a double scalar re-read inside the loop
     // would cost a conversion on the FP64 pipe per use)
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(256) sigma_kernel(SigmaArgs<R> A)
     __shared__ R s_k[4];
     if (tid == 0) {
         if (f32) {
-            const float4 k4 = A.kcs[jidx];
+            const float4 k4 = A.kcs[j];
             s_k[0] = (R)k4.x; s_k[1] = (R)k4.y; s_k[2] = (R)k4.z; s_k[3] = (R)k4.w;
         } else {
             double sx, cx, sy, cy;
@@ -293,7 +307,7 @@ __global__ void __launch_bounds__(256) sigma_kernel(SigmaArgs<R> A)
         R *rec = s_rec + (size_t)REC * i;
         if (f32) {
             // k_j + p as FP32 hi/lo pairs from the per-call table
-            const float4 k4 = A.kp[(long)jidx * M + p];
+            const float4 k4 = A.kp[(long)j * M + p];
             rec[0] = (R)k4.x;
             rec[10] = (R)k4.y;
             rec[1] = (R)k4.z;
@@ -370,8 +384,9 @@ __global__ void __launch_bounds__(256) sigma_kernel(SigmaArgs<R> A)
                     cw = project32_guarded(x, y, Na, inv_dth, dth, jc);
                     if (cw == -1) {
                         // near a wedge boundary: float-float decision on the FP32 pipes
+                        float margin;
                         cw = project_ff((float)r[0], (float)r[10], (float)r[1], (float)r[11], (float)qx, qxl,
-                                        (float)qy, qyl, jc, Na, s_bnd);
+                                        (float)qy, qyl, jc, Na, s_bnd, margin);
                     } else if (cw == -2) {
                         // zone edge or origin: the exact FP64 projection
                         const int p = a * P + (i % nt) * nr + i / nt;
@@ -487,6 +502,7 @@ __global__ void __launch_bounds__(256) sigma_kernel(SigmaArgs<R> A)
 constexpr int SF_QPT = 2;
 constexpr int SF_QB = 4;        // default blocks of 256 SF_QPT loop points q per CTA
 constexpr int SF_PCH = 1024;    // loop points p staged per pass
+constexpr int SF_QCAP = 1024;   // guarded pairs queued per pass
 constexpr int SF_SLOTS = 257;   // per-patch slots: c in 0..N (c = N is patch 0 again), padded to 257
 
 struct SigmaFastArgs {
@@ -494,11 +510,25 @@ struct SigmaFastArgs {
     FineTable<float> fine;
     const double *V, *Z, *kx64, *ky64, *kf;
     const float *xij_f, *qxl, *qyl;
+    double fold0, fold1;    // last doubles k with rint(k / 2 pi) = 0 and < 2
     const float4 *kp, *kcs, *bnd;
+    const int2 *kfx, *pfx;  // k_j + p and the fine points in fixed point
     const uint8_t *ptab;
     const uint8_t *rtab;    // patch of r per (target, p, q) (RT launches; rtab_build_kernel)
     const int *jlist;
+    // sym.mode == 2: target slots 0 .. N-1 are the patches or, where the C4v test
+    // of (V, Z) holds, the n_list targets of jlist (the other slots return)
+    SymMode sym;
+    int n_list;
+    const double *K;        // Katanin factors (interaction-flow lines; the GL kernels)
     double *sig;
+    // pairs on a boundary between patches met by a reduced launch, and per patch
+    // its own slope less its representative's (sigma_fix_kernel); only_full: run
+    // only when there were more pairs than the record holds
+    int4 *events;
+    unsigned *nevents, max_events;
+    bool only_full;
+    double *corr;
     float t, tp, mu, eta2, invT, cT, twoT, fourT;   // cT = log2(e) / T
     float tln2, kchord, eta2x4;                     // T ln 2, 4 T^2 + eta^2, 4 eta^2
     float inv_dth, dth;                             // N / 2 pi, 2 pi / N
@@ -508,9 +538,42 @@ struct SigmaFastArgs {
     // grid mode: pole energies E binned from e_min in bins of h, moments 0..4
     // of the offset from the bin centre, hist[target][moment][bin] (FP64)
     double *hist;
-    float e_min, inv_h, h;
-    int nbins;
+    float h;
+    // bin of E: c_int + rint(x), x = E / h + c_frac (1 / h = inv_h + inv_h_lo, so
+    // that the offset x - rint(x) keeps FP32 accuracy at every bin)
+    float inv_h, inv_h_lo, c_frac;
+    int nbins, c_int;
+    float w_max;            // largest quadrature weight
 };
+
+// Target of slot z; false where the slot has none.
+__device__ __forceinline__ bool sigma_target(const SigmaFastArgs &A, int z, int &j, bool &sym)
+{
+    sym = A.sym.mode == 2 ? sym_compact(A.sym) : A.jlist != nullptr;
+    if (sym && A.sym.mode == 2 && z >= A.n_list) return false;
+    j = sym ? A.jlist[z] : z;
+    return true;
+}
+
+// A target on a mirror line of the zone (the line through k_j, j a multiple of
+// N/8, which reflects patch a to 2j - a) has a sum symmetric under that mirror:
+// keep the patches a on one side of it with weight fac = 2 and half of each patch
+// the mirror maps onto itself (P loop points: angular index t < n_theta / 2).
+// fac = 0: the mirror patch carries this one.  mirror 2 leaves out the zone-edge
+// targets (j a multiple of N/4).
+__device__ __forceinline__ void mirror_part(int mirror, int N, int j, int a, int &fac, int &P)
+{
+    fac = 1;
+    if (!mirror || (8 * j) % N != 0 || (mirror == 2 && (4 * j) % N == 0)) return;
+    const int ma = ((2 * j - a) % N + N) % N;
+    if (ma == a) {
+        fac = 2;
+        P /= 2;
+    } else {
+        const int rel = ((a - j) % N + N) % N;
+        fac = (rel > 0 && 2 * rel < N) ? 2 : 0;
+    }
+}
 
 __device__ __forceinline__ float ex2_approx(float x)
 {
@@ -545,12 +608,30 @@ __device__ __forceinline__ int fx_patch(int kpx, int kpy, int qx, int qy, const 
     return e + (cr >= 0.f ? 1 : 0);
 }
 
+// The same for a pair that fx_patch left undecided, where r lies near the origin
+// (cells of three or more wedges, 1 % of all pairs at 48 patches and 4 % at 96):
+// the wedges are cones, so the table's cell of 2^s r decides as well, s <= 6
+// keeping the scaled position error below the cells' margin.
+__device__ __forceinline__ int fx_zoom(int kpx, int kpy, int qx, int qy, const unsigned char *tabc, const float2 *ray,
+                                       bool &slow)
+{
+    const int X = (int)((unsigned)kpx - (unsigned)qx);
+    const int Y = (int)((unsigned)kpy - (unsigned)qy);
+    const int s = min(max(__clz(max(abs(X), abs(Y))) - 1, 0), 6);
+    const float x = __int2float_rn(X), y = __int2float_rn(Y);
+    const int e = tabc[((Y << s) >> 24) * kProjStride + ((X << s) >> 24)];
+    const float2 rr = ray[e + 1];
+    const float cr = rr.x * y - rr.y * x;
+    slow = fmaxf(fabsf(x), fabsf(y)) > kFxEdge || fabsf(cr) < kFxGuard;
+    return e + (cr >= 0.f ? 1 : 0);
+}
+
 struct SfSmem {
-    size_t rA, rB, cz, ray, cd, rC, tab, hist, total;
+    size_t rA, rB, cz, ray, cd, ck, rC, tab, queue, total;
 };
 
-// nbins > 0: a histogram of nbins x 5 FP32 moments follows the table (grid mode)
-__host__ __device__ inline SfSmem sf_smem_layout(int pch, int nbins = 0)
+// (a launch that reads the patch table has no use for the queue)
+__host__ __device__ inline SfSmem sf_smem_layout(int pch, bool rt)
 {
     SfSmem L;
     L.rA = 0;                                  // pch + 1 records: room for a pad record
@@ -560,29 +641,108 @@ __host__ __device__ inline SfSmem sf_smem_layout(int pch, int nbins = 0)
     L.cd = L.ray + (size_t)8 * SF_SLOTS;
     L.rC = (L.cd + (size_t)4 * SF_SLOTS + 15) / 16 * 16;
     L.tab = (L.rC + (size_t)4 * (pch + 1) + 15) / 16 * 16;
-    L.hist = L.tab + ((size_t)kProjW * kProjStride + 15) / 16 * 16;
-    L.total = L.hist + (size_t)5 * 4 * nbins;
+    L.queue = L.tab + ((size_t)kProjW * kProjStride + 15) / 16 * 16;
+    L.ck = L.queue + (size_t)4 * (1 + SF_QCAP);
+    L.total = rt ? L.queue : L.ck + (size_t)4 * SF_SLOTS;
     return L;
 }
 
 // Patch of r for a lane that left the table path: near a ray or the origin
-// (float-float ray tests) or near the zone edge (FP64 projection).
-__device__ __noinline__ int sf_slow_patch(const SigmaFastArgs &A, int jidx, int j, int p, int q, float x, float y,
-                                          bool edge, const float4 *bnd)
+// (float-float ray tests) or near the zone edge.  There the FP64 fold decides: its
+// count rint(k / 2 pi) changes where k passes fold0 (pi) and fold1 (3 pi), the
+// last doubles of the lower count, so two FP64 additions and comparisons per
+// component give the folded momentum of project_fp64, and the wedge follows from
+// FP32 and float-float ray tests; only within 1e-11 of a ray, or of the origin,
+// does the FP64 projection run (its atan2 and divisions, 170 instructions at 64
+// clocks each per warp, made the CTAs of coinciding p and q the tail of the launch:
+// np48, Z of a symmetric vertex 4.5 -> 3.9 ms).  flags: 1 near the zone edge, 2
+// record a pair within 1e-9 of a ray or of the zone edge in A.events (correcting
+// its image targets on the spot cost the pair loop 600 bytes of spills).
+__device__ __noinline__ int sf_slow_patch(const SigmaFastArgs &A, int j, int p, int q, float x, float y, int flags,
+                                          const float4 *bnd)
 {
     const int N = A.pb.N;
-    int c = -2;
-    if (!edge) {
+    float margin = 0.f;
+    auto record = [&](int c) {
+        if (!(flags & 2)) return;
+        const unsigned n = atomicAdd(A.nevents, 1u);
+        if (n < A.max_events) A.events[n] = make_int4(j, p, q, c);
+    };
+    if (!(flags & 1)) {
         int jc;
-        c = project32_guarded(x, y, N, A.inv_dth, A.dth, jc);
+        const int c = project32_guarded(x, y, N, A.inv_dth, A.dth, jc);
+        if (c >= 0) return c;
         if (c == -1) {
-            const float4 k4 = A.kp[(long)jidx * A.pb.M + p];
-            c = project_ff(k4.x, k4.y, k4.z, k4.w, A.fine.kx[q], A.qxl[q], A.fine.ky[q], A.qyl[q], jc, N, bnd);
+            const float4 k4 = A.kp[(long)j * A.pb.M + p];
+            const int r = project_ff(k4.x, k4.y, k4.z, k4.w, A.fine.kx[q], A.qxl[q], A.fine.ky[q], A.qyl[q], jc, N, bnd,
+                                     margin);
+            if (margin < 1e-9f) record(r);
+            return r;
         }
     }
-    if (c < 0)
-        c = project_fp64((A.kf[2 * j] + A.kx64[p]) - A.kx64[q], (A.kf[2 * j + 1] + A.ky64[p]) - A.ky64[q], A.pb);
+    const double kx = (A.kf[2 * j] + A.kx64[p]) - A.kx64[q], ky = (A.kf[2 * j + 1] + A.ky64[p]) - A.ky64[q];
+    const double nx = kx > A.fold0 ? -kTwoPi : (kx < -A.fold0 ? kTwoPi : 0.0);
+    const double ny = ky > A.fold0 ? -kTwoPi : (ky < -A.fold0 ? kTwoPi : 0.0);
+    const double fx = kx + nx, fy = ky + ny;
+    const float xh = (float)fx, yh = (float)fy, xl = (float)(fx - (double)xh), yl = (float)(fy - (double)yh);
+    const float r2 = xh * xh + yh * yh;
+    if (kx > A.fold1 || kx < -A.fold1 || ky > A.fold1 || ky < -A.fold1 || r2 < 1e-8f) {
+        const int c = project_fp64(kx, ky, A.pb);
+        record(c);
+        return c;
+    }
+    // distance to the zone edge: pi = 3.14159274f - 8.7422777e-8f
+    const float ex = (3.14159274f - fabsf(xh)) - (copysignf(xl, xh * xl) + 8.7422777e-8f);
+    const float ey = (3.14159274f - fabsf(yh)) - (copysignf(yl, yh * yl) + 8.7422777e-8f);
+    int jc;
+    rint_add(atan2_poly(yh, xh) * A.inv_dth, jc);
+    int c = rays_ff(xh, xl, yh, yl, jc, N, bnd, margin);
+    if (margin < 1e-11f) c = project_fp64(kx, ky, A.pb);
+    if (fminf(fminf(fabsf(ex), fabsf(ey)), margin) < 1e-9f) record(c);
     return c;
+}
+
+// Chord term of one pair with r in patch c, in FP64 from the tables (rare).
+__device__ __noinline__ double sf_pair_term(const SigmaFastArgs &A, int j, int p, int q, int c)
+{
+    const int N = A.pb.N, PP = A.pb.P, a = p / PP, b = q / PP;
+    auto z = [&](int k) { return A.Z ? A.Z[k] : 1.0; };
+    const bool qp = A.pb.propagator == QPFRG_PROP_QP;
+    const double Za = z(a), Zb = z(b), Zc = z(c), invT = A.invT;
+    const double cx = cos(A.kf[2 * j] + A.kx64[p] - A.kx64[q]), cy = cos(A.kf[2 * j + 1] + A.ky64[p] - A.ky64[q]);
+    const double xp = (qp ? Za : 1.0) * A.fine.xi[p], xq = (qp ? Zb : 1.0) * A.fine.xi[q];
+    const double xr = (qp ? Zc : 1.0) * (-2.0 * A.pb.t * (cx + cy) - 4.0 * A.pb.tp * cx * cy - A.pb.mu);
+    auto f = [&](double x) { return 1.0 / (1.0 + exp(x * invT)); };
+    const double F = f(xp) * f(-xq) * f(-xr) + f(-xp) * f(xq) * f(xr);
+    const double *V = A.V + ((long)j * N + a) * N;
+    double amp = (double)A.fine.w[p] * A.fine.w[q] * Za * Zb * Zc * (2.0 * V[b] * V[b] - V[b] * V[c]) * F;
+    if (A.K)
+        amp *= (A.K[a] * Za * (Zb + Zc) + A.K[b] * Zb * (Za + Zc) + A.K[c] * Zc * (Za + Zb)) * (1.0 / 6.0);
+    const double d0 = A.xij_f[j] - (xq + xr - xp), dp = d0 + A.twoT, dm = d0 - A.twoT;
+    return amp * ((double)A.eta2 - dp * dm) / ((dp * dp + A.eta2) * (dm * dm + A.eta2));
+}
+
+// A recorded pair (p, q) of target j, patch c, lies on a boundary: every image
+// target that copies j's sum is corrected where its own pair is decided
+// otherwise, so that each patch keeps its own sum.
+__global__ void __launch_bounds__(128) sigma_fix_kernel(SigmaFastArgs A)
+{
+    const int N = A.pb.N, PP = A.pb.P, nt = A.pb.n_theta, nr = A.pb.n_r;
+    const unsigned n = min(*A.nevents, A.max_events);
+    auto image = [&](int g, int k) {
+        const int a = k / PP, l = k - a * PP, t = l / nr, s = l - t * nr;
+        return c4v_apply(g, a, N, 1) * PP + ((g & 4) ? nt - 1 - t : t) * nr + s;
+    };
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < 7u * n; i += gridDim.x * blockDim.x) {
+        const int4 e = A.events[i / 7u];
+        const int g = 1 + (int)(i % 7u), j = e.x, jg = c4v_apply(g, j, N, 1);
+        bool seen = jg == j;       // one element per image target
+        for (int k = 1; k < g; ++k) seen |= c4v_apply(k, j, N, 1) == jg;
+        if (seen) continue;
+        const int pg = image(g, e.y), qg = image(g, e.z);
+        const int own = sf_slow_patch(A, jg, pg, qg, 0.f, 0.f, 1, A.bnd), copied = c4v_apply(g, e.w, N, 1);
+        if (own != copied) atomicAdd(&A.corr[jg], sf_pair_term(A, jg, pg, qg, own) - sf_pair_term(A, jg, pg, qg, copied));
+    }
 }
 
 // The patch of r = k_j + p - q for every target of the list (position jidx),
@@ -617,8 +777,7 @@ __global__ void __launch_bounds__(256) rtab_build_kernel(SigmaFastArgs A, uint8_
             ray[i] = i <= N ? make_float2(bd.x, bd.z) : make_float2(0.f, 0.f);
         }
         for (int i = tid; i < PP; i += blockDim.x) {
-            const float4 k4 = A.kp[(long)jidx * M + a * PP + i];
-            rec[i] = make_int2(angle_fx((double)k4.x + (double)k4.y), angle_fx((double)k4.z + (double)k4.w));
+            rec[i] = A.kfx[(long)j * M + a * PP + i];
         }
     }
     __syncthreads();
@@ -627,7 +786,7 @@ __global__ void __launch_bounds__(256) rtab_build_kernel(SigmaFastArgs A, uint8_
     if (iq >= M) return;
     const int b = iq / PP, rem = iq - b * PP;
     const int qq = b * PP + (rem % A.pb.n_theta) * A.pb.n_r + rem / A.pb.n_theta;
-    const int qx = angle_fx(A.kx64[qq]), qy = angle_fx(A.ky64[qq]);
+    const int qx = A.pfx[qq].x, qy = A.pfx[qq].y;
     // the thread's P bytes, as P/8 words of eight records (P a multiple of 16)
     uint2 *out = reinterpret_cast<uint2 *>(rtab) + ((long)jidx * N + a) * (long)(PP / 8) * M + iq;
     for (int i0 = 0; i0 < PP; i0 += 8) {
@@ -638,9 +797,10 @@ __global__ void __launch_bounds__(256) rtab_build_kernel(SigmaFastArgs A, uint8_
             float x, y;
             bool slow;
             int c = fx_patch(kr.x, kr.y, qx, qy, tabc, ray, x, y, slow);
+            if (slow) c = fx_zoom(kr.x, kr.y, qx, qy, tabc, ray, slow);
             if (slow) {
                 const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
-                c = sf_slow_patch(A, jidx, j, p, qq, x * kRadPerFx, y * kRadPerFx, edge, A.bnd);
+                c = sf_slow_patch(A, j, p, qq, x * kRadPerFx, y * kRadPerFx, edge ? 1 : 0, A.bnd);
             }
             w[(i - i0) >> 2] |= (unsigned)c << (8 * ((i - i0) & 3));
         }
@@ -652,34 +812,29 @@ __global__ void __launch_bounds__(256) rtab_build_kernel(SigmaFastArgs A, uint8_
 // multiple of 256 SF_QPT), so the vertex weight is a per-patch table:
 // cz[c] = (Z_c (2 V_jab^2 - V_jab V_jac), -, -2t l_c, -mu l_c); otherwise
 // cz[c] = (Z_c, Z_c V_jac, -2t l_c, -mu l_c) and the weight is formed per pair.
-template <bool TP0, bool UNIB, bool RT>
+// GL: the interaction flow's line weights, (1/6)[K_a Z_a (Z_b + Z_c) + K_b Z_b
+// (Z_a + Z_c) + K_c Z_c (Z_a + Z_b)] times Z_a Z_b Z_c.
+template <bool TP0, bool UNIB, bool RT, bool GL>
 __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
 {
     const int N = A.pb.N, M = A.pb.M;
     const int a = blockIdx.y, jidx = blockIdx.z;
-    const int j = A.jlist ? A.jlist[jidx] : jidx;
+    int j;
+    bool sym = true;
+    if (RT) {                   // the table's targets
+        j = A.jlist[jidx];
+    } else {
+        if (A.only_full && *A.nevents <= A.max_events) return;
+        if (!sigma_target(A, jidx, j, sym)) return;      // uniform over the CTA
+    }
     const int tid = threadIdx.x;
     const bool qp = A.pb.propagator == QPFRG_PROP_QP;
-    // A target on a mirror line of the zone (theta_j = 0 or pi/4) has a sum
-    // symmetric under that mirror: keep the patches a on one side of it with
-    // weight 2 and half of each patch the mirror maps onto itself.
-    int fac = 1, P = A.pb.P;
-    if (A.mirror) {
-        int ma = -1;
-        if (j == 0) ma = (N - a) % N;
-        else if (8 * j == N) ma = ((N / 4 - a) % N + N) % N;
-        if (ma == a) {
-            fac = 2;
-            P = A.pb.P / 2;     // angular index t < n_theta / 2
-        } else if (ma >= 0) {
-            const int rel = j == 0 ? a : ((a - N / 8) % N + N) % N;
-            fac = (rel > 0 && 2 * rel < N) ? 2 : 0;
-        }
-    }
+    int fac, P = A.pb.P;
+    mirror_part(sym ? A.mirror : 0, N, j, a, fac, P);
     if (fac == 0) return;       // the mirror patch carries this one (uniform over the CTA)
     const int PP = A.pb.P;      // points per patch (record and loop-point indexing)
     const int pch = P < SF_PCH ? P : SF_PCH;
-    const SfSmem L = sf_smem_layout(pch);
+    const SfSmem L = sf_smem_layout(pch, RT);
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *rA = reinterpret_cast<float4 *>(smem_raw + L.rA);   // (k+p)_x, (k+p)_y (fixed point), cos of both
@@ -688,9 +843,13 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
     float2 *ray = reinterpret_cast<float2 *>(smem_raw + L.ray);
     float *cd = reinterpret_cast<float *>(smem_raw + L.cd);     // -4 t' l_c
     float *rC = reinterpret_cast<float *>(smem_raw + L.rC);     // x_j + x_p + 2T
+    float *ck = reinterpret_cast<float *>(smem_raw + L.ck);     // K_c Z_c (GL)
     unsigned char *tab = smem_raw + L.tab;
+    int &s_nq = *reinterpret_cast<int *>(smem_raw + L.queue);              // guarded pairs of a pass
+    unsigned *queue = reinterpret_cast<unsigned *>(smem_raw + L.queue) + 1;
 
     if (!RT) {
+        if (tid == 0) s_nq = 0;
         const uint4 *src = reinterpret_cast<const uint4 *>(A.ptab);
         uint4 *dst = reinterpret_cast<uint4 *>(tab);
         const int n16 = (kProjW * kProjStride + 15) / 16;
@@ -698,8 +857,11 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
     }
     const double *Vja = A.V + ((long)j * N + a) * N;
     // per-patch slots; with UNIB the weight column is filled per q block (b)
+    const float Za = A.Z ? (float)A.Z[a] : 1.f;
+    const float kza = GL ? (float)A.K[a] * Za : 0.f;
     auto fill_slots = [&](int b) {
         const float vb = UNIB ? (float)Vja[b] : 0.f;
+        const float Zb = UNIB && GL ? (A.Z ? (float)A.Z[b] : 1.f) : 0.f, kzb = UNIB && GL ? (float)A.K[b] * Zb : 0.f;
         for (int i = tid; i < SF_SLOTS; i += blockDim.x) {
             if (i <= N) {
                 const int cc = i == N ? 0 : i;
@@ -707,7 +869,10 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                 const float lz = qp ? Zc : 1.f;
                 const float vc = (float)Vja[cc];
                 const float lzc = lz * A.cT;     // energies of r in units of T / log2(e)
-                cz[i] = UNIB ? make_float4(Zc * (2.f * vb * vb - vb * vc), 0.f, -2.f * A.t * lzc, -A.mu * lzc)
+                const float kzc = GL ? (float)A.K[cc] * Zc : 0.f;
+                if (GL) ck[i] = kzc;
+                const float gl = UNIB && GL ? (kza * (Zb + Zc) + kzb * (Za + Zc) + kzc * (Za + Zb)) * (1.f / 6.f) : 1.f;
+                cz[i] = UNIB ? make_float4(gl * Zc * (2.f * vb * vb - vb * vc), 0.f, -2.f * A.t * lzc, -A.mu * lzc)
                              : make_float4(Zc, Zc * vc, -2.f * A.t * lzc, -A.mu * lzc);
                 cd[i] = -4.f * A.tp * lzc;
                 const float4 bd = A.bnd[cc];
@@ -715,15 +880,15 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             } else {
                 cz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 cd[i] = 0.f;
+                if (GL) ck[i] = 0.f;
                 ray[i] = make_float2(0.f, 0.f);
             }
         }
     };
     int b_slots = UNIB ? (blockIdx.x * A.qb * 256 * SF_QPT) / PP : 0;
     fill_slots(b_slots);
-    const float Za = A.Z ? (float)A.Z[a] : 1.f;
     const float lza = qp ? Za : 1.f;
-    const float4 kcs = A.kcs[jidx];
+    const float4 kcs = A.kcs[j];
     const float xj = A.xij_f[j];
 
     const unsigned char *tabc = tab + (kProjW / 2) * (kProjStride + 1);   // the cell of the origin
@@ -731,14 +896,13 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
     auto stage = [&](int p0, int cnt) {
         for (int i = tid; i < cnt; i += blockDim.x) {
             const int p = a * PP + p0 + i;
-            const float4 k4 = A.kp[(long)jidx * M + p];
+            const int2 kf = RT ? make_int2(0, 0) : A.kfx[(long)j * M + p];   // (the table needs no momenta)
             const float cpx = A.fine.cx[p], spx = A.fine.sx[p], cpy = A.fine.cy[p], spy = A.fine.sy[p];
             const float xp = lza * A.fine.xi[p];
             float fp, fcp;
             sfermi(xp, A.invT, fp, fcp);
             const float wp = A.fine.w[p];
-            const int kx = angle_fx((double)k4.x + (double)k4.y), ky = angle_fx((double)k4.z + (double)k4.w);
-            rA[i] = make_float4(__int_as_float(kx), __int_as_float(ky), kcs.x * cpx - kcs.y * spx,
+            rA[i] = make_float4(__int_as_float(kf.x), __int_as_float(kf.y), kcs.x * cpx - kcs.y * spx,
                                 kcs.z * cpy - kcs.w * spy);
             rB[i] = make_float4(kcs.y * cpx + kcs.x * spx, kcs.w * cpy + kcs.z * spy, wp * fp, wp * fcp);
             rC[i] = xj + xp;
@@ -772,6 +936,7 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
         float2 cq[SF_QPT], sq[SF_QPT];
         float fqp[SF_QPT], fcqp[SF_QPT], v2[SF_QPT], vab[SF_QPT], mxq[SF_QPT];
         float2 acc = make_float2(0.f, 0.f);     // the SF_QPT = 2 loop points as the two lanes
+        float ga[SF_QPT], gb[SF_QPT], gc[SF_QPT];   // GL: bracket = ga + gb Z_c + gc K_c Z_c
         int qi[SF_QPT], qx[SF_QPT], qy[SF_QPT];
         const uint8_t *rq[SF_QPT];   // RT: the patch-of-r rows of this thread's loop points q
 #pragma unroll
@@ -784,8 +949,8 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             const int qq = b * PP + (rem % A.pb.n_theta) * A.pb.n_r + rem / A.pb.n_theta;
             qi[k] = qq;
             const float Zb = A.Z ? (float)A.Z[b] : 1.f;
-            qx[k] = angle_fx(A.kx64[qq]);
-            qy[k] = angle_fx(A.ky64[qq]);
+            qx[k] = A.pfx[qq].x;
+            qy[k] = A.pfx[qq].y;
             cq[k] = make_float2(A.fine.cx[qq], A.fine.cy[qq]);
             sq[k] = make_float2(A.fine.sx[qq], A.fine.sy[qq]);
             const float xq = (qp ? Zb : 1.f) * A.fine.xi[qq];
@@ -794,6 +959,12 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             const float pref = valid ? Za * Zb * A.fine.w[qq] : 0.f;
             fqp[k] = fq * pref;
             fcqp[k] = fcq * pref;
+            if (GL && !UNIB) {
+                const float kzb = (float)A.K[b] * Zb;
+                ga[k] = (kza * Zb + kzb * Za) * (1.f / 6.f);
+                gb[k] = (kza + kzb) * (1.f / 6.f);
+                gc[k] = (Za + Zb) * (1.f / 6.f);
+            }
             vab[k] = (float)Vja[b];
             v2[k] = 2.f * vab[k] * vab[k];
             mxq[k] = -xq;
@@ -826,7 +997,8 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                         const float ex = ex2_approx(x);
                         const float a = rb[r].z * fcqp[k];
                         const float d = fmaf(rb[r].w, fqp[k], -a);
-                        const float w = UNIB ? z.x : fmaf(-vab[k], z.y, z.x * v2[k]);
+                        float w = UNIB ? z.x : fmaf(-vab[k], z.y, z.x * v2[k]);
+                        if (GL && !UNIB) w *= fmaf(gc[k], ck[c[r][k]], fmaf(gb[k], z.x, ga[k]));
                         const float sm = upp[r] + mxq[k];
                         if (k == 0) { xr.x = x; fr.x = ex; aq.x = a; dq.x = d; amp.x = w; sum.x = sm; }
                         else        { xr.y = x; fr.y = ex; aq.y = a; dq.y = d; amp.y = w; sum.y = sm; }
@@ -878,8 +1050,10 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                 }
             } else {
             // two records per iteration: the patches of all 2 x SF_QPT pairs
-            // first, one rarely taken branch for the guarded ones, then the
-            // arithmetic of all of them (one large block for the scheduler);
+            // first, one rarely taken branch that queues the guarded ones, then the
+            // arithmetic of all of them with the table's patch (one large block for
+            // the scheduler; a call for the exact patch here spilled registers in
+            // every iteration, 40 % of the time);
             // an odd count reads the zero-weight pad record after the last one;
             // the loop is unrolled four times (eight records per trip, 122
             // registers: the loop overhead amortised, more independent work)
@@ -894,7 +1068,7 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                     upp[r] = rC[i + r];
                 }
                 int c[2][SF_QPT];
-                bool slow_any = false;
+                unsigned slow_mask = 0;
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -903,27 +1077,88 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                         bool slow;
                         c[r][k] = fx_patch(__float_as_int(ra[r].x), __float_as_int(ra[r].y), qx[k], qy[k], tabc, ray,
                                            x, y, slow);
-                        slow_any |= slow;
+                        slow_mask |= slow ? 1u << (2 * r + k) : 0u;
                     }
-                if (slow_any) {
-#pragma unroll
-                    for (int r = 0; r < 2; ++r)
-#pragma unroll
-                        for (int k = 0; k < SF_QPT; ++k) {
-                            float x, y;
-                            bool slow;
-                            fx_patch(__float_as_int(ra[r].x), __float_as_int(ra[r].y), qx[k], qy[k], tabc, ray, x, y,
-                                     slow);
-                            // the pad record (weight 0) keeps its table patch
-                            if (slow && i + r < cnt) {
-                                const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
-                                c[r][k] = sf_slow_patch(A, jidx, j, a * PP + p0 + i + r, qi[k], x * kRadPerFx,
-                                                        y * kRadPerFx, edge, A.bnd);
-                            }
+                if (__any_sync(0xffffffffu, slow_mask != 0)) {
+                    // taken by the whole warp (a branch per lane left the lanes apart
+                    // for the rest of the unrolled trip: 84 instead of 40 issue slots
+                    // per pair); one copy of the code for the four pairs
+#pragma unroll 1
+                    for (int e = 0; e < 2 * SF_QPT; ++e) {
+                        const bool r1 = e >= SF_QPT, k1 = (e & 1) != 0;
+                        bool slow;
+                        const int cc = fx_zoom(__float_as_int(r1 ? ra[1].x : ra[0].x), __float_as_int(r1 ? ra[1].y : ra[0].y),
+                                               k1 ? qx[1] : qx[0], k1 ? qy[1] : qy[0], tabc, ray, slow);
+                        const bool mine = (slow_mask >> e & 1u) != 0;
+                        const int rec = i + (r1 ? 1 : 0);
+                        if (mine && slow && rec < cnt) {     // (the pad record has weight 0)
+                            const int at = atomicAdd(&s_nq, 1);
+                            if (at < SF_QCAP) queue[at] = (unsigned)rec | (unsigned)((k1 ? 256 : 0) + tid) << 12;
                         }
+                        __syncwarp();
+                        if (mine && !r1 && !k1) c[0][0] = cc;
+                        if (mine && !r1 && k1) c[0][1] = cc;
+                        if (mine && r1 && !k1) c[1][0] = cc;
+                        if (mine && r1 && k1) c[1][1] = cc;
+                    }
                 }
                 pair_math(ra, rb, upp, c);
             }
+            // the guarded pairs of this pass: where the exact patch differs from the
+            // table's, the difference of the two chord terms
+            __syncthreads();
+            const int nq = s_nq;
+            __syncthreads();
+            if (tid == 0) s_nq = 0;
+            const bool over = nq > SF_QCAP;      // more than the queue holds: look at every pair again
+            const int ntot = over ? cnt * (256 * SF_QPT) : nq;
+            for (int e = tid; e < ntot; e += 256) {
+                const unsigned en = over ? (unsigned)(e % cnt) | (unsigned)(e / cnt) << 12 : queue[e];
+                const int i = en & 4095u, iq = blk * (256 * SF_QPT) + (int)(en >> 12);
+                if (iq >= M) continue;
+                const int b = iq / PP, rem = iq - b * PP;
+                const int qq = b * PP + (rem % A.pb.n_theta) * A.pb.n_r + rem / A.pb.n_theta;
+                const float4 ra = rA[i], rb = rB[i];
+                // the patch the loop used
+                float x, y;
+                bool slow;
+                fx_patch(__float_as_int(ra.x), __float_as_int(ra.y), A.pfx[qq].x, A.pfx[qq].y, tabc, ray, x, y, slow);
+                if (!slow) continue;
+                const int c0 = fx_zoom(__float_as_int(ra.x), __float_as_int(ra.y), A.pfx[qq].x, A.pfx[qq].y, tabc, ray, slow);
+                if (!slow) continue;
+                const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
+                const bool fix = A.sym.mode == 2 && sym && (4 * j) % N != 0;   // the zone-edge targets have no images
+                const int c1 = sf_slow_patch(A, j, a * PP + p0 + i, qq, x * kRadPerFx, y * kRadPerFx,
+                                             (edge ? 1 : 0) | (fix ? 2 : 0), A.bnd);
+                if (c1 == c0) continue;
+                const float Zb = A.Z ? (float)A.Z[b] : 1.f, vb = (float)Vja[b];
+                const float xq = (qp ? Zb : 1.f) * A.fine.xi[qq];
+                float fq, fcq;
+                sfermi(xq, A.invT, fq, fcq);
+                const float pref = Za * Zb * A.fine.w[qq];
+                const float2 cr = __ffma2_rn(make_float2(ra.z, ra.w), make_float2(A.fine.cx[qq], A.fine.cy[qq]),
+                                             __fmul2_rn(make_float2(rb.x, rb.y),
+                                                        make_float2(A.fine.sx[qq], A.fine.sy[qq])));
+                const float aq = rb.z * (fcq * pref), dq = fmaf(rb.w, fq * pref, -aq);
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    const int cc = u ? c0 : c1;
+                    const float4 z = cz[cc];
+                    float xr = fmaf(cr.x + cr.y, z.z, z.w);
+                    if (!TP0) xr = fmaf(cr.x * cr.y, cd[cc], xr);
+                    float w = UNIB ? z.x : fmaf(-vb, z.y, z.x * (2.f * vb * vb));
+                    if (GL && !UNIB) {
+                        const float kzb = (float)A.K[b] * Zb;
+                        w *= ((kza * Zb + kzb * Za) + (kza + kzb) * z.x + (Za + Zb) * ck[cc]) * (1.f / 6.f);
+                    }
+                    const float F = fmaf(rcp_approx(1.f + ex2_approx(xr)), dq, aq);
+                    const float d0 = fmaf(xr, -A.tln2, rC[i] - xq);
+                    const float uu = fmaf(d0, d0, -A.kchord);
+                    const float t = w * F * uu * rcp_approx(fmaf(A.eta2x4 * d0, d0, uu * uu));
+                    acc.x += u ? -t : t;
+                }
+            }
+            __syncthreads();
             }
         }
         vsum -= (double)acc.x + (double)acc.y;   // the chord term is -u / den
@@ -945,136 +1180,218 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
     }
 }
 
-// Frequency-grid variant of sigma_fast_kernel:
-// instead of the chord slope, bin W F by pole energy E = x_q + x_r - x_p
-// (moments 0..4 of E - E_bin) in a shared-memory histogram per CTA, flushed to
-// the FP64 histogram once at the end (then sigma_grid_kernel).  A separate
-// kernel, so that the chord kernel of the flow keeps its own code generation.
-template <bool TP0, bool UNIB>
-__global__ void __launch_bounds__(256, 1) sigma_grid_fast_kernel(SigmaFastArgs A)
+// Frequency-grid variant of sigma_fast_kernel: instead of the chord slope, W F
+// binned by pole energy E = x_q + x_r - x_p (moments 0..4 of E about the bin
+// centre in units of half a bin) in a shared-memory histogram per CTA, flushed
+// to the FP64 histogram after every block of loop points q.
+//
+// What bounds it: the shared-memory adds, five or six per pair.  A float add on
+// shared memory is a compare-and-swap loop, so the histogram is 32-bit fixed
+// point with native integer reductions.  The lanes of a warp own neighbouring
+// radii of q, whose energies lie many bins apart (angular neighbours share
+// bins, and equal addresses serialise).  The scale of a flush period (1024
+// loop points q times the patch's points p) follows from a bound on the sum of
+// all its |W F| <= W_b max(f_p (1 - f_q), (1 - f_p) f_q), W_b the largest weight
+// over c, so no bin leaves +-2^30 (a pair is then hundreds of units), and one
+// addend stays below 2^21 units (rounded by adding 1.5 * 2^23, no conversion).
+// What moment 0 rounds off goes into a second word (LO) in units 2^30 / pairs
+// finer; the higher moments enter Sigma with (h/2|z - E|)^n <= 8^-n, which
+// carries their rounding below that of the FP32 pairs.  np48, 16 x 16 points, 10 targets, 512 frequencies: 26.0
+// -> 6.4 ms (58 -> 236 Gpair/s).
+//
+// Launch: grid (q splits, N patches a, targets), 512 threads, one CTA per SM
+// (the histogram).  NBS: words per moment (a constant, so that the moments are
+// immediate offsets), nbins <= NBS.
+constexpr int HF_THR = 512;
+constexpr int HF_QPT = 2;
+constexpr int HF_REC = 256;     // loop points p staged per pass
+constexpr int HF_QCAP = 1024;   // guarded pairs queued per pass
+
+struct HfSmem {
+    size_t rA, rB, cz, ray, cd, ck, wb, rC, queue, tab, hist, total;
+};
+
+__host__ __device__ inline HfSmem hf_smem_layout(int nbs, bool lo)
 {
-    const int N = A.pb.N, M = A.pb.M;
+    HfSmem L;
+    L.rA = 0;
+    L.rB = L.rA + (size_t)16 * HF_REC;
+    L.cz = L.rB + (size_t)16 * HF_REC;
+    L.ray = L.cz + (size_t)16 * SF_SLOTS;
+    L.cd = L.ray + (size_t)8 * SF_SLOTS;
+    L.ck = L.cd + (size_t)4 * SF_SLOTS;
+    L.wb = L.ck + (size_t)4 * SF_SLOTS;
+    L.rC = (L.wb + (size_t)4 * SF_SLOTS + 15) / 16 * 16;
+    L.queue = L.rC + (size_t)4 * HF_REC;
+    L.tab = L.queue + (size_t)4 * HF_QCAP;
+    L.hist = L.tab + ((size_t)kProjW * kProjStride + 15) / 16 * 16;
+    L.total = L.hist + (size_t)4 * nbs * (lo ? 6 : 5);
+    return L;
+}
+
+__device__ __forceinline__ void red_shared(unsigned addr, int v)
+{
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+template <int NBS, bool LO, bool GL>
+__global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastArgs A)
+{
+    const int N = A.pb.N, M = A.pb.M, PP = A.pb.P;
     const int a = blockIdx.y, jidx = blockIdx.z;
-    const int j = A.jlist ? A.jlist[jidx] : jidx;
+    int j;
+    bool sym;
+    if (!sigma_target(A, jidx, j, sym)) return;      // uniform over the CTA
+    int fac, P = PP;
+    mirror_part(sym ? A.mirror : 0, N, j, a, fac, P);
+    if (fac == 0) return;       // the mirror patch carries this one (uniform over the CTA)
     const int tid = threadIdx.x;
     const bool qp = A.pb.propagator == QPFRG_PROP_QP;
-    // A target on a mirror line of the zone (theta_j = 0 or pi/4) has a sum
-    // symmetric under that mirror: keep the patches a on one side of it with
-    // weight 2 and half of each patch the mirror maps onto itself.
-    // The mirror line through k_j (j a multiple of N/8) reflects patch a to 2j - a.
-    int fac = 1, P = A.pb.P;
-    if (A.mirror && (8 * j) % N == 0 && !(A.mirror == 2 && (4 * j) % N == 0)) {
-        const int ma = ((2 * j - a) % N + N) % N;
-        if (ma == a) {
-            fac = 2;
-            P = A.pb.P / 2;     // angular index t < n_theta / 2
-        } else {
-            const int rel = ((a - j) % N + N) % N;
-            fac = (rel > 0 && 2 * rel < N) ? 2 : 0;
-        }
-    }
-    if (fac == 0) return;       // the mirror patch carries this one (uniform over the CTA)
-    const int PP = A.pb.P;      // points per patch (record and loop-point indexing)
-    const int cap = SF_PCH / 2;     // room for the histogram
-    const int pch = P < cap ? P : cap;
-    const SfSmem L = sf_smem_layout(pch, A.nbins);
+    const HfSmem L = hf_smem_layout(NBS, LO);
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *rA = reinterpret_cast<float4 *>(smem_raw + L.rA);   // (k+p)_x, (k+p)_y, cos, sin of (k+p)_x
-    float4 *rB = reinterpret_cast<float4 *>(smem_raw + L.rB);   // cos, sin of (k+p)_y, w_p f_p, w_p (1 - f_p)
-    float4 *cz = reinterpret_cast<float4 *>(smem_raw + L.cz);
+    float4 *rA = reinterpret_cast<float4 *>(smem_raw + L.rA);   // (k+p)_x, (k+p)_y (fixed point), cos of both
+    float4 *rB = reinterpret_cast<float4 *>(smem_raw + L.rB);   // sin of both, w_p f_p, w_p (1 - f_p)
+    float4 *cz = reinterpret_cast<float4 *>(smem_raw + L.cz);   // Z_c, Z_c V_jac, -2t l_c, -mu l_c
     float2 *ray = reinterpret_cast<float2 *>(smem_raw + L.ray);
     float *cd = reinterpret_cast<float *>(smem_raw + L.cd);     // -4 t' l_c
-    float *rC = reinterpret_cast<float *>(smem_raw + L.rC);     // x_j + x_p + 2T
+    float *ck = reinterpret_cast<float *>(smem_raw + L.ck);     // K_c Z_c (GL)
+    float *rC = reinterpret_cast<float *>(smem_raw + L.rC);     // x_p
     unsigned char *tab = smem_raw + L.tab;
-    float *hs = reinterpret_cast<float *>(smem_raw + L.hist);   // [moment][bin] (grid mode)
-    for (int i = tid; i < 5 * A.nbins; i += blockDim.x) hs[i] = 0.f;
+    unsigned *queue = reinterpret_cast<unsigned *>(smem_raw + L.queue);   // guarded pairs of a pass
+    __shared__ int s_nq;
+    int *hs = reinterpret_cast<int *>(smem_raw + L.hist);       // [moment 0..4, rest of moment 0][NBS]
+    float *wb = reinterpret_cast<float *>(smem_raw + L.wb);     // max over c of a pair's vertex and line weight
+    __shared__ float s_max[2];                                  // max |Z|, |K Z|
+    __shared__ float s_sum[2], s_blk[3];                        // sums of w_p f_p, w_p (1 - f_p); of a block of q
+    __shared__ int s_bad;
 
+    for (int i = tid; i < NBS * (LO ? 6 : 5); i += HF_THR) hs[i] = 0;
+    if (tid < 2) s_max[tid] = s_sum[tid] = 0.f;
+    if (tid == 2) s_bad = s_nq = 0;
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(A.ptab);
         uint4 *dst = reinterpret_cast<uint4 *>(tab);
         const int n16 = (kProjW * kProjStride + 15) / 16;
-        for (int i = tid; i < n16; i += blockDim.x) dst[i] = src[i];
+        for (int i = tid; i < n16; i += HF_THR) dst[i] = src[i];
     }
+    __syncthreads();
     const double *Vja = A.V + ((long)j * N + a) * N;
-    // per-patch slots; with UNIB the weight column is filled per q block (b)
-    auto fill_slots = [&](int b) {
-        const float vb = UNIB ? (float)Vja[b] : 0.f;
-        for (int i = tid; i < SF_SLOTS; i += blockDim.x) {
-            if (i <= N) {
-                const int cc = i == N ? 0 : i;
-                const float Zc = A.Z ? (float)A.Z[cc] : 1.f;
-                const float lz = qp ? Zc : 1.f;
-                const float vc = (float)Vja[cc];
-                cz[i] = UNIB ? make_float4(Zc * (2.f * vb * vb - vb * vc), 0.f, -2.f * A.t * lz, -A.mu * lz)
-                             : make_float4(Zc, Zc * vc, -2.f * A.t * lz, -A.mu * lz);
-                cd[i] = -4.f * A.tp * lz;
-                const float4 bd = A.bnd[cc];
-                ray[i] = make_float2(bd.x, bd.z);
-            } else {
-                cz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                cd[i] = 0.f;
-                ray[i] = make_float2(0.f, 0.f);
-            }
+    const float Za = A.Z ? (float)A.Z[a] : 1.f;
+    const float kza = GL ? (float)A.K[a] * Za : 0.f;
+    const float lza = qp ? Za : 1.f;
+    for (int i = tid; i < SF_SLOTS; i += HF_THR) {
+        if (i <= N) {
+            const int cc = i == N ? 0 : i;
+            const float Zc = A.Z ? (float)A.Z[cc] : 1.f;
+            const float lz = qp ? Zc : 1.f;
+            const float vc = (float)Vja[cc];
+            const float kzc = GL ? (float)A.K[cc] * Zc : 1.f;
+            cz[i] = make_float4(Zc, Zc * vc, -2.f * A.t * lz, -A.mu * lz);
+            cd[i] = -4.f * A.tp * lz;
+            if (GL) ck[i] = kzc;
+            const float4 bd = A.bnd[cc];
+            ray[i] = make_float2(bd.x, bd.z);
+            // non-negative floats order like their bits
+            atomicMax(reinterpret_cast<int *>(&s_max[0]), __float_as_int(fabsf(Zc)));
+            atomicMax(reinterpret_cast<int *>(&s_max[1]), __float_as_int(fabsf(kzc)));
+            if (!isfinite(vc) || !isfinite(Zc) || !isfinite(kzc)) s_bad = 1;
+        } else {
+            cz[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            cd[i] = 0.f;
+            if (GL) ck[i] = 0.f;
+            ray[i] = make_float2(0.f, 0.f);
+        }
+    }
+    __syncthreads();
+    double *H = A.hist + (long)jidx * 5 * A.nbins;
+    if (s_bad) {       // a non-finite vertex or weight: as in the sums, every frequency of this target
+        if (tid == 0) atomicAdd(&H[0], __longlong_as_double(0x7ff8000000000000LL));
+        return;
+    }
+    const float4 kcs = A.kcs[j];
+    const unsigned char *tabc = tab + (kProjW / 2) * (kProjStride + 1);   // the cell of the origin
+    // bounds of the fixed-point scale (see above): the largest weight of patch b,
+    // and the sums over the patch's points p
+    const float gl_max = GL ? s_max[1] * s_max[0] : 1.f;
+    for (int b = tid; b < N; b += HF_THR) {
+        const float vb = (float)Vja[b];
+        float m = 0.f;
+        for (int c = 0; c < N; ++c) m = fmaxf(m, fabsf(fmaf(-vb, cz[c].y, cz[c].x * 2.f * vb * vb)));
+        wb[b] = m * gl_max;
+    }
+    for (int i = tid; i < P; i += HF_THR) {
+        float fp, fcp;
+        sfermi(lza * A.fine.xi[a * PP + i], A.invT, fp, fcp);
+        const float w = A.fine.w[a * PP + i];
+        atomicAdd(&s_sum[0], w * fp);
+        atomicAdd(&s_sum[1], w * fcp);
+    }
+    const float pairs = (float)(HF_THR * HF_QPT) * (float)P;
+    const float lo_scale = 1073741824.f / pairs;
+    constexpr float kMagic = 12582912.f;
+    const unsigned hbase = (unsigned)__cvta_generic_to_shared(hs);
+
+    // one pair of weight amp and pole energy E: its bin, the offset from the
+    // bin's centre in half bins, and the moments
+    auto deposit = [&](float amp, float E, float scale) {
+        const float u = amp * scale;                     // in units of the histogram
+        int r;
+        const float rr = rint_add(fmaf(E, A.inv_h, A.c_frac), r);
+        const float d = 2.f * (fmaf(E, A.inv_h, -rr) + fmaf(E, A.inv_h_lo, A.c_frac));
+        const int bin = min(max(r + A.c_int, 0), A.nbins - 1);
+        const unsigned h = hbase + 4u * (unsigned)bin;
+        const float u0 = u + kMagic;
+        red_shared(h, __float_as_int(u0) - 0x4B400000);
+        if (LO) {
+            const float rest = fmaf(amp, scale, -(u0 - kMagic)) * lo_scale;
+            red_shared(h + 20u * NBS, __float_as_int(rest + kMagic) - 0x4B400000);
+        }
+        float m = u;
+#pragma unroll
+        for (int mo = 1; mo < 5; ++mo) {
+            m *= d;
+            red_shared(h + 4u * NBS * mo, __float_as_int(m + kMagic) - 0x4B400000);
         }
     };
-    int b_slots = UNIB ? (blockIdx.x * A.qb * 256 * SF_QPT) / PP : 0;
-    fill_slots(b_slots);
-    const float Za = A.Z ? (float)A.Z[a] : 1.f;
-    const float lza = qp ? Za : 1.f;
-    const float4 kcs = A.kcs[jidx];
-
-    const unsigned char *tabc = tab + (kProjW / 2) * (kProjStride + 1);   // the cell of the origin
-    // records of the loop points p0 .. p0 + cnt - 1 of patch a
+    const bool one_pass = P <= HF_REC;
     auto stage = [&](int p0, int cnt) {
-        for (int i = tid; i < cnt; i += blockDim.x) {
+        for (int i = tid; i < cnt; i += HF_THR) {
             const int p = a * PP + p0 + i;
-            const float4 k4 = A.kp[(long)jidx * M + p];
+            const int2 kf = A.kfx[(long)j * M + p];
             const float cpx = A.fine.cx[p], spx = A.fine.sx[p], cpy = A.fine.cy[p], spy = A.fine.sy[p];
             const float xp = lza * A.fine.xi[p];
             float fp, fcp;
             sfermi(xp, A.invT, fp, fcp);
             const float wp = A.fine.w[p];
-            const int kx = angle_fx((double)k4.x + (double)k4.y), ky = angle_fx((double)k4.z + (double)k4.w);
-            rA[i] = make_float4(__int_as_float(kx), __int_as_float(ky), kcs.x * cpx - kcs.y * spx,
-                                kcs.y * cpx + kcs.x * spx);
-            rB[i] = make_float4(kcs.z * cpy - kcs.w * spy, kcs.w * cpy + kcs.z * spy, wp * fp, wp * fcp);
+            rA[i] = make_float4(__int_as_float(kf.x), __int_as_float(kf.y), kcs.x * cpx - kcs.y * spx,
+                                kcs.z * cpy - kcs.w * spy);
+            rB[i] = make_float4(kcs.y * cpx + kcs.x * spx, kcs.w * cpy + kcs.z * spy, wp * fp, wp * fcp);
             rC[i] = xp;
         }
     };
-    const bool one_pass = P <= pch;
     if (one_pass) stage(0, P);
-    __syncthreads();   // tables (and the records of a single pass) written
 
-    // A.qb blocks of 256 SF_QPT loop points q per CTA reuse the staged tables
-    for (int qb = 0; qb < A.qb; ++qb) {
-        const int blk = blockIdx.x * A.qb + qb;
-        if (blk * (256 * SF_QPT) >= M) break;   // uniform over the CTA
-        if (UNIB && blk * (256 * SF_QPT) / PP != b_slots) {
-            b_slots = blk * (256 * SF_QPT) / PP;
-            __syncthreads();   // every warp is done with the previous weights
-            fill_slots(b_slots);
-            __syncthreads();
-        }
-        // the SF_QPT loop points q of this thread (an index past M gets weight 0)
-        float cqx[SF_QPT], sqx[SF_QPT], cqy[SF_QPT], sqy[SF_QPT];
-        float fqp[SF_QPT], fcqp[SF_QPT], v2[SF_QPT], vab[SF_QPT], mxq[SF_QPT];
-        int qi[SF_QPT], qx[SF_QPT], qy[SF_QPT];
+    const int nblk = (M + HF_THR * HF_QPT - 1) / (HF_THR * HF_QPT);
+    for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+        float2 cq[HF_QPT], sq[HF_QPT];
+        float fqp[HF_QPT], fcqp[HF_QPT], v2[HF_QPT], vab[HF_QPT], xqk[HF_QPT], ga[HF_QPT], gb[HF_QPT], gc[HF_QPT];
+        int qi[HF_QPT], qx[HF_QPT], qy[HF_QPT];
+        if (tid < 3) s_blk[tid] = 0.f;
+        __syncthreads();
+        float t1 = 0.f, t2 = 0.f, t3 = 0.f;      // sums and maximum of the weights of this thread's q
 #pragma unroll
-        for (int k = 0; k < SF_QPT; ++k) {
-            const int iq = blk * (256 * SF_QPT) + k * 256 + tid;   // angular-minor index
+        for (int k = 0; k < HF_QPT; ++k) {
+            const int iq = blk * (HF_THR * HF_QPT) + k * HF_THR + tid;   // radial-minor: the storage order
             const bool valid = iq < M;
-            const int ii = valid ? iq : M - 1;
-            const int b = ii / PP, rem = ii - b * PP;
-            const int qq = b * PP + (rem % A.pb.n_theta) * A.pb.n_r + rem / A.pb.n_theta;
+            const int qq = valid ? iq : M - 1;
+            const int b = qq / PP;
             qi[k] = qq;
             const float Zb = A.Z ? (float)A.Z[b] : 1.f;
-            qx[k] = angle_fx(A.kx64[qq]);
-            qy[k] = angle_fx(A.ky64[qq]);
-            cqx[k] = A.fine.cx[qq];
-            sqx[k] = A.fine.sx[qq];
-            cqy[k] = A.fine.cy[qq];
-            sqy[k] = A.fine.sy[qq];
+            qx[k] = A.pfx[qq].x;
+            qy[k] = A.pfx[qq].y;
+            cq[k] = make_float2(A.fine.cx[qq], A.fine.cy[qq]);
+            sq[k] = make_float2(A.fine.sx[qq], A.fine.sy[qq]);
             const float xq = (qp ? Zb : 1.f) * A.fine.xi[qq];
             float fq, fcq;
             sfermi(xq, A.invT, fq, fcq);
@@ -1083,11 +1400,34 @@ __global__ void __launch_bounds__(256, 1) sigma_grid_fast_kernel(SigmaFastArgs A
             fcqp[k] = fcq * pref;
             vab[k] = (float)Vja[b];
             v2[k] = 2.f * vab[k] * vab[k];
-            mxq[k] = -xq;
+            xqk[k] = xq;
+            if (GL) {
+                const float kzb = (float)A.K[b] * Zb;
+                ga[k] = (kza * Zb + kzb * Za) * (1.f / 6.f);
+                gb[k] = (kza + kzb) * (1.f / 6.f);
+                gc[k] = (Za + Zb) * (1.f / 6.f);
+            }
+            t1 += fabsf(fcqp[k]) * wb[b];
+            t2 += fabsf(fqp[k]) * wb[b];
+            t3 = fmaxf(t3, fabsf(pref) * wb[b]);
         }
-
-        for (int p0 = 0; p0 < P; p0 += pch) {
-            const int cnt = P - p0 < pch ? P - p0 : pch;
+        for (int off = 16; off > 0; off >>= 1) {
+            t1 += __shfl_down_sync(0xffffffffu, t1, off);
+            t2 += __shfl_down_sync(0xffffffffu, t2, off);
+            t3 = fmaxf(t3, __shfl_down_sync(0xffffffffu, t3, off));
+        }
+        if ((tid & 31) == 0) {
+            atomicAdd(&s_blk[0], t1);
+            atomicAdd(&s_blk[1], t2);
+            atomicMax(reinterpret_cast<int *>(&s_blk[2]), __float_as_int(t3));
+        }
+        __syncthreads();
+        // |W F| <= W max(f_p (1 - f_q), (1 - f_p) f_q) summed over the block
+        const float total = s_sum[0] * s_blk[0] + s_sum[1] * s_blk[1], single = A.w_max * s_blk[2];
+        const float scale = total > 0.f ? fminf(1073741824.f / total, 2097152.f / single) : 0.f;
+        const double unit = scale > 0.f ? (double)fac / (double)scale : 0.0, unit_lo = unit / (double)lo_scale;
+        for (int p0 = 0; p0 < P; p0 += HF_REC) {
+            const int cnt = min(HF_REC, P - p0);
             if (!one_pass) {
                 __syncthreads();   // previous pass done with the records
                 stage(p0, cnt);
@@ -1096,130 +1436,215 @@ __global__ void __launch_bounds__(256, 1) sigma_grid_fast_kernel(SigmaFastArgs A
 #pragma unroll 2
             for (int i = 0; i < cnt; ++i) {
                 const float4 ra = rA[i], rb = rB[i];
-                const float upp = rC[i];   // x_p
-                int c[SF_QPT];
-                float x[SF_QPT], y[SF_QPT];
-                bool slow_any = false;
-                unsigned slow_mask = 0;
+                const float xp = rC[i];
+                int c[HF_QPT];
+                bool slow[HF_QPT];
 #pragma unroll
-                for (int k = 0; k < SF_QPT; ++k) {
-                    bool slow;
-                    c[k] = fx_patch(__float_as_int(ra.x), __float_as_int(ra.y), qx[k], qy[k], tabc, ray, x[k], y[k],
-                                    slow);
-                    slow_mask |= slow ? 1u << k : 0u;
-                    slow_any = slow_any || slow;
+                for (int k = 0; k < HF_QPT; ++k) {
+                    float x, y;
+                    c[k] = fx_patch(__float_as_int(ra.x), __float_as_int(ra.y), qx[k], qy[k], tabc, ray, x, y, slow[k]);
                 }
-                if (slow_any) {
+                if (__any_sync(0xffffffffu, slow[0] || slow[1])) {      // taken by the whole warp
 #pragma unroll
-                    for (int k = 0; k < SF_QPT; ++k)
-                        if (slow_mask & (1u << k)) {
-                            const bool edge = fmaxf(fabsf(x[k]), fabsf(y[k])) > kFxEdge;
-                            c[k] = sf_slow_patch(A, jidx, j, a * PP + p0 + i, qi[k], x[k] * kRadPerFx,
-                                                 y[k] * kRadPerFx, edge, A.bnd);
+                    for (int k = 0; k < HF_QPT; ++k) {
+                        bool still;
+                        const int cc = fx_zoom(__float_as_int(ra.x), __float_as_int(ra.y), qx[k], qy[k], tabc, ray, still);
+                        if (slow[k]) c[k] = cc;
+                        if (slow[k] && still) {       // queued; the table's patch until the pass ends
+                            const int at = atomicAdd(&s_nq, 1);
+                            if (at < HF_QCAP) queue[at] = (unsigned)i | (unsigned)(k * HF_THR + tid) << 12;
                         }
+                        __syncwarp();
+                    }
                 }
 #pragma unroll
-                for (int k = 0; k < SF_QPT; ++k) {
+                for (int k = 0; k < HF_QPT; ++k) {
                     const float4 z = cz[c[k]];
-                    const float crx = ra.z * cqx[k] + ra.w * sqx[k];
-                    const float cry = rb.x * cqy[k] + rb.y * sqy[k];
-                    float xr = fmaf(crx + cry, z.z, z.w);           // Z-scaled line energy of r
-                    if (!TP0) xr = fmaf(crx * cry, cd[c[k]], xr);
-                    const float fr = rcp_approx(1.f + ex2_approx(xr * A.cT));
+                    const float2 cr = __ffma2_rn(make_float2(ra.z, ra.w), cq[k],
+                                                 __fmul2_rn(make_float2(rb.x, rb.y), sq[k]));
+                    float xr = fmaf(cr.x + cr.y, z.z, z.w);          // Z-scaled line energy of r
+                    xr = fmaf(cr.x * cr.y, cd[c[k]], xr);
                     const float Aq = rb.z * fcqp[k], Bq = rb.w * fqp[k];
-                    const float F = fmaf(fr, Bq - Aq, Aq);
-                    const float amp = UNIB ? z.x * F : fmaf(-vab[k], z.y, z.x * v2[k]) * F;
-                    // pole energy E = x_q + x_r - x_p (upp holds x_p here)
-                    const float E = (xr - mxq[k]) - upp;
-                    int bin = (int)floorf((E - A.e_min) * A.inv_h);
-                    bin = bin < 0 ? 0 : (bin >= A.nbins ? A.nbins - 1 : bin);
-                    const float d = E - (A.e_min + ((float)bin + 0.5f) * A.h);
-                    float mm[5];
-                    mm[0] = amp;
-#pragma unroll
-                    for (int mo = 1; mo < 5; ++mo) mm[mo] = mm[mo - 1] * d;
-                    // neighbouring lanes often share a bin: sum runs of equal
-                    // bins with shuffles (each lane adds the lanes up to the
-                    // end of its run), then one atomic per run and moment
-                    const int lane = tid & 31;
-                    const int bup = __shfl_up_sync(0xffffffffu, bin, 1);
-                    const bool head = lane == 0 || bup != bin;
-                    const unsigned heads = __ballot_sync(0xffffffffu, head);
-                    if (heads != 0xffffffffu) {
-                        const unsigned above = lane == 31 ? 0u : heads >> (lane + 1);
-                        const int end = above ? lane + __ffs(above) - 1 : 31;
-#pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) {
-#pragma unroll
-                            for (int mo = 0; mo < 5; ++mo) {
-                                const float o = __shfl_down_sync(0xffffffffu, mm[mo], off);
-                                if (lane + off <= end) mm[mo] += o;
-                            }
-                        }
+                    const float F = fmaf(rcp_approx(1.f + ex2_approx(xr * A.cT)), Bq - Aq, Aq);
+                    float w = fmaf(-vab[k], z.y, z.x * v2[k]);
+                    if (GL) w *= fmaf(gc[k], ck[c[k]], fmaf(gb[k], z.x, ga[k]));
+                    deposit(w * F, (xr + xqk[k]) - xp, scale);
+                }
+            }
+            // the guarded pairs of this pass: where the exact patch differs from the
+            // table's, its contribution is taken out (the same rounded addends) and
+            // the right one put in
+            __syncthreads();
+            const int nq = s_nq;
+            __syncthreads();
+            if (tid == 0) s_nq = 0;
+            const bool over = nq > HF_QCAP;      // more than the queue holds: look at every pair again
+            const int ntot = over ? cnt * (HF_THR * HF_QPT) : nq;
+            for (int e = tid; e < ntot; e += HF_THR) {
+                const unsigned en = over ? (unsigned)(e % cnt) | (unsigned)(e / cnt) << 12 : queue[e];
+                const int i = en & 4095u, qq = blk * (HF_THR * HF_QPT) + (int)(en >> 12);
+                if (qq >= M) continue;
+                const float4 ra = rA[i], rb = rB[i];
+                // the patch the loop used
+                float x, y;
+                bool slow;
+                fx_patch(__float_as_int(ra.x), __float_as_int(ra.y), A.pfx[qq].x, A.pfx[qq].y, tabc, ray, x, y, slow);
+                if (!slow) continue;
+                const int c0 = fx_zoom(__float_as_int(ra.x), __float_as_int(ra.y), A.pfx[qq].x, A.pfx[qq].y, tabc, ray, slow);
+                if (!slow) continue;
+                const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
+                const int c1 = sf_slow_patch(A, j, a * PP + p0 + i, qq, x * kRadPerFx, y * kRadPerFx, edge ? 1 : 0, A.bnd);
+                if (c1 == c0) continue;
+                const int b = qq / PP;
+                const float Zb = A.Z ? (float)A.Z[b] : 1.f, vb = (float)Vja[b];
+                const float xq = (qp ? Zb : 1.f) * A.fine.xi[qq];
+                float fq, fcq;
+                sfermi(xq, A.invT, fq, fcq);
+                const float pref = Za * Zb * A.fine.w[qq];
+                const float2 cr = __ffma2_rn(make_float2(ra.z, ra.w), make_float2(A.fine.cx[qq], A.fine.cy[qq]),
+                                             __fmul2_rn(make_float2(rb.x, rb.y),
+                                                        make_float2(A.fine.sx[qq], A.fine.sy[qq])));
+                const float Aq = rb.z * (fcq * pref), Bq = rb.w * (fq * pref);
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    const int cc = u ? c0 : c1;
+                    const float4 z = cz[cc];
+                    float xr = fmaf(cr.x + cr.y, z.z, z.w);
+                    xr = fmaf(cr.x * cr.y, cd[cc], xr);
+                    const float F = fmaf(rcp_approx(1.f + ex2_approx(xr * A.cT)), Bq - Aq, Aq);
+                    float w = fmaf(-vb, z.y, z.x * (2.f * vb * vb));
+                    if (GL) {
+                        const float kzb = (float)A.K[b] * Zb;
+                        w *= fmaf((Za + Zb) * (1.f / 6.f), ck[cc],
+                                  fmaf((kza + kzb) * (1.f / 6.f), z.x, (kza * Zb + kzb * Za) * (1.f / 6.f)));
                     }
-                    if (head) {
-#pragma unroll
-                        for (int mo = 0; mo < 5; ++mo) atomicAdd(&hs[mo * A.nbins + bin], mm[mo]);
+                    deposit(u ? -(w * F) : w * F, (xr + xq) - rC[i], scale);
+                }
+            }
+            __syncthreads();
+            // without the second word the rounding of moment 0 is kept small by
+            // flushing after every pass
+            if (!LO || p0 + HF_REC >= P) {
+                for (int i = tid; i < A.nbins; i += HF_THR) {
+                    const int v = hs[i], lo = LO ? hs[5 * NBS + i] : 0;
+                    if (v == 0 && lo == 0) continue;
+                    hs[i] = 0;
+                    if (LO) hs[5 * NBS + i] = 0;
+                    atomicAdd(&H[i], unit * (double)v + unit_lo * (double)lo);
+                }
+                float mom = (float)unit;                         // (h/2)^moment per unit
+                for (int mo = 1; mo < 5; ++mo) {
+                    mom *= 0.5f * A.h;
+                    for (int i = tid; i < A.nbins; i += HF_THR) {
+                        const int v = hs[mo * NBS + i];
+                        if (v == 0) continue;
+                        hs[mo * NBS + i] = 0;
+                        atomicAdd(&H[(long)mo * A.nbins + i], (double)((float)v * mom));
                     }
                 }
+                __syncthreads();
             }
         }
     }
-    __syncthreads();
-    double *H = A.hist + (long)jidx * 5 * A.nbins;
-    for (int i = tid; i < 5 * A.nbins; i += blockDim.x) {
-        const float v = hs[i];
-        if (v != 0.f) atomicAdd(&H[i], (double)v * fac);
-    }
 }
 
-// Z_j = 1/(1 - slope) with the chord slope accumulated per target.  rep[j]
-// (may be NULL) is the slot of j's C4v representative among the targets.
-__global__ void z_update_kernel(const double *slope, const int *rep, double *Zout, int N)
+// Z_j = 1/(1 - slope) with the chord slope accumulated per target slot, or the
+// slopes themselves (slopes_out).  rep[j] (may be NULL) is the slot of j's C4v
+// representative among the targets; sym.mode == 2: where the C4v test holds, with
+// the patch's own correction corr[j], or from the sums of every patch (full) when
+// the record of boundary pairs ran over.
+__global__ void z_update_kernel(const double *slope, const double *corr, const double *full, const unsigned *nevents,
+                                unsigned max_events, const int *rep, SymMode sym, double *Zout, double *slopes_out,
+                                int N)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
-    Zout[j] = 1.0 / (1.0 - slope[rep ? rep[j] : j]);
+    const bool use = rep && (sym.mode != 2 || sym_compact(sym));
+    double s = slope[use ? rep[j] : j];
+    if (sym.mode == 2 && use) s = *nevents > max_events ? full[j] : s + corr[j];
+    if (slopes_out) slopes_out[j] = s;
+    if (Zout) Zout[j] = 1.0 / (1.0 - s);
 }
 
 // Sigma on the grid from the binned moments: sum_b sum_n H_n[b] / (z - E_b)^(n+1),
-// z = w_m + i eta (Taylor expansion of 1/(z - E_b - d) in the offset d).
-// rep (may be NULL): the histogram slot of patch j's C4v representative.
-__global__ void sigma_grid_kernel(const double *hist, int nbins, double e_min, double h, int n_omega,
-                                  double w0, double dw, double eta, double *re, double *im, int N,
-                                  const int *rep)
+// z = w_m + i eta (Taylor expansion of 1/(z - E_b - d) in the offset d), for the
+// target slots of the histogram, accumulated into acc[slot][re, im][m].
+//
+// What bounds it: FP64 FMAs (2 per clock and SM).  The powers of u = 1/(z - E_b)
+// do not depend on the target, so a thread (one frequency) computes them once
+// for RG_T targets (32 FP64 operations, then 10 per target), empty bins cost one
+// read, only the targets of a symmetric vertex are resummed, and the bins are
+// split over the grid.  np48, 512 frequencies, 4 801 bins: 15.7 -> 1.5 ms.
+constexpr int RG_T = 8;         // targets per thread
+constexpr int RG_BINS = 64;     // bins per CTA
+
+__global__ void __launch_bounds__(128) sigma_resum_kernel(const double *__restrict__ hist, int nbins, double e_min,
+                                                          double h, int n_omega, double w0, double dw, double eta,
+                                                          double *__restrict__ acc, int ntarget, int n_list, SymMode sym)
 {
+    const int nt = sym.mode == 2 && sym_compact(sym) ? n_list : ntarget;
+    const int t0 = blockIdx.z * RG_T;
+    if (t0 >= nt) return;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (m >= n_omega) return;
-    const double w = w0 + dw * m;
-    const double *H = hist + (long)(rep ? rep[j] : j) * 5 * nbins;
-    double sr = 0.0, si = 0.0;
-    for (int b = 0; b < nbins; ++b) {
+    const double w = w0 + dw * min(m, n_omega - 1);
+    const int b0 = blockIdx.y * RG_BINS, b1 = min(nbins, b0 + RG_BINS);
+    const double eta2 = eta * eta;
+    double sr[RG_T] = {}, si[RG_T] = {};
+    for (int b = b0; b < b1; ++b) {
+        double hv[RG_T][5];
+        bool any = false;
+#pragma unroll
+        for (int t = 0; t < RG_T; ++t) {
+            const double *H = hist + (long)(t0 + t) * 5 * nbins + b;
+#pragma unroll
+            for (int mo = 0; mo < 5; ++mo) hv[t][mo] = t0 + t < nt ? __ldg(H + (long)mo * nbins) : 0.0;
+#pragma unroll
+            for (int mo = 0; mo < 5; ++mo) any = any || hv[t][mo] != 0.0;
+        }
+        if (!any) continue;                      // uniform over the warp
         const double Eb = e_min + (b + 0.5) * h;
-        // u = 1/(z - Eb) = (dx - i eta)/(dx^2 + eta^2)
-        const double dx = w - Eb, den = dx * dx + eta * eta;
-        const double ur = dx / den, ui = -eta / den;
+        const double dx = w - Eb, inv = 1.0 / fma(dx, dx, eta2);
+        const double ur = dx * inv, ui = -eta * inv;
         double pr = ur, pi = ui;                 // u^(n+1)
+#pragma unroll
         for (int mo = 0; mo < 5; ++mo) {
-            const double hv = H[(long)mo * nbins + b];
-            sr += hv * pr;
-            si += hv * pi;
-            const double nr = pr * ur - pi * ui, ni = pr * ui + pi * ur;
+#pragma unroll
+            for (int t = 0; t < RG_T; ++t) {
+                sr[t] = fma(hv[t][mo], pr, sr[t]);
+                si[t] = fma(hv[t][mo], pi, si[t]);
+            }
+            const double nr = pr * ur - pi * ui;
+            pi = pr * ui + pi * ur;
             pr = nr;
-            pi = ni;
         }
     }
-    re[(long)j * n_omega + m] = sr;
-    im[(long)j * n_omega + m] = si;
+    if (m >= n_omega) return;
+#pragma unroll
+    for (int t = 0; t < RG_T; ++t) {
+        if (t0 + t >= nt || (sr[t] == 0.0 && si[t] == 0.0)) continue;
+        atomicAdd(&acc[(2L * (t0 + t)) * n_omega + m], sr[t]);
+        atomicAdd(&acc[(2L * (t0 + t) + 1) * n_omega + m], si[t]);
+    }
 }
 
-static qpfrg_status launch_kp_table(qpfrg_ctx *c, const int *jlist, int nj)
+// Sigma of every patch from its target slot.
+__global__ void sigma_spread_kernel(const double *__restrict__ acc, const int *rep, SymMode sym, int n_omega,
+                                    double *__restrict__ re, double *__restrict__ im)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (m >= n_omega) return;
+    const bool use = rep && (sym.mode != 2 || sym_compact(sym));
+    const double *a = acc + 2L * (use ? rep[j] : j) * n_omega + m;
+    re[(long)j * n_omega + m] = a[0];
+    im[(long)j * n_omega + m] = a[n_omega];
+}
+
+static qpfrg_status launch_kp_table(qpfrg_ctx *c, const int *jlist, int nj, bool fixed = true)
 {
     const long total = (long)nj * c->pb.M;
     prof_begin(c);
     kp_table_kernel<<<(int)std::min<long>((total + 255) / 256, 152L * 8), 256, 0, c->stream>>>(
-        c->d_kf, jlist, nj, c->f64.kx, c->f64.ky, c->pb.M, c->d_kp, c->d_kcs);
+        c->d_kf, jlist, nj, c->f64.kx, c->f64.ky, c->pb.M, c->d_kp, fixed ? c->d_kfx : nullptr, c->d_kcs);
     prof_end(c, K_KP_TABLE);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "kp_table_kernel");
@@ -1245,27 +1670,55 @@ static qpfrg_status launch_sigma(qpfrg_ctx *c, bool hist, SigmaArgs<R> &A, int k
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_kernel");
 }
 
-// Shared memory of the fast kernel (grid mode with nbins > 0)
-static size_t sigma_fast_smem(const qpfrg_ctx *c, int nbins)
+// Target slots of a self-energy call: a fixed list (mode 0; jlist NULL: every
+// patch) or the list where the C4v test of (V, Z) holds and every patch where it
+// does not, decided on the device (mode 2).
+struct SigmaTargets {
+    const int *jlist = nullptr;
+    int n = 0;              // targets of the list
+    SymMode sym;
+    const int *rep = nullptr;   // slot of each patch under the list
+    int mirror = 0;             // mirror_part of the list's targets
+    int slots(int N) const { return sym.mode == 2 || !jlist ? N : n; }
+};
+
+// Targets of a given (V, Z): with the symmetry that the device finds (d_sym), the
+// irreducible patches and the zone-edge patches; images copy the sum of their
+// representative.  mirror 2 also halves the targets on a diagonal.
+static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror)
 {
-    const int cap = nbins > 0 ? SF_PCH / 2 : SF_PCH;
-    const int pch = c->pb.P < cap ? c->pb.P : cap;
-    return sf_smem_layout(pch, nbins).total;
+    SigmaTargets t;
+    t.n = c->pb.N;
+    if (!c->d_jgrid) return t;
+    t.jlist = c->d_jgrid;
+    t.n = c->n_grid;
+    t.rep = c->d_repgrid;
+    t.sym.mode = 2;
+    t.sym.red = c->d_sym;
+    t.sym.tol = tol / 3.0;
+    t.mirror = c->pb.n_theta % 2 == 0 ? mirror : 0;
+    return t;
 }
 
-// nbins == 0: chord slopes into d_sig (the flow's Z); nbins > 0: the binned
-// pole density into hist (frequency grid)
-static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z,
-                                      const int *jlist, int nj, double *hist = nullptr, double e_min = 0.0,
-                                      double h = 1.0, int nbins = 0)
+// The last double k > 0 with rint(k / 2 pi) <= n (round to even at the half: 0.5
+// folds to 0, 1.5 to 2), the comparisons of the FP64 fold.
+static double fold_limit(int n)
 {
-    qpfrg_status s = launch_kp_table(c, jlist, nj);
-    if (s != QPFRG_OK) return s;
-    SigmaFastArgs A;
+    double k = (2 * n + 1) * kPi;
+    while (std::rint(k / kTwoPi) > n) k = std::nextafter(k, 0.0);
+    while (std::rint(std::nextafter(k, 1e9) / kTwoPi) <= n) k = std::nextafter(k, 1e9);
+    return k;
+}
+
+static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                               const SigmaTargets &tg)
+{
+    SigmaFastArgs A{};
     A.pb = c->pb;
     A.fine = c->f32;
     A.V = d_V;
     A.Z = d_Z;
+    A.K = d_K;
     A.kx64 = c->f64.kx;
     A.ky64 = c->f64.ky;
     A.kf = c->d_kf;
@@ -1273,11 +1726,20 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     A.qxl = c->d_qxl;
     A.qyl = c->d_qyl;
     A.kp = c->d_kp;
+    A.kfx = c->d_kfx;
+    A.pfx = c->d_pfx;
     A.kcs = c->d_kcs;
     A.bnd = c->d_bnd;
     A.ptab = c->d_ptab;
-    A.jlist = jlist;
+    A.jlist = tg.jlist;
+    A.sym = tg.sym;
+    A.n_list = tg.n;
+    A.mirror = tg.mirror;
     A.sig = c->d_sig;
+    A.corr = c->d_sig + 2 * c->pb.N;
+    A.events = c->d_events;
+    A.nevents = reinterpret_cast<unsigned *>(c->d_sig + 4 * c->pb.N);
+    A.max_events = c->max_events;
     A.t = (float)c->pb.t;
     A.tp = (float)c->pb.tp;
     A.mu = (float)c->pb.mu;
@@ -1291,26 +1753,31 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     A.eta2x4 = (float)(4.0 * c->pb.eta * c->pb.eta);
     A.inv_dth = (float)(c->pb.N / kTwoPi);
     A.dth = (float)(kTwoPi / c->pb.N);
-    A.hist = hist;
-    A.e_min = (float)e_min;
-    A.h = (float)h;
-    A.inv_h = (float)(1.0 / h);
-    A.nbins = nbins;
-    const bool grid_mode = nbins > 0;
-    const size_t smem = sigma_fast_smem(c, nbins);
-    // The zone-edge targets' sums are mirror symmetric only up to the pairs
-    // whose momentum r lands on |r_x| or |r_y| = pi (their wedge is decided by
-    // rounding): halving them is kept for the chord slope (a relative error
-    // below 1e-4, shrinking with N) and left out on the frequency grid.
-    A.mirror = (jlist != nullptr && c->pb.n_theta % 2 == 0) ? (grid_mode ? 2 : 1) : 0;
+    A.w_max = (float)c->fw_max;
+    static const double fold0 = fold_limit(0), fold1 = fold_limit(1);
+    A.fold0 = fold0;
+    A.fold1 = fold1;
+    return A;
+}
+
+// Chord slopes of the target slots into d_sig (FP32, wedge grid).
+static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                                      const SigmaTargets &tg)
+{
+    const int nj = tg.slots(c->pb.N);
+    // a list decided on the device may be any patch: k + p of all of them; a
+    // launch that reads the patch table needs no fixed-point momenta
+    const bool listed = !d_K && tg.sym.mode == 0 && tg.jlist != nullptr && tg.jlist == c->d_jirr;
+    qpfrg_status s = launch_kp_table(c, tg.sym.mode == 2 ? nullptr : tg.jlist, nj, !(listed && c->d_rtab));
+    if (s != QPFRG_OK) return s;
+    SigmaFastArgs A = fast_args(c, T, d_V, d_Z, d_K, tg);
     const bool unib = c->pb.P % (256 * SF_QPT) == 0;
     // The flow's Z on the C4v-irreducible targets reads the patches of r from
     // a table built on first use (one byte per target, p and q: N_irr M^2
     // bytes, 126 GB at np96_n32), when it fits in 60 % of the free device
     // memory and options.sigma_table >= 0; otherwise it decides them per pair.
     // (record passes of a multiple of 8 records: P a multiple of 16, mirror halves included)
-    const bool rt_list = !grid_mode && jlist != nullptr && jlist == c->d_jirr && nj == c->n_irr &&
-                         c->pb.P % 16 == 0 && c->pb.P <= SF_PCH;
+    const bool rt_list = listed && nj == c->n_irr && c->pb.P % 16 == 0 && c->pb.P <= SF_PCH;
     if (rt_list && !c->rtab_tried && c->opt.sigma_table >= 0) {
         c->rtab_tried = true;
         const size_t bytes = (size_t)nj * c->pb.N * (size_t)c->pb.P * (size_t)c->pb.M;
@@ -1333,31 +1800,87 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
         }
     }
     const bool rt = rt_list && c->d_rtab != nullptr;
+    const size_t smem = sf_smem_layout(c->pb.P < SF_PCH ? c->pb.P : SF_PCH, rt).total;
     A.rtab = rt ? c->d_rtab : nullptr;
     using Kern = void (*)(SigmaFastArgs);
-    Kern kern;
-    if (grid_mode)
-        kern = c->pb.tp == 0.0
-                   ? (unib ? sigma_grid_fast_kernel<true, true> : sigma_grid_fast_kernel<true, false>)
-                   : (unib ? sigma_grid_fast_kernel<false, true> : sigma_grid_fast_kernel<false, false>);
-    else if (rt)
-        kern = c->pb.tp == 0.0 ? (unib ? sigma_fast_kernel<true, true, true> : sigma_fast_kernel<true, false, true>)
-                               : (unib ? sigma_fast_kernel<false, true, true> : sigma_fast_kernel<false, false, true>);
-    else
-        kern = c->pb.tp == 0.0 ? (unib ? sigma_fast_kernel<true, true, false> : sigma_fast_kernel<true, false, false>)
-                               : (unib ? sigma_fast_kernel<false, true, false> : sigma_fast_kernel<false, false, false>);
+    static const Kern plain[2][2][2] = {   // [t' = 0][uniform blocks][table]
+        {{sigma_fast_kernel<false, false, false, false>, sigma_fast_kernel<false, false, true, false>},
+         {sigma_fast_kernel<false, true, false, false>, sigma_fast_kernel<false, true, true, false>}},
+        {{sigma_fast_kernel<true, false, false, false>, sigma_fast_kernel<true, false, true, false>},
+         {sigma_fast_kernel<true, true, false, false>, sigma_fast_kernel<true, true, true, false>}}};
+    static const Kern lines[2][2] = {
+        {sigma_fast_kernel<false, false, false, true>, sigma_fast_kernel<false, true, false, true>},
+        {sigma_fast_kernel<true, false, false, true>, sigma_fast_kernel<true, true, false, true>}};
+    const int tp0 = c->pb.tp == 0.0;
+    const Kern kern = d_K ? lines[tp0][unib] : plain[tp0][unib][rt];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(c, e, "sigma_fast smem attribute");
-    // grid mode: one CTA per (patch a, target) takes every q block, so that the
-    // per-CTA histogram reaches the FP64 one with few atomics per bin
     const int nqb = div_up(c->pb.M, 256 * SF_QPT);
-    A.qb = grid_mode ? nqb : (c->tune.sigma_qblocks > 0 ? c->tune.sigma_qblocks : SF_QB);
-    dim3 grid(div_up(nqb, A.qb), c->pb.N, nj);
+    A.qb = c->tune.sigma_qblocks > 0 ? c->tune.sigma_qblocks : SF_QB;
     prof_begin(c);
-    kern<<<grid, 256, smem, c->stream>>>(A);
-    prof_end(c, grid_mode ? K_SIGMA_HIST : K_SIGMA_Z);
+    kern<<<dim3(div_up(nqb, A.qb), c->pb.N, nj), 256, smem, c->stream>>>(A);
+    if (tg.sym.mode == 2) {
+        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(A);
+        // every patch, should the record have run over
+        SigmaFastArgs F = A;
+        F.only_full = true;
+        F.jlist = nullptr;
+        F.sym = SymMode();
+        F.sig = c->d_sig + 3 * c->pb.N;
+        kern<<<dim3(div_up(nqb, A.qb), c->pb.N, c->pb.N), 256, smem, c->stream>>>(F);
+    }
+    prof_end(c, K_SIGMA_Z);
     e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_fast_kernel");
+}
+
+// Words per moment of the frequency-grid histogram and whether moment 0 has a
+// second word: the smallest that holds the bins beside the projection table.
+// 227 KB of shared memory hold 6 x 5952 words or 5 x 6880.
+constexpr int kHfBins[3] = {4864, 5952, 6880};
+
+static int hist_variant(int nbins)
+{
+    for (int v = 0; v < 3; ++v)
+        if (nbins <= kHfBins[v]) return v;
+    return -1;
+}
+
+// Binned pole density of the target slots into hist (FP32, wedge grid).
+static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                                      const SigmaTargets &tg, double *hist, double e_min, double h, int nbins)
+{
+    const int nj = tg.slots(c->pb.N), N = c->pb.N, v = hist_variant(nbins);
+    qpfrg_status s = launch_kp_table(c, tg.sym.mode == 2 ? nullptr : tg.jlist, nj);
+    if (s != QPFRG_OK) return s;
+    SigmaFastArgs A = fast_args(c, T, d_V, d_Z, d_K, tg);
+    A.hist = hist;
+    const double c0 = -e_min / h - 0.5;      // bin centre b at e_min + (b + 1/2) h
+    A.c_int = (int)std::rint(c0);
+    A.c_frac = (float)(c0 - A.c_int);
+    A.inv_h = (float)(1.0 / h);
+    A.inv_h_lo = (float)(1.0 / h - (double)A.inv_h);
+    A.h = (float)h;
+    A.nbins = nbins;
+    using Kern = void (*)(SigmaFastArgs);
+    static const Kern table[3][2] = {
+        {sigma_hist_kernel<kHfBins[0], true, false>, sigma_hist_kernel<kHfBins[0], true, true>},
+        {sigma_hist_kernel<kHfBins[1], true, false>, sigma_hist_kernel<kHfBins[1], true, true>},
+        {sigma_hist_kernel<kHfBins[2], false, false>, sigma_hist_kernel<kHfBins[2], false, true>}};
+    const Kern kern = table[v][d_K ? 1 : 0];
+    const size_t smem = hf_smem_layout(kHfBins[v], v < 2).total;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(c, e, "sigma_hist smem attribute");
+    // one CTA per SM: split the q blocks until there are eight waves of the
+    // listed targets (a flush follows every block either way)
+    const int nqb = div_up(c->pb.M, HF_THR * HF_QPT);
+    const long per = (long)N * (tg.jlist ? tg.n : nj);
+    const int split = (int)std::max<long>(1, std::min<long>(nqb, (8 * 152 + per - 1) / per));
+    prof_begin(c);
+    kern<<<dim3(split, N, nj), HF_THR, smem, c->stream>>>(A);
+    prof_end(c, K_SIGMA_HIST);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_hist_kernel");
 }
 
 template <typename R>
@@ -1395,129 +1918,104 @@ static void fill_args(qpfrg_ctx *c, SigmaArgs<R> &A, const FineTable<R> &fine, d
     A.nbins = 0;
 }
 
-qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, double *d_Zout,
-                            bool use_symmetry)
+// Z or slopes of every patch from the target slots' sums in d_sig
+static qpfrg_status launch_z_update(qpfrg_ctx *c, const SigmaTargets &tg, double *Z, double *slopes)
 {
     const int N = c->pb.N;
-    // The zone edge breaks the C4v covariance of the angular projection at
-    // the rounding level (mirror pairs land on |k_x| = pi exactly), which
-    // moves Z on symmetric patches by ~1e-6: reduce in mixed precision only.
-    const bool sym = use_symmetry && c->d_jirr != nullptr && c->opt.precision != QPFRG_FP64;
-    const int nj = sym ? c->n_irr : N;
-    cudaError_t e = cudaMemsetAsync(c->d_sig, 0, 2 * (size_t)N * sizeof(double), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "memset sigma");
-    qpfrg_status s;
-    if (c->opt.precision == QPFRG_FP64) {
-        SigmaArgs<double> A;
-        fill_args(c, A, c->f64, T, d_V, d_Z);
-        A.nj = nj;
-        A.jlist = sym ? c->d_jirr : nullptr;
-        s = launch_sigma(c, false, A, K_SIGMA_Z);
-    } else if (c->d_ptab) {
-        s = launch_sigma_fast(c, T, d_V, d_Z, sym ? c->d_jirr : nullptr, nj);
-    } else {
-        SigmaArgs<float> A;
-        fill_args(c, A, c->f32, T, d_V, d_Z);
-        A.nj = nj;
-        A.jlist = sym ? c->d_jirr : nullptr;
-        s = launch_sigma(c, false, A, K_SIGMA_Z);
-    }
-    if (s != QPFRG_OK) return s;
     prof_begin(c);
-    z_update_kernel<<<div_up(N, 128), 128, 0, c->stream>>>(c->d_sig, sym ? c->d_rep : nullptr, d_Zout, N);
+    z_update_kernel<<<div_up(N, 128), 128, 0, c->stream>>>(c->d_sig, c->d_sig + 2 * N, c->d_sig + 3 * N,
+                                                              reinterpret_cast<unsigned *>(c->d_sig + 4 * N),
+                                                              c->max_events, tg.rep, tg.sym, Z, slopes, N);
     prof_end(c, K_Z_UPDATE);
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "z_update_kernel");
 }
 
-// Whether (V, Z) keep the C4v symmetry of the angular patches: flag set when
-// an image V(g k1, g k2, g k3) or Z(g k) differs from the original by more
-// than tol (1 + |v|), g running over the rotations w -> w + m N_a/4 and the
-// reflections w -> -w + m N_a/4 of the wedge w of patch j = w ns + s.
-__global__ void c4v_check_kernel(const double *V, const double *Z, int N, int ns, double tol,
-                                 unsigned long long *flag)
+// Tolerance, relative to the largest magnitudes, of the C4v test that admits the
+// reduced targets: an asymmetry enters the chord slope at first order (FP32 sums
+// carry 1e-6); the frequency grid's own accuracy is 3e-5.
+constexpr double kTolZ = 1e-6, kTolGrid = 1e-5;
+
+// state_symmetric: (V, Z) is the flow's state, symmetric by construction
+// (irreducible targets, halved on the mirror lines).
+qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, double *d_Zout,
+                            bool state_symmetric)
 {
-    const long NN = (long)N * N, n3 = NN * N;
-    const int Na = N / ns, q = Na / 4;
-    for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < n3; idx += (long)gridDim.x * blockDim.x) {
-        const int i = (int)(idx / NN), j = (int)((idx / N) % N), l = (int)(idx % N);
-        const double v = V[idx];
-        bool bad = false;
-        for (int g = 1; g < 8; ++g) {
-            const int m = g & 3, sg = g < 4 ? 1 : -1;
-            auto img = [&](int x) { return ((sg * (x / ns) + m * q) % Na + Na) % Na * ns + x % ns; };
-            const double w = V[((long)img(i) * N + img(j)) * N + img(l)];
-            bad = bad || fabs(w - v) > tol * (1.0 + fabs(v));
-            if (idx < N && Z) bad = bad || fabs(Z[img((int)idx)] - Z[idx]) > tol * (1.0 + fabs(Z[idx]));
-        }
-        if (bad) atomicOr(flag, 1ull);
+    const int N = c->pb.N;
+    cudaError_t e = cudaMemsetAsync(c->d_sig, 0, (4 * (size_t)N + 1) * sizeof(double), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "memset sigma");
+    qpfrg_status s;
+    SigmaTargets tg;
+    tg.n = N;
+    // The zone edge breaks the C4v covariance of the angular projection at
+    // the rounding level (mirror pairs land on |k_x| = pi exactly), which
+    // moves Z on symmetric patches by ~1e-6: the state's reduction in mixed
+    // precision only.
+    if (state_symmetric && c->d_jirr != nullptr && c->opt.precision != QPFRG_FP64) {
+        tg.jlist = c->d_jirr;
+        tg.n = c->n_irr;
+        tg.rep = c->d_rep;
+        tg.mirror = c->pb.n_theta % 2 == 0 ? 1 : 0;
     }
-}
-
-static qpfrg_status c4v_check(qpfrg_ctx *c, const double *d_V, const double *d_Z, bool &sym)
-{
-    sym = false;
-    const int N = c->pb.N, ns = c->pb.n_shell;
-    if ((N / ns) % 4 != 0) return QPFRG_OK;
-    cudaError_t e = cudaMemsetAsync(c->d_red, 0, sizeof(unsigned long long), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "memset symmetry flag");
-    const long n3 = (long)N * N * N;
-    c4v_check_kernel<<<(int)std::min<long>((n3 + 255) / 256, 152L * 8), 256, 0, c->stream>>>(d_V, d_Z, N, ns, 1e-5,
-                                                                                            c->d_red);
-    unsigned long long flag = 1;
-    if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&flag, c->d_red, sizeof(flag), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
-        return cuda_fail(c, e, "symmetry check");
-    sym = flag == 0;
-    return QPFRG_OK;
-}
-
-// Bin count of the frequency-grid histogram: with h = eta/4 the offset of a
-// pole from its bin centre is at most |z - E_b|/8, so the moment expansion
-// truncated after moment 4 is accurate to 8^-5 = 3e-5 relative per pole.
-static int grid_bins(const qpfrg_ctx *c, double e_min, double e_max)
-{
-    const double h_target = 0.25 * c->opt.eta;
-    int nb = (int)std::ceil((e_max - e_min) / h_target);
-    if (nb < 64) nb = 64;
-    if (nb > 1 << 16) nb = 1 << 16;
-    return nb;
+    if (c->opt.precision == QPFRG_FP64) {
+        SigmaArgs<double> A;
+        fill_args(c, A, c->f64, T, d_V, d_Z);
+        s = launch_sigma(c, false, A, K_SIGMA_Z);
+    } else if (c->d_ptab) {
+        if (!tg.jlist) {
+            tg = device_targets(c, kTolZ, 0);
+            if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1)) != QPFRG_OK) return s;
+        }
+        s = launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
+    } else {
+        SigmaArgs<float> A;
+        fill_args(c, A, c->f32, T, d_V, d_Z);
+        A.nj = tg.n;
+        A.jlist = tg.jlist;
+        s = launch_sigma(c, false, A, K_SIGMA_Z);
+    }
+    if (s != QPFRG_OK) return s;
+    return launch_z_update(c, tg, d_Zout, nullptr);
 }
 
 // Chord slopes of the two-loop term with the interaction flow's line weights
 // (Katanin factors d_K, ones without the correction) for every patch, into
-// c->d_sig: the generic kernel, exact projection.
-qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K)
+// d_slopes.  FP32 wedge grid: the targets that the C4v test of (V, Z, K) in
+// c->d_sym admits; otherwise the generic kernel for every patch.
+qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                                double *d_slopes)
 {
-    cudaError_t e = cudaMemsetAsync(c->d_sig, 0, 2 * (size_t)c->pb.N * sizeof(double), c->stream);
+    cudaError_t e = cudaMemsetAsync(c->d_sig, 0, (4 * (size_t)c->pb.N + 1) * sizeof(double), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "memset sigma");
+    SigmaTargets tg;
+    tg.n = c->pb.N;
+    qpfrg_status s;
     if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
         fill_args(c, A, c->f64, T, d_V, d_Z);
         A.K = d_K;
-        return launch_sigma(c, false, A, K_SIGMA_Z);
+        s = launch_sigma(c, false, A, K_SIGMA_Z);
+    } else if (c->d_ptab) {
+        tg = device_targets(c, kTolZ, 0);
+        s = launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
+    } else {
+        SigmaArgs<float> A;
+        fill_args(c, A, c->f32, T, d_V, d_Z);
+        A.K = d_K;
+        s = launch_sigma(c, false, A, K_SIGMA_Z);
     }
-    SigmaArgs<float> A;
-    fill_args(c, A, c->f32, T, d_V, d_Z);
-    A.K = d_K;
-    return launch_sigma(c, false, A, K_SIGMA_Z);
+    if (s != QPFRG_OK) return s;
+    return launch_z_update(c, tg, nullptr, d_slopes);
 }
 
+// d_K (interaction flow): the C4v test of (V, Z, K) is already in c->d_sym
 qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, double *d_re,
                                double *d_im, const double *d_K)
 {
     const int N = c->pb.N, n_omega = c->opt.n_omega;
-    // pole energies E = x_q + x_r - x_p lie in [2 min x - max x, 2 max x - min x]
-    double xmin = 1e300, xmax = -1e300;
-    for (int p = 0; p < c->pb.M; ++p) {
-        const double kx = c->fk[2 * p], ky = c->fk[2 * p + 1];
-        const double x = -2.0 * c->pb.t * (std::cos(kx) + std::cos(ky)) -
-                         4.0 * c->pb.tp * std::cos(kx) * std::cos(ky) - c->pb.mu;
-        xmin = x < xmin ? x : xmin;
-        xmax = x > xmax ? x : xmax;
-    }
+    // pole energies E = x_q + x_r - x_p lie in [2 min x - max x, 2 max x - min x];
     // r = k + p - q is not a fine point: bound its dispersion by the band
+    double xmin = c->fx_min, xmax = c->fx_max;
     const double band_lo = -4.0 * std::fabs(c->pb.t) - 4.0 * std::fabs(c->pb.tp) - c->pb.mu;
     const double band_hi = 4.0 * std::fabs(c->pb.t) + 4.0 * std::fabs(c->pb.tp) - c->pb.mu;
     xmin = std::fmin(xmin, band_lo);
@@ -1526,9 +2024,14 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
         xmin *= c->opt.z_max;
         xmax *= c->opt.z_max;
     }
+    // Bins of width h <= eta / 4: the offset of a pole from its bin centre is at
+    // most |z - E_b| / 8, so the moment expansion truncated after moment 4 is
+    // accurate to 8^-5 = 3e-5 relative per pole.
     const double e_min = 2.0 * xmin - xmax - 1e-9, e_max = 2.0 * xmax - xmin + 1e-9;
-    const int nbins = grid_bins(c, e_min, e_max);
-    const size_t need = (size_t)N * 5 * nbins;
+    const int nbins = (int)std::fmin(std::fmax(std::ceil((e_max - e_min) / (0.25 * c->opt.eta)), 64.0), 65536.0);
+    const double h = (e_max - e_min) / nbins;
+    // histogram, then the sums per target slot
+    const size_t hist_n = (size_t)N * 5 * nbins, need = hist_n + 2 * (size_t)N * n_omega;
     if (need > c->hist_elems) {
         if (c->d_hist) cudaFree(c->d_hist);
         c->d_hist = nullptr;
@@ -1541,17 +2044,16 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     }
     cudaError_t e = cudaMemsetAsync(c->d_hist, 0, need * sizeof(double), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "memset histogram");
-    const double h = (e_max - e_min) / nbins;
+    double *acc = c->d_hist + hist_n;
     qpfrg_status s;
-    bool sym = false;
-    if (!d_K && c->opt.precision != QPFRG_FP64 && c->d_ptab && sigma_fast_smem(c, nbins) <= 226 * 1024) {
+    SigmaTargets tg;
+    tg.n = N;
+    if (c->opt.precision != QPFRG_FP64 && c->d_ptab && hist_variant(nbins) >= 0) {
         // FP32 wedge grid: table projection, histogram in shared memory; a
-        // C4v-symmetric (V, Z) needs only the irreducible targets
-        if (c->d_jgrid) {
-            if ((s = c4v_check(c, d_V, d_Z, sym)) != QPFRG_OK) return s;
-        }
-        s = launch_sigma_fast(c, T, d_V, d_Z, sym ? c->d_jgrid : nullptr, sym ? c->n_grid : N, c->d_hist, e_min,
-                              h, nbins);
+        // C4v-symmetric (V, Z) needs only the irreducible and zone-edge targets
+        tg = device_targets(c, kTolGrid, 2);
+        if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1)) != QPFRG_OK) return s;
+        s = launch_sigma_hist(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
     } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
         fill_args(c, A, c->f64, T, d_V, d_Z);
@@ -1572,13 +2074,14 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     if (s != QPFRG_OK) return s;
     const double w0 = c->opt.omega_min;
     const double dw = n_omega > 1 ? (c->opt.omega_max - c->opt.omega_min) / (n_omega - 1) : 0.0;
-    dim3 grid(div_up(n_omega, 128), N);
+    const int nslot = tg.slots(N);
     prof_begin(c);
-    sigma_grid_kernel<<<grid, 128, 0, c->stream>>>(c->d_hist, nbins, e_min, h, n_omega, w0, dw, c->pb.eta,
-                                                   d_re, d_im, N, sym ? c->d_repgrid : nullptr);
+    sigma_resum_kernel<<<dim3(div_up(n_omega, 128), div_up(nbins, RG_BINS), div_up(nslot, RG_T)), 128, 0, c->stream>>>(
+        c->d_hist, nbins, e_min, h, n_omega, w0, dw, c->pb.eta, acc, nslot, tg.n, tg.sym);
+    sigma_spread_kernel<<<dim3(div_up(n_omega, 128), N), 128, 0, c->stream>>>(acc, tg.rep, tg.sym, n_omega, d_re, d_im);
     prof_end(c, K_SIGMA_GRID);
     e = cudaGetLastError();
-    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_grid_kernel");
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_resum_kernel");
 }
 
 }  // namespace qpfrg
