@@ -262,7 +262,7 @@ qpfrg_status setup_group(Group &g, const qpfrg_lattice *lattice, const qpfrg_fin
         return cuda_fail(c, e, "clear batch buffers");
     // every flow starts at V = U with Z = 1, C4v symmetric, and stays so:
     // the row orbits apply to the whole batch when the context built them
-    g.compact = c->rows_ok;
+    g.compact = c->rows_exact;
     double *outc = nullptr;
     std::vector<double *> poutc(F, nullptr);
     if (g.compact) {

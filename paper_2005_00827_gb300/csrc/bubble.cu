@@ -529,7 +529,7 @@ __device__ __forceinline__ void bubble_body(const BubbleArgs<R> &A, unsigned cha
             for (int im = 0; im < nimg; ++im) {
                 int Qi = kq, ai = a, g = 0;
                 if (img) {
-                    const int2 e = img[8 * (long)kq + im];
+                    const int2 e = img[kLoopImages * (long)kq + im];
                     Qi = e.x;
                     ai = e.y & 0xffff;
                     g = e.y >> 16;
@@ -692,10 +692,11 @@ qpfrg_status launch_bubbles(qpfrg_ctx *c, double lambda, const double *d_Z, bool
     c->rows_compact = sym.mode == 1;
     if (c->opt.precision == QPFRG_FP64)
         return launch_r<double>(c, lambda, d_Z, d_K, z_symmetric, c->f64, c->qpp64, c->qph64, kThrF64, sym);
-    if (c->opt.precision == QPFRG_MIXED_TC) {
+    if (c->opt.precision == QPFRG_MIXED_TC && !c->tc_ready) {
         qpfrg_status s = launch_tc_prep(c);       // B operands and V^T of this stage
         if (s != QPFRG_OK) return s;
     }
+    c->tc_ready = false;
     return launch_r<float>(c, lambda, d_Z, d_K, z_symmetric, c->f32, c->qpp32, c->qph32, kThrF32, sym);
 }
 

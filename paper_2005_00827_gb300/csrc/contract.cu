@@ -38,7 +38,8 @@ struct ContractArgs {
     const R *B;                  // bubble tables [f][row][a][b], family stride N^4
     const R *V;                  // stage vertex
     const R *P;                  // permuted views [cr, d1, d2][a][b][n]
-    const int *rep;              // compact form: transfer pair of a row
+    const int *rep;              // compact form: [family][row] transfer pair of a row
+    int n_can;                   // compact form: rows of the table (row m >= n_can holds the table row m - n_can)
     double *part;                // [split][job][row][n]
     int N, ntiles, njobs;
     int jobs[4];                 // 0 pp, 1 cr, 2 d first product, 3 d second product
@@ -93,9 +94,10 @@ __global__ void __launch_bounds__(256) contract_kernel(const ContractArgs<R> A)
         const int m = m0 + (tid >> 4) + 16 * e;
         rok[e] = m < sh.rows;
         const int mm = rok[e] ? m : 0;
-        const int Q = compact ? A.rep[mm] : mm;
+        const int Q = compact ? A.rep[mm + (job == 0 ? 0 : sh.rows)] : mm;
+        const int trow = compact && mm >= A.n_can ? mm - A.n_can : mm;
         const int q1 = Q / N, q2 = Q - q1 * N;
-        Brow[e] = A.B + (job == 0 ? 0 : NN * NN) + (long)mm * NN;
+        Brow[e] = A.B + (job == 0 ? 0 : NN * NN) + (long)trow * NN;
         frow[e] = A.V + (job == 0 ? (long)Q * N : (job == 1 ? (long)q2 * N + q1 : (long)q1 * NN + q2));
         grow[e] = A.V + (long)q1 * N + q2;   // + a N^2
     }
@@ -254,7 +256,7 @@ __global__ void expand_kernel(const ExpandArgs A)
             const int n = ch == 0 ? k3 : (ch == 1 ? k1 : k2);
             long o = (long)Q * N + n;
             if (c) {
-                const int e = __ldg(A.rowmap + Q);
+                const int e = __ldg(A.rowmap + (ch == 0 ? 0 : (long)N * N) + Q);
                 o = (long)(e & 0xffffff) * N + c4v_patch(c4v_inverse(e >> 24), n, A.ns, Na);
             }
             v += __ldg(A.outc + ch * stride + o);
@@ -300,9 +302,12 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
         is[x] = (short)c4v_apply(4, x, N, ns);
     }
     __syncthreads();
-    double m = 0.0, d = 0.0;
+    // maxima of magnitudes as integers (the bits of non-negative doubles order like
+    // the values, NaN above infinity): two FP64 subtractions per element are left
+    // on the FP64 pipe (with FP64 maxima and tests np96 took 23 us)
+    unsigned long long m = 0, d = 0;
+    const unsigned long long mag = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;
     bool fin = true;
-    const double inf = __longlong_as_double(0x7ff0000000000000LL);
     for (int r = w0; r < NN; r += ws) {
         const int i = r / N, j = r - i * N;
         const IN *row = V + (long)r * N;
@@ -312,54 +317,86 @@ __global__ void __launch_bounds__(256) stage_prep_kernel(const IN *__restrict__ 
             rs = V + ((long)is[i] * N + is[j]) * N;
         }
         for (int l = lane; l < N; l += 32) {
-            const double v = (double)row[l];
+            const IN v = row[l];
             if (Vf) Vf[(long)r * N + l] = (float)v;
             if (!sym) continue;
-            const double e = fmax(fabs((double)rr[ir[l]] - v), fabs((double)rs[is[l]] - v));
-            d = isfinite(v) ? fmax(d, e) : inf;
-            if (isfinite(v)) m = fmax(m, fabs(v));
+            const IN e1 = rr[ir[l]] - v, e2 = rs[is[l]] - v;
+            const unsigned long long b1 = (unsigned long long)__double_as_longlong((double)e1) & mag;
+            const unsigned long long b2 = (unsigned long long)__double_as_longlong((double)e2) & mag;
+            const unsigned long long bv = (unsigned long long)__double_as_longlong((double)v) & mag;
+            d = max(d, max(b1, b2));
+            if (bv < inf) m = max(m, bv);
             else fin = false;
         }
     }
     if (!sym) return;
-    auto reduce = [&](double x, unsigned long long *slot) {
-        for (int off = 16; off > 0; off >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, off));
-        // non-negative values order like their bits
-        if (lane == 0 && x > 0.0) atomicMax(slot, (unsigned long long)__double_as_longlong(x));
+    if (!fin) d = inf;
+    // one atomic a block, and only where it raises the maximum
+    auto raise = [&](unsigned long long v, unsigned long long *slot) {
+        if (v > *(volatile unsigned long long *)slot) atomicMax(slot, v);
     };
-    reduce(m, sym);
-    reduce(d, sym + 1);
+    __shared__ unsigned long long sm[8], sd[8];
+    for (int off = 16; off > 0; off >>= 1) {
+        m = max(m, __shfl_down_sync(0xffffffffu, m, off));
+        d = max(d, __shfl_down_sync(0xffffffffu, d, off));
+    }
+    if (lane == 0) {
+        sm[threadIdx.x >> 5] = m;
+        sd[threadIdx.x >> 5] = d;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < nw; ++k) {
+            m = max(m, sm[k]);
+            d = max(d, sd[k]);
+        }
+        raise(m, sym);
+        raise(d, sym + 1);
+    }
     if (!fin) atomicOr(&sym[4], 1ull);
     if (w0 == 0) {
-        double mz = 0.0, dz = 0.0;
+        unsigned long long mz = 0, dz = 0;
+        bool zfin = true;
         for (int y = lane; y < nz * N; y += 32) {
             const int x = y % N;
             const double *Zy = Z + (y - x);
             const double z = Zy[x];
-            const double e = fmax(fabs(Zy[ir[x]] - z), fabs(Zy[is[x]] - z));
-            dz = isfinite(z) ? fmax(dz, e) : inf;
-            if (isfinite(z)) mz = fmax(mz, fabs(z));
-            else fin = false;
+            const unsigned long long b1 = (unsigned long long)__double_as_longlong(Zy[ir[x]] - z) & mag;
+            const unsigned long long b2 = (unsigned long long)__double_as_longlong(Zy[is[x]] - z) & mag;
+            const unsigned long long bz = (unsigned long long)__double_as_longlong(z) & mag;
+            dz = max(dz, max(b1, b2));
+            if (bz < inf) mz = max(mz, bz);
+            else zfin = false;
         }
-        reduce(mz, sym + 2);
-        reduce(dz, sym + 3);
-        if (!fin) atomicOr(&sym[4], 1ull);
+        if (!zfin) {
+            dz = inf;
+            atomicOr(&sym[4], 1ull);
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            mz = max(mz, __shfl_down_sync(0xffffffffu, mz, off));
+            dz = max(dz, __shfl_down_sync(0xffffffffu, dz, off));
+        }
+        if (lane == 0) {
+            raise(mz, sym + 2);
+            raise(dz, sym + 3);
+        }
     }
 }
 
-// The C4v test of V and of nz arrays of N weights Z into c->d_sym (read by
+// The C4v test of V and of nz arrays of N weights Z into red (read by
 // sym_compact; nz = 0: no test), the FP32 copy
 // when Vf is given and, outside the tensor-core precision, the permuted views.
-static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const double *d_Z, int nz, float *Vf, bool operands)
+static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const double *d_Z, int nz, float *Vf, bool operands,
+                                unsigned long long *red)
 {
     const bool test = nz > 0;
     const int N = c->pb.N, ns = c->pb.n_shell;
     cudaError_t e;
-    if (test && (e = cudaMemsetAsync(c->d_sym, 0, 5 * sizeof(unsigned long long), c->stream)) != cudaSuccess)
+    if (test && (e = cudaMemsetAsync(red, 0, 5 * sizeof(unsigned long long), c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "memset symmetry test");
-    unsigned long long *sym = test ? c->d_sym : nullptr;
+    unsigned long long *sym = test ? red : nullptr;
     const bool views = operands && c->opt.precision != QPFRG_MIXED_TC;
-    const dim3 grid(std::max(1, std::min(div_up((long)N * N, 8), 304)), views ? 4 : 1);
+    const dim3 grid(std::max(1, std::min(div_up((long)N * N, 8), 608)), views ? 4 : 1);
     prof_begin(c);
     if (c->opt.precision == QPFRG_FP64 || !operands)
         stage_prep_kernel<double, double><<<grid, 256, 0, c->stream>>>((const double *)V, d_Z, nz, N, ns, sym, nullptr,
@@ -380,19 +417,19 @@ static qpfrg_status launch_prep(qpfrg_ctx *c, const void *V, bool v64, const dou
 // FP32 copy in the mixed precisions, permuted views of the SIMT contraction.
 qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz)
 {
-    return launch_prep(c, d_V, true, d_Z, nz, c->opt.precision == QPFRG_FP64 ? nullptr : c->d_Vf, true);
+    return launch_prep(c, d_V, true, d_Z, nz, c->opt.precision == QPFRG_FP64 ? nullptr : c->d_Vf, true, c->d_sym);
 }
 
 // The same of a later stage's vertex (FP64, or FP32 in mixed precision).
 qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z, int nz)
 {
     if (c->opt.precision == QPFRG_MIXED_TC) return QPFRG_OK;
-    return launch_prep(c, d_Vin, c->opt.precision == QPFRG_FP64, d_Z, nz, nullptr, true);
+    return launch_prep(c, d_Vin, c->opt.precision == QPFRG_FP64, d_Z, nz, nullptr, true, c->d_sym);
 }
 
-qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz)
+qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz, unsigned long long *red)
 {
-    return launch_prep(c, d_V, true, d_Z, nz, nullptr, false);
+    return launch_prep(c, d_V, true, d_Z, nz, nullptr, false, red);
 }
 
 // Columns per thread: the count (1..3) whose 16-wide tiles pad N least.
@@ -447,6 +484,7 @@ static qpfrg_status launch_simt(qpfrg_ctx *c, const R *V, double scale, double *
     A.V = V;
     A.P = reinterpret_cast<const R *>(c->d_views);
     A.rep = c->d_rrep;
+    A.n_can = c->n_rcan;
     A.part = c->d_partial;
     A.N = N;
     const int nb = contract_nb(N);
@@ -515,6 +553,7 @@ __device__ __forceinline__ void expand_row(const double *__restrict__ outc, cons
     const long ch_stride = (long)nr * N;
     double *row = out + ((long)k1 * N + k2) * N;
     const int e_pp = __ldg(rowmap + k1 * N + k2);
+    rowmap += N * N;             // the particle-hole family's
     for (int k3 = threadIdx.x; k3 < N; k3 += blockDim.x) {
         double v = 0.0;
         auto take = [&](int ch, int e, int n) {
@@ -559,27 +598,23 @@ qpfrg_status launch_rows_expand_batch(qpfrg_ctx *c, const TcBatch &bt)
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out)
 {
     if (c->opt.precision == QPFRG_MIXED_TC) {
-        // the weighted tables of this stage, formed into A tiles inside the contraction
+        // the weighted tables of this stage, formed into A tiles inside the
+        // contraction; representative rows go into compact rows, then expanded
         const unsigned ch = c->pb.channels;
         qpfrg_status s = QPFRG_OK;
-        // representative rows only (row orbits): into the compact rows, then expanded
-        double *dst[3] = {d_out, d_out, d_out};
-        cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)c->pb.N * c->pb.N * c->pb.N * sizeof(double), c->stream);
+        const int N = c->pb.N;
+        const bool orbits = c->rhs_sym.mode != 0;
+        const long per = orbits ? (long)c->n_rrep * N : 0;
+        cudaError_t e = cudaMemsetAsync(d_out, 0, (size_t)N * N * N * sizeof(double), c->stream);
+        if (e == cudaSuccess && orbits) e = cudaMemsetAsync(c->d_outc, 0, 3 * per * sizeof(double), c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "memset right-hand side");
-        if (c->rows_compact) {
-            const long per = (long)c->n_rrep * c->pb.N;
-            e = cudaMemsetAsync(c->d_outc, 0, 3 * per * sizeof(double), c->stream);
-            if (e != cudaSuccess) return cuda_fail(c, e, "memset representative rows");
-            for (int k = 0; k < 3; ++k) dst[k] = c->d_outc + k * per;
-        }
-        if ((ch & QPFRG_CH_PP) && (s = launch_tc_fused(c, 0, -scale, dst[0], K_TC_PP))) return s;
-        if ((ch & QPFRG_CH_CR) && (s = launch_tc_fused(c, 1, -scale, dst[1], K_TC_CR))) return s;
-        if ((ch & QPFRG_CH_D) && (s = launch_tc_fused(c, 2, scale, dst[2], K_TC_D))) return s;
-        if (c->rows_compact) {
-            const int N = c->pb.N, thr = std::min(256, (N + 31) / 32 * 32);
+        if ((ch & QPFRG_CH_PP) && (s = launch_tc_fused(c, 0, -scale, d_out, c->d_outc, K_TC_PP))) return s;
+        if ((ch & QPFRG_CH_CR) && (s = launch_tc_fused(c, 1, -scale, d_out, c->d_outc + per, K_TC_CR))) return s;
+        if ((ch & QPFRG_CH_D) && (s = launch_tc_fused(c, 2, scale, d_out, c->d_outc + 2 * per, K_TC_D))) return s;
+        if (orbits) {
             prof_begin(c);
-            rows_expand_kernel<<<dim3(N, N), thr, 0, c->stream>>>(c->d_outc, c->d_rowmap, c->n_rrep, N,
-                                                                  c->pb.n_shell, ch, d_out);
+            rows_expand_kernel<<<dim3(N, N), std::min(256, (N + 31) / 32 * 32), 0, c->stream>>>(
+                c->d_outc, c->d_rowmap, c->n_rrep, N, c->pb.n_shell, ch, d_out);
             prof_end(c, K_ROWS_EXPAND);
             e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(c, e, "rows_expand_kernel");

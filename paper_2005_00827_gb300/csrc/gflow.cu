@@ -55,13 +55,17 @@ __global__ void gflow_zka_kernel(const double *y, int N, int ns, double g, int z
     sh_min[threadIdx.x] = mn;
     sh_max[threadIdx.x] = mx;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0, lo = 1e300, hi = -1e300;
-        for (int t = 0; t < (int)blockDim.x; ++t) {   // in thread order: deterministic
-            s += sh_sum[t];
-            lo = fmin(lo, sh_min[t]);
-            hi = fmax(hi, sh_max[t]);
+    // a fixed tree: deterministic (one thread adding 256 values took 41 us)
+    for (int w = (int)blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) {
+            sh_sum[threadIdx.x] += sh_sum[threadIdx.x + w];
+            sh_min[threadIdx.x] = fmin(sh_min[threadIdx.x], sh_min[threadIdx.x + w]);
+            sh_max[threadIdx.x] = fmax(sh_max[threadIdx.x], sh_max[threadIdx.x + w]);
         }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double s = sh_sum[0], lo = sh_min[0], hi = sh_max[0];
         *Abar = a_mode == 1 ? lo : (a_mode == 2 ? hi : (a_mode == 3 ? 0.0 : s / (N / ns)));
     }
 }
@@ -159,7 +163,7 @@ qpfrg_status gflow_enqueue_stages(qpfrg_ctx *c, double x, double h)
         // the right-hand side and the self-energy decide by
         const int nz = c->pb.mode == QPFRG_GRID_LATTICE ? 0 : 2;
         if (st == 0) s = launch_stage_prep(c, c->d_V, Zs, nz);
-        else if (c->opt.precision == QPFRG_MIXED_TC && nz) s = launch_sym_test(c, Vst, Zs, nz);
+        else if (c->opt.precision == QPFRG_MIXED_TC && nz) s = launch_sym_test(c, Vst, Zs, nz, c->d_sym);
         else s = launch_stage_views(c, Vin, Zs, nz);
         if (s != QPFRG_OK) return s;
         // vertex: loop kernels with Z and K on the lines, contraction

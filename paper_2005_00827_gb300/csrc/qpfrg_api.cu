@@ -196,6 +196,7 @@ void qpfrg_destroy(qpfrg_t c)
                         c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views, c->d_kfx, c->d_pfx, c->d_events};
         for (void *p : ptrs)
             if (p) cudaFree(p);
+        if (c->ev_test) cudaEventDestroy(c->ev_test);
     }
     Profiler *p = prof_of(c);
     if (p) {
@@ -369,14 +370,17 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
         if (e == cudaSuccess) e = cudaMemset(c->d_B, 0, c->B_bytes);
         if (e != cudaSuccess) return fail(cuda_fail(c, e, "clear tensor-core operands"));
         if ((s = tc_make_maps(c)) != QPFRG_OK) return fail(s);
+        if ((e = cudaEventCreateWithFlags(&c->ev_test, cudaEventDisableTiming)) != cudaSuccess)
+            return fail(cuda_fail(c, e, "cudaEventCreate"));
     }
     if ((s = dev_alloc(c, &c->d_V, n3, "V")) || (s = dev_alloc(c, &c->d_Vs, n3, "V stage")) ||
         (s = dev_alloc(c, &c->d_k, n3, "k")) || (s = dev_alloc(c, &c->d_acc, n3, "acc")) ||
         (s = dev_alloc(c, &c->d_Vf, n3, "V fp32")) || (s = dev_alloc(c, &c->d_Z, N, "Z")) ||
         (s = dev_alloc(c, &c->d_Zwork, N, "Z work")) || (s = dev_alloc(c, &c->d_ones, N, "ones")) ||
         (s = dev_alloc(c, &c->d_sig, 4 * N + 1, "sigma chord")) || (s = dev_alloc(c, &c->d_red, 5, "reduction")) ||
-        (s = dev_alloc(c, &c->d_sym, 5, "symmetry test")))
+        (s = dev_alloc(c, &c->d_sym, 10, "symmetry tests")))
         return fail(s);
+    c->d_sym_v = c->d_sym + 5;
     if (!tcmode && (s = contract_alloc(c)) != QPFRG_OK) return fail(s);
     e = cudaMallocHost((void **)&c->h_red, 10 * sizeof(unsigned long long));
     if (e != cudaSuccess) return fail(cuda_fail(c, e, "cudaMallocHost"));
@@ -432,7 +436,8 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
     if (e != cudaSuccess) return fail(cuda_fail(c, e, "init Z"));
     c->lambda = lambda0;
     c->lambda_end = c->opt.lambda_end;
-    c->c4v_state = c->rows_state = pb.mode == QPFRG_GRID_WEDGE || pb.mode == QPFRG_GRID_SHELL;
+    c->c4v_state = pb.mode == QPFRG_GRID_WEDGE || pb.mode == QPFRG_GRID_SHELL;
+    c->rows_state = c->rows_exact;
     c->steps = 0;
     c->status = QPFRG_FLOW_RUNNING;
     c->max_abs_v = std::fabs(U);
@@ -455,7 +460,8 @@ qpfrg_status qpfrg_rhs(qpfrg_t c, double lambda, const double *d_V, const double
     qpfrg_status s;
     // row orbits need a C4v-symmetric V and Z: tested on the device, where the
     // FP64 and FP32 contractions also take the decision; the tensor-core
-    // contraction's is read back
+    // contraction's is read back (the launches of the form not taken cost its
+    // three channels more than the wait: np60 274 us against 258)
     if ((s = launch_stage_prep(c, d_V, Z, c->rows_ok ? 1 : 0)) != QPFRG_OK) return s;
     SymMode sym;
     if (c->rows_ok) {
@@ -465,8 +471,16 @@ qpfrg_status qpfrg_rhs(qpfrg_t c, double lambda, const double *d_V, const double
         if (c->opt.precision == QPFRG_MIXED_TC) {
             cudaError_t e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 4 * sizeof(unsigned long long),
                                             cudaMemcpyDeviceToHost, c->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-            if (e != cudaSuccess) return cuda_fail(c, e, "C4v test of the RHS input");
+            // the operands do not depend on the form: they are made while the host
+            // waits for the test
+            if (e == cudaSuccess) e = cudaEventRecord(c->ev_test, c->stream);
+            if (e == cudaSuccess && (s = launch_tc_prep(c)) != QPFRG_OK) return s;
+            c->tc_ready = true;
+            if (e == cudaSuccess) e = cudaEventSynchronize(c->ev_test);
+            if (e != cudaSuccess) {
+                c->tc_ready = false;
+                return cuda_fail(c, e, "C4v test of the RHS input");
+            }
             sym.mode = c4v_within(c, rows_tol(c)) ? 1 : 0;
         }
     }
@@ -730,7 +744,8 @@ static qpfrg_status make_child(qpfrg_ctx *parent, double U, double lambda0, doub
     c->max_abs_v = std::fabs(U);
     c->lambda_c = 0.0;
     c->pending = false;
-    c->c4v_state = c->rows_state = c->pb.mode == QPFRG_GRID_WEDGE || c->pb.mode == QPFRG_GRID_SHELL;
+    c->c4v_state = c->pb.mode == QPFRG_GRID_WEDGE || c->pb.mode == QPFRG_GRID_SHELL;
+    c->rows_state = c->rows_exact;
     *out = c;
     return QPFRG_OK;
 }
@@ -896,9 +911,9 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->d_acc, Z, c->pb.N * sizeof(double), cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "set_state upload");
-    qpfrg_status st = launch_sym_test(c, c->d_k, c->d_acc, 1);
+    qpfrg_status st = launch_sym_test(c, c->d_k, c->d_acc, 1, c->d_sym_v);
     if (st != QPFRG_OK) return st;
-    if ((e = cudaMemcpyAsync(&c->h_red[5], c->d_sym, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+    if ((e = cudaMemcpyAsync(&c->h_red[5], c->d_sym_v, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                              c->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state check");
@@ -920,7 +935,7 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     // of the state's symmetry).  The slopes of the self-energy ODE set Z, K and
     // A, so they have to be symmetric as well.
     const double rtol = c->opt.precision == QPFRG_FP64 ? rows_tol(c) : (c->opt.precision == QPFRG_MIXED ? 3e-7 : tol);
-    c->rows_state = c->rows_ok && c->c4v_state && (c->opt.precision == QPFRG_MIXED_TC || c4v_within(c, rtol));
+    c->rows_state = c->rows_exact && c->c4v_state && (c->opt.precision == QPFRG_MIXED_TC || c4v_within(c, rtol));
     if (c->d_gy && c->rows_state) c->rows_state = slopes_symmetric(c, Z + c->pb.N, rtol);
     c->status = hd.status;
     c->steps = (int)hd.steps;

@@ -229,6 +229,9 @@ __host__ __device__ inline int c4v_apply(int g, int j, int N, int ns)
     return (r < 0 ? r + Na : r) * ns + sh;
 }
 
+// image rows of one evaluated loop-kernel row: C4v and the exchange
+constexpr int kLoopImages = 16;
+
 // inverse element: rotations by m -> by 4 - m; every reflection is an involution
 __host__ __device__ inline int c4v_inverse(int g) { return (g & 4) ? g : ((4 - (g & 3)) & 3); }
 
@@ -277,7 +280,7 @@ struct qpfrg_ctx {
     std::vector<qpfrg::LoopGroup> lgroups;
     int *d_lrepQ = nullptr;      // transfer Q of each representative row (families concatenated)
     int *d_lnimg = nullptr;      // number of image rows of each representative
-    int2 *d_limg = nullptr;      // 8 slots per representative: (Q', a' | g << 16)
+    int2 *d_limg = nullptr;      // kLoopImages slots per representative: (Q', a' | g << 16)
     int4 *d_ltask = nullptr;     // (family, patch, first representative, count) per CTA
     long n_lrep = 0;
     int ltask_qchunk = 0, n_ltask = 0;
@@ -290,15 +293,24 @@ struct qpfrg_ctx {
     // only representative rows are tabled and contracted and the result is
     // expanded (contract.cu).  Built when every loop-kernel row is covariant.
     bool rows_ok = false;
+    // no pair is a row for itself: a symmetric state keeps its symmetry over the
+    // stages of a step (else only a given, tested vertex takes the row orbits)
+    bool rows_exact = false;
     bool rows_compact = false;   // the table of the current RHS holds representative rows only
     bool rows_state = false;     // the flow state is symmetric enough for the row orbits
     qpfrg::SymMode rhs_sym;      // form of the current RHS
-    unsigned long long *d_sym = nullptr;   // C4v test of a right-hand side's inputs (SymMode::red)
+    cudaEvent_t ev_test = nullptr;   // the test's result is on the host
+    bool tc_ready = false;       // the tensor-core operands of the current RHS are enqueued
+    // C4v tests (SymMode::red, 5 words each): of a right-hand side's inputs, and of
+    // other vertices (self-energies, state images)
+    unsigned long long *d_sym = nullptr, *d_sym_v = nullptr;
     double *d_partial = nullptr; // partial rows of the SIMT contraction [split][job][row][n]
     void *d_views = nullptr;     // permuted views of the stage vertex [cr, d1, d2][a][b][n] (FP64 or FP32)
-    int n_rrep = 0;
-    int *d_rrep = nullptr;       // Q of each representative row
-    int *d_rowmap = nullptr;     // per Q: representative index | g << 24, Q = g rep
+    // Rows n_rcan .. n_rrep - 1 are the exchanged pairs of rows 0 ..: same transfer
+    // momentum, same table row (symmetry.cu)
+    int n_rrep = 0, n_rcan = 0;
+    int *d_rrep = nullptr;       // [family][row]: Q of each representative row
+    int *d_rowmap = nullptr;     // [family][Q]: row | g << 24, Q = g rep
     int4 *d_rtask = nullptr;     // (family, patch, first representative, count) per loop-kernel CTA
     int rtask_qchunk = 0, n_rtask = 0;
     double *d_outc = nullptr;    // [channel][representative][n] contraction rows
@@ -407,8 +419,8 @@ qpfrg_status row_tasks(qpfrg_ctx *c, int qchunk, int *ntask);
 // V input is FP64 (precision FP64) or FP32 (MIXED); its permuted views are
 // those of the last launch_stage_prep / launch_stage_views.
 qpfrg_status contract_alloc(qpfrg_ctx *c);
-// the C4v test of V (FP64) and nz weight arrays alone, into c->d_sym
-qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz);
+// the C4v test of V (FP64) and nz weight arrays alone, into red
+qpfrg_status launch_sym_test(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz, unsigned long long *red);
 qpfrg_status launch_stage_prep(qpfrg_ctx *c, const double *d_V, const double *d_Z, int nz);
 qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d_Z = nullptr, int nz = 0);
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out);
@@ -475,7 +487,7 @@ qpfrg_status flow_batch_device(const qpfrg_lattice *lattice, const qpfrg_fine_gr
 // tc_prep.cu / tc_fused.cu: tensor-core contraction
 qpfrg_status launch_tc_prep(qpfrg_ctx *c);
 qpfrg_status tc_make_maps(qpfrg_ctx *c);   // TMA maps of the tensor-core operand tiles
-qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, int kid);
+qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, double *outc, int kid);
 
 // ode.cu
 qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_V,

@@ -1682,10 +1682,10 @@ struct SigmaTargets {
     int slots(int N) const { return sym.mode == 2 || !jlist ? N : n; }
 };
 
-// Targets of a given (V, Z): with the symmetry that the device finds (d_sym), the
+// Targets of a given (V, Z): with the symmetry that the device finds (red), the
 // irreducible patches and the zone-edge patches; images copy the sum of their
 // representative.  mirror 2 also halves the targets on a diagonal.
-static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror)
+static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror, const unsigned long long *red)
 {
     SigmaTargets t;
     t.n = c->pb.N;
@@ -1694,7 +1694,7 @@ static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror)
     t.n = c->n_grid;
     t.rep = c->d_repgrid;
     t.sym.mode = 2;
-    t.sym.red = c->d_sym;
+    t.sym.red = red;
     t.sym.tol = tol / 3.0;
     t.mirror = c->pb.n_theta % 2 == 0 ? mirror : 0;
     return t;
@@ -1963,8 +1963,8 @@ qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const dou
         s = launch_sigma(c, false, A, K_SIGMA_Z);
     } else if (c->d_ptab) {
         if (!tg.jlist) {
-            tg = device_targets(c, kTolZ, 0);
-            if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1)) != QPFRG_OK) return s;
+            tg = device_targets(c, kTolZ, 0, c->d_sym_v);
+            if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         }
         s = launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
     } else {
@@ -1996,7 +1996,7 @@ qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const
         A.K = d_K;
         s = launch_sigma(c, false, A, K_SIGMA_Z);
     } else if (c->d_ptab) {
-        tg = device_targets(c, kTolZ, 0);
+        tg = device_targets(c, kTolZ, 0, c->d_sym);
         s = launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
     } else {
         SigmaArgs<float> A;
@@ -2051,8 +2051,8 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     if (c->opt.precision != QPFRG_FP64 && c->d_ptab && hist_variant(nbins) >= 0) {
         // FP32 wedge grid: table projection, histogram in shared memory; a
         // C4v-symmetric (V, Z) needs only the irreducible and zone-edge targets
-        tg = device_targets(c, kTolGrid, 2);
-        if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1)) != QPFRG_OK) return s;
+        tg = device_targets(c, kTolGrid, 2, d_K ? c->d_sym : c->d_sym_v);
+        if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         s = launch_sigma_hist(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
     } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;

@@ -10,6 +10,13 @@
 // the patch projection is covariant, proj(g k) = g proj(k), the Z-free binned
 // loop kernels satisfy
 //     B_f[g Q][g a][g b] = B_f[Q][a][b].
+// Exchange: the transfer pairs (x, y) and (y, x) have the same momentum
+// k_F(x) + k_F(y), and (x, y) and (y', x') the same k_F(x) - k_F(y), x' = x + N_a/2
+// the patch opposite to x, so that B_pp[x,y] = B_pp[y,x] and B_ph[x,y] =
+// B_ph[y',x'] row by row, columns in place.  The exchange commutes with C4v; the
+// orbits below are those of the 16 elements (g, s): first the exchange if s,
+// then g.  That halves the loop-kernel evaluations (np96, 32 x 32 points, row
+// orbits: 394 -> 229 us a launch).
 // So one row per orbit of (Q, a) is evaluated and written to every image,
 // its columns permuted by g (the Z weights and vertex factors are applied per
 // image).  Covariance is not assumed: check_covariance_kernel compares every
@@ -29,21 +36,22 @@
 
 namespace qpfrg {
 
-// flag[f][Q N + a] = 1 where the partner-map row (f, Q, a) is not the image
-// of its representative's row under g.  rep[Q N + a] = representative's Q N + a,
-// gof[Q N + a] = g with (Q, a) = g (representative).
+// flag[f][Q N + a] = 1 where the partner-map row (f, Q, a) is not the image of its
+// representative's row under g.  rep[f][Q N + a] = representative's Q N + a,
+// gof[f][Q N + a] = g with (Q, a) = g, after an exchange perhaps, of the
+// representative.
 __global__ void check_covariance_kernel(const uint8_t *__restrict__ part, const int *__restrict__ rep,
                                         const uint8_t *__restrict__ gof, uint8_t *__restrict__ flag, int N, int M,
                                         int P, int nt, int nr, int ns)
 {
     const int Q = blockIdx.x, f = blockIdx.y;
-    const long NN = (long)N * N;
+    const long NN = (long)N * N, fo = (long)f * NN * N;
     __shared__ int bad;
     for (int a = 0; a < N; ++a) {
         const long row = (long)Q * N + a;
-        const int r = rep[row];
+        const int r = rep[fo + row];
         if (r == row) continue;                    // uniform over the block
-        const int g = gof[row];
+        const int g = gof[fo + row];
         const int Qr = r / N, ar = r - Qr * N;
         const uint8_t *src = part + ((long)f * NN + Qr) * (long)M + (long)ar * P;
         const uint8_t *dst = part + ((long)f * NN + Q) * (long)M + (long)a * P;
@@ -63,52 +71,160 @@ __global__ void check_covariance_kernel(const uint8_t *__restrict__ part, const 
     }
 }
 
-// Row orbits of the contraction: the representative of the
-// transfer pair Q = (x, y) is its image g Q = (g x, g y) with the smallest
-// index; rowmap[Q] = (representative index | g << 24) with Q = g rep.  Only
-// built when every loop-kernel row passed the covariance check, so that the
-// table rows of the images are exactly the representative's, permuted.
-static qpfrg_status build_row_orbits(qpfrg_ctx *c)
+// (x, y) exchanged, with the same transfer momentum in family f (0 pp, 1 ph)
+static void exchange(int f, int N, int ns, int &x, int &y)
+{
+    const int u = x;
+    x = f == 0 ? y : c4v_apply(2, y, N, ns);
+    y = f == 0 ? u : c4v_apply(2, u, N, ns);
+}
+
+// Row orbits of the contraction: rowmap[f][Q] = (row | g << 24) with Q = g
+// rrep[f][row].  The first n_rcan rows are one pair of each orbit under C4v and
+// exchange, the same in both families: the rows of the table, those first whose
+// exchanged pair lies in another C4v orbit.  The others
+// are these exchanged pairs, in the same order: row n_rcan + i holds the table row
+// i.  A pair Q that failed the covariance check (own[Q]: a momentum on a boundary
+// between patches or shells, decided by rounding) is a row for itself, so that the
+// table rows of the remaining images are exactly the representative's, permuted.
+// (The exchanged row of an orbit may be such a pair: it then stands for the other
+// images only.)  exch = false: every C4v orbit is a row of the table.
+static qpfrg_status build_row_orbits(qpfrg_ctx *c, bool exch, const std::vector<uint8_t> &own)
 {
     const int N = c->pb.N, ns = c->pb.n_shell;
     const long NN = (long)N * N;
-    std::vector<int> repidx(NN, -1), reps, rowmap(NN);
-    // in increasing Q the representative (the orbit's smallest index, <= Q)
-    // is always met first
-    for (long Q = 0; Q < NN; ++Q) {
-        const int x = (int)(Q / N), y = (int)(Q - (long)x * N);
-        long best = -1;
-        int bg = 0;
-        for (int g = 0; g < 8; ++g) {
-            const long gQ = (long)c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns);
-            if (best < 0 || gQ < best) {
-                best = gQ;
-                bg = g;
+    std::vector<int> paired, single;
+    std::vector<uint8_t> seen(NN, 0);
+    for (long Q0 = 0; Q0 < NN; ++Q0) {
+        if (seen[Q0]) continue;
+        // the orbit of Q0; its row is the smallest pair that passed the check
+        // (none did: they are all rows for themselves)
+        long can = NN;
+        int x = (int)(Q0 / N), y = (int)(Q0 - (long)x * N);
+        for (int k = 0; k < (exch ? 2 : 1); ++k) {
+            for (int g = 0; g < 8; ++g) {
+                const long Q = (long)c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns);
+                seen[Q] = 1;
+                if (!own[Q]) can = std::min(can, Q);
             }
+            std::swap(x, y);      // exchanges of both families share their C4v orbit
         }
-        if (best == Q) {
-            repidx[Q] = (int)reps.size();
-            reps.push_back((int)Q);
-        }
-        // bg maps Q onto its representative: Q = bg^-1 rep
-        rowmap[Q] = repidx[best] | (c4v_inverse(bg) << 24);
+        if (can == NN) continue;
+        bool other = exch;        // the exchanged pair lies in another C4v orbit
+        x = (int)(can / N);
+        y = (int)(can - (long)x * N);
+        for (int g = 0; g < 8 && other; ++g)
+            other = (long)c4v_apply(g, y, N, ns) * N + c4v_apply(g, x, N, ns) != can;
+        (other ? paired : single).push_back((int)can);
     }
-    const int nr = (int)reps.size();
+    const size_t norb = single.size();
+    for (long Q = 0; Q < NN; ++Q)
+        if (own[Q]) single.push_back((int)Q);
+    const int npar = (int)paired.size(), ncan = npar + (int)single.size(), nr = ncan + npar;
+    std::vector<int> reps(2 * (size_t)nr), rowmap(2 * NN);
+    for (int f = 0; f < 2; ++f) {
+        int *rep = reps.data() + (size_t)f * nr, *map = rowmap.data() + f * NN;
+        std::copy(paired.begin(), paired.end(), rep);
+        std::copy(single.begin(), single.end(), rep + npar);
+        for (int i = 0; i < npar; ++i) {
+            int x = paired[i] / N, y = paired[i] - x * N;
+            exchange(f, N, ns, x, y);
+            rep[ncan + i] = x * N + y;
+        }
+        for (int m = 0; m < nr; ++m)
+            for (int g = 7; g >= 0 && !(m >= npar + (int)norb && m < ncan); --g) {
+                const int x = rep[m] / N, y = rep[m] - x * N;
+                map[c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns)] = m | (g << 24);
+            }
+        for (int m = npar + (int)norb; m < ncan; ++m) map[rep[m]] = m;
+    }
     cudaError_t e;
-    if ((e = cudaMalloc((void **)&c->d_rrep, nr * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc((void **)&c->d_rowmap, NN * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc((void **)&c->d_rtask, (2L * N * ((nr + 7) / 8) + 8) * sizeof(int4))) != cudaSuccess ||
+    if ((e = cudaMalloc((void **)&c->d_rrep, 2 * (size_t)nr * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc((void **)&c->d_rowmap, 2 * NN * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc((void **)&c->d_rtask, (2L * N * ((ncan + 7) / 8) + 8) * sizeof(int4))) != cudaSuccess ||
         (c->opt.precision == QPFRG_MIXED_TC &&
          (e = cudaMalloc((void **)&c->d_outc, 3L * nr * N * sizeof(double))) != cudaSuccess))
         return cuda_fail(c, e, "cudaMalloc(row orbits)");
-    e = cudaMemcpy(c->d_rrep, reps.data(), nr * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->d_rowmap, rowmap.data(), NN * sizeof(int), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(c->d_rrep, reps.data(), reps.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_rowmap, rowmap.data(), 2 * NN * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload row orbits");
     c->n_rrep = nr;
+    c->n_rcan = ncan;
     c->rtask_qchunk = 0;
     c->loop_evals_rows = 2LL * nr * c->pb.M;
     c->rows_ok = true;
+    c->rows_exact = std::count(own.begin(), own.end(), 1) == 0;
     return QPFRG_OK;
+}
+
+// Representatives (rep, gof as check_covariance_kernel reads them) of every row
+// (f, Q, a) under C4v and, where exch[f], the exchange: the image with the
+// smallest (a, Q), whose patch lies in the fundamental domain 0..N/8.
+static void row_representatives(int N, int ns, const bool (&exch)[2], std::vector<int> &rep, std::vector<uint8_t> &gof)
+{
+    const long NN = (long)N * N, rows = NN * N;
+    std::vector<int> ap(8 * (size_t)N);              // g on a patch
+    for (int g = 0; g < 8; ++g)
+        for (int j = 0; j < N; ++j) ap[(size_t)g * N + j] = c4v_apply(g, j, N, ns);
+    // per patch the elements that take it to its smallest image
+    std::vector<int> amin(N), ng(N), gl(8 * (size_t)N);
+    for (int a = 0; a < N; ++a) {
+        int m = a;
+        for (int g = 0; g < 8; ++g) m = std::min(m, ap[(size_t)g * N + a]);
+        amin[a] = m;
+        for (int g = 0; g < 8; ++g)
+            if (ap[(size_t)g * N + a] == m) gl[8 * (size_t)a + ng[a]++] = g;
+    }
+    for (int f = 0; f < 2; ++f)
+        for (int x = 0; x < N; ++x)
+            for (int y = 0; y < N; ++y) {
+                int ex = x, ey = y;
+                exchange(f, N, ns, ex, ey);
+                for (int a = 0; a < N; ++a) {
+                    int best = -1, bg = 0;
+                    for (int k = 0; k < ng[a]; ++k) {
+                        const int g = gl[8 * (size_t)a + k];
+                        const int *A = &ap[(size_t)g * N];
+                        int Q = A[x] * N + A[y];
+                        if (exch[f]) Q = std::min(Q, A[ex] * N + A[ey]);
+                        if (best < 0 || Q < best) {
+                            best = Q;
+                            bg = g;
+                        }
+                    }
+                    const long row = ((long)x * N + y) * N + a;
+                    rep[f * rows + row] = (int)((long)best * N + amin[a]);
+                    gof[f * rows + row] = (uint8_t)c4v_inverse(bg);    // (Q, a) = g^-1 applied to the representative
+                }
+            }
+}
+
+// flag[f][row] = 1 where a partner-map row is not its representative's image
+static qpfrg_status check_rows(qpfrg_ctx *c, const std::vector<int> &rep, const std::vector<uint8_t> &gof,
+                               std::vector<uint8_t> &flag)
+{
+    const size_t n = rep.size();
+    const long NN = (long)c->pb.N * c->pb.N;
+    int *d_rep = nullptr;
+    uint8_t *d_g = nullptr, *d_flag = nullptr;
+    cudaError_t e;
+    if ((e = cudaMalloc((void **)&d_rep, n * sizeof(int))) == cudaSuccess &&
+        (e = cudaMalloc((void **)&d_g, n)) == cudaSuccess && (e = cudaMalloc((void **)&d_flag, n)) == cudaSuccess) {
+        e = cudaMemcpyAsync(d_rep, rep.data(), n * sizeof(int), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_g, gof.data(), n, cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_flag, 0, n, c->stream);
+        if (e == cudaSuccess) {
+            check_covariance_kernel<<<dim3((unsigned)NN, 2), 256, 0, c->stream>>>(
+                c->d_part, d_rep, d_g, d_flag, c->pb.N, c->pb.M, c->pb.P, c->pb.n_theta, c->pb.n_r, c->pb.n_shell);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(flag.data(), d_flag, n, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    }
+    cudaFree(d_rep);
+    cudaFree(d_g);
+    cudaFree(d_flag);
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "partner-map covariance check");
 }
 
 qpfrg_status build_loop_orbits(qpfrg_ctx *c)
@@ -120,61 +236,37 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
     const int N = c->pb.N, ns = c->pb.n_shell;
     if ((N / ns) % 4 != 0) return QPFRG_OK;
     const long NN = (long)N * N, rows = NN * N;
-    // canonical representative of every (Q, a): the image with the smallest
-    // (a, Q); its patch lies in the fundamental domain 0..N/8
-    std::vector<int> rep(rows);
-    std::vector<uint8_t> gof(rows);
-    for (int x = 0; x < N; ++x)
-        for (int y = 0; y < N; ++y)
-            for (int a = 0; a < N; ++a) {
-                long best = -1;
-                int bg = 0;
-                for (int g = 0; g < 8; ++g) {
-                    const long ga = c4v_apply(g, a, N, ns);
-                    const long gQ = (long)c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns);
-                    const long key = ga * NN + gQ;
-                    if (best < 0 || key < best) {
-                        best = key;
-                        bg = g;
-                    }
-                }
-                const long ra = best / NN, rQ = best - ra * NN;
-                const long row = ((long)x * N + y) * N + a;
-                rep[row] = (int)(rQ * N + ra);
-                gof[row] = (uint8_t)c4v_inverse(bg);    // (Q, a) = g^-1 applied to the representative
-            }
-    int *d_rep = nullptr;
-    uint8_t *d_g = nullptr, *d_flag = nullptr;
-    auto release = [&]() {
-        cudaFree(d_rep);
-        cudaFree(d_g);
-        cudaFree(d_flag);
-    };
-    cudaError_t e;
-    if ((e = cudaMalloc((void **)&d_rep, rows * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc((void **)&d_g, rows)) != cudaSuccess || (e = cudaMalloc((void **)&d_flag, 2 * rows)) != cudaSuccess) {
-        release();
-        return cuda_fail(c, e, "cudaMalloc(loop orbits)");
+    std::vector<int> rep(2 * rows);
+    std::vector<uint8_t> gof(2 * rows), flag(2 * rows);
+    // Where rows differ, C4v alone may leave fewer of them (opposite Fermi momenta
+    // are opposite to rounding only): the grouping with fewer rows to evaluate
+    bool exch[2] = {true, true};
+    cudaError_t e = cudaSuccess;
+    auto differ = [&](const std::vector<uint8_t> &v) { return (long)std::count(v.begin(), v.end(), 1); };
+    row_representatives(N, ns, exch, rep, gof);
+    qpfrg_status st = check_rows(c, rep, gof, flag);
+    const long d16 = st == QPFRG_OK ? differ(flag) : 0;
+    if (d16 > 0) {
+        std::vector<int> rep8(2 * rows);
+        std::vector<uint8_t> gof8(2 * rows), flag8(2 * rows);
+        const bool none[2] = {false, false};
+        row_representatives(N, ns, none, rep8, gof8);
+        st = check_rows(c, rep8, gof8, flag8);
+        const long d8 = differ(flag8);
+        if (st == QPFRG_OK && (d8 == 0 || d8 + rows / 4 < d16 + rows / 8)) {
+            exch[0] = exch[1] = false;
+            rep.swap(rep8);
+            gof.swap(gof8);
+            flag.swap(flag8);
+        }
     }
-    std::vector<uint8_t> flag(2 * rows);
-    e = cudaMemcpyAsync(d_rep, rep.data(), rows * sizeof(int), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_g, gof.data(), rows, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_flag, 0, 2 * rows, c->stream);
-    if (e == cudaSuccess) {
-        check_covariance_kernel<<<dim3((unsigned)NN, 2), 256, 0, c->stream>>>(c->d_part, d_rep, d_g, d_flag, N, c->pb.M,
-                                                                          c->pb.P, c->pb.n_theta, c->pb.n_r, ns);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(flag.data(), d_flag, 2 * rows, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    release();
-    if (e != cudaSuccess) return cuda_fail(c, e, "partner-map covariance check");
+    if (st != QPFRG_OK) return st;
 
     // representatives per family grouped by patch, each with its images;
     // rows whose partner bytes broke covariance are representatives of themselves
     struct Rep {
         int a, Q, n;
-        int2 img[8];
+        int2 img[kLoopImages];
     };
     std::vector<Rep> reps[2];
     long mism = 0;
@@ -189,16 +281,18 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
                 reps[f].push_back(r);
                 continue;
             }
-            if (rep[row] != row) continue;
+            if (rep[f * rows + row] != row) continue;
             Rep r{a, Q, 0, {}};
-            const int x = Q / N, y = Q - x * N;
-            for (int g = 0; g < 8; ++g) {
-                const int Qi = c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns), ai = c4v_apply(g, a, N, ns);
-                const long irow = (long)Qi * N + ai;
-                if (fl[irow]) continue;                // evaluated by itself
-                bool dup = false;
-                for (int k = 0; k < r.n; ++k) dup |= r.img[k].x == Qi && (r.img[k].y & 0xffff) == ai;
-                if (!dup) r.img[r.n++] = make_int2(Qi, ai | (g << 16));
+            for (int s = 0; s < (exch[f] ? 2 : 1); ++s) {
+                int x = Q / N, y = Q - x * N;
+                if (s) exchange(f, N, ns, x, y);
+                for (int g = 0; g < 8; ++g) {
+                    const int Qi = c4v_apply(g, x, N, ns) * N + c4v_apply(g, y, N, ns), ai = c4v_apply(g, a, N, ns);
+                    if (fl[(long)Qi * N + ai]) continue;   // evaluated by itself
+                    bool dup = false;
+                    for (int k = 0; k < r.n; ++k) dup |= r.img[k].x == Qi && (r.img[k].y & 0xffff) == ai;
+                    if (!dup) r.img[r.n++] = make_int2(Qi, ai | (g << 16));
+                }
             }
             reps[f].push_back(r);
         }
@@ -206,7 +300,7 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
     }
     const long nrep = (long)reps[0].size() + (long)reps[1].size();
     std::vector<int> hQ(nrep), hn(nrep);
-    std::vector<int2> himg(8 * nrep, make_int2(0, 0));
+    std::vector<int2> himg(kLoopImages * nrep, make_int2(0, 0));
     c->lgroups.clear();
     long k = 0, evals = 0;
     for (int f = 0; f < 2; ++f) {
@@ -215,7 +309,7 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
             const Rep &r = reps[f][i];
             hQ[k] = r.Q;
             hn[k] = r.n;
-            for (int m = 0; m < r.n; ++m) himg[8 * k + m] = r.img[m];
+            for (int m = 0; m < r.n; ++m) himg[kLoopImages * k + m] = r.img[m];
             evals += c->pb.P;
             const bool last = i + 1 == reps[f].size() || reps[f][i + 1].a != r.a;
             if (last) {
@@ -226,21 +320,27 @@ qpfrg_status build_loop_orbits(qpfrg_ctx *c)
     }
     if ((e = cudaMalloc((void **)&c->d_lrepQ, nrep * sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_lnimg, nrep * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc((void **)&c->d_limg, 8 * nrep * sizeof(int2))) != cudaSuccess ||
+        (e = cudaMalloc((void **)&c->d_limg, kLoopImages * nrep * sizeof(int2))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_ltask, (nrep + 2 * (long)N + 8) * sizeof(int4))) != cudaSuccess)
         return cuda_fail(c, e, "cudaMalloc(loop representatives)");
     e = cudaMemcpy(c->d_lrepQ, hQ.data(), nrep * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_lnimg, hn.data(), nrep * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->d_limg, himg.data(), 8 * nrep * sizeof(int2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(c->d_limg, himg.data(), kLoopImages * nrep * sizeof(int2), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload loop representatives");
     c->n_lrep = nrep;
     c->ltask_qchunk = 0;
     c->loop_evals_red = evals;
     c->loop_mismatch_rows = mism;
     c->loop_red = true;
-    if (mism == 0 && c->opt.no_loop_symmetry == 0)
-        return build_row_orbits(c);
-    return QPFRG_OK;
+    if (c->opt.no_loop_symmetry != 0) return QPFRG_OK;
+    std::vector<uint8_t> own(NN, 0);
+    for (int f = 0; f < 2; ++f)
+        for (long row = 0; row < rows; ++row)
+            if (flag[f * rows + row]) own[row / N] = 1;
+    // row orbits while the pairs of their own leave at least half of the saving
+    if (std::count(own.begin(), own.end(), 1) > NN / 2) return QPFRG_OK;
+    return build_row_orbits(c, exch[0], own);
 }
 
 // Tasks of the reduced loop-kernel launch for a chunk size: (family, patch,
@@ -282,7 +382,7 @@ qpfrg_status row_tasks(qpfrg_ctx *c, int qchunk, int *ntask)
     std::vector<int4> t;
     for (int f = 0; f < 2; ++f)
         for (int a = 0; a < c->pb.N; ++a)
-            for (int s0 = 0; s0 < c->n_rrep; s0 += qchunk) t.push_back(make_int4(f, a, s0, std::min(qchunk, c->n_rrep - s0)));
+            for (int s0 = 0; s0 < c->n_rcan; s0 += qchunk) t.push_back(make_int4(f, a, s0, std::min(qchunk, c->n_rcan - s0)));
     cudaError_t e = cudaMemcpyAsync(c->d_rtask, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload row tasks");

@@ -77,18 +77,22 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float x0, float x1)
 }  // namespace
 
 struct TcFusedArgs {
-    int M, Ncol, Npad, N;             // valid rows, valid columns, padded columns, patches
-    int nkb_total, kb_per_split;      // 64-wide k blocks of the padded reduction; per CTA along grid.y
+    int Ncol, Npad, N;                // valid columns, padded columns, patches
+    int nkb_total;                    // 64-wide k blocks of the padded reduction
     int nkb_half;                     // k blocks per half of the d reduction (Kp / 64)
     long RT, KB;                      // row tiles and k blocks per family of the tiled table
     int ch;                           // 0 pp, 1 cr, 2 d
-    // row orbits: A row m is the transfer pair rows[m] (table row m of the
-    // compact table), output row m of out[m][n]; nullptr: row m is Q = m,
-    // written to the channel's place in the N^3 output
+    // form 0, every row: row m is Q = m, written to the channel's place in the N^3
+    // output; form 1, row orbits: A row m is the transfer pair rows[m], output row m
+    // of outc[m][n].  Row tiles 0 .. t1 - 1 hold rows 0 .. m1 - 1, tile t1 + i the
+    // rows m1 + 128 i .. M - 1, which read the table tile i again (the exchanged pairs
+    // of the row orbits; without them t1 = all tiles, m1 = M); kb_per k blocks per CTA
+    int M, m1, t1, kb_per;
     const int *rows;
+    int form;
     const float *Vf, *VT;             // stage vertex [k1][k2][k3]; factor tables of cr and d (tc_prep)
     int fw;                           // row stride of the staged factor rows (odd), 0: not staged
-    double *out;
+    double *out, *outc;
     double scale;
     unsigned *err;
     TcBatch batch;
@@ -135,8 +139,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     __shared__ int abort_flag;
 
     // the flow of this CTA (batched launch) or the context's single flow
+    const bool compact = A.form != 0;
+    const int *rows = compact ? A.rows : nullptr;
+    const int bx = blockIdx.x, by = blockIdx.y;
     const float *Vf = A.Vf, *VT = A.VT;
-    double *out = A.out;
+    double *out = compact ? A.outc : A.out;
     double scale = A.scale;
     const CUtensorMap *mtab = &mTab, *mhi = &mBhi, *mlo = &mBlo;
     if (A.batch.nflows) {
@@ -148,15 +155,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
         mtab = Bt.tab_maps + Bt.slot_tab[sf];
         Vf = Bt.Vf[f];
         VT = Bt.VT[f];
-        out = Bt.outc ? Bt.outc[f] + (long)A.ch * A.M * A.N : Bt.out[f];
+        out = compact ? Bt.outc[f] + (long)A.ch * A.M * A.N : Bt.out[f];
         scale *= exp(Bt.x[f] + Bt.cst * h);      // dV/d ln T = T dV/dT at the stage temperature
         mhi = Bt.maps + 6L * f + 2 * A.ch;
         mlo = mhi + 1;
     }
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int m0 = blockIdx.x * BM;
-    const int kb0 = blockIdx.y * A.kb_per_split;
-    const int kb1 = min(A.nkb_total, kb0 + A.kb_per_split);
+    const bool sec = bx >= A.t1;
+    const int tile = sec ? bx - A.t1 : bx;                      // table tile
+    const int m0 = (sec ? A.m1 : 0) + tile * BM, mend = sec ? A.M : A.m1;
+    const int kb0 = by * A.kb_per;
+    const int kb1 = min(A.nkb_total, kb0 + A.kb_per);
     const int nkb = kb1 - kb0;
     const int Npad = A.Npad, N = A.N;
     const int NN = N * N;
@@ -196,8 +205,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
         // lanes l and l + 16 the two halves (columns 0-31, 32-63) of row 16 w + l ----
         const int lane = tid & 31;
         const int rr = (warp << 4) | (lane & 15), hh = lane >> 4;
-        const bool valid = m0 + rr < A.M;
-        const int Q = !valid ? 0 : (A.rows ? A.rows[m0 + rr] : m0 + rr);   // transfer pair of the row
+        const bool valid = m0 + rr < mend;
+        const int Q = !valid ? 0 : (rows ? rows[m0 + rr] : m0 + rr);   // transfer pair of the row
         // raw row rr of the half h (columns 32 h .. 32 h + 31), 16-byte chunk c:
         // h 16 KB + rr 128 + (c ^ (rr % 8)) 16 (128-byte swizzle); A_hi row rr,
         // 8-wide k chunk kc: rr 128 + (kc ^ (rr % 8)) 16, A_lo the same + 16 KB
@@ -334,7 +343,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
     } else if (tid == kCopyWarp * 32 && nkb > 0) {
         // ---- table and B copies: stage s is refilled as soon as the products
         // of its previous block are done ----
-        const long tile0 = ((long)fam * A.RT + blockIdx.x) * A.KB;   // first k block of this row tile
+        const long tile0 = ((long)fam * A.RT + tile) * A.KB;   // first k block of this row tile
         int issued = 0;
         for (; issued < nkb; ++issued) {
             const int s = issued % S;
@@ -421,13 +430,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
         for (int c0 = 16 * (warp >> 2); c0 < Npad; c0 += 32) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)c0, v);
-            if (Q < A.M) {
+            if (Q < mend) {
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
                     const int n = c0 + q;
                     if (n >= A.Ncol) continue;
                     long o;
-                    if (A.ch == 0 || A.rows) o = (long)Q * N + n;                // (i, j, n); compact rows [m][n]
+                    if (A.ch == 0 || rows) o = (long)Q * N + n;                // (i, j, n); compact rows [m][n]
                     else if (A.ch == 1) o = (long)n * NN + (long)qb * N + qa;     // (n, j, l)
                     else o = ((long)qa * N + n) * N + qb;                         // (i, n, l)
                     atomicAdd(&out[o], scale * (double)v[q]);
@@ -452,16 +461,17 @@ static qpfrg_status launch_fused(qpfrg_ctx *c, int ch, TcFusedArgs &A, int nz, i
         c->err = "tensor-core contraction: unsupported shape";
         return QPFRG_ERR_UNSUPPORTED;
     }
-    const int M = A.rows ? c->n_rrep : (int)NN;
-    const int mtiles = div_up(M, tc::BM);
     const int nkb = (int)(Kp / tc::BK);
     const int nkb_half = (int)(t.Kp / tc::BK);
+    A.M = A.form ? c->n_rrep : (int)NN;
+    A.m1 = A.form ? c->n_rcan : A.M;
+    A.t1 = div_up(A.m1, tc::BM);
+    const int mtiles = A.t1 + div_up(A.M - A.m1, tc::BM);
     // split K so that the grid fills whole waves of the 152 SMs (one CTA per SM)
     int splits = 1;
     double best = -1.0;
     for (int sp = 1; sp <= std::max(1, nkb / 4) && sp <= 16; ++sp) {
-        const int ctas = mtiles * sp * nz;
-        const double waves = (double)ctas / 152.0, fill = waves / std::ceil(waves);
+        const double waves = (double)(mtiles * sp * nz) / 152.0, fill = waves / std::ceil(waves);
         const double score = fill - 0.02 * std::ceil(waves);
         if (score > best + 1e-9) {
             best = score;
@@ -469,14 +479,14 @@ static qpfrg_status launch_fused(qpfrg_ctx *c, int ch, TcFusedArgs &A, int nz, i
         }
     }
     if (c->tune.tc_splits[ch] > 0) splits = std::min(c->tune.tc_splits[ch], nkb);
-    const int kb_per = div_up(nkb, splits);
-    splits = div_up(nkb, kb_per);
+    A.kb_per = div_up(nkb, splits);
+    splits = div_up(nkb, A.kb_per);
     // the factor rows the widest split touches, staged in shared memory when
     // they fit beside at least two stages (row stride odd)
     int wmax = 1;
     for (int y = 0; y < splits; ++y) {
         int lo[2], n[2];
-        factor_segments(ch, N, y * kb_per, std::min(nkb, (y + 1) * kb_per), nkb_half, lo, n);
+        factor_segments(ch, N, y * A.kb_per, std::min(nkb, (y + 1) * A.kb_per), nkb_half, lo, n);
         wmax = std::max(wmax, n[0] + n[1]);
     }
     const int fw = wmax | 1;
@@ -506,13 +516,11 @@ static qpfrg_status launch_fused(qpfrg_ctx *c, int ch, TcFusedArgs &A, int nz, i
     const KernT kern = table[S - 2][(N & 7) == 0 ? 1 : 0][stg ? 1 : 0];
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(c, e, "tc_fused smem attribute");
-    A.M = M;
     A.Ncol = N;
     A.Npad = Npad;
     A.N = N;
     A.nkb_total = nkb;
-    A.kb_per_split = kb_per;
-    A.nkb_half = (int)(t.Kp / tc::BK);
+    A.nkb_half = nkb_half;
     A.RT = t.RT;
     A.KB = t.KB;
     A.ch = ch;
@@ -526,16 +534,19 @@ static qpfrg_status launch_fused(qpfrg_ctx *c, int ch, TcFusedArgs &A, int nz, i
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "tc_fused_kernel");
 }
 
-// Host launcher of channel ch (0 pp, 1 cr, 2 d): out += scale * A B^T with A
-// formed from the weighted loop-kernel table of the context.
-qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, int kid)
+// Host launcher of channel ch (0 pp, 1 cr, 2 d): out (every row) or outc (row
+// orbits) += scale * A B^T with A formed from the weighted loop-kernel table of the
+// context, in the form of the context's right-hand side.
+qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, double *outc, int kid)
 {
     TcFusedArgs A{};
     A.Vf = c->d_Vf;
     A.VT = c->tc.VT;
     A.out = out;
+    A.outc = outc;
     A.scale = scale;
-    A.rows = c->rows_compact ? c->d_rrep : nullptr;
+    A.form = c->rhs_sym.mode;
+    A.rows = A.form ? c->d_rrep + (ch == 0 ? 0 : c->n_rrep) : nullptr;
     return launch_fused(c, ch, A, 1, kid);
 }
 
@@ -546,7 +557,8 @@ qpfrg_status launch_tc_fused_batch(qpfrg_ctx *c, int ch, const TcBatch &bt, doub
     TcFusedArgs A{};
     A.scale = sign;
     A.batch = bt;
-    A.rows = bt.outc ? c->d_rrep : nullptr;
+    A.form = bt.outc ? 1 : 0;
+    A.rows = bt.outc ? c->d_rrep + (ch == 0 ? 0 : c->n_rrep) : nullptr;
     return launch_fused(c, ch, A, bt.nflows, K_TC_PP + ch);
 }
 

@@ -33,11 +33,71 @@ struct TcPrepArgs {
 // Job blockIdx.y: 0, 1, 2 the pp, cr, d operands, one thread per row n and
 // 8 consecutive k (one 16-byte chunk of hi and of lo in the tile layout;
 // neighbouring threads take neighbouring rows, so the pp reads are coalesced);
-// 3, 4, 5 the three factor tables, one element per thread.  32-bit indices:
+// 3, 4, 5 the three factor tables, one element per thread (N a multiple of 8: job
+// 2 is the d operand and the factor tables, tc_prep_turn).  32-bit indices:
 // N <= 256 keeps N^3 and Npad K_pd below 2^31.
+__device__ __forceinline__ uint32_t bf16_pair(float x0, float x1, uint32_t &lo)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __low2float(h), x1 - __high2float(h));
+    lo = *reinterpret_cast<const uint32_t *>(&l);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// The operands whose source runs along another index than their rows, for N a
+// multiple of 8: the d operand and the three factor tables are transposes, at a
+// fixed third index f, of S1[x][y] = V[x,f,y] and S2[x][y] = V[f,x,y]:
+//   Bd row f: k = y N + x from S1, Kp + y N + x from S2;
+//   VT0[y,f][x] = S1,  VT1[f,y][x] = 2 S2 - S1,  VT2[f,y][x] = -S2.
+// A block turns 32 x 32 tiles of both through shared memory, so that reads and
+// factor writes are 128 contiguous bytes (reading them element by element moved
+// 32 bytes for 4: np96 34 -> 17 us, 224 patches 370 -> 153 us a stage).
+__device__ __forceinline__ void tc_prep_turn(const TcPrepArgs &t)
+{
+    __shared__ float s1[32][33], s2[32][33];
+    const int N = t.N, NN = N * N, Kp = (int)t.Kp, nt = (N + 31) / 32, tid = threadIdx.x;
+    const float *V = t.V;
+    float *VT0 = t.VT, *VT1 = VT0 + (long)NN * N, *VT2 = VT1 + (long)NN * N;
+    for (int it = blockIdx.x; it < N * nt * nt; it += gridDim.x) {
+        const int f = it / (nt * nt), r = it - f * nt * nt, x0 = (r / nt) * 32, y0 = (r % nt) * 32;
+        __syncthreads();
+        for (int e = tid; e < 1024; e += 256) {
+            const int x = x0 + (e >> 5), y = y0 + (e & 31);
+            const bool ok = x < N && y < N;
+            s1[e >> 5][e & 31] = ok ? V[(x * N + f) * N + y] : 0.f;
+            s2[e >> 5][e & 31] = ok ? V[(f * N + x) * N + y] : 0.f;
+        }
+        __syncthreads();
+        for (int e = tid; e < 1024; e += 256) {
+            const int x = x0 + (e & 31), y = y0 + (e >> 5);
+            if (x >= N || y >= N) continue;
+            const float a = s1[e & 31][e >> 5], b = s2[e & 31][e >> 5];
+            VT0[(y * N + f) * N + x] = a;
+            VT1[(f * N + y) * N + x] = 2.f * b - a;
+            VT2[(f * N + y) * N + x] = -b;
+        }
+        // one 8-wide chunk of one half per thread (N a multiple of 8: a chunk lies in one y)
+        const int half = tid >> 7, yy = (tid >> 2) & 31, xx = (tid & 3) * 8;
+        if (x0 + xx < N && y0 + yy < N) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = half ? s2[xx + u][yy] : s1[xx + u][yy];
+            uint4 hi, lo;
+            hi.x = bf16_pair(v[0], v[1], lo.x);
+            hi.y = bf16_pair(v[2], v[3], lo.y);
+            hi.z = bf16_pair(v[4], v[5], lo.z);
+            hi.w = bf16_pair(v[6], v[7], lo.w);
+            const long o = tile_index(f, (long)half * Kp + (y0 + yy) * N + x0 + xx, t.Npad, 2L * Kp);
+            *reinterpret_cast<uint4 *>(t.Bd[0] + o) = hi;
+            *reinterpret_cast<uint4 *>(t.Bd[1] + o) = lo;
+        }
+    }
+}
+
 __device__ __forceinline__ void tc_prep_body(const TcPrepArgs &t)
 {
     const int N = t.N, Npad = t.Npad, job = blockIdx.y;
+    if (job == 2 && N % 8 == 0) return tc_prep_turn(t);
     const int NN = N * N, Kp = (int)t.Kp;
     const float *V = t.V;
     const int stride = gridDim.x * blockDim.x;
@@ -72,10 +132,7 @@ __device__ __forceinline__ void tc_prep_body(const TcPrepArgs &t)
                         ++a;
                     }
                 }
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[0], x[1]);
-                const __nv_bfloat162 l2 = __floats2bfloat162_rn(x[0] - __low2float(h2), x[1] - __high2float(h2));
-                hp[e / 2] = *reinterpret_cast<const uint32_t *>(&h2);
-                lp[e / 2] = *reinterpret_cast<const uint32_t *>(&l2);
+                hp[e / 2] = bf16_pair(x[0], x[1], lp[e / 2]);
             }
             // k0 % 8 == 0: the chunk's 8 elements are contiguous in the tile (16-byte aligned)
             const long o = tile_index(n, k0, Npad, K);
@@ -129,7 +186,7 @@ qpfrg_status launch_tc_prep_batch(qpfrg_ctx *c, const TcPrepFlow *d_flows, const
     t.Kp = c->tc.Kp;
     t.Kpd = c->tc.Kpd;
     prof_begin(c);
-    tc_prep_batch_kernel<<<dim3(blocks, 6, nflows), 256, 0, c->stream>>>(t, d_flows, d_status, d_h_tab, step, nflows);
+    tc_prep_batch_kernel<<<dim3(blocks, N % 8 == 0 ? 3 : 6, nflows), 256, 0, c->stream>>>(t, d_flows, d_status, d_h_tab, step, nflows);
     prof_end(c, K_TC_PREP);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "tc_prep_batch_kernel");
@@ -154,7 +211,7 @@ qpfrg_status launch_tc_prep(qpfrg_ctx *c)
     }
     t.VT = c->tc.VT;
     prof_begin(c);
-    tc_prep_kernel<<<dim3(blocks, 6), 256, 0, c->stream>>>(t);
+    tc_prep_kernel<<<dim3(blocks, N % 8 == 0 ? 3 : 6), 256, 0, c->stream>>>(t);
     prof_end(c, K_TC_PREP);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "tc_prep_kernel");

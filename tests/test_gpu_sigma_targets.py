@@ -22,10 +22,10 @@ GEO = [  # N, nt, nr, tp, propagator, eta
     (8, 4, 4, -0.2, 0, 0.02), (8, 4, 4, 0.0, 0, 0.0145), (8, 4, 4, 0.0, 0, 0.01)]
 
 
-def run(N, nt, nr, tp, prop, eta, V, Z, T, w, lam=None):
+def run(N, nt, nr, tp, prop, eta, V, Z, T, w, prec=api.QPFRG_MIXED):
     import torch
     new = lambda *n: torch.full(n, float("nan"), dtype=torch.float64, device="cuda")  # noqa: E731
-    with api.Context(N, nt, nr, U=2.0, tp=tp, precision=api.QPFRG_MIXED, propagator=prop, eta=eta, n_omega=len(w),
+    with api.Context(N, nt, nr, U=2.0, tp=tp, precision=prec, propagator=prop, eta=eta, n_omega=len(w),
                      omega_min=w[0], omega_max=w[-1]) as c:
         zo, re, im = new(N), new(N, len(w)), new(N, len(w))
         api.qpfrg_selfenergy(c.h, T, torch.from_numpy(V.ravel().copy()).cuda(), torch.from_numpy(Z.copy()).cuda(), re, im, zo)
@@ -89,3 +89,4 @@ def test_interaction_flow_lines(N, nt, nr, skew):
     sl, sg = slice(n3 + N, n3 + 3 * N), slice(n3 + 3 * N, None)
     assert np.abs(a[sl] - b[sl]).max() < 1e-5 * np.abs(b[sl]).max()
     assert np.abs(a[sg] - b[sg]).max() < TOL_W * np.abs(b[sg]).max()
+
