@@ -510,6 +510,8 @@ struct SigmaFastArgs {
     FineTable<float> fine;
     const double *V, *Z, *kx64, *ky64, *kf;
     const float *xij_f, *qxl, *qyl;
+    const double *xi64, *w64, *xij64;   // dispersion and weight of the fine points, xi(k_F(j))
+    double T64;
     double fold0, fold1;    // last doubles k with rint(k / 2 pi) = 0 and < 2
     const float4 *kp, *kcs, *bnd;
     const int2 *kfx, *pfx;  // k_j + p and the fine points in fixed point
@@ -652,8 +654,8 @@ __host__ __device__ inline SfSmem sf_smem_layout(int pch, bool rt)
 // count rint(k / 2 pi) changes where k passes fold0 (pi) and fold1 (3 pi), the
 // last doubles of the lower count, so two FP64 additions and comparisons per
 // component give the folded momentum of project_fp64, and the wedge follows from
-// FP32 and float-float ray tests; only within 1e-11 of a ray, or of the origin,
-// does the FP64 projection run (its atan2 and divisions, 170 instructions at 64
+// FP32 and float-float ray tests; only within 1e-11 of a ray (where the FP64
+// rounding decides), or of the origin, does the FP64 projection run (its atan2 and divisions, 170 instructions at 64
 // clocks each per warp, made the CTAs of coinciding p and q the tail of the launch:
 // np48, Z of a symmetric vertex 4.5 -> 3.9 ms).  flags: 1 near the zone edge, 2
 // record a pair within 1e-9 of a ray or of the zone edge in A.events (correcting
@@ -676,8 +678,10 @@ __device__ __noinline__ int sf_slow_patch(const SigmaFastArgs &A, int j, int p, 
             const float4 k4 = A.kp[(long)j * A.pb.M + p];
             const int r = project_ff(k4.x, k4.y, k4.z, k4.w, A.fine.kx[q], A.qxl[q], A.fine.ky[q], A.qyl[q], jc, N, bnd,
                                      margin);
-            if (margin < 1e-9f) record(r);
-            return r;
+            if (margin >= 1e-11f) {
+                if (margin < 1e-9f) record(r);
+                return r;
+            }
         }
     }
     const double kx = (A.kf[2 * j] + A.kx64[p]) - A.kx64[q], ky = (A.kf[2 * j + 1] + A.ky64[p]) - A.ky64[q];
@@ -708,18 +712,18 @@ __device__ __noinline__ double sf_pair_term(const SigmaFastArgs &A, int j, int p
     const int N = A.pb.N, PP = A.pb.P, a = p / PP, b = q / PP;
     auto z = [&](int k) { return A.Z ? A.Z[k] : 1.0; };
     const bool qp = A.pb.propagator == QPFRG_PROP_QP;
-    const double Za = z(a), Zb = z(b), Zc = z(c), invT = A.invT;
+    const double Za = z(a), Zb = z(b), Zc = z(c), invT = 1.0 / A.T64, eta2 = A.pb.eta * A.pb.eta;
     const double cx = cos(A.kf[2 * j] + A.kx64[p] - A.kx64[q]), cy = cos(A.kf[2 * j + 1] + A.ky64[p] - A.ky64[q]);
-    const double xp = (qp ? Za : 1.0) * A.fine.xi[p], xq = (qp ? Zb : 1.0) * A.fine.xi[q];
+    const double xp = (qp ? Za : 1.0) * A.xi64[p], xq = (qp ? Zb : 1.0) * A.xi64[q];
     const double xr = (qp ? Zc : 1.0) * (-2.0 * A.pb.t * (cx + cy) - 4.0 * A.pb.tp * cx * cy - A.pb.mu);
     auto f = [&](double x) { return 1.0 / (1.0 + exp(x * invT)); };
     const double F = f(xp) * f(-xq) * f(-xr) + f(-xp) * f(xq) * f(xr);
     const double *V = A.V + ((long)j * N + a) * N;
-    double amp = (double)A.fine.w[p] * A.fine.w[q] * Za * Zb * Zc * (2.0 * V[b] * V[b] - V[b] * V[c]) * F;
+    double amp = A.w64[p] * A.w64[q] * Za * Zb * Zc * (2.0 * V[b] * V[b] - V[b] * V[c]) * F;
     if (A.K)
         amp *= (A.K[a] * Za * (Zb + Zc) + A.K[b] * Zb * (Za + Zc) + A.K[c] * Zc * (Za + Zb)) * (1.0 / 6.0);
-    const double d0 = A.xij_f[j] - (xq + xr - xp), dp = d0 + A.twoT, dm = d0 - A.twoT;
-    return amp * ((double)A.eta2 - dp * dm) / ((dp * dp + A.eta2) * (dm * dm + A.eta2));
+    const double d0 = A.xij64[j] - (xq + xr - xp), dp = d0 + 2.0 * A.T64, dm = d0 - 2.0 * A.T64;
+    return amp * (eta2 - dp * dm) / ((dp * dp + eta2) * (dm * dm + eta2));
 }
 
 // A recorded pair (p, q) of target j, patch c, lies on a boundary: every image
@@ -1548,6 +1552,176 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     }
 }
 
+// FP64 self-energy of the wedge grid: the sum of sigma_kernel<double>, with the
+// patches of r decided as in the FP32 kernels (fixed-point table, exact near the
+// boundaries) and, for the chord, the targets that a symmetric (V, Z) needs.
+//
+// What bounds it: FP64 instructions, 64 clocks each per warp and scheduler.
+// sigma_kernel<double> issued about 180 per pair, 100 of them for the projection
+// (atan2 and three divisions); here about 55: the projection runs on the integer
+// and FP32 pipes, and F and the chord term share one division,
+//   F = (A + B e) / (1 + e) for x_r > 0, (A e + B) / (1 + e) otherwise, e = exp(-|x_r|/T),
+//   A = w_p f_p (1 - f_q), B = w_p (1 - f_p) f_q.
+// np16, 8 x 8 points, Z of a symmetric vertex (7 of 16 targets): 4.82 -> 0.83 ms.
+// Launch: grid (ceil(M / 256), N patches a, target slots), 256 threads, one q each.
+// GL: the interaction flow's line weights.  HIST: binned pole weights (every patch).
+struct Sigma64Args {
+    SigmaFastArgs a;
+    FineTable<double> f;
+    double *hist;
+    double e_min, inv_h;
+    int nbins;
+};
+constexpr int S64_REC = 128;    // loop points p staged per pass
+struct S64Rec {
+    double cx, sx, cy, sy, x, wf, wfc;   // cos, sin of k + p, x_p, w_p f_p, w_p (1 - f_p)
+    int kx, ky;                          // k + p in fixed point
+};
+
+template <bool TP0, bool GL, bool HIST>
+__global__ void __launch_bounds__(256) sigma64_kernel(const Sigma64Args S)
+{
+    const SigmaFastArgs &A = S.a;
+    const int N = A.pb.N, M = A.pb.M, PP = A.pb.P;
+    const int a = blockIdx.y, jidx = blockIdx.z, tid = threadIdx.x;
+    int j;
+    bool sym;
+    if (A.only_full && *A.nevents <= A.max_events) return;
+    if (!sigma_target(A, jidx, j, sym)) return;      // uniform over the CTA
+    const bool qp = A.pb.propagator == QPFRG_PROP_QP;
+    const double T = A.T64, invT = 1.0 / T, eta2 = A.pb.eta * A.pb.eta;
+
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    S64Rec *rec = reinterpret_cast<S64Rec *>(smem_raw);
+    double2 *zv = reinterpret_cast<double2 *>(rec + S64_REC);          // Z_c, Z_c V_jac
+    double *kz = reinterpret_cast<double *>(zv + SF_SLOTS);            // K_c Z_c (GL)
+    float2 *ray = reinterpret_cast<float2 *>(kz + (GL ? SF_SLOTS : 0));
+    const unsigned char *tabc = A.ptab + (kProjW / 2) * (kProjStride + 1);   // the cell of the origin
+    const double *Vja = A.V + ((long)j * N + a) * N;
+    for (int i = tid; i < SF_SLOTS; i += 256) {
+        const int c = i < N ? i : 0;
+        const bool ok = i <= N;
+        const double Zc = A.Z ? A.Z[c] : 1.0;
+        zv[i] = ok ? make_double2(Zc, Zc * Vja[c]) : make_double2(0.0, 0.0);
+        if (GL) kz[i] = ok ? A.K[c] * Zc : 0.0;
+        const float4 bd = A.bnd[c];
+        ray[i] = ok ? make_float2(bd.x, bd.z) : make_float2(0.f, 0.f);
+    }
+    const double Za = A.Z ? A.Z[a] : 1.0;
+    double skx, ckx, sky, cky;
+    sincos(A.kf[2 * j], &skx, &ckx);
+    sincos(A.kf[2 * j + 1], &sky, &cky);
+    auto fermi = [&](double x, double &f, double &fc) {
+        const double e = exp(-fabs(x) * invT), hi = 1.0 / (1.0 + e), lo = e * hi;
+        f = x > 0.0 ? lo : hi;
+        fc = x > 0.0 ? hi : lo;
+    };
+
+    const int q = blockIdx.x * 256 + tid;
+    const bool valid = q < M;
+    const int qq = valid ? q : M - 1, b = qq / PP;
+    const int qx = A.pfx[qq].x, qy = A.pfx[qq].y;
+    const double cqx = S.f.cx[qq], sqx = S.f.sx[qq], cqy = S.f.cy[qq], sqy = S.f.sy[qq];
+    const double Zb = A.Z ? A.Z[b] : 1.0;
+    const double xq = (qp ? Zb : 1.0) * S.f.xi[qq];
+    double fq, fcq;
+    fermi(xq, fq, fcq);
+    const double pref = valid ? Za * Zb * S.f.w[qq] : 0.0;
+    fq *= pref;
+    fcq *= pref;
+    const double vab = Vja[b], v2 = 2.0 * vab * vab, dq = A.xij64[j] - xq, twoT = 2.0 * T;
+    double ga = 0.0, gb = 0.0, gc = 0.0;     // GL: bracket = ga + gb Z_c + gc K_c Z_c
+    if (GL) {
+        const double kza = A.K[a] * Za, kzb = A.K[b] * Zb;
+        ga = (kza * Zb + kzb * Za) * (1.0 / 6.0);
+        gb = (kza + kzb) * (1.0 / 6.0);
+        gc = (Za + Zb) * (1.0 / 6.0);
+    }
+    double acc = 0.0;
+    for (int p0 = 0; p0 < PP; p0 += S64_REC) {
+        const int cnt = min(S64_REC, PP - p0);
+        __syncthreads();         // the slots written, the previous pass done
+        for (int i = tid; i < cnt; i += 256) {
+            const int p = a * PP + p0 + i;
+            S64Rec r;
+            const double cpx = S.f.cx[p], spx = S.f.sx[p], cpy = S.f.cy[p], spy = S.f.sy[p];
+            r.cx = ckx * cpx - skx * spx;
+            r.sx = skx * cpx + ckx * spx;
+            r.cy = cky * cpy - sky * spy;
+            r.sy = sky * cpy + cky * spy;
+            r.x = (qp ? Za : 1.0) * S.f.xi[p];
+            double f, fc;
+            fermi(r.x, f, fc);
+            r.wf = S.f.w[p] * f;
+            r.wfc = S.f.w[p] * fc;
+            const int2 k = A.kfx[(long)j * M + p];
+            r.kx = k.x;
+            r.ky = k.y;
+            rec[i] = r;
+        }
+        __syncthreads();
+        for (int i = 0; i < cnt; ++i) {
+            const S64Rec &r = rec[i];
+            float x, y;
+            bool slow;
+            int c = fx_patch(r.kx, r.ky, qx, qy, tabc, ray, x, y, slow);
+            if (__any_sync(0xffffffffu, slow)) {          // taken by the whole warp
+                bool still;
+                const int cc = fx_zoom(r.kx, r.ky, qx, qy, tabc, ray, still);
+                if (slow) c = cc;
+                if (slow && still) {
+                    const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
+                    // (the zone-edge targets have no images)
+                    const bool fix = !HIST && A.sym.mode == 2 && sym && (4 * j) % N != 0 && valid;
+                    c = sf_slow_patch(A, j, a * PP + p0 + i, qq, x * kRadPerFx, y * kRadPerFx,
+                                      (edge ? 1 : 0) | (fix ? 2 : 0), A.bnd);
+                }
+                __syncwarp();
+            }
+            const double crx = r.cx * cqx + r.sx * sqx, cry = r.cy * cqy + r.sy * sqy;
+            double xr = -2.0 * A.pb.t * (crx + cry) - A.pb.mu;
+            if (!TP0) xr -= 4.0 * A.pb.tp * crx * cry;
+            const double2 z = zv[c];
+            if (qp) xr *= z.x;
+            const double e = exp(-fabs(xr) * invT), An = r.wf * fcq, Bn = r.wfc * fq;
+            double w = fma(-vab, z.y, z.x * v2) * (xr > 0.0 ? fma(Bn, e, An) : fma(An, e, Bn));
+            if (GL) w *= fma(gc, kz[c], fma(gb, z.x, ga));
+            if (HIST) {
+                const double E = xq + xr - r.x, amp = w / (1.0 + e);
+                int bin = (int)floor((E - S.e_min) * S.inv_h);
+                bin = bin < 0 ? 0 : (bin >= S.nbins ? S.nbins - 1 : bin);
+                const double d = E - (S.e_min + (bin + 0.5) / S.inv_h);
+                double *h = S.hist + (long)jidx * 5 * S.nbins + bin;
+                double m = amp;
+                if (valid) {
+#pragma unroll
+                    for (int mo = 0; mo < 5; ++mo) {
+                        atomicAdd(h + (long)mo * S.nbins, m);
+                        m *= d;
+                    }
+                }
+            } else {
+                // chord slope of Re 1/(w - E + i eta) over w = xi_j +- 2T:
+                // (eta^2 - d+ d-) / ((d+^2 + eta^2)(d-^2 + eta^2))
+                const double d0 = dq - xr + r.x, dp = d0 + twoT, dm = d0 - twoT;
+                acc += w * fma(-dp, dm, eta2) / ((1.0 + e) * (fma(dp, dp, eta2) * fma(dm, dm, eta2)));
+            }
+        }
+    }
+    if constexpr (!HIST) {
+        __shared__ double red[8];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+        if ((tid & 31) == 0) red[tid >> 5] = acc;
+        __syncthreads();
+        if (tid == 0) {
+            double v = 0.0;
+            for (int i = 0; i < 8; ++i) v += red[i];
+            atomicAdd(&A.sig[jidx], v);
+        }
+    }
+}
+
 // Z_j = 1/(1 - slope) with the chord slope accumulated per target slot, or the
 // slopes themselves (slopes_out).  rep[j] (may be NULL) is the slot of j's C4v
 // representative among the targets; sym.mode == 2: where the C4v test holds, with
@@ -1754,6 +1928,10 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     A.inv_dth = (float)(c->pb.N / kTwoPi);
     A.dth = (float)(kTwoPi / c->pb.N);
     A.w_max = (float)c->fw_max;
+    A.xi64 = c->f64.xi;
+    A.w64 = c->f64.w;
+    A.xij64 = c->d_xij;
+    A.T64 = T;
     static const double fold0 = fold_limit(0), fold1 = fold_limit(1);
     A.fold0 = fold0;
     A.fold1 = fold1;
@@ -1883,6 +2061,47 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_hist_kernel");
 }
 
+// FP64 chord slopes of the target slots into d_sig or, with nbins, the binned
+// pole weights of every patch into hist.
+static qpfrg_status launch_sigma64(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
+                                   const SigmaTargets &tg, double *hist = nullptr, double e_min = 0.0, double h = 1.0,
+                                   int nbins = 0)
+{
+    const int N = c->pb.N, nj = tg.slots(N);
+    qpfrg_status s = launch_kp_table(c, nullptr, N);
+    if (s != QPFRG_OK) return s;
+    Sigma64Args S{};
+    S.a = fast_args(c, T, d_V, d_Z, d_K, tg);
+    S.f = c->f64;
+    S.hist = hist;
+    S.e_min = e_min;
+    S.inv_h = 1.0 / h;
+    S.nbins = nbins;
+    using Kern = void (*)(const Sigma64Args);
+    static const Kern table[2][2][2] = {   // [t' = 0][lines][histogram]
+        {{sigma64_kernel<false, false, false>, sigma64_kernel<false, false, true>},
+         {sigma64_kernel<false, true, false>, sigma64_kernel<false, true, true>}},
+        {{sigma64_kernel<true, false, false>, sigma64_kernel<true, false, true>},
+         {sigma64_kernel<true, true, false>, sigma64_kernel<true, true, true>}}};
+    const Kern kern = table[c->pb.tp == 0.0][d_K ? 1 : 0][nbins > 0 ? 1 : 0];
+    const size_t smem = S64_REC * sizeof(S64Rec) + SF_SLOTS * (sizeof(double2) + (d_K ? sizeof(double) : 0) + sizeof(float2));
+    const dim3 grid(div_up(c->pb.M, 256), N, nj);
+    prof_begin(c);
+    kern<<<grid, 256, smem, c->stream>>>(S);
+    if (tg.sym.mode == 2 && nbins == 0) {
+        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(S.a);
+        Sigma64Args F = S;       // every patch, should the record have run over
+        F.a.only_full = true;
+        F.a.jlist = nullptr;
+        F.a.sym = SymMode();
+        F.a.sig = c->d_sig + 3 * N;
+        kern<<<dim3(grid.x, N, N), 256, smem, c->stream>>>(F);
+    }
+    prof_end(c, nbins > 0 ? K_SIGMA_HIST : K_SIGMA_Z);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma64_kernel");
+}
+
 template <typename R>
 static void fill_args(qpfrg_ctx *c, SigmaArgs<R> &A, const FineTable<R> &fine, double T, const double *d_V,
                       const double *d_Z)
@@ -1957,16 +2176,17 @@ qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const dou
         tg.rep = c->d_rep;
         tg.mirror = c->pb.n_theta % 2 == 0 ? 1 : 0;
     }
-    if (c->opt.precision == QPFRG_FP64) {
+    if (c->d_ptab) {
+        const bool fp64 = c->opt.precision == QPFRG_FP64;
+        if (!tg.jlist) {
+            tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, 0, c->d_sym_v);
+            if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
+        }
+        s = fp64 ? launch_sigma64(c, T, d_V, d_Z, nullptr, tg) : launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
+    } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
         fill_args(c, A, c->f64, T, d_V, d_Z);
         s = launch_sigma(c, false, A, K_SIGMA_Z);
-    } else if (c->d_ptab) {
-        if (!tg.jlist) {
-            tg = device_targets(c, kTolZ, 0, c->d_sym_v);
-            if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
-        }
-        s = launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
     } else {
         SigmaArgs<float> A;
         fill_args(c, A, c->f32, T, d_V, d_Z);
@@ -1990,14 +2210,15 @@ qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const
     SigmaTargets tg;
     tg.n = c->pb.N;
     qpfrg_status s;
-    if (c->opt.precision == QPFRG_FP64) {
+    if (c->d_ptab) {
+        const bool fp64 = c->opt.precision == QPFRG_FP64;
+        tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, 0, c->d_sym);
+        s = fp64 ? launch_sigma64(c, T, d_V, d_Z, d_K, tg) : launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
+    } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
         fill_args(c, A, c->f64, T, d_V, d_Z);
         A.K = d_K;
         s = launch_sigma(c, false, A, K_SIGMA_Z);
-    } else if (c->d_ptab) {
-        tg = device_targets(c, kTolZ, 0, c->d_sym);
-        s = launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
     } else {
         SigmaArgs<float> A;
         fill_args(c, A, c->f32, T, d_V, d_Z);
@@ -2054,6 +2275,8 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
         tg = device_targets(c, kTolGrid, 2, d_K ? c->d_sym : c->d_sym_v);
         if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         s = launch_sigma_hist(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
+    } else if (c->opt.precision == QPFRG_FP64 && c->d_ptab) {
+        s = launch_sigma64(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
     } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
         fill_args(c, A, c->f64, T, d_V, d_Z);

@@ -90,3 +90,33 @@ def test_interaction_flow_lines(N, nt, nr, skew):
     assert np.abs(a[sl] - b[sl]).max() < 1e-5 * np.abs(b[sl]).max()
     assert np.abs(a[sg] - b[sg]).max() < TOL_W * np.abs(b[sg]).max()
 
+
+# FP64: sums of 1e5 .. 1e7 pairs of relative rounding 1e-15: 1e-12 on Z; the grid's
+# moment expansion 8^-5
+@pytest.mark.parametrize("kind", ["sym", "asym", "one_entry"])
+@pytest.mark.parametrize("geo", [g for g in GEO if g[1] % 2 == 0 and g[1] < 20])
+def test_selfenergy_fp64(geo, kind):
+    """The FP64 kernel (passes of 128 records, decisions by table)."""
+    N, nt, nr, tp, prop, eta = geo
+    T, w = 0.2, np.linspace(-3.0, 3.0, 17)
+    V = inputs.random_vertex(N, 2.0, seed=N + nt, c4v=kind != "asym")
+    Z = inputs.z_profile(N, "aniso")
+    if kind == "one_entry":
+        V[N // 2, 1, N - 1] *= 1.5
+    o = Oracle(N, nt, nr, tp=tp, prop_mode=prop, eta=eta)
+    zo, sig = run(N, nt, nr, tp, prop, eta, V, Z, T, w, prec=api.QPFRG_FP64)
+    assert np.abs(zo - o.zfactor(T, V, Z)).max() < 1e-12
+    for j in (0, 1, N // 2, N - 1):
+        ref = o.sigma(T, V, Z, j, w)
+        assert np.abs(sig[j] - ref).max() < TOL_W * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("kind", ["sym", "asym"])
+def test_selfenergy_fp64_several_passes(kind):
+    """144 loop points per patch (two passes of records); the patches on the
+    diagonals, whose pairs lie on no boundary."""
+    N, T, w = 8, 0.2, np.linspace(-3.0, 3.0, 9)
+    V, Z = inputs.random_vertex(N, 2.0, seed=5, c4v=kind == "sym"), inputs.z_profile(N, "aniso")
+    zo, sig = run(N, 12, 12, 0.0, 1, 0.05, V, Z, T, w, prec=api.QPFRG_FP64)
+    ref = Oracle(N, 12, 12, prop_mode=1, eta=0.05).zfactor(T, V, Z)
+    assert np.abs(zo - ref)[1::2].max() < 1e-12
