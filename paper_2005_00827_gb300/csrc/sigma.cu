@@ -9,14 +9,16 @@
 // (definition_Z), with the slope the chord of Re Sigma over xi_j +- 2T
 // ("from outside", Sec. 3.1.1).
 //
-// sigma_kernel<R,false> evaluates Re Sigma exactly at the two chord frequencies.
-// Launch shape: grid (q blocks, patch a of p, target j), 256 threads, one q
-// per thread; the CTA stages patch a's points (k_j + p, cos/sin, Fermi
-// factors) and the vertex row V[j][a][:] in shared memory and loops over
-// them.  In the flow only the C4v-irreducible patches 0..N/8 are evaluated
-// (the vertex and Z keep the lattice symmetry) and Z is copied to their
-// images.  sigma_kernel<R,true> bins W F by pole energy E with moments 0..4 for
-// the frequency grid; sigma_grid_kernel resums the moments on the grid.
+// Wedge grid: sigma_fast_kernel (FP32) and sigma64_kernel evaluate Re Sigma
+// exactly at the two chord frequencies; sigma_hist_kernel (FP32) and
+// sigma64_kernel<HIST> bin W F by pole energy E with moments 0..4 for the
+// frequency grid, which sigma_resum_kernel resums and sigma_spread_kernel copies
+// to the images.  Lattice and shell modes: sigma_kernel<R,HIST>.  Each CTA
+// stages the points of one patch a of p (k_j + p, cos/sin, Fermi factors) and
+// the vertex row V[j][a][:] in shared memory and loops over them with its q.
+// In the mixed flow the C4v-irreducible patches 0..N/8 are evaluated (the vertex
+// and Z keep the lattice symmetry), of a given vertex the targets that a C4v
+// test on the device admits; Z is copied to their images.
 #include <algorithm>
 
 #include "atan_poly.h"
@@ -1562,7 +1564,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
 // and FP32 pipes, and F and the chord term share one division,
 //   F = (A + B e) / (1 + e) for x_r > 0, (A e + B) / (1 + e) otherwise, e = exp(-|x_r|/T),
 //   A = w_p f_p (1 - f_q), B = w_p (1 - f_p) f_q.
-// np16, 8 x 8 points, Z of a symmetric vertex (7 of 16 targets): 4.82 -> 0.83 ms.
+// np16, 8 x 8 points, Z of a symmetric vertex (6 of 16 targets): 4.82 -> 0.83 ms.
 // Launch: grid (ceil(M / 256), N patches a, target slots), 256 threads, one q each.
 // GL: the interaction flow's line weights.  HIST: binned pole weights (every patch).
 struct Sigma64Args {
@@ -1994,7 +1996,9 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(c, e, "sigma_fast smem attribute");
     const int nqb = div_up(c->pb.M, 256 * SF_QPT);
-    A.qb = c->tune.sigma_qblocks > 0 ? c->tune.sigma_qblocks : SF_QB;
+    // equal shares of at most SF_QB blocks (4 + 2 of 6 blocks left the GPU to the
+    // larger half)
+    A.qb = c->tune.sigma_qblocks > 0 ? c->tune.sigma_qblocks : div_up(nqb, div_up(nqb, SF_QB));
     prof_begin(c);
     kern<<<dim3(div_up(nqb, A.qb), c->pb.N, nj), 256, smem, c->stream>>>(A);
     if (tg.sym.mode == 2) {
