@@ -10,7 +10,8 @@
 // flow that clamps at this step -- and every running flow contracts the table
 // of its slot with its own vertex on the tensor cores:
 //   per stage: loop table per active slot | operands of every flow |
-//              3 batched contractions    | batched RK update
+//              3 batched contractions    | batched RK update (on the
+//              representative rows of the row orbits, then the FP32 vertex)
 //   per step:  a finalize kernel: max|V| and finiteness -> status, Lambda_c,
 //              and the slots still in use at the next step.
 // The schedule (per step and flow: h, slot) is fixed on the host from the
@@ -38,22 +39,30 @@ struct FlowArrays {
     double *x, *m_old, *lambda_c, *max_v;
 };
 
-// RK4 bookkeeping of every running flow with a step, grid.y = flow; k (and
-// the representative rows outc of the row orbits, nc values per flow) are
-// cleared after use (the contractions add into them); the final stage also
-// refreshes the FP32 copy for the next step and reduces max|V| and finiteness.
+// Initial state of the flows, grid.y = flow: V = U (nv values) and its FP32 copy (nf).
+__global__ void fill_batch_kernel(const double *U, double *V, long nv, float *Vf, long nf)
+{
+    const int f = blockIdx.y;
+    const double u = U[f];
+    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
+    for (long i = t; i < nv; i += nt) V[f * nv + i] = u;
+    for (long i = t; i < nf; i += nt) Vf[f * nf + i] = (float)u;
+}
+
+// RK4 bookkeeping of every running flow with a step where every row is contracted
+// (with row orbits: launch_rows_rk_batch), grid.y = flow; k is cleared after use
+// (the contractions add into it); the final stage also refreshes the FP32 copy
+// for the next step and reduces max|V| and finiteness.
 __global__ void rk_batch_kernel(int stage, const TcPrepFlow *pf, double *const *V, double *const *k,
-                                double *const *acc, double *const *outc, long nc, const double *h_tab,
-                                const int *status, int step, int nflows, unsigned long long *red, long n)
+                                double *const *acc, const double *h_tab, const int *status, int step, int nflows,
+                                unsigned long long *red, long n)
 {
     const int f = blockIdx.y;
     const double h = h_tab[(long)step * nflows + f];
     if (status[f] != QPFRG_FLOW_RUNNING || h == 0.0) return;
     double *Vf64 = V[f], *kf = k[f], *af = acc[f];
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < nc; i += (long)gridDim.x * blockDim.x)
-        outc[f][i] = 0.0;
     float *Vf = const_cast<float *>(pf[f].Vf);
-    const double c_next = stage == 3 ? h : 0.5 * h;
+    const double c_next = stage == 3 ? h : 0.5 * h, h6 = h / 6.0;
     double m = 0.0;
     bool bad = false;
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
@@ -63,7 +72,7 @@ __global__ void rk_batch_kernel(int stage, const TcPrepFlow *pf, double *const *
             af[i] = stage == 1 ? ki : af[i] + 2.0 * ki;
             Vf[i] = (float)(Vf64[i] + c_next * ki);
         } else {
-            const double v = Vf64[i] + h / 6.0 * (af[i] + ki);
+            const double v = Vf64[i] + h6 * (af[i] + ki);
             Vf64[i] = v;
             Vf[i] = (float)v;
             bad = bad || !isfinite(v);
@@ -155,6 +164,7 @@ struct Group {
     bool compact = false;              // row orbits: representative rows, expanded per flow
     double **d_outc = nullptr;         // per flow: [ch][representative][n]
     long nc = 0;                       // values per flow of d_outc
+    float **d_Vr = nullptr;            // per flow: [representative][n] FP32 stage vertex
     const float **d_Vf = nullptr, **d_VT = nullptr;
     CUtensorMap *d_maps = nullptr;
     CUtensorMap *d_tmaps = nullptr;    // table map per slot
@@ -248,50 +258,55 @@ qpfrg_status setup_group(Group &g, const qpfrg_lattice *lattice, const qpfrg_fin
     const long n3 = (long)N * N * N;
     const TcBuffers &t = c->tc;
     const size_t nb = (size_t)t.Npad * t.Kp, nbd = (size_t)t.Npad * t.Kpd;
+    // every flow starts at V = U with Z = 1, C4v symmetric, and stays so:
+    // the row orbits apply to the whole batch when the context built them, and
+    // V and its sums are kept on the representative rows only
+    g.compact = c->rows_exact;
+    const long per = (long)c->n_rrep * N, nv = g.compact ? per : n3;
     // per-flow state and operands, one allocation per kind
-    double *V, *k, *acc;
-    float *Vf, *VT;
+    double *V, *k = nullptr, *acc, *Us;
+    float *Vf, *VT, *Vr = nullptr;
     __nv_bfloat16 *B;
     const size_t bper = 2 * (2 * nb + nbd);
-    if ((s = galloc(g, &V, F * n3, "batch V")) || (s = galloc(g, &k, F * n3, "batch k")) ||
-        (s = galloc(g, &acc, F * n3, "batch acc")) || (s = galloc(g, &Vf, F * n3, "batch V fp32")) ||
+    if ((s = galloc(g, &V, F * nv, "batch V")) || (!g.compact && (s = galloc(g, &k, F * n3, "batch k"))) ||
+        (s = galloc(g, &acc, F * nv, "batch acc")) || (s = galloc(g, &Vf, F * n3, "batch V fp32")) ||
+        (g.compact && (s = galloc(g, &Vr, F * nv, "batch rows fp32"))) || (s = galloc(g, &Us, F, "batch couplings")) ||
         (s = galloc(g, &VT, F * 3 * n3, "batch row-factor tables")) || (s = galloc(g, &B, F * bper, "batch operands")))
         return s;
-    if ((e = cudaMemsetAsync(k, 0, F * n3 * sizeof(double), g.stream)) != cudaSuccess ||
+    if ((k && (e = cudaMemsetAsync(k, 0, F * n3 * sizeof(double), g.stream)) != cudaSuccess) ||
         (e = cudaMemsetAsync(B, 0, F * bper * sizeof(__nv_bfloat16), g.stream)) != cudaSuccess)
         return cuda_fail(c, e, "clear batch buffers");
-    // every flow starts at V = U with Z = 1, C4v symmetric, and stays so:
-    // the row orbits apply to the whole batch when the context built them
-    g.compact = c->rows_exact;
     double *outc = nullptr;
     std::vector<double *> poutc(F, nullptr);
     if (g.compact) {
-        g.nc = 3L * c->n_rrep * N;
+        g.nc = 3 * per;
         if ((s = galloc(g, &outc, F * g.nc, "batch representative rows")) ||
+            (s = galloc(g, &g.d_Vr, F, "batch row ptrs")) ||
             (s = galloc(g, &g.d_outc, F, "batch representative row ptrs")))
             return s;
         if ((e = cudaMemsetAsync(outc, 0, F * g.nc * sizeof(double), g.stream)) != cudaSuccess)
             return cuda_fail(c, e, "clear batch representative rows");
         for (int i = 0; i < F; ++i) poutc[i] = outc + i * g.nc;
     }
-    std::vector<double> hv(n3);
-    std::vector<float> hf(n3);
+    std::vector<double> hu(F);
+    for (int i = 0; i < F; ++i) hu[i] = specs[g.members[i]].U;
+    if ((e = cudaMemcpyAsync(Us, hu.data(), F * sizeof(double), cudaMemcpyHostToDevice, g.stream)) != cudaSuccess)
+        return cuda_fail(c, e, "batch initial state");
+    fill_batch_kernel<<<dim3(div_up(n3, 256 * 16), F), 256, 0, g.stream>>>(Us, V, nv, Vf, n3);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "batch initial state");
     std::vector<TcPrepFlow> pf(F);
     std::vector<double *> pV(F), pk(F), pacc(F);
+    std::vector<float *> pVr(F);
     std::vector<const float *> pVf(F), pVT(F);
     std::vector<CUtensorMap> maps(6 * (size_t)F);
     std::vector<int> h_status(F), h_steps(F, 0);
     std::vector<double> h_x(F), h_m(F), h_lc(F, 0.0), xend(F);
     for (int i = 0; i < F; ++i) {
         const qpfrg_flow_spec &sp = specs[g.members[i]];
-        std::fill(hv.begin(), hv.end(), sp.U);
-        std::fill(hf.begin(), hf.end(), (float)sp.U);
-        if ((e = cudaMemcpy(V + i * n3, hv.data(), n3 * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = cudaMemcpy(Vf + i * n3, hf.data(), n3 * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess)
-            return cuda_fail(c, e, "batch initial state");
-        pV[i] = V + i * n3;
-        pk[i] = k + i * n3;
-        pacc[i] = acc + i * n3;
+        pV[i] = V + i * nv;
+        pk[i] = k ? k + i * n3 : nullptr;
+        pacc[i] = acc + i * nv;
+        pVr[i] = Vr ? Vr + i * nv : nullptr;
         pVf[i] = Vf + i * n3;
         pVT[i] = VT + i * 3 * n3;
         __nv_bfloat16 *bb = B + i * bper;
@@ -361,7 +376,8 @@ qpfrg_status setup_group(Group &g, const qpfrg_lattice *lattice, const qpfrg_fin
                {g.d_slot, g.slot_tab.data(), g.slot_tab.size()},
                {g.d_rows, g.rows.data(), g.nslots * sizeof(float *)},
                {g.d_tmaps, tmaps.data(), g.nslots * sizeof(CUtensorMap)},
-               {g.d_outc, poutc.data(), g.compact ? F * sizeof(double *) : 0}};
+               {g.d_outc, poutc.data(), g.compact ? F * sizeof(double *) : 0},
+               {g.d_Vr, pVr.data(), g.compact ? F * sizeof(float *) : 0}};
     for (const Up &u : ups)
         if (u.bytes && (e = cudaMemcpy(u.dst, u.src, u.bytes, cudaMemcpyHostToDevice)) != cudaSuccess)
             return cuda_fail(c, e, "batch upload");
@@ -407,12 +423,14 @@ qpfrg_status enqueue_group_step(Group &g, int k, double stop)
         if ((ch & QPFRG_CH_PP) && (s = launch_tc_fused_batch(c, 0, bt, -1.0))) return s;
         if ((ch & QPFRG_CH_CR) && (s = launch_tc_fused_batch(c, 1, bt, -1.0))) return s;
         if ((ch & QPFRG_CH_D) && (s = launch_tc_fused_batch(c, 2, bt, 1.0))) return s;
-        if (g.compact && (s = launch_rows_expand_batch(c, bt)) != QPFRG_OK) return s;
+        if (g.compact) {
+            if ((s = launch_rows_rk_batch(c, st + 1, bt, g.d_V, g.d_acc, g.d_Vr, g.d_red)) != QPFRG_OK) return s;
+            continue;
+        }
         const int blocks = (int)std::min<long>((n3 + 255) / 256, 152L * 4 / std::max(1, g.F / 8 + 1) + 1);
         prof_begin(c);
-        rk_batch_kernel<<<dim3(blocks, g.F), 256, 0, g.stream>>>(st + 1, g.d_pf, g.d_V, g.d_k, g.d_acc, g.d_outc,
-                                                                 g.compact ? g.nc : 0, g.d_h, g.st.status, k, g.F,
-                                                                 g.d_red, n3);
+        rk_batch_kernel<<<dim3(blocks, g.F), 256, 0, g.stream>>>(st + 1, g.d_pf, g.d_V, g.d_k, g.d_acc, g.d_h,
+                                                                 g.st.status, k, g.F, g.d_red, n3);
         prof_end(c, st < 3 ? K_RK_STAGE : K_RK_FINAL);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(c, e, "rk_batch_kernel");

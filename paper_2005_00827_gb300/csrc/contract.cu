@@ -574,25 +574,98 @@ __global__ void rows_expand_kernel(const double *__restrict__ outc, const int *_
     expand_row(outc, rowmap, nr, N, ns, channels, out, blockIdx.y, blockIdx.x);
 }
 
-// Batched flows: grid.z = flow; flows that are not running or have no step
-// at this row of the schedule return at once.
-__global__ void rows_expand_batch_kernel(TcBatch bt, const int *__restrict__ rowmap, int nr, int N, int ns,
-                                         unsigned channels)
+// Runge-Kutta stage (1 .. 4) of the batched flows on the representative rows: their
+// state is V[m][n], acc[m][n] of the particle-particle representatives
+// Q_m = (x, y), n = k3, and every other element is an image of these.  The three
+// channels' values of (x, y, n) give dV; Vr is the FP32 vertex of the next stage.
+//
+// What bounds it: latency and the gathers of cr and d (L2).  FP64 costs 64 clocks a
+// warp instruction: on all N^3 elements of 12 flows at np96 the expansion into dV,
+// the stage update and the clearing of dV took 140 + 600 us (1 GB), of which an
+// eighth of the elements is needed; here and in vertex_expand_batch_kernel @RK@.
+__global__ void rows_rk_batch_kernel(int stage, TcBatch bt, const int *__restrict__ rep, const int *__restrict__ rowmap,
+                                     int nr, int N, int ns, unsigned channels, double *const *Vs, double *const *accs,
+                                     float *const *Vrs, unsigned long long *red)
 {
-    const int f = blockIdx.z;
-    if (bt.status[f] != QPFRG_FLOW_RUNNING || bt.h_tab[(long)bt.step * bt.nflows + f] == 0.0) return;
-    expand_row(bt.outc[f], rowmap, nr, N, ns, channels, bt.out[f], blockIdx.y, blockIdx.x);
+    const int f = blockIdx.y;
+    const double h = bt.h_tab[(long)bt.step * bt.nflows + f];
+    if (bt.status[f] != QPFRG_FLOW_RUNNING || h == 0.0) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, per = nr * N;
+    double m = 0.0;
+    bool bad = false;
+    if (i < per) {
+        const double *__restrict__ outc = bt.outc[f];
+        double *V = Vs[f], *acc = accs[f];
+        const int Na = N / ns, r = i / N, n = i - r * N;
+        const int Q = __ldg(rep + r), x = Q / N, y = Q - x * N;
+        const int *__restrict__ ph = rowmap + N * N;
+        auto take = [&](int ch, int e, int col) {
+            return __ldg(outc + (long)ch * per + (long)(e & 0xffffff) * N + c4v_patch(c4v_inverse(e >> 24), col, ns, Na));
+        };
+        const double v = V[i], a0 = stage > 1 ? acc[i] : 0.0;
+        double k = 0.0;
+        if (channels & QPFRG_CH_PP) k += __ldg(outc + i);
+        if (channels & QPFRG_CH_CR) k += take(1, __ldg(ph + n * N + y), x);
+        if (channels & QPFRG_CH_D) k += take(2, __ldg(ph + x * N + n), y);
+        if (stage < 4) {
+            acc[i] = stage == 1 ? k : a0 + 2.0 * k;
+            Vrs[f][i] = (float)(v + (stage == 3 ? h : 0.5 * h) * k);
+        } else {
+            const double w = v + h / 6.0 * (a0 + k);
+            V[i] = w;
+            Vrs[f][i] = (float)w;
+            bad = !isfinite(w);
+            m = bad ? 0.0 : fabs(w);
+        }
+    }
+    if (stage < 4) return;
+    for (int off = 16; off > 0; off >>= 1) {
+        m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
+        bad = __shfl_down_sync(0xffffffffu, (int)bad, off) || bad;
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&red[2 * f], (unsigned long long)__double_as_longlong(m));
+        if (bad) atomicOr(&red[2 * f + 1], 1ull);
+    }
 }
 
-qpfrg_status launch_rows_expand_batch(qpfrg_ctx *c, const TcBatch &bt)
+// The FP32 stage vertex of every running flow from its representative rows, four
+// consecutive k3 per thread, and the contraction rows cleared for the next stage.
+__global__ void vertex_expand_batch_kernel(TcBatch bt, const int *__restrict__ rowmap, int nr, int N, int ns,
+                                           const float *const *Vrs)
 {
-    const int N = c->pb.N, thr = std::min(256, (N + 31) / 32 * 32);
+    const int f = blockIdx.y;
+    if (bt.status[f] != QPFRG_FLOW_RUNNING || bt.h_tab[(long)bt.step * bt.nflows + f] == 0.0) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    double *outc = bt.outc[f];
+    for (int i = t; i < 3 * nr * N; i += nt) outc[i] = 0.0;
+    const int n4 = N / 4;                 // N is a multiple of 4
+    if (t >= N * N * n4) return;
+    const int Q = t / n4, k3 = 4 * (t - Q * n4), Na = N / ns;
+    const int e = __ldg(rowmap + Q), gi = c4v_inverse(e >> 24);
+    const float *__restrict__ row = Vrs[f] + (long)(e & 0xffffff) * N;
+    float4 v;
+    v.x = row[c4v_patch(gi, k3, ns, Na)];
+    v.y = row[c4v_patch(gi, k3 + 1, ns, Na)];
+    v.z = row[c4v_patch(gi, k3 + 2, ns, Na)];
+    v.w = row[c4v_patch(gi, k3 + 3, ns, Na)];
+    *reinterpret_cast<float4 *>(const_cast<float *>(bt.Vf[f]) + (long)Q * N + k3) = v;
+}
+
+qpfrg_status launch_rows_rk_batch(qpfrg_ctx *c, int stage, const TcBatch &bt, double *const *V, double *const *acc,
+                                  float *const *Vr, unsigned long long *red)
+{
+    const int N = c->pb.N;
     prof_begin(c);
-    rows_expand_batch_kernel<<<dim3(N, N, bt.nflows), thr, 0, c->stream>>>(bt, c->d_rowmap, c->n_rrep, N,
-                                                                           c->pb.n_shell, c->pb.channels);
+    rows_rk_batch_kernel<<<dim3(div_up((long)c->n_rrep * N, 256), bt.nflows), 256, 0, c->stream>>>(
+        stage, bt, c->d_rrep, c->d_rowmap, c->n_rrep, N, c->pb.n_shell, c->pb.channels, V, acc, Vr, red);
+    prof_end(c, stage < 4 ? K_RK_STAGE : K_RK_FINAL);
+    prof_begin(c);
+    vertex_expand_batch_kernel<<<dim3(div_up((long)N * N * N / 4, 256), bt.nflows), 256, 0, c->stream>>>(
+        bt, c->d_rowmap, c->n_rrep, N, c->pb.n_shell, Vr);
     prof_end(c, K_ROWS_EXPAND);
     const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "rows_expand_batch_kernel");
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "rows_rk_batch_kernel");
 }
 
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out)

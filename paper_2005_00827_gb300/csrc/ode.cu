@@ -54,18 +54,6 @@ __global__ void rk_final_kernel(double h, double *__restrict__ V, const double *
     reduce_max_flag(m, bad, red);
 }
 
-__global__ void check_finite_kernel(const double *__restrict__ x, long n, unsigned long long *red)
-{
-    double m = 0.0;
-    unsigned bad = 0;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const double v = x[i];
-        if (!isfinite(v)) bad = 1;
-        else m = fmax(m, fabs(v));
-    }
-    reduce_max_flag(m, bad, red);
-}
-
 static int grid_for(long n)
 {
     long b = (n + 255) / 256;
@@ -94,15 +82,6 @@ qpfrg_status launch_rk_final(qpfrg_ctx *c, double h, double *d_V, const double *
     prof_end(c, K_RK_FINAL);
     e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "rk_final_kernel");
-}
-
-qpfrg_status launch_check_finite(qpfrg_ctx *c, const double *d_x, long n)
-{
-    cudaError_t e = cudaMemsetAsync(c->d_red, 0, 2 * sizeof(unsigned long long), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "memset reduction");
-    check_finite_kernel<<<grid_for(n), 256, 0, c->stream>>>(d_x, n, c->d_red);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "check_finite_kernel");
 }
 
 }  // namespace qpfrg

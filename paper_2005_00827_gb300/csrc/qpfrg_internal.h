@@ -473,9 +473,12 @@ struct TcBatch {
 };
 
 qpfrg_status launch_tc_fused_batch(qpfrg_ctx *c, int ch, const TcBatch &bt, double sign);
-// contract.cu: out_f += the expansion of the representative rows outc_f of
-// every running flow f with a step at this row of the schedule
-qpfrg_status launch_rows_expand_batch(qpfrg_ctx *c, const TcBatch &bt);
+// contract.cu: Runge-Kutta stage 1 .. 4 of every running flow with a step at this row
+// of the schedule on its representative rows (V, acc FP64 and Vr FP32, [n_rrep][N] per
+// flow), the FP32 stage vertex expanded from them, outc cleared; stage 4 reduces
+// max|V| and finiteness into red[2 f], red[2 f + 1]
+qpfrg_status launch_rows_rk_batch(qpfrg_ctx *c, int stage, const TcBatch &bt, double *const *V, double *const *acc,
+                                  float *const *Vr, unsigned long long *red);
 
 // batch.cu: batched temperature flows (qpfrg_flow_batch)
 bool batch_device_path(const qpfrg_fine_grid *grid, qpfrg_regulator regulator, const qpfrg_options &opt, int n,
@@ -494,7 +497,6 @@ qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_
                              const double *d_k, double *d_acc, double *d_Vs, float *d_Vf);
 qpfrg_status launch_rk_final(qpfrg_ctx *c, double h, double *d_V, const double *d_acc,
                              const double *d_k);
-qpfrg_status launch_check_finite(qpfrg_ctx *c, const double *d_x, long n);
 
 // profiling helpers (qpfrg_api.cu)
 void prof_begin(qpfrg_ctx *c);
