@@ -133,8 +133,8 @@ typedef struct {
                                     each patch-count group (qpfrg_autotune) before stepping */
     int no_loop_symmetry;        /* 0: C4v reductions on (wedge and shell modes): one
                                     loop-kernel row per orbit of (transfer, patch), and
-                                    with QPFRG_MIXED_TC and a C4v-symmetric V and Z one
-                                    contraction row per orbit of transfers, expanded;
+                                    with a C4v-symmetric V and Z one contraction row per
+                                    orbit of transfers, expanded;
                                     2: the loop-kernel orbits only; other nonzero: every
                                     loop-kernel row and every contraction row evaluated */
     /* interaction flow only: the self-energy ODE of App. A.2-A.5 (state V,
@@ -188,11 +188,14 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
  * d_V: N^3 FP64 input, d_Z: N FP64 input (NULL = all ones), d_dV: N^3 FP64
  * output (may not alias d_V).  lambda = T (T-flow, > 0) or g (g-flow).
  * Uses the context's precision.  The context's flow state is not changed.
- * With QPFRG_MIXED_TC and the contraction's row orbits available (see
- * qpfrg_rhs_work) the call first tests V and Z for C4v symmetry on the device
- * (1e-12 of max|V|, max|Z|) and waits for that test on the context's stream:
- * a symmetric input contracts one row per orbit of transfer pairs, any other
- * every row.  Otherwise the work is only enqueued. */
+ * Where the row orbits are available (see qpfrg_rhs_work) the call tests V and
+ * Z for C4v symmetry on the device (of max|V|, max|Z|: 1e-12, FP64 1e-14; an
+ * Inf or NaN is not symmetric): a symmetric input contracts one row per orbit
+ * of transfer pairs, any other every row.  With QPFRG_FP64 and QPFRG_MIXED the
+ * device takes that decision and the work is only enqueued; with
+ * QPFRG_MIXED_TC the host waits for the test on the context's stream.
+ * Deviations are tested image by image under the two generators of C4v, each
+ * within a third of the tolerance. */
 qpfrg_status qpfrg_rhs(qpfrg_t ctx, double lambda, const double *d_V, const double *d_Z,
                        double *d_dV);
 
@@ -205,7 +208,12 @@ qpfrg_status qpfrg_rhs(qpfrg_t ctx, double lambda, const double *d_V, const doub
  * and Z_j = 1/(1 - [Re Sigma(xi_j+2T) - Re Sigma(xi_j-2T)]/(4T)).
  * d_sigma_re/d_sigma_im: N x n_omega FP64 outputs (may be NULL when
  * n_omega == 0; the frequency grid is binned, see the design notes);
- * d_Z_out: N FP64 output (may be NULL).  Regulator must be TEMPERATURE
+ * d_Z_out: N FP64 output (may be NULL).  In wedge mode V and Z are tested for
+ * C4v symmetry on the device (1e-6 of the maxima for Z and 1e-5 for the grid,
+ * FP64 Z 1e-14; FP64 evaluates the grid at every patch): a symmetric input
+ * evaluates the targets that differ under C4v, and images whose momenta on a
+ * wedge boundary are decided otherwise than their representative's get that
+ * difference added.  Regulator must be TEMPERATURE
  * (QPFRG_ERR_UNSUPPORTED otherwise). */
 qpfrg_status qpfrg_selfenergy(qpfrg_t ctx, double lambda, const double *d_V, const double *d_Z,
                               double *d_sigma_re, double *d_sigma_im, double *d_Z_out);
@@ -274,8 +282,8 @@ qpfrg_status qpfrg_get_state(qpfrg_t ctx, void *h_buf, size_t bytes);
 /* Replace the flow state by h_buf (as written by qpfrg_get_state; host,
  * page-locked memory preferred).  The image is uploaded into scratch space and
  * checked on the device (finiteness, max|V|, C4v symmetry of the state, which
- * selects the self-energy's irreducible targets); synchronises the context's
- * stream.  Returns QPFRG_ERR_INVALID on a wrong header or size,
+ * selects the self-energy's irreducible targets and the row orbits);
+ * synchronises the context's stream.  Returns QPFRG_ERR_INVALID on a wrong header or size,
  * QPFRG_ERR_NONFINITE (state unchanged) when V or Z holds NaN/Inf.  Between
  * steps only (it reuses the RK scratch buffers). */
 qpfrg_status qpfrg_set_state(qpfrg_t ctx, const void *h_buf, size_t bytes);
@@ -331,19 +339,25 @@ qpfrg_status qpfrg_profile_get(qpfrg_t ctx, int id, double *ms, long long *launc
  * checks byte by byte on its partner maps at creation (rows that differ are
  * evaluated by themselves; C4v moves the wedge of a patch and keeps its
  * energy shell).  With quasi-particle lines (QPFRG_PROP_QP) the
- * reduction needs a C4v-symmetric Z.  With QPFRG_MIXED_TC, every row
- * covariant and a C4v-symmetric V and Z (the flow's state, or a qpfrg_rhs
- * input that passes a device test at 1e-12 relative), each channel's output
- * is C4v invariant too: then only one output row per orbit of transfer pairs
- * Q = (x, y) is tabled (all its patches a) and contracted, and every other
- * row is its representative's with the columns permuted (row orbits).
- *   loop_evals: loop-kernel evaluations of the context's last RHS;
+ * reduction needs a C4v-symmetric Z.  With a C4v-symmetric V and Z (the
+ * flow's state, or a qpfrg_rhs input that passes the device test), each
+ * channel's output is C4v invariant too: then only one output row per orbit of
+ * transfer pairs Q = (x, y) is tabled (all its patches a) and contracted, and
+ * every other row is its representative's with the columns permuted (row
+ * orbits).  Pairs whose rows break covariance are contraction rows of their
+ * own; a flow takes the row orbits only where no pair does.  The pairs (x, y)
+ * and (y, x) of the particle-particle family, and (x, y) and (y', x') of the
+ * particle-hole family, x' opposite to x, have the same transfer momentum:
+ * their rows of the table are the same and are evaluated once.
+ *   loop_evals: loop-kernel evaluations of the context's last RHS, a row of
+ *     the table that two contraction rows share counted for each of them;
  *   loop_evals_full: 2 N^2 M, the evaluations of the unreduced RHS;
  *   rows_unreduced: rows evaluated by themselves because the covariance check
  *     failed for them;
  *   contraction_rows: rows of each channel GEMM in the last RHS (N^2, or the
  *     number of row orbits).
- * All outputs may be NULL; loop_evals equals loop_evals_full when the
+ * Where the device decided the form of the last RHS the call waits for it on
+ * the context's stream.  All outputs may be NULL; loop_evals equals loop_evals_full when the
  * reduction is off (lattice mode, no_loop_symmetry). */
 qpfrg_status qpfrg_rhs_work(qpfrg_t ctx, long long *loop_evals, long long *loop_evals_full,
                             long long *rows_unreduced, long long *contraction_rows);

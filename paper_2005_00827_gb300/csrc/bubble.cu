@@ -14,9 +14,9 @@
 // Launch shape: one CTA of 8 warps per (patch a, chunk of Q, family) -- or,
 // in wedge mode, per task of the C4v-reduced launch (symmetry.cu: one row per
 // orbit of (Q, a) under the point group, written to every image row with its
-// columns permuted; or, for the tensor-core contraction of a C4v-symmetric
-// state, the representative transfer pairs of the row orbits with every patch
-// a, each row written once to the compact table).  The CTA stages its wedge's
+// columns permuted; or, for a C4v-symmetric state, the representative transfer
+// pairs of the row orbits with every patch a, each row written once to the
+// compact table; the form may be decided on the device, SymMode).  The CTA stages its wedge's
 // fine points in shared
 // memory; each warp takes one transfer at a time, streams its partner-patch
 // bytes (coalesced) and bins the loop kernels into a private row of N
