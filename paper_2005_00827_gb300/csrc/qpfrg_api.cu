@@ -192,7 +192,7 @@ void qpfrg_destroy(qpfrg_t c)
                         c->d_part, c->d_B, c->d_ones, c->d_sig, c->d_hist, c->d_jirr, c->d_rep,
                         c->tc.Bpp[0], c->tc.Bpp[1], c->tc.Bcr[0], c->tc.Bcr[1], c->tc.Bd[0], c->tc.Bd[1],
                         c->tc.VT, c->d_tc_err, c->d_xij, c->d_bnd, c->d_qxl, c->d_qyl, c->d_kp, c->d_kcs, c->d_xij_f,
-                        c->d_ptab, c->d_jgrid, c->d_repgrid, c->d_lrepQ, c->d_lnimg, c->d_limg, c->d_ltask,
+                        c->d_ptab, c->d_jgrid, c->d_repgrid, c->d_owngrid, c->d_lrepQ, c->d_lnimg, c->d_limg, c->d_ltask,
                         c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views, c->d_kfx, c->d_pfx, c->d_events};
         for (void *p : ptrs)
             if (p) cudaFree(p);
@@ -418,9 +418,18 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
                 jgrid.push_back(m * q);
             }
             c->n_grid = (int)jgrid.size();
+            std::vector<int> own(N, -1);
+            for (int k = 0; k < c->n_grid; ++k) own[jgrid[k]] = k;
+            for (int j = 0; j < (int)N; ++j)
+                if (own[j] < 0) {
+                    own[j] = (int)jgrid.size();
+                    jgrid.push_back(j);
+                }
             if ((s = dev_alloc(c, &c->d_jgrid, jgrid.size(), "grid targets")) ||
-                (s = dev_alloc(c, &c->d_repgrid, N, "grid representatives")))
+                (s = dev_alloc(c, &c->d_repgrid, N, "grid representatives")) ||
+                (s = dev_alloc(c, &c->d_owngrid, N, "grid slots")))
                 return fail(s);
+            cudaMemcpy(c->d_owngrid, own.data(), N * sizeof(int), cudaMemcpyHostToDevice);
             cudaMemcpy(c->d_jgrid, jgrid.data(), jgrid.size() * sizeof(int), cudaMemcpyHostToDevice);
             cudaMemcpy(c->d_repgrid, repgrid.data(), N * sizeof(int), cudaMemcpyHostToDevice);
         }

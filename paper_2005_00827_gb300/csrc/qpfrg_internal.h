@@ -344,8 +344,9 @@ struct qpfrg_ctx {
     // targets of the frequency-grid self-energy of a C4v-symmetric state: the
     // irreducible patches plus the zone-edge patches N/4, N/2, 3N/4, whose sums
     // differ from patch 0's where a momentum lands on |k_x| or |k_y| = pi
-    int *d_jgrid = nullptr;
+    int *d_jgrid = nullptr;      // these n_grid patches, then every other one
     int *d_repgrid = nullptr;    // slot of each patch's representative in d_jgrid
+    int *d_owngrid = nullptr;    // slot of each patch itself
     int n_grid = 0;
     bool c4v_state = false;      // flow state V, Z is C4v symmetric
     double *d_hist = nullptr;    // Sigma frequency-grid histogram (lazily sized)

@@ -520,15 +520,18 @@ struct SigmaFastArgs {
     const uint8_t *ptab;
     const uint8_t *rtab;    // patch of r per (target, p, q) (RT launches; rtab_build_kernel)
     const int *jlist;
-    // sym.mode == 2: target slots 0 .. N-1 are the patches or, where the C4v test
-    // of (V, Z) holds, the n_list targets of jlist (the other slots return)
+    // sym.mode == 2: jlist holds every patch, its first n_list the targets that a
+    // C4v-symmetric (V, Z) needs (the other slots then return); own[j]: slot of j
     SymMode sym;
     int n_list;
+    const int *own;
     const double *K;        // Katanin factors (interaction-flow lines; the GL kernels)
     double *sig;
     // pairs on a boundary between patches met by a reduced launch, and per patch
-    // its own slope less its representative's (sigma_fix_kernel); only_full: run
-    // only when there were more pairs than the record holds
+    // its own slope less its representative's (sigma_fix_kernel; the frequency grid:
+    // its own histogram less its representative's, in its slot); nevents[0] their
+    // number, nevents[1] the corrections made; only_full: run only when there were
+    // more pairs than the record holds
     int4 *events;
     unsigned *nevents, max_events;
     bool only_full;
@@ -536,8 +539,7 @@ struct SigmaFastArgs {
     float t, tp, mu, eta2, invT, cT, twoT, fourT;   // cT = log2(e) / T
     float tln2, kchord, eta2x4;                     // T ln 2, 4 T^2 + eta^2, 4 eta^2
     float inv_dth, dth;                             // N / 2 pi, 2 pi / N
-    int mirror;     // n_theta even and symmetric targets: 1 halves every mirror-line target,
-                    // 2 all but the zone-edge ones (j a multiple of N/4)
+    int mirror;     // n_theta even and symmetric targets: halve the mirror-line targets
     int qb;         // blocks of 256 SF_QPT loop points q per CTA
     // grid mode: pole energies E binned from e_min in bins of h, moments 0..4
     // of the offset from the bin centre, hist[target][moment][bin] (FP64)
@@ -547,6 +549,7 @@ struct SigmaFastArgs {
     // that the offset x - rint(x) keeps FP32 accuracy at every bin)
     float inv_h, inv_h_lo, c_frac;
     int nbins, c_int;
+    double e_min, h64;
     float w_max;            // largest quadrature weight
 };
 
@@ -555,7 +558,7 @@ __device__ __forceinline__ bool sigma_target(const SigmaFastArgs &A, int z, int 
 {
     sym = A.sym.mode == 2 ? sym_compact(A.sym) : A.jlist != nullptr;
     if (sym && A.sym.mode == 2 && z >= A.n_list) return false;
-    j = sym ? A.jlist[z] : z;
+    j = A.jlist ? A.jlist[z] : z;
     return true;
 }
 
@@ -563,12 +566,11 @@ __device__ __forceinline__ bool sigma_target(const SigmaFastArgs &A, int z, int 
 // N/8, which reflects patch a to 2j - a) has a sum symmetric under that mirror:
 // keep the patches a on one side of it with weight fac = 2 and half of each patch
 // the mirror maps onto itself (P loop points: angular index t < n_theta / 2).
-// fac = 0: the mirror patch carries this one.  mirror 2 leaves out the zone-edge
-// targets (j a multiple of N/4).
+// fac = 0: the mirror patch carries this one.
 __device__ __forceinline__ void mirror_part(int mirror, int N, int j, int a, int &fac, int &P)
 {
     fac = 1;
-    if (!mirror || (8 * j) % N != 0 || (mirror == 2 && (4 * j) % N == 0)) return;
+    if (!mirror || (8 * j) % N != 0) return;
     const int ma = ((2 * j - a) % N + N) % N;
     if (ma == a) {
         fac = 2;
@@ -708,13 +710,14 @@ __device__ __noinline__ int sf_slow_patch(const SigmaFastArgs &A, int j, int p, 
     return c;
 }
 
-// Chord term of one pair with r in patch c, in FP64 from the tables (rare).
-__device__ __noinline__ double sf_pair_term(const SigmaFastArgs &A, int j, int p, int q, int c)
+// Weight W F and pole energy E of one pair with r in patch c, in FP64 from the
+// tables (rare).
+__device__ __noinline__ double sf_pair_weight(const SigmaFastArgs &A, int j, int p, int q, int c, double &E)
 {
     const int N = A.pb.N, PP = A.pb.P, a = p / PP, b = q / PP;
     auto z = [&](int k) { return A.Z ? A.Z[k] : 1.0; };
     const bool qp = A.pb.propagator == QPFRG_PROP_QP;
-    const double Za = z(a), Zb = z(b), Zc = z(c), invT = 1.0 / A.T64, eta2 = A.pb.eta * A.pb.eta;
+    const double Za = z(a), Zb = z(b), Zc = z(c), invT = 1.0 / A.T64;
     const double cx = cos(A.kf[2 * j] + A.kx64[p] - A.kx64[q]), cy = cos(A.kf[2 * j + 1] + A.ky64[p] - A.ky64[q]);
     const double xp = (qp ? Za : 1.0) * A.xi64[p], xq = (qp ? Zb : 1.0) * A.xi64[q];
     const double xr = (qp ? Zc : 1.0) * (-2.0 * A.pb.t * (cx + cy) - 4.0 * A.pb.tp * cx * cy - A.pb.mu);
@@ -724,17 +727,19 @@ __device__ __noinline__ double sf_pair_term(const SigmaFastArgs &A, int j, int p
     double amp = A.w64[p] * A.w64[q] * Za * Zb * Zc * (2.0 * V[b] * V[b] - V[b] * V[c]) * F;
     if (A.K)
         amp *= (A.K[a] * Za * (Zb + Zc) + A.K[b] * Zb * (Za + Zc) + A.K[c] * Zc * (Za + Zb)) * (1.0 / 6.0);
-    const double d0 = A.xij64[j] - (xq + xr - xp), dp = d0 + 2.0 * A.T64, dm = d0 - 2.0 * A.T64;
-    return amp * (eta2 - dp * dm) / ((dp * dp + eta2) * (dm * dm + eta2));
+    E = xq + xr - xp;
+    return amp;
 }
 
 // A recorded pair (p, q) of target j, patch c, lies on a boundary: every image
 // target that copies j's sum is corrected where its own pair is decided
-// otherwise, so that each patch keeps its own sum.
-__global__ void __launch_bounds__(128) sigma_fix_kernel(SigmaFastArgs A)
+// otherwise, so that each patch keeps its own sum.  hist: the difference goes into
+// the image's own slot of the frequency grid's histogram, else into its slope.
+__global__ void __launch_bounds__(128) sigma_fix_kernel(SigmaFastArgs A, double *hist)
 {
+    if (*A.nevents > A.max_events) return;      // every patch is summed
     const int N = A.pb.N, PP = A.pb.P, nt = A.pb.n_theta, nr = A.pb.n_r;
-    const unsigned n = min(*A.nevents, A.max_events);
+    const unsigned n = *A.nevents;
     auto image = [&](int g, int k) {
         const int a = k / PP, l = k - a * PP, t = l / nr, s = l - t * nr;
         return c4v_apply(g, a, N, 1) * PP + ((g & 4) ? nt - 1 - t : t) * nr + s;
@@ -747,7 +752,22 @@ __global__ void __launch_bounds__(128) sigma_fix_kernel(SigmaFastArgs A)
         if (seen) continue;
         const int pg = image(g, e.y), qg = image(g, e.z);
         const int own = sf_slow_patch(A, jg, pg, qg, 0.f, 0.f, 1, A.bnd), copied = c4v_apply(g, e.w, N, 1);
-        if (own != copied) atomicAdd(&A.corr[jg], sf_pair_term(A, jg, pg, qg, own) - sf_pair_term(A, jg, pg, qg, copied));
+        if (own == copied) continue;
+        atomicAdd(A.nevents + 1, 1u);
+        for (int u = 0; u < 2; ++u) {
+            double E, amp = sf_pair_weight(A, jg, pg, qg, u ? copied : own, E);
+            if (u) amp = -amp;
+            if (hist) {
+                const int bin = (int)fmin(fmax(floor((E - A.e_min) / A.h64), 0.0), A.nbins - 1.0);
+                const double d = E - (A.e_min + (bin + 0.5) * A.h64);
+                double *H = hist + (long)A.own[jg] * 5 * A.nbins + bin;
+                for (int mo = 0; mo < 5; ++mo, amp *= d) atomicAdd(H + (long)mo * A.nbins, amp);
+            } else {
+                const double eta2 = A.pb.eta * A.pb.eta;
+                const double d0 = A.xij64[jg] - E, dp = d0 + 2.0 * A.T64, dm = d0 - 2.0 * A.T64;
+                atomicAdd(&A.corr[jg], amp * (eta2 - dp * dm) / ((dp * dp + eta2) * (dm * dm + eta2)));
+            }
+        }
     }
 }
 
@@ -1247,10 +1267,9 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     const int a = blockIdx.y, jidx = blockIdx.z;
     int j;
     bool sym;
+    if (A.only_full && *A.nevents <= A.max_events) return;
     if (!sigma_target(A, jidx, j, sym)) return;      // uniform over the CTA
-    int fac, P = PP;
-    mirror_part(sym ? A.mirror : 0, N, j, a, fac, P);
-    if (fac == 0) return;       // the mirror patch carries this one (uniform over the CTA)
+    const int P = PP;
     const int tid = threadIdx.x;
     const bool qp = A.pb.propagator == QPFRG_PROP_QP;
     const HfSmem L = hf_smem_layout(NBS, LO);
@@ -1431,7 +1450,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
         // |W F| <= W max(f_p (1 - f_q), (1 - f_p) f_q) summed over the block
         const float total = s_sum[0] * s_blk[0] + s_sum[1] * s_blk[1], single = A.w_max * s_blk[2];
         const float scale = total > 0.f ? fminf(1073741824.f / total, 2097152.f / single) : 0.f;
-        const double unit = scale > 0.f ? (double)fac / (double)scale : 0.0, unit_lo = unit / (double)lo_scale;
+        const double unit = scale > 0.f ? 1.0 / (double)scale : 0.0, unit_lo = unit / (double)lo_scale;
         for (int p0 = 0; p0 < P; p0 += HF_REC) {
             const int cnt = min(HF_REC, P - p0);
             if (!one_pass) {
@@ -1499,7 +1518,9 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                 const int c0 = fx_zoom(__float_as_int(ra.x), __float_as_int(ra.y), A.pfx[qq].x, A.pfx[qq].y, tabc, ray, slow);
                 if (!slow) continue;
                 const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
-                const int c1 = sf_slow_patch(A, j, a * PP + p0 + i, qq, x * kRadPerFx, y * kRadPerFx, edge ? 1 : 0, A.bnd);
+                const bool fix = A.sym.mode == 2 && sym && (4 * j) % N != 0;   // the zone-edge targets have no images
+                const int c1 = sf_slow_patch(A, j, a * PP + p0 + i, qq, x * kRadPerFx, y * kRadPerFx,
+                                             (edge ? 1 : 0) | (fix ? 2 : 0), A.bnd);
                 if (c1 == c0) continue;
                 const int b = qq / PP;
                 const float Zb = A.Z ? (float)A.Z[b] : 1.f, vb = (float)Vja[b];
@@ -1726,17 +1747,17 @@ __global__ void __launch_bounds__(256) sigma64_kernel(const Sigma64Args S)
 
 // Z_j = 1/(1 - slope) with the chord slope accumulated per target slot, or the
 // slopes themselves (slopes_out).  rep[j] (may be NULL) is the slot of j's C4v
-// representative among the targets; sym.mode == 2: where the C4v test holds, with
+// representative among the targets, own[j] its own (NULL: j); sym.mode == 2: where the C4v test holds, with
 // the patch's own correction corr[j], or from the sums of every patch (full) when
 // the record of boundary pairs ran over.
 __global__ void z_update_kernel(const double *slope, const double *corr, const double *full, const unsigned *nevents,
-                                unsigned max_events, const int *rep, SymMode sym, double *Zout, double *slopes_out,
-                                int N)
+                                unsigned max_events, const int *rep, const int *own, SymMode sym, double *Zout,
+                                double *slopes_out, int N)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
     const bool use = rep && (sym.mode != 2 || sym_compact(sym));
-    double s = slope[use ? rep[j] : j];
+    double s = slope[use ? rep[j] : (own ? own[j] : j)];
     if (sym.mode == 2 && use) s = *nevents > max_events ? full[j] : s + corr[j];
     if (slopes_out) slopes_out[j] = s;
     if (Zout) Zout[j] = 1.0 / (1.0 - s);
@@ -1756,9 +1777,12 @@ constexpr int RG_BINS = 64;     // bins per CTA
 
 __global__ void __launch_bounds__(128) sigma_resum_kernel(const double *__restrict__ hist, int nbins, double e_min,
                                                           double h, int n_omega, double w0, double dw, double eta,
-                                                          double *__restrict__ acc, int ntarget, int n_list, SymMode sym)
+                                                          double *__restrict__ acc, int ntarget, int n_list, SymMode sym,
+                                                          const unsigned *nevents, unsigned max_events)
 {
-    const int nt = sym.mode == 2 && sym_compact(sym) ? n_list : ntarget;
+    // the slots past the list hold the corrections of the images, or their own sums
+    const bool more = sym.mode == 2 && (nevents[1] != 0 || nevents[0] > max_events);
+    const int nt = sym.mode == 2 && !more && sym_compact(sym) ? n_list : ntarget;
     const int t0 = blockIdx.z * RG_T;
     if (t0 >= nt) return;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1803,16 +1827,26 @@ __global__ void __launch_bounds__(128) sigma_resum_kernel(const double *__restri
     }
 }
 
-// Sigma of every patch from its target slot.
-__global__ void sigma_spread_kernel(const double *__restrict__ acc, const int *rep, SymMode sym, int n_omega,
-                                    double *__restrict__ re, double *__restrict__ im)
+// Sigma of every patch from its target slot; an image adds the correction in its
+// own slot, which holds its whole sum when the record of boundary pairs ran over.
+__global__ void sigma_spread_kernel(const double *__restrict__ acc, const int *rep, const int *own, SymMode sym,
+                                    const unsigned *nevents, unsigned max_events, int n_omega, double *__restrict__ re,
+                                    double *__restrict__ im)
 {
     const int m = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (m >= n_omega) return;
     const bool use = rep && (sym.mode != 2 || sym_compact(sym));
-    const double *a = acc + 2L * (use ? rep[j] : j) * n_omega + m;
-    re[(long)j * n_omega + m] = a[0];
-    im[(long)j * n_omega + m] = a[n_omega];
+    const int so = own ? own[j] : j, sr = use ? rep[j] : so;
+    const bool full = use && own && *nevents > max_events;
+    const double *a = acc + 2L * (full ? so : sr) * n_omega + m;
+    double x = a[0], y = a[n_omega];
+    if (use && own && so != sr && !full) {
+        a = acc + 2L * so * n_omega + m;
+        x += a[0];
+        y += a[n_omega];
+    }
+    re[(long)j * n_omega + m] = x;
+    im[(long)j * n_omega + m] = y;
 }
 
 static qpfrg_status launch_kp_table(qpfrg_ctx *c, const int *jlist, int nj, bool fixed = true)
@@ -1854,14 +1888,15 @@ struct SigmaTargets {
     int n = 0;              // targets of the list
     SymMode sym;
     const int *rep = nullptr;   // slot of each patch under the list
+    const int *own = nullptr;   // slot of each patch where every patch is evaluated (mode 2)
     int mirror = 0;             // mirror_part of the list's targets
     int slots(int N) const { return sym.mode == 2 || !jlist ? N : n; }
 };
 
 // Targets of a given (V, Z): with the symmetry that the device finds (red), the
-// irreducible patches and the zone-edge patches; images copy the sum of their
-// representative.  mirror 2 also halves the targets on a diagonal.
-static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror, const unsigned long long *red)
+// irreducible patches and the zone-edge patches, unhalved (every boundary pair is
+// met); images copy the sum of their representative and correct it.
+static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, const unsigned long long *red)
 {
     SigmaTargets t;
     t.n = c->pb.N;
@@ -1869,10 +1904,10 @@ static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, int mirror, c
     t.jlist = c->d_jgrid;
     t.n = c->n_grid;
     t.rep = c->d_repgrid;
+    t.own = c->d_owngrid;
     t.sym.mode = 2;
     t.sym.red = red;
     t.sym.tol = tol / 3.0;
-    t.mirror = c->pb.n_theta % 2 == 0 ? mirror : 0;
     return t;
 }
 
@@ -1910,6 +1945,7 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     A.jlist = tg.jlist;
     A.sym = tg.sym;
     A.n_list = tg.n;
+    A.own = tg.own;
     A.mirror = tg.mirror;
     A.sig = c->d_sig;
     A.corr = c->d_sig + 2 * c->pb.N;
@@ -2002,7 +2038,7 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     prof_begin(c);
     kern<<<dim3(div_up(nqb, A.qb), c->pb.N, nj), 256, smem, c->stream>>>(A);
     if (tg.sym.mode == 2) {
-        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(A);
+        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(A, nullptr);
         // every patch, should the record have run over
         SigmaFastArgs F = A;
         F.only_full = true;
@@ -2044,6 +2080,8 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     A.inv_h_lo = (float)(1.0 / h - (double)A.inv_h);
     A.h = (float)h;
     A.nbins = nbins;
+    A.e_min = e_min;
+    A.h64 = h;
     using Kern = void (*)(SigmaFastArgs);
     static const Kern table[3][2] = {
         {sigma_hist_kernel<kHfBins[0], true, false>, sigma_hist_kernel<kHfBins[0], true, true>},
@@ -2060,6 +2098,16 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     const int split = (int)std::max<long>(1, std::min<long>(nqb, (8 * 152 + per - 1) / per));
     prof_begin(c);
     kern<<<dim3(split, N, nj), HF_THR, smem, c->stream>>>(A);
+    if (tg.sym.mode == 2) {
+        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(A, hist);
+        // the images' own sums, should the record have run over
+        SigmaFastArgs F = A;
+        F.only_full = true;
+        F.jlist = tg.jlist + tg.n;
+        F.hist = hist + (long)tg.n * 5 * nbins;
+        F.sym = SymMode();
+        if (N > tg.n) kern<<<dim3(1, N, N - tg.n), HF_THR, smem, c->stream>>>(F);
+    }
     prof_end(c, K_SIGMA_HIST);
     e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_hist_kernel");
@@ -2093,7 +2141,7 @@ static qpfrg_status launch_sigma64(qpfrg_ctx *c, double T, const double *d_V, co
     prof_begin(c);
     kern<<<grid, 256, smem, c->stream>>>(S);
     if (tg.sym.mode == 2 && nbins == 0) {
-        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(S.a);
+        sigma_fix_kernel<<<152, 128, 0, c->stream>>>(S.a, nullptr);
         Sigma64Args F = S;       // every patch, should the record have run over
         F.a.only_full = true;
         F.a.jlist = nullptr;
@@ -2148,7 +2196,7 @@ static qpfrg_status launch_z_update(qpfrg_ctx *c, const SigmaTargets &tg, double
     prof_begin(c);
     z_update_kernel<<<div_up(N, 128), 128, 0, c->stream>>>(c->d_sig, c->d_sig + 2 * N, c->d_sig + 3 * N,
                                                               reinterpret_cast<unsigned *>(c->d_sig + 4 * N),
-                                                              c->max_events, tg.rep, tg.sym, Z, slopes, N);
+                                                              c->max_events, tg.rep, tg.own, tg.sym, Z, slopes, N);
     prof_end(c, K_Z_UPDATE);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "z_update_kernel");
@@ -2183,7 +2231,7 @@ qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const dou
     if (c->d_ptab) {
         const bool fp64 = c->opt.precision == QPFRG_FP64;
         if (!tg.jlist) {
-            tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, 0, c->d_sym_v);
+            tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, c->d_sym_v);
             if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         }
         s = fp64 ? launch_sigma64(c, T, d_V, d_Z, nullptr, tg) : launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
@@ -2216,7 +2264,7 @@ qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const
     qpfrg_status s;
     if (c->d_ptab) {
         const bool fp64 = c->opt.precision == QPFRG_FP64;
-        tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, 0, c->d_sym);
+        tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, c->d_sym);
         s = fp64 ? launch_sigma64(c, T, d_V, d_Z, d_K, tg) : launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
     } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
@@ -2270,13 +2318,16 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     cudaError_t e = cudaMemsetAsync(c->d_hist, 0, need * sizeof(double), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "memset histogram");
     double *acc = c->d_hist + hist_n;
+    unsigned *nevents = reinterpret_cast<unsigned *>(c->d_sig + 4 * N);
+    if ((e = cudaMemsetAsync(nevents, 0, 2 * sizeof(unsigned), c->stream)) != cudaSuccess)
+        return cuda_fail(c, e, "memset boundary pairs");
     qpfrg_status s;
     SigmaTargets tg;
     tg.n = N;
     if (c->opt.precision != QPFRG_FP64 && c->d_ptab && hist_variant(nbins) >= 0) {
         // FP32 wedge grid: table projection, histogram in shared memory; a
         // C4v-symmetric (V, Z) needs only the irreducible and zone-edge targets
-        tg = device_targets(c, kTolGrid, 2, d_K ? c->d_sym : c->d_sym_v);
+        tg = device_targets(c, kTolGrid, d_K ? c->d_sym : c->d_sym_v);
         if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         s = launch_sigma_hist(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
     } else if (c->opt.precision == QPFRG_FP64 && c->d_ptab) {
@@ -2304,8 +2355,9 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     const int nslot = tg.slots(N);
     prof_begin(c);
     sigma_resum_kernel<<<dim3(div_up(n_omega, 128), div_up(nbins, RG_BINS), div_up(nslot, RG_T)), 128, 0, c->stream>>>(
-        c->d_hist, nbins, e_min, h, n_omega, w0, dw, c->pb.eta, acc, nslot, tg.n, tg.sym);
-    sigma_spread_kernel<<<dim3(div_up(n_omega, 128), N), 128, 0, c->stream>>>(acc, tg.rep, tg.sym, n_omega, d_re, d_im);
+        c->d_hist, nbins, e_min, h, n_omega, w0, dw, c->pb.eta, acc, nslot, tg.n, tg.sym, nevents, c->max_events);
+    sigma_spread_kernel<<<dim3(div_up(n_omega, 128), N), 128, 0, c->stream>>>(acc, tg.rep, tg.own, tg.sym, nevents,
+                                                                             c->max_events, n_omega, d_re, d_im);
     prof_end(c, K_SIGMA_GRID);
     e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_resum_kernel");
