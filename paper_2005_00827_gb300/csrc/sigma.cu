@@ -1260,6 +1260,16 @@ __device__ __forceinline__ void red_shared(unsigned addr, int v)
     asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
+// A pole outside the bins (quasi-particle lines with a weight above z_max): the
+// moments about the edge bin, which are far from one half bin (rare).
+__device__ __noinline__ void hist_outside(const SigmaFastArgs &A, double *H, float amp, float E)
+{
+    const int bin = E < A.e_min + 0.5 * A.nbins * A.h64 ? 0 : A.nbins - 1;
+    const double d = (double)E - (A.e_min + (bin + 0.5) * A.h64);
+    double m = amp;
+    for (int mo = 0; mo < 5; ++mo, m *= d) atomicAdd(H + (long)mo * A.nbins + bin, m);
+}
+
 template <int NBS, bool LO, bool GL>
 __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastArgs A)
 {
@@ -1361,10 +1371,14 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     // bin's centre in half bins, and the moments
     auto deposit = [&](float amp, float E, float scale) {
         const float u = amp * scale;                     // in units of the histogram
-        int r;
+        int r;                                           // (past +-2^22: no bin either)
         const float rr = rint_add(fmaf(E, A.inv_h, A.c_frac), r);
         const float d = 2.f * (fmaf(E, A.inv_h, -rr) + fmaf(E, A.inv_h_lo, A.c_frac));
-        const int bin = min(max(r + A.c_int, 0), A.nbins - 1);
+        const int bin = r + A.c_int;
+        if ((unsigned)bin >= (unsigned)A.nbins) {
+            hist_outside(A, H, amp, E);
+            return;
+        }
         const unsigned h = hbase + 4u * (unsigned)bin;
         const float u0 = u + kMagic;
         red_shared(h, __float_as_int(u0) - 0x4B400000);
