@@ -1262,11 +1262,10 @@ __device__ __forceinline__ void red_shared(unsigned addr, int v)
 
 // A pole outside the bins (quasi-particle lines with a weight above z_max): the
 // moments about the edge bin, which are far from one half bin (rare).
-__device__ __noinline__ void hist_outside(const SigmaFastArgs &A, double *H, float amp, float E)
+__device__ __noinline__ void hist_outside(const SigmaFastArgs &A, double *H, double m, float E)
 {
     const int bin = E < A.e_min + 0.5 * A.nbins * A.h64 ? 0 : A.nbins - 1;
     const double d = (double)E - (A.e_min + (bin + 0.5) * A.h64);
-    double m = amp;
     for (int mo = 0; mo < 5; ++mo, m *= d) atomicAdd(H + (long)mo * A.nbins + bin, m);
 }
 
@@ -1352,8 +1351,13 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     for (int b = tid; b < N; b += HF_THR) {
         const float vb = (float)Vja[b];
         float m = 0.f;
-        for (int c = 0; c < N; ++c) m = fmaxf(m, fabsf(fmaf(-vb, cz[c].y, cz[c].x * 2.f * vb * vb)));
-        wb[b] = m * gl_max;
+        bool fin = true;         // (fmaxf drops a NaN)
+        for (int c = 0; c < N; ++c) {
+            const float w = fabsf(fmaf(-vb, cz[c].y, cz[c].x * 2.f * vb * vb));
+            m = fmaxf(m, w);
+            fin = fin && w <= 3e38f;
+        }
+        wb[b] = fin ? m * gl_max : __int_as_float(0x7f800000);
     }
     for (int i = tid; i < P; i += HF_THR) {
         float fp, fcp;
@@ -1369,14 +1373,14 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
 
     // one pair of weight amp and pole energy E: its bin, the offset from the
     // bin's centre in half bins, and the moments
-    auto deposit = [&](float amp, float E, float scale) {
+    auto deposit = [&](float amp, float E, float scale, float lift) {
         const float u = amp * scale;                     // in units of the histogram
         int r;                                           // (past +-2^22: no bin either)
         const float rr = rint_add(fmaf(E, A.inv_h, A.c_frac), r);
         const float d = 2.f * (fmaf(E, A.inv_h, -rr) + fmaf(E, A.inv_h_lo, A.c_frac));
         const int bin = r + A.c_int;
         if ((unsigned)bin >= (unsigned)A.nbins) {
-            hist_outside(A, H, amp, E);
+            hist_outside(A, H, (double)amp / lift, E);
             return;
         }
         const unsigned h = hbase + 4u * (unsigned)bin;
@@ -1462,9 +1466,22 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
         }
         __syncthreads();
         // |W F| <= W max(f_p (1 - f_q), (1 - f_p) f_q) summed over the block
-        const float total = s_sum[0] * s_blk[0] + s_sum[1] * s_blk[1], single = A.w_max * s_blk[2];
+        float total = s_sum[0] * s_blk[0] + s_sum[1] * s_blk[1], single = A.w_max * s_blk[2];
+        if (!(total <= 3e38f && single <= 3e38f)) {      // a weight overflows: as non-finite ones
+            if (tid == 0) atomicAdd(&H[0], __longlong_as_double(0x7ff8000000000000LL));
+            return;
+        }
+        // a small block is raised by a power of two, so that the scale stays finite
+        const float lift = total < 1e-20f ? 1.2089258e24f : 1.f;
+        total *= lift;
+        single *= lift;
+#pragma unroll
+        for (int k = 0; k < HF_QPT; ++k) {
+            fqp[k] *= lift;
+            fcqp[k] *= lift;
+        }
         const float scale = total > 0.f ? fminf(1073741824.f / total, 2097152.f / single) : 0.f;
-        const double unit = scale > 0.f ? 1.0 / (double)scale : 0.0, unit_lo = unit / (double)lo_scale;
+        const double unit = scale > 0.f ? 1.0 / ((double)scale * (double)lift) : 0.0, unit_lo = unit / (double)lo_scale;
         for (int p0 = 0; p0 < P; p0 += HF_REC) {
             const int cnt = min(HF_REC, P - p0);
             if (!one_pass) {
@@ -1507,7 +1524,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                     const float F = fmaf(rcp_approx(1.f + ex2_approx(xr * A.cT)), Bq - Aq, Aq);
                     float w = fmaf(-vab[k], z.y, z.x * v2[k]);
                     if (GL) w *= fmaf(gc[k], ck[c[k]], fmaf(gb[k], z.x, ga[k]));
-                    deposit(w * F, (xr + xqk[k]) - xp, scale);
+                    deposit(w * F, (xr + xqk[k]) - xp, scale, lift);
                 }
             }
             // the guarded pairs of this pass: where the exact patch differs from the
@@ -1541,7 +1558,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                 const float xq = (qp ? Zb : 1.f) * A.fine.xi[qq];
                 float fq, fcq;
                 sfermi(xq, A.invT, fq, fcq);
-                const float pref = Za * Zb * A.fine.w[qq];
+                const float pref = Za * Zb * A.fine.w[qq] * lift;
                 const float2 cr = __ffma2_rn(make_float2(ra.z, ra.w), make_float2(A.fine.cx[qq], A.fine.cy[qq]),
                                              __fmul2_rn(make_float2(rb.x, rb.y),
                                                         make_float2(A.fine.sx[qq], A.fine.sy[qq])));
@@ -1559,7 +1576,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                         w *= fmaf((Za + Zb) * (1.f / 6.f), ck[cc],
                                   fmaf((kza + kzb) * (1.f / 6.f), z.x, (kza * Zb + kzb * Za) * (1.f / 6.f)));
                     }
-                    deposit(u ? -(w * F) : w * F, (xr + xq) - rC[i], scale);
+                    deposit(u ? -(w * F) : w * F, (xr + xq) - rC[i], scale, lift);
                 }
             }
             __syncthreads();
@@ -1573,14 +1590,15 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                     if (LO) hs[5 * NBS + i] = 0;
                     atomicAdd(&H[i], unit * (double)v + unit_lo * (double)lo);
                 }
-                float mom = (float)unit;                         // (h/2)^moment per unit
+                float mom = scale > 0.f ? 1.f / scale : 0.f;     // (h/2)^moment per lifted unit
                 for (int mo = 1; mo < 5; ++mo) {
                     mom *= 0.5f * A.h;
                     for (int i = tid; i < A.nbins; i += HF_THR) {
                         const int v = hs[mo * NBS + i];
                         if (v == 0) continue;
                         hs[mo * NBS + i] = 0;
-                        atomicAdd(&H[(long)mo * A.nbins + i], (double)((float)v * mom));
+                        const double x = (double)((float)v * mom);
+                        atomicAdd(&H[(long)mo * A.nbins + i], lift == 1.f ? x : x / (double)lift);
                     }
                 }
                 __syncthreads();

@@ -1,5 +1,6 @@
 """Ranges of the frequency grid's fixed-point histogram (mixed precision) against
-the FP64 call, which bins alike: pole energies outside the bins."""
+the FP64 call, which bins alike: pole energies outside the bins, and weights whose sums are near
+or past the ends of FP32."""
 import numpy as np
 import pytest
 
@@ -18,3 +19,33 @@ def test_weights_above_z_max(z, sym):
     V, Z = inputs.random_vertex(N, 2.0, seed=1, c4v=sym), np.full(N, z)
     ref, got = (sigma(N, 4, 6, 0.0, 1, p, V, Z, 0.2, w) for p in (api.QPFRG_FP64, api.QPFRG_MIXED))
     assert_every_patch(got, ref)
+
+
+@pytest.mark.parametrize("e", [-50, -45, -36, -33, -30, 30, 50])
+def test_scaled_vertex(e):
+    """Sigma is quadratic in V: the histogram's scale follows the vertex, also where
+    the sum of a block's weights is near the end of FP32's range."""
+    N, w = 12, np.linspace(-3.0, 3.0, 9)
+    V, Z = inputs.random_vertex(N, 2.0, seed=4, c4v=False), inputs.z_profile(N, "aniso")
+    ref, got = (sigma(N, 5, 4, 0.0, 0, api.QPFRG_MIXED, V * s, Z, 0.2, w) for s in (1.0, 2.0 ** e))
+    assert_every_patch(got * 2.0 ** (-2 * e), ref)
+
+
+@pytest.mark.parametrize("big", [3e19, -3e19, 1e30])
+def test_overflowing_weight_is_not_finite(big):
+    """A finite entry whose square leaves FP32: its target has no finite value, the
+    others theirs."""
+    N, w = 8, np.linspace(-3.0, 3.0, 9)
+    V, Z = inputs.random_vertex(N, 2.0, seed=4, c4v=False), np.ones(N)
+    ref = sigma(N, 4, 4, 0.0, 0, api.QPFRG_MIXED, V, Z, 0.2, w)
+    V[5, 2, 3] = big
+    got = sigma(N, 4, 4, 0.0, 0, api.QPFRG_MIXED, V, Z, 0.2, w)
+    rest = np.arange(N) != 5
+    assert not np.isfinite(got[5]).any()
+    assert_every_patch(got[rest], ref[rest])
+
+
+def test_overflowing_symmetric_vertex_is_not_finite():
+    N, w = 8, np.linspace(-3.0, 3.0, 9)
+    got = sigma(N, 4, 4, 0.0, 0, api.QPFRG_MIXED, np.full((N, N, N), 2e19), np.ones(N), 0.2, w)
+    assert not np.isfinite(got).any()
