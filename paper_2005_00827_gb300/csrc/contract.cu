@@ -188,7 +188,11 @@ __global__ void __launch_bounds__(256) contract_kernel(const ContractArgs<R> A)
 
 // Channel rows outc[0 pp, 1 cr, 2 d][row][n] = the signed sums of the partial
 // rows over splits (and both products of d), in split order, so that the result
-// does not depend on the launch; then out[k1,k2,k3] = scale * (pp + cr + d): pp
+// does not depend on the launch.  Compact form: a mirror that leaves the row's pair
+// in place takes column n to an equal one up to rounding; both get the sum of the
+// lower one, so that the expanded right-hand side is C4v symmetric to the last bit (a
+// flow keeps its symmetry, and takes the same form when it is resumed from an image).
+// Then out[k1,k2,k3] = scale * (pp + cr + d): pp
 // row (k1,k2) column k3, cr row (k3,k2) column k1, d row (k1,k3) column k2.
 // Compact form: row Q = g rep at column n is the representative's at g^-1 n.
 // Two launches: an expansion that summed the splits itself read each partial
@@ -197,6 +201,7 @@ struct ExpandArgs {
     const double *part;
     double *outc;
     const int *rowmap;
+    const uint8_t *rstab;
     double *out;
     double scale;
     int N, ns, njobs;
@@ -204,31 +209,6 @@ struct ExpandArgs {
     int rows[2], splits[2];
     SymMode sym;
 };
-
-__global__ void __launch_bounds__(128) reduce_kernel(const ExpandArgs A)
-{
-    const int c = sym_compact(A.sym) ? 1 : 0, ch = blockIdx.y, nj = A.count[ch], ns = A.splits[c];
-    if (nj == 0) return;
-    const long stride = (long)A.rows[c] * A.N, per = stride * A.njobs;
-    const double *src = A.part + A.first[ch] * stride;
-    for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < stride; o += (long)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        // 16 loads in flight (one after the other they cost 18 us at 32 partial rows)
-        for (int j = 0; j < nj; ++j)
-            for (int k0 = 0; k0 < ns; k0 += 16) {
-                double t[16];
-#pragma unroll
-                for (int u = 0; u < 16; ++u) t[u] = k0 + u < ns ? __ldg(src + (k0 + u) * per + j * stride + o) : 0.0;
-                // as a tree: an FP64 add waits long for its operands
-#pragma unroll
-                for (int w = 8; w > 0; w >>= 1)
-#pragma unroll
-                    for (int u = 0; u < w; ++u) t[u] += t[u + w];
-                v += t[0];
-            }
-        A.outc[ch * stride + o] = ch < 2 ? -v : v;
-    }
-}
 
 // C4v element g on patch j (wedge part, ns shells per wedge, Na wedges)
 __device__ __forceinline__ int c4v_patch(int g, int j, int ns, int Na)
@@ -238,6 +218,36 @@ __device__ __forceinline__ int c4v_patch(int g, int j, int ns, int Na)
     int r = (g & 4) ? off - w : w + off;      // in (-Na, 2 Na)
     r = r >= Na ? r - Na : (r < 0 ? r + Na : r);
     return r * ns + sh;
+}
+
+__global__ void __launch_bounds__(128) reduce_kernel(const ExpandArgs A)
+{
+    const int c = sym_compact(A.sym) ? 1 : 0, ch = blockIdx.y, nj = A.count[ch], ns = A.splits[c];
+    if (nj == 0) return;
+    const long stride = (long)A.rows[c] * A.N, per = stride * A.njobs;
+    const double *src = A.part + A.first[ch] * stride;
+    for (long o = blockIdx.x * (long)blockDim.x + threadIdx.x; o < stride; o += (long)gridDim.x * blockDim.x) {
+        double v = 0.0;
+        long oc = o;
+        if (c) {
+            const int row = (int)(o / A.N), n = (int)(o - (long)row * A.N), s = __ldg(A.rstab + row);
+            if (s) oc = o + min(0, c4v_patch(s, n, A.ns, A.N / A.ns) - n);
+        }
+        // 16 loads in flight (one after the other they cost 18 us at 32 partial rows)
+        for (int j = 0; j < nj; ++j)
+            for (int k0 = 0; k0 < ns; k0 += 16) {
+                double t[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) t[u] = k0 + u < ns ? __ldg(src + (k0 + u) * per + j * stride + oc) : 0.0;
+                // as a tree: an FP64 add waits long for its operands
+#pragma unroll
+                for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+                    for (int u = 0; u < w; ++u) t[u] += t[u + w];
+                v += t[0];
+            }
+        A.outc[ch * stride + o] = ch < 2 ? -v : v;
+    }
 }
 
 // Block (k2, k1).
@@ -516,6 +526,7 @@ static qpfrg_status launch_simt(qpfrg_ctx *c, const R *V, double scale, double *
     E.part = c->d_partial;
     E.outc = c->d_outc;
     E.rowmap = c->d_rowmap;
+    E.rstab = c->d_rstab;
     E.out = out;
     E.scale = scale;
     E.N = N;

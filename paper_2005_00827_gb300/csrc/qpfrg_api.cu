@@ -193,7 +193,7 @@ void qpfrg_destroy(qpfrg_t c)
                         c->tc.Bpp[0], c->tc.Bpp[1], c->tc.Bcr[0], c->tc.Bcr[1], c->tc.Bd[0], c->tc.Bd[1],
                         c->tc.VT, c->d_tc_err, c->d_xij, c->d_bnd, c->d_qxl, c->d_qyl, c->d_kp, c->d_kcs, c->d_xij_f,
                         c->d_ptab, c->d_jgrid, c->d_repgrid, c->d_owngrid, c->d_lrepQ, c->d_lnimg, c->d_limg, c->d_ltask,
-                        c->d_rtab, c->d_rrep, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views, c->d_kfx, c->d_pfx, c->d_events};
+                        c->d_rtab, c->d_rrep, c->d_rstab, c->d_rowmap, c->d_rtask, c->d_outc, c->d_sym, c->d_partial, c->d_views, c->d_kfx, c->d_pfx, c->d_events};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         if (c->ev_test) cudaEventDestroy(c->ev_test);
@@ -939,13 +939,16 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
                              c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state (self-energy ODE)");
     c->c4v_state = wedge && c4v_within(c, tol);
-    // The row orbits: every precision's contraction stays within its own
-    // rounding of the unreduced one (the tensor-core flow keeps the tolerance
-    // of the state's symmetry).  The slopes of the self-energy ODE set Z, K and
-    // A, so they have to be symmetric as well.
-    const double rtol = c->opt.precision == QPFRG_FP64 ? rows_tol(c) : (c->opt.precision == QPFRG_MIXED ? 3e-7 : tol);
-    c->rows_state = c->rows_exact && c->c4v_state && (c->opt.precision == QPFRG_MIXED_TC || c4v_within(c, rtol));
-    if (c->d_gy && c->rows_state) c->rows_state = slopes_symmetric(c, Z + c->pb.N, rtol);
+    // The row orbits, as the flow that wrote the image took them: where every stage
+    // is tested on the device, left to that test; otherwise a flow's state is
+    // symmetric to the last bit (FP64 and FP32 contraction) or to the tolerance of the
+    // state's symmetry (tensor cores; there the slopes of the self-energy ODE, which set
+    // Z, K and A, to the 1e-4 of that flow).
+    c->rows_state = c->rows_exact;
+    if (c->opt.precision == QPFRG_MIXED_TC)
+        c->rows_state = c->rows_exact && c->c4v_state && (!c->d_gy || slopes_symmetric(c, Z + c->pb.N, 1e-4));
+    else if (!stage_tested(c))
+        c->rows_state = c->rows_exact && c4v_within(c, c->opt.precision == QPFRG_FP64 ? rows_tol(c) : 3e-7);
     c->status = hd.status;
     c->steps = (int)hd.steps;
     c->lambda = hd.lambda;

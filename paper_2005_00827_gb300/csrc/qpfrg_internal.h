@@ -311,6 +311,7 @@ struct qpfrg_ctx {
     int n_rrep = 0, n_rcan = 0;
     int *d_rrep = nullptr;       // [family][row]: Q of each representative row
     int *d_rowmap = nullptr;     // [family][Q]: row | g << 24, Q = g rep
+    uint8_t *d_rstab = nullptr;  // [row]: the mirror (4 .. 7) that leaves its pair in place, 0: none
     int4 *d_rtask = nullptr;     // (family, patch, first representative, count) per loop-kernel CTA
     int rtask_qchunk = 0, n_rtask = 0;
     double *d_outc = nullptr;    // [channel][representative][n] contraction rows
@@ -396,13 +397,18 @@ inline double rows_tol(const qpfrg_ctx *c) { return c->opt.precision == QPFRG_FP
 // self-energies that evaluate every patch, the zone-edge patches differ by what
 // the wedge decision of momenta on |k| = pi does (1e-7 .. 1e-5): the stage's test
 // decides on the device, in FP32 within the rounding of its right-hand side.
+inline bool stage_tested(const qpfrg_ctx *c)
+{
+    return c->opt.precision != QPFRG_MIXED_TC &&
+           (c->opt.sigma_ode || (c->opt.precision == QPFRG_FP64 && c->opt.z_feedback));
+}
 inline SymMode state_form(const qpfrg_ctx *c)
 {
     SymMode s;
     if (!c->rows_ok || !c->rows_state) return s;
     s.mode = 1;
+    if (!stage_tested(c)) return s;
     const bool fp64 = c->opt.precision == QPFRG_FP64;
-    if (c->opt.precision == QPFRG_MIXED_TC || !(c->opt.sigma_ode || (fp64 && c->opt.z_feedback))) return s;
     s.mode = 2;
     s.red = c->d_sym;
     s.tol = (fp64 ? rows_tol(c) : 1e-6) / 3.0;

@@ -139,14 +139,21 @@ static qpfrg_status build_row_orbits(qpfrg_ctx *c, bool exch, const std::vector<
             }
         for (int m = npar + (int)norb; m < ncan; ++m) map[rep[m]] = m;
     }
+    std::vector<uint8_t> stab(nr, 0);      // the same in both families; rows of their own have no images
+    for (int m = 0; m < nr; ++m)
+        for (int g = 4; g < 8 && (m < npar + (int)norb || m >= ncan); ++g)
+            if (c4v_apply(g, reps[m] / N, N, ns) == reps[m] / N && c4v_apply(g, reps[m] % N, N, ns) == reps[m] % N)
+                stab[m] = (uint8_t)g;
     cudaError_t e;
     if ((e = cudaMalloc((void **)&c->d_rrep, 2 * (size_t)nr * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc((void **)&c->d_rstab, nr)) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_rowmap, 2 * NN * sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_rtask, (2L * N * ((ncan + 7) / 8) + 8) * sizeof(int4))) != cudaSuccess ||
         (c->opt.precision == QPFRG_MIXED_TC &&
          (e = cudaMalloc((void **)&c->d_outc, 3L * nr * N * sizeof(double))) != cudaSuccess))
         return cuda_fail(c, e, "cudaMalloc(row orbits)");
     e = cudaMemcpy(c->d_rrep, reps.data(), reps.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_rstab, stab.data(), nr, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_rowmap, rowmap.data(), 2 * NN * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(c, e, "upload row orbits");
     c->n_rrep = nr;
