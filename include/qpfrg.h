@@ -209,7 +209,7 @@ qpfrg_status qpfrg_rhs(qpfrg_t ctx, double lambda, const double *d_V, const doub
  * d_sigma_re/d_sigma_im: N x n_omega FP64 outputs (may be NULL when
  * n_omega == 0; the frequency grid is binned, see the design notes);
  * d_Z_out: N FP64 output (may be NULL).  In wedge mode V and Z are tested for
- * C4v symmetry on the device (1e-6 of the maxima for Z and 1e-5 for the grid,
+ * C4v symmetry on the device (1e-12 of the maxima for Z and 1e-5 for the grid,
  * FP64 Z 1e-14; FP64 evaluates the grid at every patch): a symmetric input
  * evaluates the targets that differ under C4v, and images whose momenta on a
  * wedge boundary are decided otherwise than their representative's get that

@@ -948,7 +948,7 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     if (c->opt.precision == QPFRG_MIXED_TC)
         c->rows_state = c->rows_exact && c->c4v_state && (!c->d_gy || slopes_symmetric(c, Z + c->pb.N, 1e-4));
     else if (!stage_tested(c))
-        c->rows_state = c->rows_exact && c4v_within(c, c->opt.precision == QPFRG_FP64 ? rows_tol(c) : 3e-7);
+        c->rows_state = c->rows_exact && c4v_within(c, rows_tol(c));
     c->status = hd.status;
     c->steps = (int)hd.steps;
     c->lambda = hd.lambda;

@@ -389,14 +389,14 @@ qpfrg_status upload_geometry(qpfrg_ctx *c);
 // orbits), kept in c->rhs_sym for the contraction of the same RHS.
 qpfrg_status launch_bubbles(qpfrg_ctx *c, double lambda, const double *d_Z, bool z_symmetric,
                             const double *d_K, const SymMode &sym);
-// tolerance of the C4v test that admits the row orbits, relative to the
-// maxima: a few roundings of the precision that computes the right-hand side
-// (an input asymmetry enters its result at first order)
+// tolerance of the C4v test that admits the row orbits and the reduced targets,
+// relative to the maxima: an input asymmetry enters the result at first order, and
+// what is dropped stays below the rounding of the precision that computes it
 inline double rows_tol(const qpfrg_ctx *c) { return c->opt.precision == QPFRG_FP64 ? 1e-14 : 1e-12; }
 // the form of a right-hand side of the flow state.  Where the weights come from
 // self-energies that evaluate every patch, the zone-edge patches differ by what
-// the wedge decision of momenta on |k| = pi does (1e-7 .. 1e-5): the stage's test
-// decides on the device, in FP32 within the rounding of its right-hand side.
+// the wedge decision of momenta on |k| = pi does (1e-9 .. 1e-5): the stage's test
+// decides on the device.
 inline bool stage_tested(const qpfrg_ctx *c)
 {
     return c->opt.precision != QPFRG_MIXED_TC &&
@@ -408,10 +408,9 @@ inline SymMode state_form(const qpfrg_ctx *c)
     if (!c->rows_ok || !c->rows_state) return s;
     s.mode = 1;
     if (!stage_tested(c)) return s;
-    const bool fp64 = c->opt.precision == QPFRG_FP64;
     s.mode = 2;
     s.red = c->d_sym;
-    s.tol = (fp64 ? rows_tol(c) : 1e-6) / 3.0;
+    s.tol = rows_tol(c) / 3.0;
     return s;
 }
 

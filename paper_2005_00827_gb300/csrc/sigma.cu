@@ -2235,9 +2235,10 @@ static qpfrg_status launch_z_update(qpfrg_ctx *c, const SigmaTargets &tg, double
 }
 
 // Tolerance, relative to the largest magnitudes, of the C4v test that admits the
-// reduced targets: an asymmetry enters the chord slope at first order (FP32 sums
-// carry 1e-6); the frequency grid's own accuracy is 3e-5.
-constexpr double kTolZ = 1e-6, kTolGrid = 1e-5;
+// reduced targets of the temperature flow's frequency grid, whose own accuracy is
+// 3e-5 (Z, the slopes and the interaction flow's grid, which is integrated: rows_tol,
+// so that no difference of an input above rounding is dropped).
+constexpr double kTolGrid = 1e-5;
 
 // state_symmetric: (V, Z) is the flow's state, symmetric by construction
 // (irreducible targets, halved on the mirror lines).
@@ -2263,7 +2264,7 @@ qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const dou
     if (c->d_ptab) {
         const bool fp64 = c->opt.precision == QPFRG_FP64;
         if (!tg.jlist) {
-            tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, c->d_sym_v);
+            tg = device_targets(c, rows_tol(c), c->d_sym_v);
             if (tg.sym.mode == 2 && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         }
         s = fp64 ? launch_sigma64(c, T, d_V, d_Z, nullptr, tg) : launch_sigma_fast(c, T, d_V, d_Z, nullptr, tg);
@@ -2296,7 +2297,7 @@ qpfrg_status launch_sigma_lines(qpfrg_ctx *c, double T, const double *d_V, const
     qpfrg_status s;
     if (c->d_ptab) {
         const bool fp64 = c->opt.precision == QPFRG_FP64;
-        tg = device_targets(c, fp64 ? rows_tol(c) : kTolZ, c->d_sym);
+        tg = device_targets(c, rows_tol(c), c->d_sym);
         s = fp64 ? launch_sigma64(c, T, d_V, d_Z, d_K, tg) : launch_sigma_fast(c, T, d_V, d_Z, d_K, tg);
     } else if (c->opt.precision == QPFRG_FP64) {
         SigmaArgs<double> A;
@@ -2359,7 +2360,7 @@ qpfrg_status launch_sigma_grid(qpfrg_ctx *c, double T, const double *d_V, const 
     if (c->opt.precision != QPFRG_FP64 && c->d_ptab && hist_variant(nbins) >= 0) {
         // FP32 wedge grid: table projection, histogram in shared memory; a
         // C4v-symmetric (V, Z) needs only the irreducible and zone-edge targets
-        tg = device_targets(c, kTolGrid, d_K ? c->d_sym : c->d_sym_v);
+        tg = device_targets(c, d_K ? rows_tol(c) : kTolGrid, d_K ? c->d_sym : c->d_sym_v);
         if (tg.sym.mode == 2 && !d_K && (s = launch_sym_test(c, d_V, d_Z, 1, c->d_sym_v)) != QPFRG_OK) return s;
         s = launch_sigma_hist(c, T, d_V, d_Z, d_K, tg, c->d_hist, e_min, h, nbins);
     } else if (c->opt.precision == QPFRG_FP64 && c->d_ptab) {
