@@ -54,6 +54,24 @@ __global__ void rk_final_kernel(double h, double *__restrict__ V, const double *
     reduce_max_flag(m, bad, red);
 }
 
+// Every image of a state under C4v (wedge w -> +-w + m N_a/4 of patch j = w ns + s, the
+// shell s kept): sets *flag where one differs by more than tv (V) or tz (Z).
+__global__ void state_images_kernel(const double *__restrict__ V, const double *__restrict__ Z, int N, int ns, double tv,
+                                    double tz, unsigned long long *flag)
+{
+    const long NN = (long)N * N;
+    bool bad = false;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < NN * N; i += (long)gridDim.x * blockDim.x) {
+        const int k1 = (int)(i / NN), k2 = (int)(i / N % N), k3 = (int)(i % N);
+        for (int g = 1; g < 8; ++g) {
+            auto at = [&](int k) { return (long)c4v_apply(g, k, N, ns); };
+            bad = bad || fabs(V[(at(k1) * N + at(k2)) * N + at(k3)] - V[i]) > tv;
+            if (i < N) bad = bad || fabs(Z[at((int)i)] - Z[i]) > tz;
+        }
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1ull);
+}
+
 static int grid_for(long n)
 {
     long b = (n + 255) / 256;
@@ -70,6 +88,17 @@ qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_
     prof_end(c, K_RK_STAGE);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "rk_stage_kernel");
+}
+
+qpfrg_status launch_state_images(qpfrg_ctx *c, const double *d_V, const double *d_Z, double tv, double tz,
+                                 unsigned long long *flag)
+{
+    cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(*flag), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "memset state images");
+    state_images_kernel<<<grid_for((long)c->pb.N * c->pb.N * c->pb.N), 256, 0, c->stream>>>(d_V, d_Z, c->pb.N, c->pb.n_shell,
+                                                                                         tv, tz, flag);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "state_images_kernel");
 }
 
 qpfrg_status launch_rk_final(qpfrg_ctx *c, double h, double *d_V, const double *d_acc, const double *d_k)

@@ -929,6 +929,19 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     if (c->h_red[9]) return set_err(c, QPFRG_ERR_NONFINITE, "state image holds NaN or Inf");
     double m = 0.0;
     std::memcpy(&m, &c->h_red[5], sizeof(double));
+    // symmetric: every image within tol.  The generators decide that below a third of
+    // it and above it; between the two every image is looked at
+    bool sym = wedge && c4v_within(c, tol);
+    if (wedge && !sym && c4v_within(c, 3.0 * tol)) {
+        double mz;
+        std::memcpy(&mz, &c->h_red[7], sizeof(double));
+        if ((st = launch_state_images(c, c->d_k, c->d_acc, tol * m, tol * mz, c->d_sym_v + 4)) != QPFRG_OK) return st;
+        if ((e = cudaMemcpyAsync(&c->h_red[9], c->d_sym_v + 4, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                 c->stream)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
+            return cuda_fail(c, e, "set_state symmetry check");
+        sym = c->h_red[9] == 0;
+    }
     if ((e = cudaMemcpyAsync(c->d_V, c->d_k, n3_of(c) * sizeof(double), cudaMemcpyDeviceToDevice, c->stream)) !=
             cudaSuccess ||
         (e = cudaMemcpyAsync(c->d_Z, c->d_acc, c->pb.N * sizeof(double), cudaMemcpyDeviceToDevice, c->stream)) !=
@@ -938,7 +951,7 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
         (e = cudaMemcpyAsync(c->d_gy, Z + c->pb.N, gflow_small_len(c) * sizeof(double), cudaMemcpyHostToDevice,
                              c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state (self-energy ODE)");
-    c->c4v_state = wedge && c4v_within(c, tol);
+    c->c4v_state = sym;
     // The row orbits, as the flow that wrote the image took them: where every stage
     // is tested on the device, left to that test; otherwise a flow's state is
     // symmetric to the last bit (FP64 and FP32 contraction) or to the tolerance of the

@@ -501,6 +501,9 @@ qpfrg_status launch_tc_fused(qpfrg_ctx *c, int ch, double scale, double *out, do
 // ode.cu
 qpfrg_status launch_rk_stage(qpfrg_ctx *c, int stage, double h, const double *d_V,
                              const double *d_k, double *d_acc, double *d_Vs, float *d_Vf);
+// *flag (device) set where an image of (V, Z) under C4v differs by more than tv, tz
+qpfrg_status launch_state_images(qpfrg_ctx *c, const double *d_V, const double *d_Z, double tv, double tz,
+                                 unsigned long long *flag);
 qpfrg_status launch_rk_final(qpfrg_ctx *c, double h, double *d_V, const double *d_acc,
                              const double *d_k);
 

@@ -48,3 +48,19 @@ def test_interaction_flow(N, nt, nr, prec):
     for (va, ra), (vb, rb) in zip(one, two):
         assert ra == rb
         assert np.abs(va - vb).max() < 1e-6 * np.abs(va).max()
+
+
+@pytest.mark.parametrize("off,sym", [(0.2e-5, True), (0.7e-5, True), (0.95e-5, True), (1.2e-5, False), (4e-5, False)])
+@pytest.mark.parametrize("entry", [(1, 2, 3), (0, 5, 5)])
+def test_image_symmetric_to_the_stated_tolerance(entry, off, sym):
+    """A tensor-core state counts as symmetric while every image is within 1e-5 of the
+    largest entry, also where a single generator moves an entry by more than a third."""
+    N = 16
+    with api.Context(N, 4, 4, U=2.0, precision=api.QPFRG_MIXED_TC) as c:
+        img = bytearray(api.qpfrg_get_state(c.h))
+        V = inputs.random_vertex(N, 2.0, seed=3)
+        V[entry] += off * np.abs(V).max()
+        img[64:] = np.concatenate([V.ravel(), np.ones(N)]).tobytes()
+        api.qpfrg_set_state(c.h, bytes(img))
+        api.qpfrg_step(c.h, 1)
+        assert (api.qpfrg_rhs_work(c.h)["contraction_rows"] < N * N) == sym
