@@ -283,7 +283,8 @@ qpfrg_status qpfrg_get_state(qpfrg_t ctx, void *h_buf, size_t bytes);
  * page-locked memory preferred).  The image is uploaded into scratch space and
  * checked on the device (finiteness, max|V|, C4v symmetry of the state, which
  * selects the self-energy's irreducible targets and the row orbits);
- * synchronises the context's stream.  Returns QPFRG_ERR_INVALID on a wrong header or size,
+ * synchronises the context's stream, after which h_buf has been read (it may be
+ * reused or freed on return).  Returns QPFRG_ERR_INVALID on a wrong header or size,
  * QPFRG_ERR_NONFINITE (state unchanged) when V or Z holds NaN/Inf.  Between
  * steps only (it reuses the RK scratch buffers). */
 qpfrg_status qpfrg_set_state(qpfrg_t ctx, const void *h_buf, size_t bytes);

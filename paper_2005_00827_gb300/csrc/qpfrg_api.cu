@@ -919,6 +919,10 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     cudaError_t e = cudaMemcpyAsync(c->d_k, V, n3_of(c) * sizeof(double), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->d_acc, Z, c->pb.N * sizeof(double), cudaMemcpyHostToDevice, c->stream);
+    // (the self-energy ODE's part as well, before the wait below: the caller may reuse
+    // a page-locked image as soon as this call returns)
+    if (e == cudaSuccess && c->d_gy)
+        e = cudaMemcpyAsync(c->d_gys, Z + c->pb.N, gflow_small_len(c) * sizeof(double), cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "set_state upload");
     qpfrg_status st = launch_sym_test(c, c->d_k, c->d_acc, 1, c->d_sym_v);
     if (st != QPFRG_OK) return st;
@@ -948,7 +952,7 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
             cudaSuccess)
         return cuda_fail(c, e, "set_state");
     if (c->d_gy &&
-        (e = cudaMemcpyAsync(c->d_gy, Z + c->pb.N, gflow_small_len(c) * sizeof(double), cudaMemcpyHostToDevice,
+        (e = cudaMemcpyAsync(c->d_gy, c->d_gys, gflow_small_len(c) * sizeof(double), cudaMemcpyDeviceToDevice,
                              c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "set_state (self-energy ODE)");
     c->c4v_state = sym;
