@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(256) sigma_kernel(SigmaArgs<R> A)
 constexpr int SF_QPT = 2;
 constexpr int SF_QB = 4;        // default blocks of 256 SF_QPT loop points q per CTA
 constexpr int SF_PCH = 1024;    // loop points p staged per pass
-constexpr int SF_QCAP = 1024;   // guarded pairs queued per pass
+constexpr int SF_QCAP = 896;    // guarded pairs queued per pass (two CTAs per SM, see sf_smem_layout)
 constexpr int SF_SLOTS = 257;   // per-patch slots: c in 0..N (c = N is patch 0 again), padded to 257
 
 struct SigmaFastArgs {
@@ -637,9 +637,9 @@ struct SfSmem {
 };
 
 // (a launch that reads the patch table has no use for the queue)
-__host__ __device__ inline SfSmem sf_smem_layout(int pch, bool rt)
+__host__ __device__ constexpr SfSmem sf_smem_layout(int pch, bool rt)
 {
-    SfSmem L;
+    SfSmem L{};
     L.rA = 0;                                  // pch + 1 records: room for a pad record
     L.rB = L.rA + (size_t)16 * (pch + 1);
     L.cz = L.rB + (size_t)16 * (pch + 1);
@@ -652,6 +652,10 @@ __host__ __device__ inline SfSmem sf_smem_layout(int pch, bool rt)
     L.total = rt ? L.queue : L.ck + (size_t)4 * SF_SLOTS;
     return L;
 }
+// Two CTAs per SM at the longest pass (32 x 32 points): each takes its layout, 256
+// bytes of static shared memory and the 1 KB that the SM reserves.  A queue of 1024
+// pairs left one CTA: Z of an unsymmetric vertex, np48, 32 x 32, 149 -> 197 ms.
+static_assert(2 * (sf_smem_layout(SF_PCH, false).total + 256 + 1024) <= 228 * 1024, "two CTAs per SM");
 
 // Patch of r for a lane that left the table path: near a ray or the origin
 // (float-float ray tests) or near the zone edge.  There the FP64 fold decides: its
