@@ -1113,8 +1113,10 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                     // taken by the whole warp (a branch per lane left the lanes apart
                     // for the rest of the unrolled trip: 84 instead of 40 issue slots
                     // per pair); one copy of the code for the four pairs
+                    unsigned todo = __reduce_or_sync(0xffffffffu, slow_mask);
 #pragma unroll 1
-                    for (int e = 0; e < 2 * SF_QPT; ++e) {
+                    for (; todo; todo &= todo - 1) {
+                        const int e = __ffs(todo) - 1;
                         const bool r1 = e >= SF_QPT, k1 = (e & 1) != 0;
                         bool slow;
                         const int cc = fx_zoom(__float_as_int(r1 ? ra[1].x : ra[0].x), __float_as_int(r1 ? ra[1].y : ra[0].y),
