@@ -404,11 +404,6 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
             return fail(s);
         cudaMemcpy(c->d_jirr, jirr.data(), jirr.size() * sizeof(int), cudaMemcpyHostToDevice);
         cudaMemcpy(c->d_rep, rep.data(), N * sizeof(int), cudaMemcpyHostToDevice);
-        if (c->d_ptab) {
-            // boundary pairs of the reduced self-energies: eight per loop point and target
-            c->max_events = (unsigned)std::min<long>(1L << 21, 8L * pb.M * c->n_irr);
-            if ((s = dev_alloc(c, &c->d_events, c->max_events, "boundary pairs")) != QPFRG_OK) return fail(s);
-        }
         if (pb.mode == QPFRG_GRID_WEDGE) {
             // frequency grid of the wedge kernels: zone-edge patches j = m N/4
             // get slots of their own
@@ -432,6 +427,7 @@ qpfrg_status qpfrg_create(const qpfrg_lattice *lattice, int n_p, const qpfrg_fin
             cudaMemcpy(c->d_owngrid, own.data(), N * sizeof(int), cudaMemcpyHostToDevice);
             cudaMemcpy(c->d_jgrid, jgrid.data(), jgrid.size() * sizeof(int), cudaMemcpyHostToDevice);
             cudaMemcpy(c->d_repgrid, repgrid.data(), N * sizeof(int), cudaMemcpyHostToDevice);
+            if ((s = sigma_plan(c)) != QPFRG_OK) return fail(s);
         }
     }
 

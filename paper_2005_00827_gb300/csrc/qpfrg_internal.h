@@ -338,7 +338,7 @@ struct qpfrg_ctx {
     double *d_gzka = nullptr, *d_gt2 = nullptr;
     double *d_sig = nullptr;     // chord slopes per target slot, per patch, corrections, slopes of every patch (N each), count of d_events
     int4 *d_events = nullptr;    // pairs on a boundary between patches (sigma.cu)
-    unsigned max_events = 0;
+    unsigned max_events = 0;     // room for them; 0: every patch is summed (sigma_plan)
     int *d_jirr = nullptr;       // C4v-irreducible patches 0..N/8 (wedge mode)
     int *d_rep = nullptr;        // slot of each patch's representative in d_jirr
     int n_irr = 0;
@@ -432,6 +432,7 @@ qpfrg_status launch_stage_views(qpfrg_ctx *c, const void *d_Vin, const double *d
 qpfrg_status launch_contractions(qpfrg_ctx *c, const void *d_Vin, double scale, double *d_out);
 
 // sigma.cu
+qpfrg_status sigma_plan(qpfrg_ctx *c);     // whether reduced targets pay, once per context
 qpfrg_status launch_sigma_z(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z,
                             double *d_Zout, bool state_symmetric);
 // d_K: the interaction flow's line weights with these Katanin factors (the

@@ -515,6 +515,7 @@ struct SigmaFastArgs {
     const double *xi64, *w64, *xij64;   // dispersion and weight of the fine points, xi(k_F(j))
     double T64;
     double fold0, fold1;    // last doubles k with rint(k / 2 pi) = 0 and < 2
+    double dth64;           // 2 pi / N
     const float4 *kp, *kcs, *bnd;
     const int2 *kfx, *pfx;  // k_j + p and the fine points in fixed point
     const uint8_t *ptab;
@@ -709,7 +710,10 @@ __device__ __noinline__ int sf_slow_patch(const SigmaFastArgs &A, int j, int p, 
     int jc;
     rint_add(atan2_poly(yh, xh) * A.inv_dth, jc);
     int c = rays_ff(xh, xl, yh, yl, jc, N, bnd, margin);
-    if (margin < 1e-11f) c = project_fp64(kx, ky, A.pb);
+    if (margin < 1e-11f) {       // project_fp64 of the folded momentum
+        c = (int)floor(atan2(fy, fx) / A.dth64 + 0.5);
+        c = c < 0 ? c + N : (c >= N ? c - N : c);
+    }
     if (fminf(fminf(fabsf(ex), fabsf(ey)), margin) < 1e-9f) record(c);
     return c;
 }
@@ -772,6 +776,32 @@ __global__ void __launch_bounds__(128) sigma_fix_kernel(SigmaFastArgs A, double 
                 atomicAdd(&A.corr[jg], amp * (eta2 - dp * dm) / ((dp * dp + eta2) * (dm * dm + eta2)));
             }
         }
+    }
+}
+
+// Number of boundary pairs among n pairs of the list's targets, every pair
+// (stride 1) or a sample: *A.nevents (sigma_plan).
+__global__ void boundary_count_kernel(const SigmaFastArgs A, unsigned n, unsigned long long stride)
+{
+    const unsigned long long M = A.pb.M, all = M * M * A.n_list;
+    const unsigned char *tabc = A.ptab + (kProjW / 2) * (kProjStride + 1);   // the cell of the origin
+    __shared__ float2 ray[SF_SLOTS];
+    for (int i = threadIdx.x; i < SF_SLOTS; i += blockDim.x) {
+        const float4 bd = A.bnd[i < A.pb.N ? i : 0];
+        ray[i] = i <= A.pb.N ? make_float2(bd.x, bd.z) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned long long k = i * stride % all;
+        const int q = (int)(k % M), p = (int)(k / M % M), j = A.jlist[k / M / M];
+        if ((4 * j) % A.pb.N == 0) continue;
+        const int2 kp = A.kfx[(long)j * A.pb.M + p], kq = A.pfx[q];
+        float x, y;
+        bool slow;
+        fx_patch(kp.x, kp.y, kq.x, kq.y, tabc, ray, x, y, slow);
+        if (slow) fx_zoom(kp.x, kp.y, kq.x, kq.y, tabc, ray, slow);
+        const bool edge = fmaxf(fabsf(x), fabsf(y)) > kFxEdge;
+        if (slow) sf_slow_patch(A, j, p, q, x * kRadPerFx, y * kRadPerFx, edge ? 3 : 2, A.bnd);
     }
 }
 
@@ -1086,9 +1116,17 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             // every iteration, 40 % of the time);
             // an odd count reads the zero-weight pad record after the last one;
             // the loop is unrolled four times (eight records per trip, 122
-            // registers: the loop overhead amortised, more independent work)
+            // registers: the loop overhead amortised, more independent work).
+            // The queue is settled after a chunk of records that leaves it a quarter
+            // full, and at the end of the pass.  A chunk is 16 records, then four times
+            // the last while few pairs are queued: where the lattice's mirror lies on a
+            // boundary (N = 4 mod 8) up to 6 % of the pairs are exact ties, which a queue
+            // per pass could not hold: N = 60, 10 x 14 points, 55 ms against 8.5 without.
+            int sub = 16, kept = 0, settled = 0;
+            for (int i0 = 0; i0 < cnt;) {
+            const int i1 = min(cnt, i0 + sub);
 #pragma unroll 4
-            for (int i = 0; i < cnt; i += 2) {
+            for (int i = i0; i < i1; i += 2) {
                 float4 ra[2], rb[2];
                 float upp[2];
 #pragma unroll
@@ -1136,16 +1174,21 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                 }
                 pair_math(ra, rb, upp, c);
             }
-            // the guarded pairs of this pass: where the exact patch differs from the
-            // table's, the difference of the two chord terms
+            // the guarded pairs: where the exact patch differs from the table's, the
+            // difference of the two chord terms
             __syncthreads();
             const int nq = s_nq;
             __syncthreads();
+            const int added = nq - kept, nrec = i1 - settled;
+            sub = added > SF_QCAP / 4 ? max(16, sub / 4) : (added < 16 ? min(SF_PCH, 4 * sub) : sub);
+            kept = nq;
+            i0 = i1;
+            if (i1 < cnt && nq <= SF_QCAP / 4) continue;     // uniform over the CTA
             if (tid == 0) s_nq = 0;
             const bool over = nq > SF_QCAP;      // more than the queue holds: look at every pair again
-            const int ntot = over ? cnt * (256 * SF_QPT) : nq;
+            const int ntot = over ? nrec * (256 * SF_QPT) : nq;
             for (int e = tid; e < ntot; e += 256) {
-                const unsigned en = over ? (unsigned)(e % cnt) | (unsigned)(e / cnt) << 12 : queue[e];
+                const unsigned en = over ? (unsigned)(settled + e % nrec) | (unsigned)(e / nrec) << 12 : queue[e];
                 const int i = en & 4095u, iq = blk * (256 * SF_QPT) + (int)(en >> 12);
                 if (iq >= M) continue;
                 const int b = iq / PP, rem = iq - b * PP;
@@ -1191,6 +1234,9 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                 }
             }
             __syncthreads();
+            kept = 0;
+            settled = i1;
+            }
             }
         }
         vsum -= (double)acc.x + (double)acc.y;   // the chord term is -u / den
@@ -1495,8 +1541,12 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                 stage(p0, cnt);
                 __syncthreads();
             }
+            // the queue is settled in chunks, as in sigma_fast_kernel
+            int sub = 8, kept = 0, settled = 0;
+            for (int i0 = 0; i0 < cnt;) {
+            const int i1 = min(cnt, i0 + sub);
 #pragma unroll 2
-            for (int i = 0; i < cnt; ++i) {
+            for (int i = i0; i < i1; ++i) {
                 const float4 ra = rA[i], rb = rB[i];
                 const float xp = rC[i];
                 int c[HF_QPT];
@@ -1533,17 +1583,22 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                     deposit(w * F, (xr + xqk[k]) - xp, scale, lift);
                 }
             }
-            // the guarded pairs of this pass: where the exact patch differs from the
-            // table's, its contribution is taken out (the same rounded addends) and
-            // the right one put in
+            // the guarded pairs: where the exact patch differs from the table's, its
+            // contribution is taken out (the same rounded addends) and the right one
+            // put in
             __syncthreads();
             const int nq = s_nq;
             __syncthreads();
+            const int added = nq - kept, nrec = i1 - settled;
+            sub = added > HF_QCAP / 4 ? max(8, sub / 4) : (added < 16 ? 4 * sub : sub);
+            kept = nq;
+            i0 = i1;
+            if (i1 < cnt && nq <= HF_QCAP / 4) continue;     // uniform over the CTA
             if (tid == 0) s_nq = 0;
             const bool over = nq > HF_QCAP;      // more than the queue holds: look at every pair again
-            const int ntot = over ? cnt * (HF_THR * HF_QPT) : nq;
+            const int ntot = over ? nrec * (HF_THR * HF_QPT) : nq;
             for (int e = tid; e < ntot; e += HF_THR) {
-                const unsigned en = over ? (unsigned)(e % cnt) | (unsigned)(e / cnt) << 12 : queue[e];
+                const unsigned en = over ? (unsigned)(settled + e % nrec) | (unsigned)(e / nrec) << 12 : queue[e];
                 const int i = en & 4095u, qq = blk * (HF_THR * HF_QPT) + (int)(en >> 12);
                 if (qq >= M) continue;
                 const float4 ra = rA[i], rb = rB[i];
@@ -1586,6 +1641,9 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                 }
             }
             __syncthreads();
+            kept = 0;
+            settled = i1;
+            }
             // without the second word the rounding of moment 0 is kept small by
             // flushing after every pass
             if (!LO || p0 + HF_REC >= P) {
@@ -1938,7 +1996,7 @@ static SigmaTargets device_targets(const qpfrg_ctx *c, double tol, const unsigne
 {
     SigmaTargets t;
     t.n = c->pb.N;
-    if (!c->d_jgrid) return t;
+    if (!c->max_events) return t;
     t.jlist = c->d_jgrid;
     t.n = c->n_grid;
     t.rep = c->d_repgrid;
@@ -2011,7 +2069,46 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     static const double fold0 = fold_limit(0), fold1 = fold_limit(1);
     A.fold0 = fold0;
     A.fold1 = fold1;
+    A.dth64 = kTwoPi / c->pb.N;
     return A;
+}
+
+// Once per context: whether the reduced targets pay.  A boundary pair costs
+// corrections of up to seven images in FP64 (7.5 ns, as long as the sums of 1800 FP32 or
+// 85 FP64 pairs), so the list is used where the pairs that it saves cost twice that;
+// the record of pairs is sized for them.  Generic grids have few; with N = 4 mod 8, mu
+// and t' = 0 the lattice's mirror is a boundary between wedges and up to 6 % of the
+// pairs lie on it: every patch is summed.  Counted where there are at most 2^22 pairs,
+// else estimated from a sample (0.1 % of 2^22 to 1.5 %).
+qpfrg_status sigma_plan(qpfrg_ctx *c)
+{
+    c->max_events = 0;
+    if (!c->d_ptab || !c->d_jgrid) return QPFRG_OK;
+    qpfrg_status s = launch_kp_table(c, nullptr, c->pb.N);
+    if (s != QPFRG_OK) return s;
+    SigmaTargets tg;
+    tg.jlist = c->d_jgrid;
+    tg.n = c->n_grid;
+    SigmaFastArgs A = fast_args(c, 1.0, nullptr, nullptr, nullptr, tg);
+    const double M = c->pb.M, all = M * M * c->n_grid;
+    const double n = std::fmin(all, 4194304.0);
+    // an odd stride near the golden section of all pairs spreads the sample evenly
+    const unsigned long long stride = n < all ? (unsigned long long)(0.6180339887498949 * all) | 1ull : 1ull;
+    cudaError_t e = cudaMemsetAsync(A.nevents, 0, sizeof(unsigned), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "memset boundary pairs");
+    boundary_count_kernel<<<152 * 4, 256, 0, c->stream>>>(A, (unsigned)n, stride);
+    unsigned found = 0;
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&found, A.nevents, sizeof(found), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
+        return cuda_fail(c, e, "boundary pairs");
+    const double pairs = found * (all / n), worth = c->opt.precision == QPFRG_FP64 ? 170.0 : 3600.0;
+    const double cap = std::fmin(1.25 * pairs + 4096.0, 2097152.0);
+    if (pairs * worth > (c->pb.N - c->n_grid) * M * M) return QPFRG_OK;
+    if ((e = cudaMalloc((void **)&c->d_events, (size_t)cap * sizeof(int4))) != cudaSuccess)
+        return cuda_fail(c, e, "cudaMalloc(boundary pairs)");
+    c->max_events = (unsigned)cap;
+    return QPFRG_OK;
 }
 
 // Chord slopes of the target slots into d_sig (FP32, wedge grid).
