@@ -1279,7 +1279,8 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
 //
 // Launch: grid (q splits, N patches a, targets), 512 threads, one CTA per SM
 // (the histogram).  NBS: words per moment (a constant, so that the moments are
-// immediate offsets), nbins <= NBS.
+// immediate offsets), nbins <= NBS.  HALF: nbins <= 2 NBS, each half of the bins by
+// CTAs of its own that walk every pair (even and odd blockIdx.x).
 constexpr int HF_THR = 512;
 constexpr int HF_QPT = 2;
 constexpr int HF_REC = 256;     // loop points p staged per pass
@@ -1289,9 +1290,9 @@ struct HfSmem {
     size_t rA, rB, cz, ray, cd, ck, wb, rC, queue, tab, hist, total;
 };
 
-__host__ __device__ inline HfSmem hf_smem_layout(int nbs, bool lo)
+__host__ __device__ constexpr HfSmem hf_smem_layout(int nbs, bool lo)
 {
-    HfSmem L;
+    HfSmem L{};
     L.rA = 0;
     L.rB = L.rA + (size_t)16 * HF_REC;
     L.cz = L.rB + (size_t)16 * HF_REC;
@@ -1321,7 +1322,7 @@ __device__ __noinline__ void hist_outside(const SigmaFastArgs &A, double *H, dou
     for (int mo = 0; mo < 5; ++mo, m *= d) atomicAdd(H + (long)mo * A.nbins + bin, m);
 }
 
-template <int NBS, bool LO, bool GL>
+template <int NBS, bool LO, bool GL, bool HALF>
 __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastArgs A)
 {
     const int N = A.pb.N, M = A.pb.M, PP = A.pb.P;
@@ -1391,6 +1392,9 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     }
     __syncthreads();
     double *H = A.hist + (long)jidx * 5 * A.nbins;
+    // the bins bin0 .. bin0 + nb - 1 of this CTA
+    const bool upper = HALF && (blockIdx.x & 1);
+    const int bin0 = upper ? NBS : 0, nb = HALF ? (upper ? A.nbins - NBS : NBS) : A.nbins;
     if (s_bad) {       // a non-finite vertex or weight: as in the sums, every frequency of this target
         if (tid == 0) atomicAdd(&H[0], __longlong_as_double(0x7ff8000000000000LL));
         return;
@@ -1430,9 +1434,9 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
         int r;                                           // (past +-2^22: no bin either)
         const float rr = rint_add(fmaf(E, A.inv_h, A.c_frac), r);
         const float d = 2.f * (fmaf(E, A.inv_h, -rr) + fmaf(E, A.inv_h_lo, A.c_frac));
-        const int bin = r + A.c_int;
-        if ((unsigned)bin >= (unsigned)A.nbins) {
-            hist_outside(A, H, (double)amp / lift, E);
+        const int bin = r + A.c_int - bin0;
+        if ((unsigned)bin >= (unsigned)nb) {
+            if (!HALF || (!upper && (unsigned)bin >= (unsigned)A.nbins)) hist_outside(A, H, (double)amp / lift, E);
             return;
         }
         const unsigned h = hbase + 4u * (unsigned)bin;
@@ -1468,7 +1472,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     if (one_pass) stage(0, P);
 
     const int nblk = (M + HF_THR * HF_QPT - 1) / (HF_THR * HF_QPT);
-    for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    for (int blk = HALF ? blockIdx.x >> 1 : blockIdx.x; blk < nblk; blk += HALF ? gridDim.x >> 1 : gridDim.x) {
         float2 cq[HF_QPT], sq[HF_QPT];
         float fqp[HF_QPT], fcqp[HF_QPT], v2[HF_QPT], vab[HF_QPT], xqk[HF_QPT], ga[HF_QPT], gb[HF_QPT], gc[HF_QPT];
         int qi[HF_QPT], qx[HF_QPT], qy[HF_QPT];
@@ -1647,22 +1651,22 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
             // without the second word the rounding of moment 0 is kept small by
             // flushing after every pass
             if (!LO || p0 + HF_REC >= P) {
-                for (int i = tid; i < A.nbins; i += HF_THR) {
+                for (int i = tid; i < nb; i += HF_THR) {
                     const int v = hs[i], lo = LO ? hs[5 * NBS + i] : 0;
                     if (v == 0 && lo == 0) continue;
                     hs[i] = 0;
                     if (LO) hs[5 * NBS + i] = 0;
-                    atomicAdd(&H[i], unit * (double)v + unit_lo * (double)lo);
+                    atomicAdd(&H[bin0 + i], unit * (double)v + unit_lo * (double)lo);
                 }
                 float mom = scale > 0.f ? 1.f / scale : 0.f;     // (h/2)^moment per lifted unit
                 for (int mo = 1; mo < 5; ++mo) {
                     mom *= 0.5f * A.h;
-                    for (int i = tid; i < A.nbins; i += HF_THR) {
+                    for (int i = tid; i < nb; i += HF_THR) {
                         const int v = hs[mo * NBS + i];
                         if (v == 0) continue;
                         hs[mo * NBS + i] = 0;
                         const double x = (double)((float)v * mom);
-                        atomicAdd(&H[(long)mo * A.nbins + i], lift == 1.f ? x : x / (double)lift);
+                        atomicAdd(&H[(long)mo * A.nbins + bin0 + i], lift == 1.f ? x : x / (double)lift);
                     }
                 }
                 __syncthreads();
@@ -2187,16 +2191,16 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     return e == cudaSuccess ? QPFRG_OK : cuda_fail(c, e, "sigma_fast_kernel");
 }
 
-// Words per moment of the frequency-grid histogram and whether moment 0 has a
-// second word: the smallest that holds the bins beside the projection table.
-// 227 KB of shared memory hold 6 x 5952 words or 5 x 6880.
-constexpr int kHfBins[3] = {4864, 5952, 6880};
+// Words per moment of the frequency-grid histogram: 227 KB of shared memory hold,
+// beside the projection table, 6 x 5952 (a second word of moment 0) or 5 x 7136.
+// More bins than that: two halves of 6 words each, which walk the pairs twice.
+constexpr int kHfBins = 5952, kHfBinsOne = 7136;
+static_assert(hf_smem_layout(kHfBins, true).total + 64 <= 227 * 1024 &&
+                  hf_smem_layout(kHfBinsOne, false).total + 64 <= 227 * 1024, "shared memory of the histogram");
 
 static int hist_variant(int nbins)
 {
-    for (int v = 0; v < 3; ++v)
-        if (nbins <= kHfBins[v]) return v;
-    return -1;
+    return nbins <= kHfBins ? 0 : (nbins <= kHfBinsOne ? 1 : (nbins <= 2 * kHfBins ? 2 : -1));
 }
 
 // Binned pole density of the target slots into hist (FP32, wedge grid).
@@ -2219,11 +2223,11 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     A.h64 = h;
     using Kern = void (*)(SigmaFastArgs);
     static const Kern table[3][2] = {
-        {sigma_hist_kernel<kHfBins[0], true, false>, sigma_hist_kernel<kHfBins[0], true, true>},
-        {sigma_hist_kernel<kHfBins[1], true, false>, sigma_hist_kernel<kHfBins[1], true, true>},
-        {sigma_hist_kernel<kHfBins[2], false, false>, sigma_hist_kernel<kHfBins[2], false, true>}};
+        {sigma_hist_kernel<kHfBins, true, false, false>, sigma_hist_kernel<kHfBins, true, true, false>},
+        {sigma_hist_kernel<kHfBinsOne, false, false, false>, sigma_hist_kernel<kHfBinsOne, false, true, false>},
+        {sigma_hist_kernel<kHfBins, true, false, true>, sigma_hist_kernel<kHfBins, true, true, true>}};
     const Kern kern = table[v][d_K ? 1 : 0];
-    const size_t smem = hf_smem_layout(kHfBins[v], v < 2).total;
+    const size_t smem = v == 1 ? hf_smem_layout(kHfBinsOne, false).total : hf_smem_layout(kHfBins, true).total;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(c, e, "sigma_hist smem attribute");
     // one CTA per SM: split the q blocks until there are eight waves of the
@@ -2232,7 +2236,8 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     const long per = (long)N * (tg.jlist ? tg.n : nj);
     const int split = (int)std::max<long>(1, std::min<long>(nqb, (8 * 152 + per - 1) / per));
     prof_begin(c);
-    kern<<<dim3(split, N, nj), HF_THR, smem, c->stream>>>(A);
+    const int halves = v == 2 ? 2 : 1;
+    kern<<<dim3(split * halves, N, nj), HF_THR, smem, c->stream>>>(A);
     if (tg.sym.mode == 2) {
         sigma_fix_kernel<<<152, 128, 0, c->stream>>>(A, hist);
         // the images' own sums, should the record have run over
@@ -2241,7 +2246,7 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
         F.jlist = tg.jlist + tg.n;
         F.hist = hist + (long)tg.n * 5 * nbins;
         F.sym = SymMode();
-        if (N > tg.n) kern<<<dim3(1, N, N - tg.n), HF_THR, smem, c->stream>>>(F);
+        if (N > tg.n) kern<<<dim3(halves, N, N - tg.n), HF_THR, smem, c->stream>>>(F);
     }
     prof_end(c, K_SIGMA_HIST);
     e = cudaGetLastError();

@@ -17,9 +17,9 @@ GEO = [(12, 4, 4, 0.0, 0), (20, 4, 4, 0.0, 0), (16, 5, 4, 0.0, 0), (12, 5, 4, 0.
        (8, 5, 4, -0.2, 1), (48, 5, 4, 0.0, 0), (16, 8, 6, 0.0, 0)]
 
 
-def sigma(N, nt, nr, tp, prop, prec, V, Z, T, w):
+def sigma(N, nt, nr, tp, prop, prec, V, Z, T, w, eta=0.05):
     import torch
-    with api.Context(N, nt, nr, U=2.0, tp=tp, precision=prec, propagator=prop, eta=0.05, n_omega=len(w), omega_min=w[0],
+    with api.Context(N, nt, nr, U=2.0, tp=tp, precision=prec, propagator=prop, eta=eta, n_omega=len(w), omega_min=w[0],
                      omega_max=w[-1]) as c:
         re, im = (torch.full((N, len(w)), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2))
         api.qpfrg_selfenergy(c.h, T, torch.from_numpy(V.ravel()).cuda(), torch.from_numpy(Z).cuda(), re, im, None)
