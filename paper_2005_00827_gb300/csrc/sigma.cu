@@ -516,6 +516,7 @@ struct SigmaFastArgs {
     double T64;
     double fold0, fold1;    // last doubles k with rint(k / 2 pi) = 0 and < 2
     double dth64;           // 2 pi / N
+    int sub0;               // records of a pass's first chunk (queue of guarded pairs)
     const float4 *kp, *kcs, *bnd;
     const int2 *kfx, *pfx;  // k_j + p and the fine points in fixed point
     const uint8_t *ptab;
@@ -1118,11 +1119,12 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             // the loop is unrolled four times (eight records per trip, 122
             // registers: the loop overhead amortised, more independent work).
             // The queue is settled after a chunk of records that leaves it a quarter
-            // full, and at the end of the pass.  A chunk is 16 records, then four times
+            // full, and at the end of the pass.  The first chunk is 16 records, or 256
+            // where boundary pairs are known to be few (sigma_plan), the next four times
             // the last while few pairs are queued: where the lattice's mirror lies on a
             // boundary (N = 4 mod 8) up to 6 % of the pairs are exact ties, which a queue
             // per pass could not hold: N = 60, 10 x 14 points, 55 ms against 8.5 without.
-            int sub = 16, kept = 0, settled = 0;
+            int sub = A.sub0, kept = 0, settled = 0;
             for (int i0 = 0; i0 < cnt;) {
             const int i1 = min(cnt, i0 + sub);
 #pragma unroll 4
@@ -1546,7 +1548,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                 __syncthreads();
             }
             // the queue is settled in chunks, as in sigma_fast_kernel
-            int sub = 8, kept = 0, settled = 0;
+            int sub = A.sub0 / 2, kept = 0, settled = 0;
             for (int i0 = 0; i0 < cnt;) {
             const int i1 = min(cnt, i0 + sub);
 #pragma unroll 2
@@ -2074,6 +2076,7 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     A.fold0 = fold0;
     A.fold1 = fold1;
     A.dth64 = kTwoPi / c->pb.N;
+    A.sub0 = c->max_events > 0 ? 256 : 16;
     return A;
 }
 
