@@ -258,6 +258,7 @@ def run_qpfrg(args):
     # launch shapes measured on this context's own state (untimed)
     tuning = api.qpfrg_autotune(ctx.h, 1.0) if not args.no_autotune else None
     work = api.qpfrg_rhs_work(ctx.h)
+    evaluated = api.qpfrg_rhs_evaluated(ctx.h)
     for _ in range(args.warmup):
         api.qpfrg_step(ctx.h, 1)
     barrier()
@@ -368,7 +369,7 @@ def run_qpfrg(args):
     roof = None
     if dom in ("bubble", "sigma_z"):
         if dom == "bubble":
-            units = bubble_units(N, M, work["loop_evals"])
+            units = bubble_units(N, M, evaluated["loop_evals"])
             fp32, ex2, rcp = BUBBLE_FP32_PER_EVAL, BUBBLE_EX2_PER_EVAL, BUBBLE_RCP_PER_EVAL
             built = BUBBLE_ISSUE_AS_BUILT
         else:
@@ -393,7 +394,7 @@ def run_qpfrg(args):
     rhs_roof = {}
     if "bubble" in kern:
         evals = 2.0 * N * N * M
-        red = bubble_units(N, M, work["loop_evals"])
+        red = bubble_units(N, M, evaluated["loop_evals"])
         b_s = kern["bubble"][0] / kern["bubble"][1] / 1e3
         b_peak = N_SM * clk_mhz * 1e6 / alu_clk_per_unit(BUBBLE_FP32_PER_EVAL, BUBBLE_EX2_PER_EVAL,
                                                           BUBBLE_RCP_PER_EVAL, rates)
@@ -403,14 +404,15 @@ def run_qpfrg(args):
     tc = [k for k in ("tc_fused_pp", "tc_fused_cr", "tc_fused_d") if k in kern]
     if len(tc) == 3:
         # The channel GEMMs stream the FP32 weighted table: pp its pp family
-        # (R rows of N^2 floats), cr the ph family, d the ph family twice
-        # (K = 2 N^2): 16 R N^2 bytes per RHS, against the HBM copy peak.  On
+        # (T rows of N^2 floats), cr the ph family, d the ph family twice
+        # (K = 2 N^2): 16 T N^2 bytes per RHS, against the HBM copy peak.  On
         # the tensor cores: three BF16 products (hi hi, hi lo, lo hi) of R rows,
         # N columns and K = N^2 (pp, cr) + 2 N^2 (d): 24 R N^3 flop per RHS.
-        # R = N^2, or the row orbits of a C4v-symmetric state (their table,
-        # written by the loop kernels just before, mostly stays in L2).
+        # R = T = N^2, or the row orbits of a C4v-symmetric state, of which two share
+        # a table row where an exchange of the pair leads to another orbit (their
+        # table, written by the loop kernels just before, mostly stays in L2).
         R = float(work.get("contraction_rows") or N * N)
-        nbytes, flop = 16.0 * R * N ** 2, 24.0 * R * N ** 3
+        nbytes, flop = 16.0 * evaluated["table_rows"] * N ** 2, 24.0 * R * N ** 3
         t_s = sum(kern[k][0] / kern[k][1] for k in tc) / 1e3
         bf16 = float(peaks.get("bf16_tflops", 1900.0))
         rhs_roof["tc_fused"] = {"bound": "hbm", "achieved": nbytes / t_s / 1e9, "peak": hbm, "unit": "GB/s",
@@ -432,7 +434,7 @@ def run_qpfrg(args):
                    "precision": args.precision, "l2": "inputs larger than L2 (partner maps "
                    f"{2 * N * N * M / 1e9:.2f} GB, bubble tables)", "parallelism": "replicas",
                    "tuning": tuning},
-        "e2e": e2e, "gpu_launches": int(sum(v[1] for v in prof.values())), "rhs_work": work,
+        "e2e": e2e, "gpu_launches": int(sum(v[1] for v in prof.values())), "rhs_work": {**work, "evaluated": evaluated},
         "sigma_table_bytes": table_bytes,
         "kernels_ms": {k: round(v[0], 3) for k, v in kern.items()},
         "kernel_launches": {k: v[1] for k, v in kern.items()},

@@ -350,8 +350,9 @@ qpfrg_status qpfrg_profile_get(qpfrg_t ctx, int id, double *ms, long long *launc
  * and (y, x) of the particle-particle family, and (x, y) and (y', x') of the
  * particle-hole family, x' opposite to x, have the same transfer momentum:
  * their rows of the table are the same and are evaluated once.
- *   loop_evals: loop-kernel evaluations of the context's last RHS, a row of
- *     the table that two contraction rows share counted for each of them;
+ *   loop_evals: loop-kernel evaluations that the contraction rows of the
+ *     context's last RHS stand for: a row of the table that two of them share
+ *     counts for each (qpfrg_rhs_evaluated counts it once);
  *   loop_evals_full: 2 N^2 M, the evaluations of the unreduced RHS;
  *   rows_unreduced: rows evaluated by themselves because the covariance check
  *     failed for them;
@@ -362,6 +363,13 @@ qpfrg_status qpfrg_profile_get(qpfrg_t ctx, int id, double *ms, long long *launc
  * reduction is off (lattice mode, no_loop_symmetry). */
 qpfrg_status qpfrg_rhs_work(qpfrg_t ctx, long long *loop_evals, long long *loop_evals_full,
                             long long *rows_unreduced, long long *contraction_rows);
+
+/* What the last RHS computed, each row once (outputs may be NULL; waits as
+ * qpfrg_rhs_work):
+ *   loop_evals: loop-kernel evaluations of one RHS;
+ *   table_rows: rows of the loop-kernel table per family that the contraction
+ *     reads (N^2, or one per orbit of transfer pairs under C4v and exchange). */
+qpfrg_status qpfrg_rhs_evaluated(qpfrg_t ctx, long long *loop_evals, long long *table_rows);
 
 /* The patch-of-r table of the flow's self-energy (options.sigma_table),
  * for verification: *bytes = its size (0 while not built: it is built by the

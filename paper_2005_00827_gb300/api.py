@@ -32,6 +32,7 @@ EXPORTS = (
     "qpfrg_geometry", "qpfrg_set_profiling", "qpfrg_profile_reset", "qpfrg_profile_count",
     "qpfrg_profile_name", "qpfrg_profile_get", "qpfrg_last_error", "qpfrg_version", "qpfrg_destroy",
     "qpfrg_zfactor_static", "qpfrg_flow_batch", "qpfrg_autotune", "qpfrg_set_tuning", "qpfrg_rhs_work",
+    "qpfrg_rhs_evaluated",
     "qpfrg_spectral", "qpfrg_read_sigma_flow", "qpfrg_sigma_table", "qpfrg_alu_rates",
 )
 
@@ -146,6 +147,8 @@ def load(build_if_missing: bool = True):
     L.qpfrg_sigma_table.argtypes = [_P, C.POINTER(C.c_size_t), C.c_longlong, C.c_longlong, _P]
     L.qpfrg_sigma_table.restype = C.c_int
     L.qpfrg_rhs_work.restype = C.c_int
+    L.qpfrg_rhs_evaluated.argtypes = [_P] + [C.POINTER(C.c_longlong)] * 2
+    L.qpfrg_rhs_evaluated.restype = C.c_int
     L.qpfrg_destroy.argtypes = [_P]
     L.qpfrg_destroy.restype = None
     for name in ("qpfrg_create", "qpfrg_rhs", "qpfrg_selfenergy", "qpfrg_step", "qpfrg_flow",
@@ -320,12 +323,20 @@ def qpfrg_read_sigma_flow(ctx, slopes, sigma, zka):
 
 
 def qpfrg_rhs_work(ctx) -> dict:
-    """Loop-kernel evaluations of the last RHS (C4v-reduced) and of the full
+    """Loop-kernel evaluations that the rows of the last RHS stand for and of the full
     one, the rows evaluated by themselves because their partner maps broke
     covariance, and the rows of each channel GEMM (N^2, or the row orbits)."""
     a, b, r, m = C.c_longlong(), C.c_longlong(), C.c_longlong(), C.c_longlong()
     _check(ctx, load().qpfrg_rhs_work(ctx, C.byref(a), C.byref(b), C.byref(r), C.byref(m)))
     return dict(loop_evals=a.value, loop_evals_full=b.value, rows_unreduced=r.value, contraction_rows=m.value)
+
+
+def qpfrg_rhs_evaluated(ctx) -> dict:
+    """Loop-kernel evaluations of the last RHS and rows of its table per family,
+    each counted once."""
+    a, b = C.c_longlong(), C.c_longlong()
+    _check(ctx, load().qpfrg_rhs_evaluated(ctx, C.byref(a), C.byref(b)))
+    return dict(loop_evals=a.value, table_rows=b.value)
 
 
 def qpfrg_sigma_table(ctx, offset=0, count=0):

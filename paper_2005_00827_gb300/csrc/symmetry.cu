@@ -426,11 +426,9 @@ extern "C" qpfrg_status qpfrg_sigma_table(qpfrg_t c, size_t *bytes, long long of
     return e == cudaSuccess ? QPFRG_OK : qpfrg::cuda_fail(c, e, "qpfrg_sigma_table");
 }
 
-extern "C" qpfrg_status qpfrg_rhs_work(qpfrg_t c, long long *loop_evals, long long *loop_evals_full,
-                                       long long *rows_unreduced, long long *contraction_rows)
+// c->rows_compact of the last RHS
+static qpfrg_status read_form(qpfrg_ctx *c)
 {
-    if (!c) return QPFRG_ERR_INVALID;
-    const long long full = 2LL * c->pb.N * c->pb.N * c->pb.M;
     if (c->rhs_sym.mode == 2) {     // the form was decided on the device: read the test
         double r[4];
         cudaError_t e = cudaMemcpyAsync(r, c->d_sym, sizeof(r), cudaMemcpyDeviceToHost, c->stream);
@@ -439,6 +437,27 @@ extern "C" qpfrg_status qpfrg_rhs_work(qpfrg_t c, long long *loop_evals, long lo
         const double tol = c->rhs_sym.tol;
         c->rows_compact = r[1] <= tol * r[0] && r[3] <= tol * r[2];
     }
+    return QPFRG_OK;
+}
+
+extern "C" qpfrg_status qpfrg_rhs_evaluated(qpfrg_t c, long long *loop_evals, long long *table_rows)
+{
+    if (!c) return QPFRG_ERR_INVALID;
+    const qpfrg_status s = read_form(c);
+    if (s != QPFRG_OK) return s;
+    const long long NN = (long long)c->pb.N * c->pb.N, rows = c->rows_compact ? c->n_rcan : NN;
+    if (table_rows) *table_rows = rows;
+    if (loop_evals) *loop_evals = !c->rows_compact && c->loop_red ? c->loop_evals_red : 2 * rows * c->pb.M;
+    return QPFRG_OK;
+}
+
+extern "C" qpfrg_status qpfrg_rhs_work(qpfrg_t c, long long *loop_evals, long long *loop_evals_full,
+                                       long long *rows_unreduced, long long *contraction_rows)
+{
+    if (!c) return QPFRG_ERR_INVALID;
+    const long long full = 2LL * c->pb.N * c->pb.N * c->pb.M;
+    const qpfrg_status s = read_form(c);
+    if (s != QPFRG_OK) return s;
     if (loop_evals) *loop_evals = c->rows_compact ? c->loop_evals_rows : (c->loop_red ? c->loop_evals_red : full);
     if (loop_evals_full) *loop_evals_full = full;
     if (rows_unreduced) *rows_unreduced = c->loop_red ? c->loop_mismatch_rows : 0;
