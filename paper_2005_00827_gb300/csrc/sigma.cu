@@ -20,6 +20,7 @@
 // and Z keep the lattice symmetry), of a given vertex the targets that a C4v
 // test on the device admits; Z is copied to their images.
 #include <algorithm>
+#include <cstdlib>
 
 #include "atan_poly.h"
 #include "qpfrg_internal.h"
@@ -517,6 +518,7 @@ struct SigmaFastArgs {
     double fold0, fold1;    // last doubles k with rint(k / 2 pi) = 0 and < 2
     double dth64;           // 2 pi / N
     int sub0;               // records of a pass's first chunk (queue of guarded pairs)
+    int qcap;               // guarded pairs that the queue holds
     const float4 *kp, *kcs, *bnd;
     const int2 *kfx, *pfx;  // k_j + p and the fine points in fixed point
     const uint8_t *ptab;
@@ -1165,7 +1167,7 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
                         const int rec = i + (r1 ? 1 : 0);
                         if (mine && slow && rec < cnt) {     // (the pad record has weight 0)
                             const int at = atomicAdd(&s_nq, 1);
-                            if (at < SF_QCAP) queue[at] = (unsigned)rec | (unsigned)((k1 ? 256 : 0) + tid) << 12;
+                            if (at < A.qcap) queue[at] = (unsigned)rec | (unsigned)((k1 ? 256 : 0) + tid) << 12;
                         }
                         __syncwarp();
                         if (mine && !r1 && !k1) c[0][0] = cc;
@@ -1182,12 +1184,12 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             const int nq = s_nq;
             __syncthreads();
             const int added = nq - kept, nrec = i1 - settled;
-            sub = added > SF_QCAP / 4 ? max(16, sub / 4) : (added < 16 ? min(SF_PCH, 4 * sub) : sub);
+            sub = added > A.qcap / 4 ? max(16, sub / 4) : (added < 16 ? min(SF_PCH, 4 * sub) : sub);
             kept = nq;
             i0 = i1;
-            if (i1 < cnt && nq <= SF_QCAP / 4) continue;     // uniform over the CTA
+            if (i1 < cnt && nq <= A.qcap / 4) continue;     // uniform over the CTA
             if (tid == 0) s_nq = 0;
-            const bool over = nq > SF_QCAP;      // more than the queue holds: look at every pair again
+            const bool over = nq > A.qcap;      // more than the queue holds: look at every pair again
             const int ntot = over ? nrec * (256 * SF_QPT) : nq;
             for (int e = tid; e < ntot; e += 256) {
                 const unsigned en = over ? (unsigned)(settled + e % nrec) | (unsigned)(e / nrec) << 12 : queue[e];
@@ -1570,7 +1572,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
                         if (slow[k]) c[k] = cc;
                         if (slow[k] && still) {       // queued; the table's patch until the pass ends
                             const int at = atomicAdd(&s_nq, 1);
-                            if (at < HF_QCAP) queue[at] = (unsigned)i | (unsigned)(k * HF_THR + tid) << 12;
+                            if (at < A.qcap) queue[at] = (unsigned)i | (unsigned)(k * HF_THR + tid) << 12;
                         }
                         __syncwarp();
                     }
@@ -1596,12 +1598,12 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
             const int nq = s_nq;
             __syncthreads();
             const int added = nq - kept, nrec = i1 - settled;
-            sub = added > HF_QCAP / 4 ? max(8, sub / 4) : (added < 16 ? 4 * sub : sub);
+            sub = added > A.qcap / 4 ? max(8, sub / 4) : (added < 16 ? 4 * sub : sub);
             kept = nq;
             i0 = i1;
-            if (i1 < cnt && nq <= HF_QCAP / 4) continue;     // uniform over the CTA
+            if (i1 < cnt && nq <= A.qcap / 4) continue;     // uniform over the CTA
             if (tid == 0) s_nq = 0;
-            const bool over = nq > HF_QCAP;      // more than the queue holds: look at every pair again
+            const bool over = nq > A.qcap;      // more than the queue holds: look at every pair again
             const int ntot = over ? nrec * (HF_THR * HF_QPT) : nq;
             for (int e = tid; e < ntot; e += HF_THR) {
                 const unsigned en = over ? (unsigned)(settled + e % nrec) | (unsigned)(e / nrec) << 12 : queue[e];
@@ -2023,6 +2025,13 @@ static double fold_limit(int n)
     return k;
 }
 
+// A smaller capacity for tests of what happens when it is exceeded.
+static int test_limit(const char *name, int given)
+{
+    const char *s = std::getenv(name);
+    return s ? std::min(given, std::max(0, std::atoi(s))) : given;
+}
+
 static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const double *d_Z, const double *d_K,
                                const SigmaTargets &tg)
 {
@@ -2077,6 +2086,7 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     A.fold1 = fold1;
     A.dth64 = kTwoPi / c->pb.N;
     A.sub0 = c->max_events > 0 ? 256 : 16;
+    A.qcap = test_limit("QPFRG_TEST_QUEUE", 1 << 20);
     return A;
 }
 
@@ -2114,7 +2124,7 @@ qpfrg_status sigma_plan(qpfrg_ctx *c)
     if (pairs * worth > (c->pb.N - c->n_grid) * M * M) return QPFRG_OK;
     if ((e = cudaMalloc((void **)&c->d_events, (size_t)cap * sizeof(int4))) != cudaSuccess)
         return cuda_fail(c, e, "cudaMalloc(boundary pairs)");
-    c->max_events = (unsigned)cap;
+    c->max_events = (unsigned)std::max(1, test_limit("QPFRG_TEST_BOUNDARY_PAIRS", (int)cap));
     return QPFRG_OK;
 }
 
@@ -2129,6 +2139,7 @@ static qpfrg_status launch_sigma_fast(qpfrg_ctx *c, double T, const double *d_V,
     qpfrg_status s = launch_kp_table(c, tg.sym.mode == 2 ? nullptr : tg.jlist, nj, !(listed && c->d_rtab));
     if (s != QPFRG_OK) return s;
     SigmaFastArgs A = fast_args(c, T, d_V, d_Z, d_K, tg);
+    A.qcap = std::min(A.qcap, SF_QCAP);
     const bool unib = c->pb.P % (256 * SF_QPT) == 0;
     // The flow's Z on the C4v-irreducible targets reads the patches of r from
     // a table built on first use (one byte per target, p and q: N_irr M^2
@@ -2214,6 +2225,7 @@ static qpfrg_status launch_sigma_hist(qpfrg_ctx *c, double T, const double *d_V,
     qpfrg_status s = launch_kp_table(c, tg.sym.mode == 2 ? nullptr : tg.jlist, nj);
     if (s != QPFRG_OK) return s;
     SigmaFastArgs A = fast_args(c, T, d_V, d_Z, d_K, tg);
+    A.qcap = std::min(A.qcap, HF_QCAP);
     A.hist = hist;
     const double c0 = -e_min / h - 0.5;      // bin centre b at e_min + (b + 1/2) h
     A.c_int = (int)std::rint(c0);
