@@ -325,7 +325,9 @@ qpfrg_status qpfrg_geometry(qpfrg_t ctx, int *n_p, int *n_fine, double *h_kf, do
 /* Kernel timing with CUDA events on the context's stream (off by default).
  * qpfrg_profile_get returns the accumulated device milliseconds and launch
  * count of kernel id (0 <= id < qpfrg_profile_count()); names via
- * qpfrg_profile_name.  qpfrg_profile_reset clears the counters. */
+ * qpfrg_profile_name (the FP64 and FP32 contraction is one launch for all
+ * channels, counted as contract_pp; contract_cr and contract_d stay 0).
+ * qpfrg_profile_reset clears the counters. */
 qpfrg_status qpfrg_set_profiling(qpfrg_t ctx, int on);
 qpfrg_status qpfrg_profile_reset(qpfrg_t ctx);
 int          qpfrg_profile_count(void);

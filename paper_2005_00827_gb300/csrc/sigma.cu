@@ -540,7 +540,7 @@ struct SigmaFastArgs {
     unsigned *nevents, max_events;
     bool only_full;
     double *corr;
-    float t, tp, mu, eta2, invT, cT, twoT, fourT;   // cT = log2(e) / T
+    float t, tp, mu, invT, cT;                      // cT = log2(e) / T
     float tln2, kchord, eta2x4;                     // T ln 2, 4 T^2 + eta^2, 4 eta^2
     float inv_dth, dth;                             // N / 2 pi, 2 pi / N
     int mirror;     // n_theta even and symmetric targets: halve the mirror-line targets
@@ -1000,7 +1000,7 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
         float fqp[SF_QPT], fcqp[SF_QPT], v2[SF_QPT], vab[SF_QPT], mxq[SF_QPT];
         float2 acc = make_float2(0.f, 0.f);     // the SF_QPT = 2 loop points as the two lanes
         float ga[SF_QPT], gb[SF_QPT], gc[SF_QPT];   // GL: bracket = ga + gb Z_c + gc K_c Z_c
-        int qi[SF_QPT], qx[SF_QPT], qy[SF_QPT];
+        int qx[SF_QPT], qy[SF_QPT];
         const uint8_t *rq[SF_QPT];   // RT: the patch-of-r rows of this thread's loop points q
 #pragma unroll
         for (int k = 0; k < SF_QPT; ++k) {
@@ -1010,7 +1010,6 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
             rq[k] = RT ? A.rtab + (((long)jidx * N + a) * (long)(PP / 8) * M + ii) * 8 : nullptr;
             const int b = ii / PP, rem = ii - b * PP;
             const int qq = b * PP + (rem % A.pb.n_theta) * A.pb.n_r + rem / A.pb.n_theta;
-            qi[k] = qq;
             const float Zb = A.Z ? (float)A.Z[b] : 1.f;
             qx[k] = A.pfx[qq].x;
             qy[k] = A.pfx[qq].y;
@@ -1479,7 +1478,7 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
     for (int blk = HALF ? blockIdx.x >> 1 : blockIdx.x; blk < nblk; blk += HALF ? gridDim.x >> 1 : gridDim.x) {
         float2 cq[HF_QPT], sq[HF_QPT];
         float fqp[HF_QPT], fcqp[HF_QPT], v2[HF_QPT], vab[HF_QPT], xqk[HF_QPT], ga[HF_QPT], gb[HF_QPT], gc[HF_QPT];
-        int qi[HF_QPT], qx[HF_QPT], qy[HF_QPT];
+        int qx[HF_QPT], qy[HF_QPT];
         if (tid < 3) s_blk[tid] = 0.f;
         __syncthreads();
         float t1 = 0.f, t2 = 0.f, t3 = 0.f;      // sums and maximum of the weights of this thread's q
@@ -1489,7 +1488,6 @@ __global__ void __launch_bounds__(HF_THR, 1) sigma_hist_kernel(const SigmaFastAr
             const bool valid = iq < M;
             const int qq = valid ? iq : M - 1;
             const int b = qq / PP;
-            qi[k] = qq;
             const float Zb = A.Z ? (float)A.Z[b] : 1.f;
             qx[k] = A.pfx[qq].x;
             qy[k] = A.pfx[qq].y;
@@ -2066,11 +2064,8 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
     A.t = (float)c->pb.t;
     A.tp = (float)c->pb.tp;
     A.mu = (float)c->pb.mu;
-    A.eta2 = (float)(c->pb.eta * c->pb.eta);
     A.invT = (float)(1.0 / T);
     A.cT = (float)(1.4426950408889634 / T);
-    A.twoT = (float)(2.0 * T);
-    A.fourT = (float)(4.0 * T);
     A.tln2 = (float)(0.6931471805599453 * T);
     A.kchord = (float)(4.0 * T * T + c->pb.eta * c->pb.eta);
     A.eta2x4 = (float)(4.0 * c->pb.eta * c->pb.eta);
