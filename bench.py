@@ -58,11 +58,11 @@ SIGMA_FP32_PER_PAIR, SIGMA_EX2_PER_PAIR, SIGMA_RCP_PER_PAIR = 20, 1, 3
 # FP32x2 instruction counts one half per pair); the loop kernels' measured
 # instructions per computed evaluation on the representative rows of the row
 # orbits (ncu smsp__inst_executed x 32 / evaluations at np96_n32:
-# 3.29e8 x 32 / 2.27e8)
-BUBBLE_ISSUE_AS_BUILT, SIGMA_ISSUE_AS_BUILT = 46.4, 36
+# 1.778e8 x 32 / 1.205e8)
+BUBBLE_ISSUE_AS_BUILT, SIGMA_ISSUE_AS_BUILT = 47.2, 36
 # the self-energy pair with its patch read from the patch-of-r table: measured
 # instructions per pair (ncu smsp__inst_executed x 32 / pairs at np48_n16:
-# 7.03e8 x 32 / 9.06e8)
+# 7.02e8 x 32 / 9.06e8)
 SIGMA_ISSUE_AS_BUILT_TABLE = 24.8
 ISSUE_LANES_PER_SM, NOMINAL_MUFU_PER_SM, N_SM = 128, 16, 152
 
@@ -117,12 +117,12 @@ def cpu_info():
 # SHA-256 of that text is recorded with the capture; profiles/ holds the summary.
 TRAFFIC = {
     # the kernel with its patch-of-r table: DRAM bytes per (p, q) pair from a
-    # full capture at np48_n16 (907.7 MB read + 3.3 MB written for 9.06e8
-    # pairs: 1.0055 B per pair, the table's byte), scaled to the bench
+    # full capture at np48_n16 (906.5 MB read + 3.1 MB written for 9.06e8
+    # pairs: 1.0040 B per pair, the table's byte), scaled to the bench
     # workload's pairs (the table grows with the pairs)
-    ("sigma_z", "np96_n32"): {"bytes": 116.61e9, "source": "paper_2005_00827_gb300/csrc/sigma.cu",
+    ("sigma_z", "np96_n32"): {"bytes": 116.43e9, "source": "paper_2005_00827_gb300/csrc/sigma.cu",
                               "kernel": "sigma_fast_kernel", "scaled_from": "np48_n16",
-                              "sha256": "85cf7d0d4dc108c73efa7da72ebd52256686955594627914ddebb3dd2bbc19e1"},
+                              "sha256": "ee4afdb5d4f23edbec985e877a26222eaf08e46dce55c5b16d0e2c3bbe52f072"},
 }
 
 

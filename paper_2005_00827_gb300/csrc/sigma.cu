@@ -2091,7 +2091,7 @@ static SigmaFastArgs fast_args(qpfrg_ctx *c, double T, const double *d_V, const 
 // the record of pairs is sized for them.  Generic grids have few; with N = 4 mod 8, mu
 // and t' = 0 the lattice's mirror is a boundary between wedges and up to 6 % of the
 // pairs lie on it: every patch is summed.  Counted where there are at most 2^22 pairs,
-// else estimated from a sample (0.1 % of 2^22 to 1.5 %).
+// else estimated from a sample.
 qpfrg_status sigma_plan(qpfrg_ctx *c)
 {
     c->max_events = 0;
@@ -2115,8 +2115,10 @@ qpfrg_status sigma_plan(qpfrg_ctx *c)
         (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "boundary pairs");
     const double pairs = found * (all / n), worth = c->opt.precision == QPFRG_FP64 ? 170.0 : 3600.0;
-    const double cap = std::fmin(1.25 * pairs + 4096.0, 2097152.0);
-    if (pairs * worth > (c->pb.N - c->n_grid) * M * M) return QPFRG_OK;
+    // room for them, and for what a sample may have missed (np96, 32 x 32 points: some
+    // 1e6 of 1.5e11 pairs are some 30 of the sample): at most 512 MB
+    const double cap = n < all ? (found + 6.0 * std::sqrt((double)found) + 36.0) * (all / n) : pairs + 64.0;
+    if (pairs * worth > (c->pb.N - c->n_grid) * M * M || cap > 33554432.0) return QPFRG_OK;
     if ((e = cudaMalloc((void **)&c->d_events, (size_t)cap * sizeof(int4))) != cudaSuccess)
         return cuda_fail(c, e, "cudaMalloc(boundary pairs)");
     c->max_events = (unsigned)std::max(1, test_limit("QPFRG_TEST_BOUNDARY_PAIRS", (int)cap));

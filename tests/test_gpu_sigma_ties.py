@@ -51,3 +51,24 @@ def test_ties_cost_little(sym):
         V, Z = inputs.random_vertex(N, 2.0, seed=N, c4v=s), inputs.z_profile(N, "aniso")
         per.append(run(N, 8, 8, api.QPFRG_MIXED, V, Z, np.zeros(1), 5)[2] / N ** 3)
     assert per[0] < 3.5 * per[1]
+
+
+def test_reduced_targets_pay_on_the_largest_grid():
+    """96 patches, 32 x 32 points: 16 of 96 targets, a million boundary pairs."""
+    import torch
+    N, ms = 96, {}
+    with api.Context(N, 32, 32, U=2.0, precision=api.QPFRG_MIXED, sigma_table=-1, n_omega=9, omega_min=-3.0,
+                     omega_max=3.0) as c:
+        z, re, im = (torch.zeros(*s, dtype=torch.float64, device="cuda") for s in ((N,), (N, 9), (N, 9)))
+        Z = torch.from_numpy(inputs.z_profile(N, "aniso")).cuda()
+        for sym in (True, False):
+            V = torch.from_numpy(inputs.random_vertex(N, 2.0, seed=N, c4v=sym).ravel()).cuda()
+            for name, args in (("Z", (None, None, z)), ("grid", (re, im, None))):
+                api.qpfrg_selfenergy(c.h, 0.2, V, Z, *args)
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                api.qpfrg_selfenergy(c.h, 0.2, V, Z, *args)
+                b.record()
+                torch.cuda.synchronize()
+                ms[name, sym] = a.elapsed_time(b)
+    assert all(ms[n, True] < 0.3 * ms[n, False] for n in ("Z", "grid"))
