@@ -213,8 +213,10 @@ qpfrg_status qpfrg_rhs(qpfrg_t ctx, double lambda, const double *d_V, const doub
  * FP64 Z 1e-14; FP64 evaluates the grid at every patch): a symmetric input
  * evaluates the targets that differ under C4v, and images whose momenta on a
  * wedge boundary are decided otherwise than their representative's get that
- * difference added.  Regulator must be TEMPERATURE
- * (QPFRG_ERR_UNSUPPORTED otherwise). */
+ * difference added to Z and to the grid.  Where such momenta are so many that this
+ * costs more than it saves (n_p = 4 mod 8 at half filling without t': percents of all
+ * pairs; counted once per context) every patch is evaluated.  Regulator must be
+ * TEMPERATURE (QPFRG_ERR_UNSUPPORTED otherwise). */
 qpfrg_status qpfrg_selfenergy(qpfrg_t ctx, double lambda, const double *d_V, const double *d_Z,
                               double *d_sigma_re, double *d_sigma_im, double *d_Z_out);
 

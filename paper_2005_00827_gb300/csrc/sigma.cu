@@ -18,7 +18,8 @@
 // the vertex row V[j][a][:] in shared memory and loops over them with its q.
 // In the mixed flow the C4v-irreducible patches 0..N/8 are evaluated (the vertex
 // and Z keep the lattice symmetry), of a given vertex the targets that a C4v
-// test on the device admits; Z is copied to their images.
+// test on the device admits; their sums are copied to the images, which decide the
+// pairs on a boundary between patches themselves (sigma_fix_kernel).
 #include <algorithm>
 #include <cstdlib>
 
@@ -1277,8 +1278,8 @@ __global__ void __launch_bounds__(256, 2) sigma_fast_kernel(SigmaFastArgs A)
 // addend stays below 2^21 units (rounded by adding 1.5 * 2^23, no conversion).
 // What moment 0 rounds off goes into a second word (LO) in units 2^30 / pairs
 // finer; the higher moments enter Sigma with (h/2|z - E|)^n <= 8^-n, which
-// carries their rounding below that of the FP32 pairs.  np48, 16 x 16 points, 10 targets, 512 frequencies: 26.0
-// -> 6.4 ms (58 -> 236 Gpair/s).
+// carries their rounding below that of the FP32 pairs.  np48, 16 x 16 points, 10
+// targets, 512 frequencies: 26.0 -> 7.0 ms (58 -> 216 Gpair/s).
 //
 // Launch: grid (q splits, N patches a, targets), 512 threads, one CTA per SM
 // (the histogram).  NBS: words per moment (a constant, so that the moments are
