@@ -267,7 +267,7 @@ __global__ void expand_kernel(const ExpandArgs A)
             long o = (long)Q * N + n;
             if (c) {
                 const int e = __ldg(A.rowmap + (ch == 0 ? 0 : (long)N * N) + Q);
-                o = (long)(e & 0xffffff) * N + c4v_patch(c4v_inverse(e >> 24), n, A.ns, Na);
+                o = (long)(e & 0xfffff) * N + c4v_patch(c4v_inverse(e >> 24), n, A.ns, Na);
             }
             v += __ldg(A.outc + ch * stride + o);
         }
@@ -555,7 +555,8 @@ static qpfrg_status launch_simt(qpfrg_ctx *c, const R *V, double scale, double *
 // so row Q = g rep of a channel at column n is the representative's row at
 // column g^-1 n.  One thread per output triple (k1, k2, k3) adds the three
 // channels' values: pp row (k1, k2) column k3, cr row (k3, k2) column k1,
-// d row (k1, k3) column k2 (the row/column roles of the channel GEMMs above).
+// d row (k1, k3) column k2 (the row/column roles of the channel GEMMs above).  Columns
+// that a mirror of the row exchanges read the lower one (as reduce_kernel).
 // Row (k1, k2) of out, threads over k3.
 __device__ __forceinline__ void expand_row(const double *__restrict__ outc, const int *__restrict__ rowmap, int nr,
                                            int N, int ns, unsigned channels, double *__restrict__ out, int k1, int k2)
@@ -568,8 +569,10 @@ __device__ __forceinline__ void expand_row(const double *__restrict__ outc, cons
     for (int k3 = threadIdx.x; k3 < N; k3 += blockDim.x) {
         double v = 0.0;
         auto take = [&](int ch, int e, int n) {
-            const int m = e & 0xffffff, gi = c4v_inverse(e >> 24);
-            v += __ldg(outc + ch * ch_stride + (long)m * N + c4v_patch(gi, n, ns, Na));
+            const int m = e & 0xfffff, gi = c4v_inverse(e >> 24), s = (e >> 20) & 15;
+            int col = c4v_patch(gi, n, ns, Na);
+            if (s) col = min(col, c4v_patch(s, col, ns, Na));
+            v += __ldg(outc + ch * ch_stride + (long)m * N + col);
         };
         if (channels & QPFRG_CH_PP) take(0, e_pp, k3);
         if (channels & QPFRG_CH_CR) take(1, __ldg(rowmap + k3 * N + k2), k1);
@@ -612,7 +615,7 @@ __global__ void rows_rk_batch_kernel(int stage, TcBatch bt, const int *__restric
         const int Q = __ldg(rep + r), x = Q / N, y = Q - x * N;
         const int *__restrict__ ph = rowmap + N * N;
         auto take = [&](int ch, int e, int col) {
-            return __ldg(outc + (long)ch * per + (long)(e & 0xffffff) * N + c4v_patch(c4v_inverse(e >> 24), col, ns, Na));
+            return __ldg(outc + (long)ch * per + (long)(e & 0xfffff) * N + c4v_patch(c4v_inverse(e >> 24), col, ns, Na));
         };
         const double v = V[i], a0 = stage > 1 ? acc[i] : 0.0;
         double k = 0.0;
@@ -655,7 +658,7 @@ __global__ void vertex_expand_batch_kernel(TcBatch bt, const int *__restrict__ r
     if (t >= N * N * n4) return;
     const int Q = t / n4, k3 = 4 * (t - Q * n4), Na = N / ns;
     const int e = __ldg(rowmap + Q), gi = c4v_inverse(e >> 24);
-    const float *__restrict__ row = Vrs[f] + (long)(e & 0xffffff) * N;
+    const float *__restrict__ row = Vrs[f] + (long)(e & 0xfffff) * N;
     float4 v;
     v.x = row[c4v_patch(gi, k3, ns, Na)];
     v.y = row[c4v_patch(gi, k3 + 1, ns, Na)];

@@ -310,7 +310,7 @@ struct qpfrg_ctx {
     // momentum, same table row (symmetry.cu)
     int n_rrep = 0, n_rcan = 0;
     int *d_rrep = nullptr;       // [family][row]: Q of each representative row
-    int *d_rowmap = nullptr;     // [family][Q]: row | g << 24, Q = g rep
+    int *d_rowmap = nullptr;     // [family][Q]: row | d_rstab << 20 | g << 24, Q = g rep
     uint8_t *d_rstab = nullptr;  // [row]: the mirror (4 .. 7) that leaves its pair in place, 0: none
     int4 *d_rtask = nullptr;     // (family, patch, first representative, count) per loop-kernel CTA
     int rtask_qchunk = 0, n_rtask = 0;

@@ -80,8 +80,8 @@ static void exchange(int f, int N, int ns, int &x, int &y)
     y = f == 0 ? u : c4v_apply(2, u, N, ns);
 }
 
-// Row orbits of the contraction: rowmap[f][Q] = (row | g << 24) with Q = g
-// rrep[f][row].  The first n_rcan rows are one pair of each orbit under C4v and
+// Row orbits of the contraction: rowmap[f][Q] = (row | s << 20 | g << 24) with Q = g
+// rrep[f][row], s the mirror that leaves the row's pair in place (0: none).  The first n_rcan rows are one pair of each orbit under C4v and
 // exchange, the same in both families: the rows of the table, those first whose
 // exchanged pair lies in another C4v orbit.  The others
 // are these exchanged pairs, in the same order: row n_rcan + i holds the table row
@@ -144,6 +144,7 @@ static qpfrg_status build_row_orbits(qpfrg_ctx *c, bool exch, const std::vector<
         for (int g = 4; g < 8 && (m < npar + (int)norb || m >= ncan); ++g)
             if (c4v_apply(g, reps[m] / N, N, ns) == reps[m] / N && c4v_apply(g, reps[m] % N, N, ns) == reps[m] % N)
                 stab[m] = (uint8_t)g;
+    for (int &e : rowmap) e |= stab[e & 0xfffff] << 20;
     cudaError_t e;
     if ((e = cudaMalloc((void **)&c->d_rrep, 2 * (size_t)nr * sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc((void **)&c->d_rstab, nr)) != cudaSuccess ||

@@ -50,6 +50,19 @@ def test_interaction_flow(N, nt, nr, prec):
         assert np.abs(va - vb).max() < 1e-6 * np.abs(va).max()
 
 
+@pytest.mark.parametrize("zfb", [0, 1])
+@pytest.mark.parametrize("N,nt,nr", [(16, 4, 4), (24, 4, 6), (60, 4, 4)])
+def test_tensor_core_flow_keeps_its_symmetry(N, nt, nr, zfb):
+    """To the last bit, whatever the order of its atomic sums; Z of the state then needs
+    the irreducible targets only."""
+    with api.Context(N, nt, nr, U=3.0, lambda0=0.5, precision=api.QPFRG_MIXED_TC, z_feedback=zfb) as c:
+        state, rows = steps(c, 6)[-1]
+    V, Z = state[:N ** 3].reshape(N, N, N), state[N ** 3:]
+    assert rows < N * N
+    for g in map(list, inputs.c4v_patch_maps(N)):
+        assert np.array_equal(V[np.ix_(g, g, g)], V) and np.array_equal(Z[g], Z)
+
+
 @pytest.mark.parametrize("off,sym", [(0.2e-5, True), (0.7e-5, True), (0.95e-5, True), (1.2e-5, False), (4e-5, False)])
 @pytest.mark.parametrize("entry", [(1, 2, 3), (0, 5, 5)])
 def test_image_symmetric_to_the_stated_tolerance(entry, off, sym):
