@@ -954,9 +954,9 @@ qpfrg_status qpfrg_set_state(qpfrg_t c, const void *h_buf, size_t bytes)
     c->c4v_state = sym;
     // The row orbits, as the flow that wrote the image took them: where every stage
     // is tested on the device, left to that test; otherwise a flow's state is
-    // symmetric to the last bit (FP64 and FP32 contraction) or to the tolerance of the
-    // state's symmetry (tensor cores; there the slopes of the self-energy ODE, which set
-    // Z, K and A, to the 1e-4 of that flow).
+    // symmetric to the last bit.  The tensor-core precision takes them for any image that
+    // counts as symmetric (and whose slopes of the self-energy ODE, which set Z, K and A,
+    // are so to the 1e-4 of that flow).
     c->rows_state = c->rows_exact;
     if (c->opt.precision == QPFRG_MIXED_TC)
         c->rows_state = c->rows_exact && c->c4v_state && (!c->d_gy || slopes_symmetric(c, Z + c->pb.N, 1e-4));
